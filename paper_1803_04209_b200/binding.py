@@ -478,8 +478,8 @@ class Fitter:
 
     def capture_elbo_grad(self, xhat, eps):
         """Capture elbo_grad(xhat, eps) in a CUDA graph.  xhat and eps are fixed tensors: the caller refills them (on the
-        current stream) before every replay_elbo_grad().  A step is some 150 small dependent launches, so a replay
-        costs a fraction of launching them one by one."""
+        current stream) before every replay_elbo_grad().  A step is nine dependent launches; a replay takes their launch
+        cost off the host."""
         import torch
         self.elbo_grad(xhat, eps)                      # once outside the capture
         torch.cuda.current_stream().synchronize()

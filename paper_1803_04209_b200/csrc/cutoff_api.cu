@@ -1823,10 +1823,9 @@ int cutoff_elbo_grad(int device, int32_t n_workers, int32_t latent_dim, int32_t 
 int cutoff_adam_step(int device, int64_t n, float* params, const float* grads, float* m, float* v, int32_t t, float lr,
                      float beta1, float beta2, float eps, float clip_norm, float grad_scale, float* norm_out, void* workspace,
                      size_t workspace_bytes, void* stream) {
-    constexpr int kParts = 256;
     if (device < 0 || n < 1 || !params || !grads || !m || !v || t < 1 || !(lr > 0.f) || !(beta1 >= 0.f && beta1 < 1.f) ||
         !(beta2 >= 0.f && beta2 < 1.f) || !(eps > 0.f) || !(clip_norm > 0.f) || !norm_out || !workspace ||
-        workspace_bytes < kParts * sizeof(double))
+        workspace_bytes < fit::kNormParts * sizeof(double))
         return CUTOFF_ERR_BAD_ARG;
     cutoff_ctx* none = nullptr;
     DeviceGuard guard(device);
@@ -1834,12 +1833,12 @@ int cutoff_adam_step(int device, int64_t n, float* params, const float* grads, f
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     double* partial = static_cast<double*>(workspace);
     const int64_t want = (n + fit::kNormThreads - 1) / fit::kNormThreads;
-    const int parts = static_cast<int>(want < kParts ? want : kParts);
+    const int parts = static_cast<int>(want < fit::kNormParts ? want : fit::kNormParts);
     fit::k_sumsq_partial<<<parts, fit::kNormThreads, 0, s>>>(grads, n, grad_scale, partial);
-    fit::k_norm_finish<<<1, 32, 0, s>>>(partial, parts, norm_out);
     const float corr1 = 1.f - std::pow(beta1, static_cast<float>(t)), corr2 = 1.f - std::pow(beta2, static_cast<float>(t));
-    fit::k_adam<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(params, grads, m, v, n, grad_scale, norm_out, clip_norm, lr,
-                                                                      beta1, beta2, eps, corr1, corr2);
+    const int64_t most = 8 * 148;                     // a few CTAs per SM: each adds the partial sums up first
+    fit::k_adam<<<static_cast<unsigned>(want < most ? want : most), fit::kNormThreads, 0, s>>>(
+        params, grads, m, v, n, grad_scale, partial, parts, norm_out, clip_norm, lr, beta1, beta2, eps, corr1, corr2);
     return cudaGetLastError() == cudaSuccess ? CUTOFF_OK : CUTOFF_ERR_CUDA;
 }
 

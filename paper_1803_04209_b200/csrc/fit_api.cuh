@@ -21,165 +21,183 @@ inline Layout layout(long long N, long long D, long long H) {
     return l;
 }
 
-// floats of workspace for a batch of B windows of W vectors
-inline long long workspace_floats(long long N, long long D, long long H, long long W, long long B) {
-    const long long bh = B * H, bd = B * D;
-    return 2 * bh                     // a0, b0 broadcast
-         + 2 * W * bh                 // a, b
-         + (W + 1) * bd               // z (index 0: z0 broadcast)
-         + W * (2 * bh + 4 * bd)      // comb, h_out | mu, pre_sig, sigma, dz of the transition density
-         + W * (2 * bh)               // u, v
-         + W * (B * 2 * D)            // transition head, then its gradient
-         + W * (B * 2 * N)            // emission head, then its gradient
-         + 2 * W * bh                 // g_a, g_b
-         + 3 * bd                     // g_z, g_z_next, g_z_prev
-         + 2 * bd                     // d_mu, d_pre_sig
-         + 4 * bh;                    // pre_c / d_h, d_v / d_u / d_pre_c, d_pre, carry
+inline long long tiles_of(long long n) { return (n + kTile - 1) / kTile; }
+
+// Parts a product's K is split into so that its tiles fill the GPU about twice (a tile of 64 x 64 alone takes
+// K * 32 clocks of an SM), at least 128 long each.
+inline int k_part_of(long long tiles, long long K) {
+    long long parts = (2 * 148 + tiles - 1) / tiles;
+    if (parts > 16) parts = 16;
+    long long len = (K + parts - 1) / parts;
+    if (len < 128) len = 128;
+    return static_cast<int>((len + kTileK - 1) / kTileK * kTileK);
+}
+inline int parts_of(long long K, int k_part) { return static_cast<int>((K + k_part - 1) / k_part); }
+
+// Everything the passes keep, as offsets (floats, multiples of 4) into the workspace.
+struct Workspace {
+    long long proj, a, b, comb, hout, mu, presig, z, u, v, dhz, dzt, path, dhx, part, dv_parts, dv, du, dpc, dh, dmu, dps, gz0,
+        dpf, dpb, ca, cb, total;
+    int proj_k, proj_parts, dv_k, dv_parts_n;
+};
+
+inline Workspace workspace(long long N, long long D, long long H, long long W, long long B) {
+    const long long R = B * W, rh = R * H, rd = R * D, sh = B * (W + 1) * H, sd = B * (W + 1) * D;
+    Workspace w;
+    w.proj_k = k_part_of(tiles_of(R) * 2 * tiles_of(H), N);
+    w.proj_parts = parts_of(N, w.proj_k);
+    w.dv_k = k_part_of(tiles_of(R) * tiles_of(H), 2 * N);
+    w.dv_parts_n = parts_of(2 * N, w.dv_k);
+    long long o = 0;
+    const auto take = [&](long long n) { const long long r = o; o += (n + 3) / 4 * 4; return r; };
+    w.proj = take(w.proj_parts * 2 * rh);
+    w.a = take(sh); w.b = take(sh);
+    w.comb = take(rh); w.hout = take(rh); w.mu = take(rd); w.presig = take(rd); w.z = take(sd); w.u = take(rh); w.v = take(rh);
+    w.dhz = take(2 * rd); w.dzt = take(rd); w.path = take(B);
+    w.dhx = take(R * 2 * N);
+    w.part = take((N + kHeadWorkers - 1) / kHeadWorkers * R);
+    w.dv_parts = take(w.dv_parts_n * rh);
+    w.dv = take(rh); w.du = take(rh); w.dpc = take(rh); w.dh = take(rh); w.dmu = take(rd); w.dps = take(rd); w.gz0 = take(B * D);
+    w.dpf = take(rh); w.dpb = take(rh); w.ca = take(B * H); w.cb = take(B * H);
+    w.total = o;
+    return w;
 }
 
-struct Launcher {
-    cudaStream_t s;
-    void gemm(const float* A, long long a_m, long long a_k, const float* Bm, long long b_k, long long b_n, float* C, long long c_m,
-              const float* bias, int M, int N, int K, int acc) const {
-        Gemm g{A, a_m, a_k, Bm, b_k, b_n, C, c_m, bias, M, N, K, acc};
-        dim3 grid((N + kGemmTile - 1) / kGemmTile, (M + kGemmTile - 1) / kGemmTile);
-        k_gemm<<<grid, 256, 0, s>>>(g);
+inline long long workspace_floats(long long N, long long D, long long H, long long W, long long B) { return workspace(N, D, H, W, B).total; }
+
+// A kernel that may begin while the one before it is still running (it waits by itself before it touches its results).
+template <typename... KArgs, typename... Args>
+inline void launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t s, bool dependent, Args... args) {
+    if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+struct ProductBuilder {
+    ProductList list{};
+    int tiles = 0;
+    ProductBuilder() { list.n = 0; }
+    void add(const Operand& a, const Operand& b, float* c, long long ldc, float* a_sums, int K) {
+        Product& p = list.p[list.n++];
+        p.a = a; p.b = b; p.c = c; p.ldc = ldc; p.a_sums = a_sums; p.K = K;
+        p.tile0 = tiles;
+        p.tiles_n = b.rows > 0 ? static_cast<int>(tiles_of(b.rows)) : 1;
+        tiles += static_cast<int>(tiles_of(a.rows)) * p.tiles_n;
     }
-    // Y[M x O] (+)= X[M x K] W[O x K]^T + bias
-    void linear(const float* X, long long ldx, const float* Wt, const float* bias, float* Y, int M, int O, int K, int acc = 0) const {
-        gemm(X, ldx, 1, Wt, 1, K, Y, O, bias, M, O, K, acc);
+    template <bool AK, bool BK>
+    void run(bool vec, int k_part, int parts, long long part_stride, cudaStream_t s, bool dependent) {
+        list.k_part = k_part;
+        list.part_stride = part_stride;
+        if (vec) launch(k_products<AK, BK, true>, dim3(tiles, parts), kGemmThreads, 0, s, dependent, list);
+        else launch(k_products<AK, BK, false>, dim3(tiles, parts), kGemmThreads, 0, s, dependent, list);
     }
-    // dX[M x K] (+)= dY[M x O] W[O x K]
-    void input_grad(const float* dY, const float* Wt, float* dX, int M, int O, int K, int acc) const {
-        gemm(dY, O, 1, Wt, K, 1, dX, K, nullptr, M, K, O, acc);
-    }
-    // dW[O x K] += dY[M x O]^T X[M x K];  db[O] += column sums of dY
-    void weight_grad(const float* dY, const float* X, long long ldx, float* dW, float* db, int M, int O, int K) const {
-        gemm(dY, 1, O, X, ldx, 1, dW, K, nullptr, O, K, M, 1);
-        if (db) k_colsum_rows<<<(O + 255) / 256, 256, 0, s>>>(dY, M, O, db, 1);
-    }
-    static unsigned blocks(long long n) { return static_cast<unsigned>((n + 255) / 256); }
 };
 
 // Enqueue forward (+ backward if grads) on `stream`.  All pointers are device pointers.
 inline void elbo_grad(int N, int D, int H, int W, int B, const float* p, const float* xhat, const float* eps, float* elbo,
                       float* grads, float* ws, cudaStream_t stream) {
     const Layout L = layout(N, D, H);
-    auto w = [&](int i) { return p + L.off[i]; };
-    auto g = [&](int i) { return grads + L.off[i]; };
-    const Launcher run{stream};
-    const long long bh = static_cast<long long>(B) * H, bd = static_cast<long long>(B) * D;
-    float* cur = ws;
-    auto take = [&](long long n) { float* r = cur; cur += n; return r; };
-    float* a0b = take(bh); float* b0b = take(bh);
-    float* a = take(W * bh); float* b = take(W * bh);
-    float* z = take((W + 1) * bd);
-    float* comb = take(W * bh); float* hout = take(W * bh);
-    float* mu = take(W * bd); float* presig = take(W * bd); float* sigma = take(W * bd); float* dzt = take(W * bd);
-    float* u = take(W * bh); float* v = take(W * bh);
-    float* headz = take(static_cast<long long>(W) * B * 2 * D);
-    float* headx = take(static_cast<long long>(W) * B * 2 * N);
-    float* g_a = take(W * bh); float* g_b = take(W * bh);
-    float* g_z = take(bd); float* g_zn = take(bd); float* g_zp = take(bd);
-    float* d_mu = take(bd); float* d_ps = take(bd);
-    float* t1 = take(bh); float* t2 = take(bh); float* d_pre = take(bh); float* carry = take(bh);
+    const Workspace o = workspace(N, D, H, W, B);
+    const auto w = [&](int i) { return p + L.off[i]; };
+    const auto g = [&](int i) { return grads + L.off[i]; };
+    const int R = B * W;
+    const long long rh = static_cast<long long>(R) * H;
     const bool back = grads != nullptr;
-    const long long xs = static_cast<long long>(W) * N;           // stride between windows in xhat
-    const int es = W * D;                                         // stride between windows in eps
+    const auto aligned = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
+    // 16-byte loads: every tensor and every row then starts on 16 bytes
+    const bool vec = N % 4 == 0 && D % 4 == 0 && H % 4 == 0 && aligned(p) && aligned(xhat) && aligned(ws);
+    const bool vec_h = H % 4 == 0 && vec;
 
-    cudaMemsetAsync(elbo, 0, sizeof(float) * B, stream);
-    if (back) cudaMemsetAsync(dzt, 0, sizeof(float) * W * bd, stream);
-    k_broadcast_rows<<<Launcher::blocks(bh), 256, 0, stream>>>(a0b, w(ia0), B, H);
-    k_broadcast_rows<<<Launcher::blocks(bh), 256, 0, stream>>>(b0b, w(ib0), B, H);
-    k_broadcast_rows<<<Launcher::blocks(bd), 256, 0, stream>>>(z, w(iz0), B, D);
-    // ---- encoder RNNs ------------------------------------------------------------------------------------------
-    for (int t = 0; t < W; ++t) {
-        float* at = a + t * bh;
-        run.linear(xhat + static_cast<long long>(t) * N, xs, w(iWxf), w(ibf), at, B, H, N);
-        run.linear(t > 0 ? a + (t - 1) * bh : a0b, H, w(iWhf), nullptr, at, B, H, H, 1);
-        k_relu<<<Launcher::blocks(bh), 256, 0, stream>>>(at, bh);
+    // ---- forward -------------------------------------------------------------------------------------------------
+    {
+        ProductBuilder q;                                     // input projections of both RNNs, K = N in parts
+        const Operand x{xhat, N, R, 0, 0};
+        q.add(x, Operand{w(iWxf), N, H, 0, 0}, ws + o.proj, 2 * H, nullptr, N);
+        q.add(x, Operand{w(iWxb), N, H, 0, 0}, ws + o.proj + H, 2 * H, nullptr, N);
+        q.run<true, true>(vec, o.proj_k, o.proj_parts, 2 * rh, stream, false);
     }
-    for (int t = W - 1; t >= 0; --t) {
-        float* bt = b + t * bh;
-        run.linear(xhat + static_cast<long long>(t) * N, xs, w(iWxb), w(ibb), bt, B, H, N);
-        run.linear(t + 1 < W ? b + (t + 1) * bh : b0b, H, w(iWhb), nullptr, bt, B, H, H, 1);
-        k_relu<<<Launcher::blocks(bh), 256, 0, stream>>>(bt, bh);
+    const bool wh_staged = H <= kRnnSmemH;
+    {
+        RnnArgs a{};
+        a.proj = ws + o.proj; a.n_parts = o.proj_parts; a.part_stride = 2 * rh;
+        a.Wh[0] = w(iWhf); a.Wh[1] = w(iWhb); a.bias[0] = w(ibf); a.bias[1] = w(ibb); a.init[0] = w(ia0); a.init[1] = w(ib0);
+        a.state[0] = ws + o.a; a.state[1] = ws + o.b; a.B = B; a.W = W; a.H = H;
+        const dim3 grid((B + kRnnRows - 1) / kRnnRows, 2);
+        const size_t smem = rnn_smem_bytes(H, wh_staged);
+        if (vec_h) launch(k_rnn_forward<true>, grid, kRnnThreads, smem, stream, true, a, wh_staged ? 1 : 0);
+        else launch(k_rnn_forward<false>, grid, kRnnThreads, smem, stream, true, a, wh_staged ? 1 : 0);
     }
-    // ---- guide chain and the two densities along the sampled path --------------------------------------------------
-    for (int t = 0; t < W; ++t) {
-        const float* zp = z + t * bd;
-        float* zt = z + (t + 1) * bd;
-        run.linear(zp, D, w(iWz), w(ibz), t1, B, H, D);
-        k_combine<<<Launcher::blocks(bh), 256, 0, stream>>>(t1, a + t * bh, b + t * bh, comb + t * bh, hout + t * bh, bh);
-        run.linear(hout + t * bh, H, w(iWmu), w(ibmu), mu + t * bd, B, D, H);
-        run.linear(mu + t * bd, D, w(iWsig), w(ibsig), presig + t * bd, B, D, D);
-        k_guide_sample<<<(B + 127) / 128, 128, 0, stream>>>(mu + t * bd, presig + t * bd, eps + t * D, es, sigma + t * bd, zt, elbo, B, D);
-        float* ut = u + t * bh;
-        run.linear(zp, D, w(iW1), w(ib1), ut, B, H, D);
-        k_relu<<<Launcher::blocks(bh), 256, 0, stream>>>(ut, bh);
-        float* hz = headz + static_cast<long long>(t) * B * 2 * D;
-        run.linear(ut, H, w(iW2), w(ib2), hz, B, 2 * D, H);
-        k_gauss_density<<<B, kDensityThreads, 0, stream>>>(hz, zt, D, D, elbo, back ? hz : nullptr, back ? dzt + t * bd : nullptr);
-        float* vt = v + t * bh;
-        run.linear(zt, D, w(iW3), w(ib3), vt, B, H, D);
-        k_relu<<<Launcher::blocks(bh), 256, 0, stream>>>(vt, bh);
-        float* hx = headx + static_cast<long long>(t) * B * 2 * N;
-        run.linear(vt, H, w(iW4), w(ib4), hx, B, 2 * N, H);
-        k_gauss_density<<<B, kDensityThreads, 0, stream>>>(hx, xhat + static_cast<long long>(t) * N, xs, N, elbo, back ? hx : nullptr, nullptr);
+    PathArgs a{};
+    a.Wz = w(iWz); a.bz = w(ibz); a.Wmu = w(iWmu); a.bmu = w(ibmu); a.Wsig = w(iWsig); a.bsig = w(ibsig); a.z0 = w(iz0);
+    a.W1 = w(iW1); a.b1 = w(ib1); a.W2 = w(iW2); a.b2 = w(ib2); a.W3 = w(iW3); a.b3 = w(ib3);
+    a.a = ws + o.a; a.b = ws + o.b; a.eps = eps;
+    a.comb = ws + o.comb; a.hout = ws + o.hout; a.mu = ws + o.mu; a.presig = ws + o.presig; a.z = ws + o.z; a.u = ws + o.u;
+    a.v = ws + o.v; a.dhz = ws + o.dhz; a.dzt = ws + o.dzt; a.path = ws + o.path;
+    a.dv_parts = ws + o.dv_parts; a.n_parts = o.dv_parts_n; a.part_stride = rh;
+    a.dv = ws + o.dv; a.du = ws + o.du; a.dpc = ws + o.dpc; a.dh = ws + o.dh; a.dmu = ws + o.dmu; a.dps = ws + o.dps;
+    a.gz0 = ws + o.gz0; a.B = B; a.W = W; a.D = D; a.H = H;
+    const size_t path_scratch = path_scratch_floats(D, H) * sizeof(float);
+    const size_t path_full = path_scratch + path_weight_floats(D, H) * sizeof(float);
+    const int staged = path_full <= 200 * 1024 ? 1 : 0;
+    const size_t path_smem = staged ? path_full : path_scratch;
+    launch(k_path_forward, dim3(B), kPathThreads, path_smem, stream, true, a, staged);
+    const int head_tiles = (N + kHeadWorkers - 1) / kHeadWorkers;
+    {
+        const dim3 grid(head_tiles, static_cast<unsigned>(tiles_of(R)));
+        float* dhx = back ? ws + o.dhx : nullptr;
+        if (vec) launch(k_emission_density<true>, grid, kGemmThreads, 0, stream, true, ws + o.v, w(iW4), w(ib4), xhat, R, N, H, dhx, ws + o.part);
+        else launch(k_emission_density<false>, grid, kGemmThreads, 0, stream, true, ws + o.v, w(iW4), w(ib4), xhat, R, N, H, dhx, ws + o.part);
     }
+    launch(k_elbo_finish, dim3((B + 3) / 4), 128, 0, stream, true, ws + o.part, head_tiles, R, W, B, ws + o.path, elbo);
     if (!back) return;
-    // ---- backward ---------------------------------------------------------------------------------------------------
-    cudaMemsetAsync(grads, 0, sizeof(float) * L.off[kTensors], stream);
-    cudaMemsetAsync(g_zn, 0, sizeof(float) * bd, stream);
-    for (int t = W - 1; t >= 0; --t) {
-        const float* zp = z + t * bd;
-        const float* zt = z + (t + 1) * bd;
-        const float* dhx = headx + static_cast<long long>(t) * B * 2 * N;
-        const float* dhz = headz + static_cast<long long>(t) * B * 2 * D;
-        // d ELBO / d z_t so far: from step t+1, and from z_t as the target of the transition density
-        cudaMemcpyAsync(g_z, g_zn, sizeof(float) * bd, cudaMemcpyDeviceToDevice, stream);
-        k_add<<<Launcher::blocks(bd), 256, 0, stream>>>(g_z, dzt + t * bd, bd);
-        // emission density
-        run.weight_grad(dhx, v + t * bh, H, g(iW4), g(ib4), B, 2 * N, H);
-        run.input_grad(dhx, w(iW4), t2, B, 2 * N, H, 0);
-        k_relu_back<<<Launcher::blocks(bh), 256, 0, stream>>>(t2, v + t * bh, bh);
-        run.weight_grad(t2, zt, D, g(iW3), g(ib3), B, H, D);
-        run.input_grad(t2, w(iW3), g_z, B, H, D, 1);
-        // transition density
-        run.weight_grad(dhz, u + t * bh, H, g(iW2), g(ib2), B, 2 * D, H);
-        run.input_grad(dhz, w(iW2), t2, B, 2 * D, H, 0);
-        k_relu_back<<<Launcher::blocks(bh), 256, 0, stream>>>(t2, u + t * bh, bh);
-        run.weight_grad(t2, zp, D, g(iW1), g(ib1), B, H, D);
-        run.input_grad(t2, w(iW1), g_zp, B, H, D, 0);
-        // guide
-        k_guide_back<<<Launcher::blocks(bd), 256, 0, stream>>>(g_z, eps + t * D, es, sigma + t * bd, presig + t * bd, d_mu, d_ps, B, D);
-        run.weight_grad(d_ps, mu + t * bd, D, g(iWsig), g(ibsig), B, D, D);
-        run.input_grad(d_ps, w(iWsig), d_mu, B, D, D, 1);
-        run.weight_grad(d_mu, hout + t * bh, H, g(iWmu), g(ibmu), B, D, H);
-        run.input_grad(d_mu, w(iWmu), t1, B, D, H, 0);
-        k_combine_back<<<Launcher::blocks(bh), 256, 0, stream>>>(t1, comb + t * bh, g_a + t * bh, g_b + t * bh, t2, bh);
-        run.weight_grad(t2, zp, D, g(iWz), g(ibz), B, H, D);
-        run.input_grad(t2, w(iWz), g_zp, B, H, D, 1);
-        float* swap = g_zn; g_zn = g_zp; g_zp = swap;
+    // ---- backward ------------------------------------------------------------------------------------------------
+    {
+        ProductBuilder q;                                     // d v = d_head W4, K = 2N in parts
+        q.add(Operand{ws + o.dhx, 2ll * N, R, 0, 0}, Operand{w(iW4), H, H, 0, 0}, ws + o.dv_parts, H, nullptr, 2 * N);
+        q.run<true, false>(vec, o.dv_k, o.dv_parts_n, rh, stream, true);
     }
-    k_colsum_rows<<<(D + 255) / 256, 256, 0, stream>>>(g_zn, B, D, g(iz0), 1);
-    // encoder RNNs
-    cudaMemsetAsync(carry, 0, sizeof(float) * bh, stream);
-    for (int t = W - 1; t >= 0; --t) {
-        k_rnn_back<<<Launcher::blocks(bh), 256, 0, stream>>>(d_pre, g_a + t * bh, carry, a + t * bh, bh);
-        run.weight_grad(d_pre, xhat + static_cast<long long>(t) * N, xs, g(iWxf), g(ibf), B, H, N);
-        run.weight_grad(d_pre, t > 0 ? a + (t - 1) * bh : a0b, H, g(iWhf), nullptr, B, H, H);
-        run.input_grad(d_pre, w(iWhf), carry, B, H, H, 0);
+    launch(k_path_backward, dim3(B), kPathThreads, path_smem, stream, true, a, staged);
+    {
+        RnnBackArgs r{};
+        r.g = ws + o.dh; r.state[0] = ws + o.a; r.state[1] = ws + o.b; r.Wh[0] = w(iWhf); r.Wh[1] = w(iWhb);
+        r.d_pre[0] = ws + o.dpf; r.d_pre[1] = ws + o.dpb; r.carry_out[0] = ws + o.ca; r.carry_out[1] = ws + o.cb;
+        r.B = B; r.W = W; r.H = H;
+        const dim3 grid((B + kRnnRows - 1) / kRnnRows, 2);
+        const size_t smem = rnn_back_smem_bytes(H, wh_staged);
+        if (vec_h) launch(k_rnn_backward<true>, grid, kRnnThreads, smem, stream, true, r, wh_staged ? 1 : 0);
+        else launch(k_rnn_backward<false>, grid, kRnnThreads, smem, stream, true, r, wh_staged ? 1 : 0);
     }
-    k_colsum_rows<<<(H + 255) / 256, 256, 0, stream>>>(carry, B, H, g(ia0), 1);
-    cudaMemsetAsync(carry, 0, sizeof(float) * bh, stream);
-    for (int t = 0; t < W; ++t) {
-        k_rnn_back<<<Launcher::blocks(bh), 256, 0, stream>>>(d_pre, g_b + t * bh, carry, b + t * bh, bh);
-        run.weight_grad(d_pre, xhat + static_cast<long long>(t) * N, xs, g(iWxb), g(ibb), B, H, N);
-        run.weight_grad(d_pre, t + 1 < W ? b + (t + 1) * bh : b0b, H, g(iWhb), nullptr, B, H, H);
-        run.input_grad(d_pre, w(iWhb), carry, B, H, H, 0);
+    {
+        // every weight gradient d W = d_out^T in over the R rows, and the biases as column sums of d_out; the largest first
+        ProductBuilder q;
+        const auto rows = [&](long long off, int ld) { return Operand{ws + off, ld, ld, 0, 0}; };
+        const auto before = [&](long long off, int ld, int first) { return Operand{ws + off, ld, ld, W, first}; };   // of [B][W + 1]
+        const Operand none{nullptr, 0, 0, 0, 0};
+        q.add(rows(o.dhx, 2 * N), rows(o.v, H), g(iW4), H, g(ib4), R);
+        q.add(rows(o.dpf, H), Operand{xhat, N, N, 0, 0}, g(iWxf), N, g(ibf), R);
+        q.add(rows(o.dpb, H), Operand{xhat, N, N, 0, 0}, g(iWxb), N, g(ibb), R);
+        q.add(rows(o.dpf, H), before(o.a, H, 0), g(iWhf), H, nullptr, R);
+        q.add(rows(o.dpb, H), before(o.b, H, 1), g(iWhb), H, nullptr, R);
+        q.add(rows(o.dv, H), before(o.z, D, 1), g(iW3), D, g(ib3), R);
+        q.add(rows(o.du, H), before(o.z, D, 0), g(iW1), D, g(ib1), R);
+        q.add(rows(o.dpc, H), before(o.z, D, 0), g(iWz), D, g(ibz), R);
+        q.add(rows(o.dhz, 2 * D), rows(o.u, H), g(iW2), H, g(ib2), R);
+        q.add(rows(o.dmu, D), rows(o.hout, H), g(iWmu), H, g(ibmu), R);
+        q.add(rows(o.dps, D), rows(o.mu, D), g(iWsig), D, g(ibsig), R);
+        q.add(rows(o.ca, H), none, nullptr, 0, g(ia0), B);
+        q.add(rows(o.cb, H), none, nullptr, 0, g(ib0), B);
+        q.add(rows(o.gz0, D), none, nullptr, 0, g(iz0), B);
+        q.run<false, false>(vec, (R + kTileK - 1) / kTileK * kTileK, 1, 0, stream, true);
     }
-    k_colsum_rows<<<(H + 255) / 256, 256, 0, stream>>>(carry, B, H, g(ib0), 1);
 }
 
 }  // namespace fit

@@ -160,3 +160,24 @@ def test_learning_calls_reject_bad_arguments():
     assert lib.cutoff_elbo_grad(0, 16, 4, 32, 1, 0, *args[6:], ws.data_ptr(), ws.numel(), None) == binding.ERR_BAD_ARG
     assert lib.cutoff_adam_step(0, n, buf.data_ptr(), buf.data_ptr(), buf.data_ptr(), buf.data_ptr(), 0, 1e-3, 0.9, 0.999,
                                 1e-8, 1.0, 1.0, buf.data_ptr(), ws.data_ptr(), ws.numel(), None) == binding.ERR_BAD_ARG
+
+
+# where the kernels change their way: tiles of 64 rows, 64 columns or 32 workers and their remainders, dimensions that are
+# no multiple of 4 (scalar loads), recurrence matrices too wide for shared memory (H > 200), latent matrices too large for
+# it (D = 64), more windows than one CTA of the recurrences takes and not a multiple of it, a product split over K
+@pytest.mark.parametrize("N,D,H,lag,B", [(1, 1, 1, 0, 1), (32, 4, 64, 0, 64), (33, 4, 68, 1, 33), (65, 8, 200, 0, 5),
+                                          (31, 5, 201, 1, 6), (64, 64, 300, 1, 3), (600, 16, 204, 3, 9)])
+def test_step_at_the_edges_of_tiles_and_of_shared_memory(N, D, H, lag, B):
+    """Bounds as above: an fp32 sum of n products errs by at most about n * 2^-24 of the sum of their magnitudes."""
+    import torch
+    w, x, eps = _case(N, D, H, lag, B, seed=1000 + N + H)
+    want_elbo, want_g = L.elbo_and_grad(w, x, eps)
+    fitter = binding.Fitter(N, D, H, lag, B, w)
+    elbo, grads = fitter.elbo_grad(torch.from_numpy(x).cuda(), torch.from_numpy(eps).cuda())
+    torch.cuda.synchronize()
+    assert np.max(np.abs(elbo.cpu().numpy() - want_elbo)) <= 2e-5 * np.max(np.abs(want_elbo))
+    got = binding.unflatten_weights(grads.cpu().numpy(), N, D, H)
+    for name in L.PARAMS:
+        denom = max(float(np.max(np.abs(want_g[name]))), 1e-6)
+        err = float(np.max(np.abs(got[name].astype(np.float64) - want_g[name]))) / denom
+        assert err <= 2e-4, f"{name}: {err:.2e}"
