@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include "kernels_model.cuh"
 #include "kernels_sort.cuh"
+#include "bucket_sort.cuh"
 #include "emit_tc.cuh"
 #include "emit_tc2.cuh"
 #include "chain_tc.cuh"
@@ -248,6 +249,26 @@ void free_all(cutoff_ctx* c) {
                 if (e) cudaEventDestroy(e);
 }
 
+// Keys per thread of the bucket sort: N / threads rounded up to a multiple of 4.
+int keys_per_thread(int n, int threads) { return ceil_div(ceil_div(n, threads), 4) * 4; }
+
+// Which rows of N <= 1024 keys are sorted by distribution and which by the register network.  Up to 128 keys the network
+// is shorter than counting and scanning (128 keys x 65536 rows: 0.033 against 0.035 ms), from 257 on it never is (300 keys x 2048 rows:
+// 0.0113 against 0.0091 ms); between, it depends on whether the longer latency of one row is hidden by the rows that
+// follow (256 keys: 2048 rows 0.0075 against 0.0086 ms, 65536 rows 0.056 against 0.049 ms; 140 keys x 16384 rows 0.0197 against 0.0172 ms).
+bool by_buckets(int n, int64_t rows) { return n > 256 || (n > 128 && rows >= 8192); }
+
+int bucket_wide_ctas(int n) {
+    switch (keys_per_thread(n, 128)) {
+        case 12: return kBucketWideCtas<12>;
+        case 16: return kBucketWideCtas<16>;
+        case 20: return kBucketWideCtas<20>;
+        case 24: return kBucketWideCtas<24>;
+        case 28: return kBucketWideCtas<28>;
+        default: return kBucketWideCtas<32>;
+    }
+}
+
 // Work split: how many samples go through chain -> emission -> sort at a time, and how many
 // CTAs the sort kernel uses per pass.
 void plan_chunks(cutoff_ctx* c, int chunk_rows_wanted) {
@@ -259,43 +280,70 @@ void plan_chunks(cutoff_ctx* c, int chunk_rows_wanted) {
     c->n_chunks = ceil_div(c->S, rows);
     // CTAs of the sort kernel per pass: enough to fill the GPU, within the partial-sum rows available
     int want, cap;
-    if (c->P <= 1024) { want = ceil_div(rows, kSortWarps); cap = c->sm_count * 2; }
-    else { want = rows; cap = c->sm_count * 8; }
+    if (c->N > 1024) { want = rows; cap = c->sm_count * bucket_wide_ctas(c->N); }
+    else if (by_buckets(c->N, rows)) { want = rows; cap = c->sm_count; }
+    else { want = ceil_div(rows, kSortWarps); cap = c->sm_count * 2; }
     if (cap > kPartialRows / c->n_chunks) cap = kPartialRows / c->n_chunks;
     c->sort_grid = want < cap ? want : cap;
 }
 
-template <int E, bool SQ>
-void launch_sort_warp_sq(cutoff_ctx* c, int count, float* partial) {
-    const size_t smem = sort_tma_smem_bytes<E>(c->ldx);
-    launch_dependent(k_sort_sum_tma<E, SQ>, dim3(c->sort_grid), dim3(kSortWarps * 32), smem, c->stream,
-                     c->d_x, c->ldx, c->N, count, partial, partial + static_cast<size_t>(kPartialRows) * c->N, c->d_state);
-}
-
 template <int E>
 void launch_sort_warp(cutoff_ctx* c, int count, float* partial) {
-    if (c->want_std) launch_sort_warp_sq<E, true>(c, count, partial);
-    else launch_sort_warp_sq<E, false>(c, count, partial);
+    float* partial_sq = partial + static_cast<size_t>(kPartialRows) * c->N;
+    const size_t smem = sort_tma_smem_bytes<E>(c->ldx);
+    if (c->want_std) launch_dependent(k_sort_sum_tma<E, true>, dim3(c->sort_grid), dim3(kSortWarps * 32), smem, c->stream, c->d_x, c->ldx, c->N, count, partial, partial_sq, c->d_state);
+    else launch_dependent(k_sort_sum_tma<E, false>, dim3(c->sort_grid), dim3(kSortWarps * 32), smem, c->stream, c->d_x, c->ldx, c->N, count, partial, partial_sq, c->d_state);
 }
 
-template <int WPR>
-void launch_sort_cta(cutoff_ctx* c, int count, float* partial) {
-    float* partial_sq = partial + static_cast<size_t>(kPartialRows) * c->N;
-    if (c->want_std) k_sort_sum_cta<WPR, true><<<c->sort_grid, WPR * 32, 0, c->stream>>>(c->d_x, c->ldx, c->N, count, partial, partial_sq);
-    else k_sort_sum_cta<WPR, false><<<c->sort_grid, WPR * 32, 0, c->stream>>>(c->d_x, c->ldx, c->N, count, partial, partial_sq);
+template <int E, bool SQ>
+void launch_bucket_warp_sq(cutoff_ctx* c, int count, float* partial) {
+    launch_dependent(k_bucket_sum_warp<E, SQ, kBulk>, dim3(c->sort_grid), dim3(kBucketWarps<E> * 32), bucket_smem_bytes<E>(), c->stream,
+                     c->d_x, c->ldx, c->N, count, partial, partial + static_cast<size_t>(kPartialRows) * c->N, c->d_state);
+}
+template <int E>
+void launch_bucket_warp(cutoff_ctx* c, int count, float* partial) {
+    if (c->want_std) launch_bucket_warp_sq<E, true>(c, count, partial);
+    else launch_bucket_warp_sq<E, false>(c, count, partial);
+}
+
+template <int E, bool SQ>
+void launch_bucket_cta_sq(cutoff_ctx* c, int count, float* partial) {
+    launch_dependent(k_bucket_sum_cta<E, SQ>, dim3(c->sort_grid), dim3(128), bucket_wide_smem_bytes<E>(), c->stream,
+                     c->d_x, c->ldx, c->N, count, partial, partial + static_cast<size_t>(kPartialRows) * c->N, c->d_state);
+}
+template <int E>
+void launch_bucket_cta(cutoff_ctx* c, int count, float* partial) {
+    if (c->want_std) launch_bucket_cta_sq<E, true>(c, count, partial);
+    else launch_bucket_cta_sq<E, false>(c, count, partial);
 }
 
 int launch_sort(cutoff_ctx* c, int count, float* partial) {
-    switch (c->P) {
-        case 32: launch_sort_warp<1>(c, count, partial); break;
-        case 64: launch_sort_warp<2>(c, count, partial); break;
-        case 128: launch_sort_warp<4>(c, count, partial); break;
-        case 256: launch_sort_warp<8>(c, count, partial); break;
-        case 512: launch_sort_warp<16>(c, count, partial); break;
-        case 1024: launch_sort_warp<32>(c, count, partial); break;
-        case 2048: launch_sort_cta<2>(c, count, partial); break;
-        case 4096: launch_sort_cta<4>(c, count, partial); break;
-        default: return CUTOFF_ERR_UNSUPPORTED;
+    if (c->N > 1024) {
+        switch (keys_per_thread(c->N, 128)) {
+            case 12: launch_bucket_cta<12>(c, count, partial); break;
+            case 16: launch_bucket_cta<16>(c, count, partial); break;
+            case 20: launch_bucket_cta<20>(c, count, partial); break;
+            case 24: launch_bucket_cta<24>(c, count, partial); break;
+            case 28: launch_bucket_cta<28>(c, count, partial); break;
+            default: launch_bucket_cta<32>(c, count, partial); break;
+        }
+    } else if (by_buckets(c->N, c->chunk_rows)) {
+        switch (keys_per_thread(c->N, 32)) {
+            case 8: launch_bucket_warp<8>(c, count, partial); break;
+            case 12: launch_bucket_warp<12>(c, count, partial); break;
+            case 16: launch_bucket_warp<16>(c, count, partial); break;
+            case 20: launch_bucket_warp<20>(c, count, partial); break;
+            case 24: launch_bucket_warp<24>(c, count, partial); break;
+            case 28: launch_bucket_warp<28>(c, count, partial); break;
+            default: launch_bucket_warp<32>(c, count, partial); break;
+        }
+    } else {
+        switch (c->P) {
+            case 32: launch_sort_warp<1>(c, count, partial); break;
+            case 64: launch_sort_warp<2>(c, count, partial); break;
+            case 128: launch_sort_warp<4>(c, count, partial); break;
+            default: launch_sort_warp<8>(c, count, partial); break;
+        }
     }
     c->launches += 1;
     return CUTOFF_OK;
@@ -601,10 +649,38 @@ cudaError_t allow_smem(Kernel kernel, size_t bytes) {
 }
 
 template <int E>
-cudaError_t allow_smem_sort() {
-    cudaError_t e = allow_smem(k_sort_sum_tma<E, false>, 100 * 1024);
-    if (e == cudaSuccess) e = allow_smem(k_sort_sum_tma<E, true>, 100 * 1024);
+cudaError_t allow_smem_bucket_warp() {
+    cudaError_t e = allow_smem(k_bucket_sum_warp<E, false, kBulk>, bucket_smem_bytes<E>());
+    if (e == cudaSuccess) e = allow_smem(k_bucket_sum_warp<E, true, kBulk>, bucket_smem_bytes<E>());
     return e;
+}
+template <int E>
+cudaError_t allow_smem_bucket_cta() {
+    cudaError_t e = allow_smem(k_bucket_sum_cta<E, false>, bucket_wide_smem_bytes<E>());
+    if (e == cudaSuccess) e = allow_smem(k_bucket_sum_cta<E, true>, bucket_wide_smem_bytes<E>());
+    return e;
+}
+cudaError_t allow_smem_sort(int n) {
+    if (n > 1024) {
+        switch (keys_per_thread(n, 128)) {
+            case 12: return allow_smem_bucket_cta<12>();
+            case 16: return allow_smem_bucket_cta<16>();
+            case 20: return allow_smem_bucket_cta<20>();
+            case 24: return allow_smem_bucket_cta<24>();
+            case 28: return allow_smem_bucket_cta<28>();
+            default: return allow_smem_bucket_cta<32>();
+        }
+    }
+    switch (n > 128 ? keys_per_thread(n, 32) : 0) {        // the network's rows fit 48 KB
+        case 0: return cudaSuccess;
+        case 8: return allow_smem_bucket_warp<8>();
+        case 12: return allow_smem_bucket_warp<12>();
+        case 16: return allow_smem_bucket_warp<16>();
+        case 20: return allow_smem_bucket_warp<20>();
+        case 24: return allow_smem_bucket_warp<24>();
+        case 28: return allow_smem_bucket_warp<28>();
+        default: return allow_smem_bucket_warp<32>();
+    }
 }
 
 template <int D>
@@ -617,15 +693,7 @@ cudaError_t allow_smem_chain() {
 
 cudaError_t set_kernel_attributes(const cutoff_ctx* c) {
     cudaError_t e = cudaSuccess;
-    switch (c->P) {
-        case 32: e = allow_smem_sort<1>(); break;
-        case 64: e = allow_smem_sort<2>(); break;
-        case 128: e = allow_smem_sort<4>(); break;
-        case 256: e = allow_smem_sort<8>(); break;
-        case 512: e = allow_smem_sort<16>(); break;
-        case 1024: e = allow_smem_sort<32>(); break;
-        default: break;
-    }
+    e = allow_smem_sort(c->N);
     if (e != cudaSuccess) return e;
     switch (c->D) {
         case 4: e = allow_smem_chain<4>(); break;
@@ -1859,10 +1927,43 @@ static __device__ __align__(256) float g_static_partial[kStaticParts * CUTOFF_ST
 
 constexpr int kMaxDevices = 64;
 float* g_static_partial_addr[kMaxDevices] = {};   // device address per GPU, filled on first use
+int g_static_sms[kMaxDevices] = {};               // its SMs
+
+// Returns the number of partial rows (CTAs).
+template <int E>
+int launch_static_network(const float* x, int ldx, int n, int n_rows, float* partial, cudaStream_t stream) {
+    const int want = ceil_div(n_rows, kSortWarps), grid = want < kStaticParts ? want : kStaticParts;
+    k_sort_sum_warp<E><<<grid, kSortWarps * 32, 0, stream>>>(x, ldx, n, n_rows, partial);
+    return grid;
+}
+
+// Rows that all start on 16 bytes come in as 16-byte chunks, others word by word (700 keys x 32768 rows: 63 against 65 us).
+template <int E>
+int launch_static_bucket(const float* x, int ldx, int n, int n_rows, float* partial, cudaStream_t stream, int sms) {
+    const int most = sms < kStaticParts ? sms : kStaticParts, grid = n_rows < most ? n_rows : most;
+    const size_t smem = bucket_smem_bytes<E>();
+    DevState* const none = nullptr;
+    const bool chunks = (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && ldx % 4 == 0;
+    if (chunks) k_bucket_sum_warp<E, false, 16><<<grid, kBucketWarps<E> * 32, smem, stream>>>(x, ldx, n, n_rows, partial, nullptr, none);
+    else k_bucket_sum_warp<E, false, 4><<<grid, kBucketWarps<E> * 32, smem, stream>>>(x, ldx, n, n_rows, partial, nullptr, none);
+    return grid;
+}
 
 template <int E>
-void launch_static_sort(const float* x, int ldx, int n, int n_rows, int grid, float* partial, cudaStream_t stream) {
-    k_sort_sum_warp<E><<<grid, kSortWarps * 32, 0, stream>>>(x, ldx, n, n_rows, partial);
+cudaError_t allow_smem_static() {
+    cudaError_t e = allow_smem(k_bucket_sum_warp<E, false, 16>, bucket_smem_bytes<E>());
+    if (e == cudaSuccess) e = allow_smem(k_bucket_sum_warp<E, false, 4>, bucket_smem_bytes<E>());
+    return e;
+}
+cudaError_t allow_smem_static_all() {
+    cudaError_t e = allow_smem_static<8>();
+    if (e == cudaSuccess) e = allow_smem_static<12>();
+    if (e == cudaSuccess) e = allow_smem_static<16>();
+    if (e == cudaSuccess) e = allow_smem_static<20>();
+    if (e == cudaSuccess) e = allow_smem_static<24>();
+    if (e == cudaSuccess) e = allow_smem_static<28>();
+    if (e == cudaSuccess) e = allow_smem_static<32>();
+    return e;
 }
 }  // namespace
 
@@ -1875,9 +1976,13 @@ extern "C" int cutoff_sorted_row_sums_static(int device, const float* x, int64_t
     DeviceGuard guard(device);
     if (guard.err != cudaSuccess) return CUTOFF_ERR_CUDA;
     if (!g_static_partial_addr[device]) {
-        // once per device, with that device current: translate the symbol into a device address
+        // once per device, with that device current: translate the symbol into a device address, let the kernels
+        // have the shared memory they need
         float* addr = nullptr;
         if (cudaGetSymbolAddress(reinterpret_cast<void**>(&addr), g_static_partial) != cudaSuccess || !addr)
+            return CUTOFF_ERR_CUDA;
+        if (allow_smem_static_all() != cudaSuccess ||
+            cudaDeviceGetAttribute(&g_static_sms[device], cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
             return CUTOFF_ERR_CUDA;
         g_static_partial_addr[device] = addr;
     }
@@ -1889,20 +1994,30 @@ extern "C" int cutoff_sorted_row_sums_static(int device, const float* x, int64_t
     // the other on the stream, so they can share the scratch array.
     for (int64_t r0 = 0; r0 < n_rows; r0 += kStaticBlockRows) {
         const int rows = static_cast<int>(n_rows - r0 < kStaticBlockRows ? n_rows - r0 : kStaticBlockRows);
-        const int want = ceil_div(rows, kSortWarps);
-        const int grid = want < kStaticParts ? want : kStaticParts;
         const float* xb = x + static_cast<size_t>(r0) * ldx;
         // every CTA of the grid writes its whole partial row (zeros if it had no sample), and the
         // column sum reads exactly `grid` rows: stale contents of the shared array are never read
-        switch (P) {
-            case 32: launch_static_sort<1>(xb, ldx, n, rows, grid, partial, s); break;
-            case 64: launch_static_sort<2>(xb, ldx, n, rows, grid, partial, s); break;
-            case 128: launch_static_sort<4>(xb, ldx, n, rows, grid, partial, s); break;
-            case 256: launch_static_sort<8>(xb, ldx, n, rows, grid, partial, s); break;
-            case 512: launch_static_sort<16>(xb, ldx, n, rows, grid, partial, s); break;
-            default: launch_static_sort<32>(xb, ldx, n, rows, grid, partial, s); break;
+        int grid = 0;
+        const int sms = g_static_sms[device];
+        if (by_buckets(n, rows)) {
+            switch (keys_per_thread(n, 32)) {
+                case 8: grid = launch_static_bucket<8>(xb, ldx, n, rows, partial, s, sms); break;
+                case 12: grid = launch_static_bucket<12>(xb, ldx, n, rows, partial, s, sms); break;
+                case 16: grid = launch_static_bucket<16>(xb, ldx, n, rows, partial, s, sms); break;
+                case 20: grid = launch_static_bucket<20>(xb, ldx, n, rows, partial, s, sms); break;
+                case 24: grid = launch_static_bucket<24>(xb, ldx, n, rows, partial, s, sms); break;
+                case 28: grid = launch_static_bucket<28>(xb, ldx, n, rows, partial, s, sms); break;
+                default: grid = launch_static_bucket<32>(xb, ldx, n, rows, partial, s, sms); break;
+            }
+        } else {
+            switch (P) {
+                case 32: grid = launch_static_network<1>(xb, ldx, n, rows, partial, s); break;
+                case 64: grid = launch_static_network<2>(xb, ldx, n, rows, partial, s); break;
+                case 128: grid = launch_static_network<4>(xb, ldx, n, rows, partial, s); break;
+                default: grid = launch_static_network<8>(xb, ldx, n, rows, partial, s); break;
+            }
         }
-        k_colsum<<<ceil_div(n, 256), 256, 0, s>>>(partial, grid, n, sums, r0 > 0 ? 1 : 0);
+        launch_dependent(k_colsum, dim3(ceil_div(n, 32)), dim3(32 * kPlainSlices), 0, s, partial, grid, n, sums, r0 > 0 ? 1 : 0);
     }
     return cudaGetLastError() == cudaSuccess ? CUTOFF_OK : CUTOFF_ERR_CUDA;
 }

@@ -193,7 +193,8 @@ __global__ void __launch_bounds__(kGemmThreads, 2) k_emission_density(const floa
     __shared__ __align__(16) TileSmem sm;
     dependency_wait();
     launch_dependents();
-    const int m0 = blockIdx.y * kTile, j0 = blockIdx.x * kHeadWorkers;
+    const int head_tiles = (N + kHeadWorkers - 1) / kHeadWorkers;          // one-dimensional grid: rows reach 2^24
+    const int m0 = blockIdx.x / head_tiles * kTile, head_tile = blockIdx.x % head_tiles, j0 = head_tile * kHeadWorkers;
     const Operand a{v, H, R, 0, 0};
     const int tid = threadIdx.x, col = tid >> 2;                             // the column of B this thread loads
     const int worker = j0 + 2 * (col >> 2) + (col & 1), head = (col >> 1) & 1;
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) k_emission_density(const floa
         }
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (tx == 0 && r < R) part[static_cast<long long>(blockIdx.x) * R + r] = s;
+        if (tx == 0 && r < R) part[static_cast<long long>(head_tile) * R + r] = s;
     }
 }
 

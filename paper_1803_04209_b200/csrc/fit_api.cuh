@@ -152,7 +152,7 @@ inline void elbo_grad(int N, int D, int H, int W, int B, const float* p, const f
     launch(k_path_forward, dim3(B), kPathThreads, path_smem, stream, true, a, staged);
     const int head_tiles = (N + kHeadWorkers - 1) / kHeadWorkers;
     {
-        const dim3 grid(head_tiles, static_cast<unsigned>(tiles_of(R)));
+        const dim3 grid(static_cast<unsigned>(head_tiles * tiles_of(R)));
         float* dhx = back ? ws + o.dhx : nullptr;
         if (vec) launch(k_emission_density<true>, grid, kGemmThreads, 0, stream, true, ws + o.v, w(iW4), w(ib4), xhat, R, N, H, dhx, ws + o.part);
         else launch(k_emission_density<false>, grid, kGemmThreads, 0, stream, true, ws + o.v, w(iW4), w(ib4), xhat, R, N, H, dhx, ws + o.part);

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_sum_tma(const float* _
 #pragma unroll
     for (int r = 0; r < (SQ ? E : 1); ++r) acc_sq[r] = 0.0f;
     const int stride = gridDim.x * kSortWarps;
-    int row = blockIdx.x * kSortWarps + warp;
+    int row = blockIdx.x + gridDim.x * warp;           // consecutive rows to different CTAs: a few rows spread over all SMs
     if (row < count && lane == 0) {
         mbar_arrive_expect_tx(bar0, row_bytes);
         bulk_load_1d(smem_u32(buf0), x + static_cast<size_t>(row) * ldx, row_bytes, bar0);
@@ -386,46 +386,6 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_sum_tma(const float* _
 #pragma unroll
             for (int w = 0; w < kSortWarps; ++w) s += stage[w * 32 * E + j];
             partial_sq[static_cast<size_t>(blockIdx.x) * N + j] = s;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
-// Sort + accumulate for wide rows (1024 < N <= 4096): a CTA of WPR = P/1024 warps per row, keys in
-// registers, running sums in registers, one partial row per CTA.
-// ---------------------------------------------------------------------------------------------
-template <int WPR, bool SQ>
-__global__ void __launch_bounds__(WPR * 32, SQ ? 3 : 4) k_sort_sum_cta(const float* __restrict__ x, int ldx, int N, int count,
-                                                            float* __restrict__ partial, float* __restrict__ partial_sq) {
-    __shared__ float xch[WPR * 1024];
-    constexpr int E = 32, T_ = WPR * 32;
-    float acc[E], acc_sq[SQ ? E : 1];
-#pragma unroll
-    for (int r = 0; r < E; ++r) acc[r] = 0.0f;
-#pragma unroll
-    for (int r = 0; r < (SQ ? E : 1); ++r) acc_sq[r] = 0.0f;
-    for (int row = blockIdx.x; row < count; row += gridDim.x) {
-        const float* src = x + static_cast<size_t>(row) * ldx;
-        float v[E];
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int e = r * T_ + threadIdx.x;            // any arrangement sorts; this one loads coalesced
-            v[r] = e < N ? src[e] : INFINITY;
-        }
-        cta_bitonic_sort<float, WPR>(v, xch);
-#pragma unroll
-        for (int r = 0; r < E; ++r) acc[r] += v[r];
-        if (SQ) {
-#pragma unroll
-            for (int r = 0; r < E; ++r) acc_sq[SQ ? r : 0] = fmaf(v[r], v[r], acc_sq[SQ ? r : 0]);
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < E; ++r) {
-        const int idx = threadIdx.x * E + r;
-        if (idx < N) {
-            partial[static_cast<size_t>(blockIdx.x) * N + idx] = acc[r];
-            if (SQ) partial_sq[static_cast<size_t>(blockIdx.x) * N + idx] = acc_sq[SQ ? r : 0];
         }
     }
 }
@@ -560,15 +520,29 @@ __global__ void __launch_bounds__(kColsumThreads) k_colsum_decide(const float* _
     }
 }
 
-// Plain column sums of partial rows (fixed order, double): one thread per column.  With `accumulate` the
-// result is added to what sums already holds.
-__global__ void __launch_bounds__(256) k_colsum(const float* __restrict__ partial, int n_part, int N,
-                                                double* __restrict__ sums, int accumulate) {
-    const int j = blockIdx.x * 256 + threadIdx.x;
-    if (j >= N) return;
-    double s = accumulate ? sums[j] : 0.0;
-    for (int p = 0; p < n_part; ++p) s += static_cast<double>(partial[static_cast<size_t>(p) * N + j]);
-    sums[j] = s;
+// Plain column sums of partial rows in a fixed order, in double: 32 columns per CTA, slice s adds rows s, s+8, ..., the
+// slices are then added in order.  With `accumulate` the result is added to what sums already holds.  (One thread per
+// column left all but three SMs idle over 256 dependent additions.)
+constexpr int kPlainSlices = 8;
+
+__global__ void __launch_bounds__(32 * kPlainSlices) k_colsum(const float* __restrict__ partial, int n_part, int N,
+                                                              double* __restrict__ sums, int accumulate) {
+    __shared__ double red[kPlainSlices][32];
+    dependency_wait();
+    const int col = threadIdx.x & 31, slice = threadIdx.x >> 5, j = blockIdx.x * 32 + col;
+    double s = 0.0;
+    if (j < N) {
+#pragma unroll 8
+        for (int p = slice; p < n_part; p += kPlainSlices) s += static_cast<double>(partial[static_cast<size_t>(p) * N + j]);
+    }
+    red[slice][col] = s;
+    __syncthreads();
+    if (slice == 0 && j < N) {
+        double total = accumulate ? sums[j] : 0.0;
+#pragma unroll
+        for (int k = 0; k < kPlainSlices; ++k) total += red[k][col];
+        sums[j] = total;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
