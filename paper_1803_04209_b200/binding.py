@@ -478,7 +478,7 @@ class Fitter:
 
     def capture_elbo_grad(self, xhat, eps):
         """Capture elbo_grad(xhat, eps) in a CUDA graph.  xhat and eps are fixed tensors: the caller refills them (on the
-        current stream) before every replay_elbo_grad().  A step is nine dependent launches; a replay takes their launch
+        current stream) before every replay_elbo_grad().  A step is eight dependent launches; a replay takes their launch
         cost off the host."""
         import torch
         self.elbo_grad(xhat, eps)                      # once outside the capture

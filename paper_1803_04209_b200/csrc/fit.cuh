@@ -5,17 +5,19 @@
 //   ELBO_b = sum_t  log p(x_t | z_t) + log p(z_t | z_{t-1}) - log q(z_t | z_{t-1}, x),     z_t = mu_t + sigma_t eps_t,
 //   log N(y; m, exp(lv)) = -1/2 [log 2 pi + lv + (y - m)^2 exp(-lv)],   log q = sum_d -1/2 log 2 pi - log sigma_d - eps_d^2 / 2.
 //
-// What bounds a step is the number of dependent launches, not its arithmetic (64 windows of the n1024 model: 1.0 G
-// multiply-adds, 28 us at the FMA rate), so the step is laid out by what depends on what.  Only the recurrences depend
-// on the previous step of a window, and only within the window: one CTA walks through all of a window's steps (of a few
-// windows' steps for the RNNs) in one launch.  Everything else is one product over all B*W (window, step) rows: the
-// input projections, the emission head with its density in the epilogue, the input gradient of the emission head, and
-// all weight gradients together in one launch over a list of products.  Nine launches per step.  Measured with Adam, 64
-// windows: N = 128, H = 128 replayed as a graph 677 -> 99 us, N = 1024, H = 256 launched one by one 2.95 -> 0.295 ms,
-// against one launch per layer, step and orientation (about 150 of them).
+// What bounds a step is the number of dependent launches and the length of its chains, not its arithmetic (64 windows of
+// the n1024 model: 1.0 G multiply-adds, 28 us at the FMA rate), so the step is laid out by what depends on what.  Only the
+// recurrences depend on the previous step of a window, and only within the window: one CTA walks through all of a
+// window's steps, a cluster through those of a few windows' RNN, in one launch.  Everything else is one product over all
+// B*W (window, step) rows: the input projections, the emission head with its density in the epilogue, the input gradient
+// of that head, and the weight gradients as a list of products in one launch.
 //
-// Rows are window-major: row r = b*W + t.  Every reduction runs in a fixed order (no floating-point atomics), so a step
-// is reproducible bit for bit.
+// Rows are window-major: row r = b*W + t.  Every sum has the order of the plain layer-by-layer evaluation: one chain of
+// fused multiply-adds over ascending k per product; a weight gradient adds the chains of the steps one after the other,
+// the step the reverse pass reaches first coming first.  No product is split over k and nothing depends on tiles,
+// clusters or the other windows, so a step is reproducible bit for bit and a change of its schedule does not change it --
+// which matters because training is not continuous: Adam turns the sign of a vanishing gradient into a full step, and a
+// ReLU whose input is within rounding of zero switches a whole row of a gradient on or off.
 #pragma once
 #include <cmath>
 
@@ -30,152 +32,189 @@ __device__ __forceinline__ float softplus_f(float v) { return v > 20.f ? v : log
 __device__ __forceinline__ float sigmoid_f(float v) { return 1.f / (1.f + expf(-v)); }
 
 // ---- tiled products ----------------------------------------------------------------------------------------------
-// C[m][n] = sum_k A(m, k) B(n, k) over 64 x 64 tiles, 16 k at a time, 4 x 4 per thread, the next slab's global loads in
-// flight while the current one is multiplied.  An operand is either "k-major" (element (m, k) at m*ld + k) or
-// "m-major" (element (m, k) at k*ld + m), so the three orientations a dense layer needs are X W^T, dY W and dY^T X.
-constexpr int kTile = 64, kTileK = 16, kGemmThreads = 256, kTilePad = kTile + 4;
+// C[m][n] = sum_k A(m, k) B(n, k).  An operand is either "k-major" (element (m, k) at m*ld + k) or "m-major" (at k*ld + m),
+// so the three orientations a dense layer needs are X W^T, dY W and dY^T X.  With n_seg > 1 the product is a sum of n_seg
+// products over K, segment s at p + s * seg; the segments' sums are added in order.
+// Two tiles: 64 x 64 with 4 x 4 results per thread where there are enough of them to fill the GPU, 16 x 32 with 2 x 2
+// where there are not -- then the time is the chain's: about 8 clocks per k (64 windows of n1024: the projections have
+// K = 1024 and 40 large or 320 small tiles, the input gradient of the emission head K = 2048 and 20 or 160).
+// The next slab's global loads are in flight while the current one is multiplied.
+template <int TM_, int TN_, int RM_, int RN_, int TK_> struct Tile {
+    static constexpr int TM = TM_, TN = TN_, RM = RM_, RN = RN_, TK = TK_;
+    static constexpr int kThreads = (TM / RM) * (TN / RN);
+    static constexpr int kAVecs = TM * TK / 4 / kThreads, kBVecs = TN * TK / 4 / kThreads;    // float4 per thread and slab
+    struct Smem {
+        float a[2][TK][TM + 4];
+        float b[2][TK][TN + 4];
+    };
+};
+using LargeTile = Tile<64, 64, 4, 4, 16>;        // 256 threads
+using SmallTile = Tile<16, 32, 2, 2, 32>;        // 128 threads
 
 struct Operand {
     const float* p;
-    long long ld;
+    long long ld, seg;
     int rows;            // valid m (the other dimension of the product is bounded by its K)
-    int skip_every;      // m-major: row k of the product is row k + k / skip_every + skip_first of the array (0: row k)
-    int skip_first;
 };
 struct Product {
     Operand a, b;
     float* c;
     long long ldc;
-    float* a_sums;       // column sums of an m-major A (bias gradient), written by the first column of tiles; or null
-    int K;
+    float* a_sums;       // sums over k and the segments of an m-major A (bias gradient), from the first column of tiles; or null
+    int K, n_seg;
     int tile0, tiles_n;  // first tile of this product in the launch, tiles per tile row
 };
 
-// One thread's share of a 64 x 16 slab: 4 values along the operand's contiguous dimension.
-template <bool K_MAJOR, bool VEC>
-__device__ __forceinline__ float4 load_slab(const Operand& o, int m0, int k0, int K, int tid) {
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
+// Vector v of a T x TK slab: 4 values along the operand's contiguous dimension.
+template <int T, int TK, bool K_MAJOR, bool VEC>
+__device__ __forceinline__ float4 load_slab(const float* base, long long ld, int rows, int m0, int k0, int K, int v) {
+    float r[4] = {0.f, 0.f, 0.f, 0.f};
     if (K_MAJOR) {
-        const int m = m0 + (tid >> 2), k = k0 + (tid & 3) * 4;
-        if (m < o.rows) {
-            const float* p = o.p + m * o.ld + k;
+        const int m = m0 + v / (TK / 4), k = k0 + v % (TK / 4) * 4;
+        if (m < rows) {
+            const float* p = base + m * ld + k;
             if (VEC && k + 3 < K) return *reinterpret_cast<const float4*>(p);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                if (k + i < K) v[i] = p[i];
+                if (k + i < K) r[i] = p[i];
         }
     } else {
-        const int k = k0 + (tid >> 4), m = m0 + (tid & 15) * 4;
+        const int k = k0 + v / (T / 4), m = m0 + v % (T / 4) * 4;
         if (k < K) {
-            const long long row = o.skip_every ? k + k / o.skip_every + o.skip_first : k;
-            const float* p = o.p + row * o.ld + m;
-            if (VEC && m + 3 < o.rows) return *reinterpret_cast<const float4*>(p);
+            const float* p = base + k * ld + m;
+            if (VEC && m + 3 < rows) return *reinterpret_cast<const float4*>(p);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                if (m + i < o.rows) v[i] = p[i];
+                if (m + i < rows) r[i] = p[i];
         }
     }
-    return make_float4(v[0], v[1], v[2], v[3]);
+    return make_float4(r[0], r[1], r[2], r[3]);
 }
-template <bool K_MAJOR>
-__device__ __forceinline__ void store_slab(float (*s)[kTilePad], const float4& v, int tid) {
+template <int T, int TK, bool K_MAJOR>
+__device__ __forceinline__ void store_slab(float (*s)[T + 4], const float4& q, int v) {
     if (K_MAJOR) {
-        const int m = tid >> 2, k = (tid & 3) * 4;
-        s[k][m] = v.x; s[k + 1][m] = v.y; s[k + 2][m] = v.z; s[k + 3][m] = v.w;
+        const int m = v / (TK / 4), k = v % (TK / 4) * 4;
+        s[k][m] = q.x; s[k + 1][m] = q.y; s[k + 2][m] = q.z; s[k + 3][m] = q.w;
     } else {
-        *reinterpret_cast<float4*>(&s[tid >> 4][(tid & 15) * 4]) = v;
+        *reinterpret_cast<float4*>(&s[v / (T / 4)][v % (T / 4) * 4]) = q;
+    }
+}
+template <int R>
+__device__ __forceinline__ void load_regs(float (&r)[R], const float* p) {
+    if (R == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p);
+        r[0] = q.x; r[1] = q.y; r[2 % R] = q.z; r[3 % R] = q.w;
+    } else {
+        const float2 q = *reinterpret_cast<const float2*>(p);
+        r[0] = q.x; r[1] = q.y;
     }
 }
 
-struct TileSmem {
-    float a[2][kTileK][kTilePad];
-    float b[2][kTileK][kTilePad];
-};
-
-// acc += A(m0.., k) B(n0.., k) for k in [k_begin, k_end).  load_b(k0) supplies the thread's share of B's slab.
-template <bool A_KMAJOR, bool B_KMAJOR, bool VEC, bool SUMS, typename LoadB>
-__device__ __forceinline__ void tile_product(TileSmem& sm, const Operand& a, int m0, int k_begin, int k_end, LoadB load_b,
-                                             float (&acc)[4][4], float& a_sum) {
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    float4 ra = load_slab<A_KMAJOR, VEC>(a, m0, k_begin, k_end, tid), rb = load_b(k_begin);
-    int buf = 0;
-    for (int k0 = k_begin; k0 < k_end; k0 += kTileK, buf ^= 1) {
-        store_slab<A_KMAJOR>(sm.a[buf], ra, tid);
-        store_slab<B_KMAJOR>(sm.b[buf], rb, tid);
-        __syncthreads();
-        if (k0 + kTileK < k_end) {
-            ra = load_slab<A_KMAJOR, VEC>(a, m0, k0 + kTileK, k_end, tid);
-            rb = load_b(k0 + kTileK);
+// acc[i][j] = sum over segments and k of A(m0 + .., k) B(n0 + .., k).  load_b(k0, s, v) supplies vector v of B's slab.
+template <typename T, bool A_KMAJOR, bool B_KMAJOR, bool VEC, bool SUMS, bool SEGMENTS, typename LoadB>
+__device__ __forceinline__ void tile_product(typename T::Smem& sm, const Operand& a, int m0, int K, int n_seg, LoadB load_b,
+                                             float (&acc)[T::RM][T::RN], float& a_sum) {
+    const int tid = threadIdx.x, tx = tid % (T::TN / T::RN), ty = tid / (T::TN / T::RN);
+    float4 ra[T::kAVecs], rb[T::kBVecs];
+    const auto fetch = [&](int k0, int s) {
+#pragma unroll
+        for (int u = 0; u < T::kAVecs; ++u)
+            ra[u] = load_slab<T::TM, T::TK, A_KMAJOR, VEC>(a.p + (SEGMENTS ? s * a.seg : 0), a.ld, a.rows, m0, k0, K, tid + u * T::kThreads);
+#pragma unroll
+        for (int u = 0; u < T::kBVecs; ++u) rb[u] = load_b(k0, s, tid + u * T::kThreads);
+    };
+    float total[T::RM][T::RN] = {};
+    fetch(0, 0);
+    int buf = 0, k0 = 0, s = 0;
+    while (true) {
+#pragma unroll
+        for (int u = 0; u < T::kAVecs; ++u) store_slab<T::TM, T::TK, A_KMAJOR>(sm.a[buf], ra[u], tid + u * T::kThreads);
+#pragma unroll
+        for (int u = 0; u < T::kBVecs; ++u) store_slab<T::TN, T::TK, B_KMAJOR>(sm.b[buf], rb[u], tid + u * T::kThreads);
+        __syncthreads();                 // one barrier per slab: the buffer written next was read before this barrier
+        int k_next = k0 + T::TK, s_next = s;
+        if (k_next >= K) { k_next = 0; ++s_next; }
+        const bool more = SEGMENTS ? s_next < n_seg : s_next == 0;
+        if (more) fetch(k_next, s_next);
+#pragma unroll
+        for (int k = 0; k < T::TK; ++k) {
+            float x[T::RM], y[T::RN];
+            load_regs<T::RM>(x, &sm.a[buf][k][T::RM * ty]);
+            load_regs<T::RN>(y, &sm.b[buf][k][T::RN * tx]);
+#pragma unroll
+            for (int i = 0; i < T::RM; ++i)
+#pragma unroll
+                for (int j = 0; j < T::RN; ++j) acc[i][j] = fmaf(x[i], y[j], acc[i][j]);
         }
+        if (SUMS && tid < T::TM) {
 #pragma unroll
-        for (int k = 0; k < kTileK; ++k) {
-            const float4 av = *reinterpret_cast<const float4*>(&sm.a[buf][k][4 * ty]);
-            const float4 bv = *reinterpret_cast<const float4*>(&sm.b[buf][k][4 * tx]);
-            const float x[4] = {av.x, av.y, av.z, av.w}, y[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(x[i], y[j], acc[i][j]);
+            for (int k = 0; k < T::TK; ++k) a_sum += sm.a[buf][k][tid];
         }
-        if (SUMS && tid < kTile) {
+        if (SEGMENTS && s_next != s) {
 #pragma unroll
-            for (int k = 0; k < kTileK; ++k) a_sum += sm.a[buf][k][tid];
+            for (int i = 0; i < T::RM; ++i)
+#pragma unroll
+                for (int j = 0; j < T::RN; ++j) { total[i][j] += acc[i][j]; acc[i][j] = 0.f; }
         }
-        // the other buffer is written next; whoever still reads this one is at most one slab behind (one barrier per slab)
+        if (!more) break;
+        k0 = k_next;
+        s = s_next;
+        buf ^= 1;
     }
-    __syncthreads();
+    if (SEGMENTS) {
+#pragma unroll
+        for (int i = 0; i < T::RM; ++i)
+#pragma unroll
+            for (int j = 0; j < T::RN; ++j) acc[i][j] = total[i][j];
+    }
 }
 
-__device__ __forceinline__ void store_tile(float* c, long long ldc, int m0, int n0, int M, int N, const float (&acc)[4][4]) {
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, n = n0 + 4 * tx;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + 4 * ty + i;
-        if (m >= M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (n + j < N) c[m * ldc + n + j] = acc[i][j];
-    }
-}
-
-// A list of products in one launch, K split over gridDim.y parts: part y goes to c + y * part_stride and whoever uses
-// the result adds the parts in order.  Parts are multiples of kTileK.
 constexpr int kMaxProducts = 16;
 struct ProductList {
     Product p[kMaxProducts];
     int n;
-    int k_part;
-    long long part_stride;
 };
 
-template <bool A_KMAJOR, bool B_KMAJOR, bool VEC>
-__global__ void __launch_bounds__(kGemmThreads, 2) k_products(const __grid_constant__ ProductList list) {
-    __shared__ __align__(16) TileSmem sm;
-    dependency_wait();
-    launch_dependents();
-    int which = 0;
-    while (which + 1 < list.n && static_cast<int>(blockIdx.x) >= list.p[which + 1].tile0) ++which;
-    const Product& q = list.p[which];
-    const int tile = blockIdx.x - q.tile0, m0 = tile / q.tiles_n * kTile, n0 = tile % q.tiles_n * kTile;
-    const int k_begin = blockIdx.y * list.k_part;
-    const int k_end = min(q.K, k_begin + list.k_part);
-    float acc[4][4] = {};
+template <typename T, bool A_KMAJOR, bool B_KMAJOR, bool VEC, bool SEGMENTS>
+__device__ __forceinline__ void run_product(typename T::Smem& sm, const Product& q, int tile) {
+    const int m0 = tile / q.tiles_n * T::TM, n0 = tile % q.tiles_n * T::TN;
     float a_sum = 0.f;
-    const auto load_b = [&](int k0) { return load_slab<B_KMAJOR, VEC>(q.b, n0, k0, k_end, threadIdx.x); };
-    if (q.b.rows == 0) {                       // column sums only: sum_k A(m, k)
-        if (threadIdx.x < kTile && m0 + static_cast<int>(threadIdx.x) < q.a.rows) {
-            for (int k = k_begin; k < k_end; ++k) a_sum += q.a.p[k * q.a.ld + m0 + threadIdx.x];
+    if (q.b.rows == 0) {                       // sums only
+        if (threadIdx.x < T::TM && m0 + static_cast<int>(threadIdx.x) < q.a.rows) {
+#pragma unroll 8
+            for (int k = 0; k < q.K; ++k) a_sum += q.a.p[k * q.a.ld + m0 + threadIdx.x];
             q.a_sums[m0 + threadIdx.x] = a_sum;
         }
         return;
     }
-    if (q.a_sums && n0 == 0) {
-        tile_product<A_KMAJOR, B_KMAJOR, VEC, true>(sm, q.a, m0, k_begin, k_end, load_b, acc, a_sum);
-        if (threadIdx.x < kTile && m0 + static_cast<int>(threadIdx.x) < q.a.rows) q.a_sums[m0 + threadIdx.x] = a_sum;
+    float acc[T::RM][T::RN] = {};
+    const auto load_b = [&](int k0, int s, int v) {
+        return load_slab<T::TN, T::TK, B_KMAJOR, VEC>(q.b.p + (SEGMENTS ? s * q.b.seg : 0), q.b.ld, q.b.rows, n0, k0, q.K, v);
+    };
+    if (SEGMENTS && q.a_sums && n0 == 0) {
+        tile_product<T, A_KMAJOR, B_KMAJOR, VEC, true, SEGMENTS>(sm, q.a, m0, q.K, q.n_seg, load_b, acc, a_sum);
+        if (threadIdx.x < T::TM && m0 + static_cast<int>(threadIdx.x) < q.a.rows) q.a_sums[m0 + threadIdx.x] = a_sum;
     } else {
-        tile_product<A_KMAJOR, B_KMAJOR, VEC, false>(sm, q.a, m0, k_begin, k_end, load_b, acc, a_sum);
+        tile_product<T, A_KMAJOR, B_KMAJOR, VEC, false, SEGMENTS>(sm, q.a, m0, q.K, q.n_seg, load_b, acc, a_sum);
     }
-    store_tile(q.c + blockIdx.y * list.part_stride, q.ldc, m0, n0, q.a.rows, q.b.rows, acc);
+    const int m = m0 + T::RM * static_cast<int>(threadIdx.x / (T::TN / T::RN)), n = n0 + T::RN * static_cast<int>(threadIdx.x % (T::TN / T::RN));
+#pragma unroll
+    for (int i = 0; i < T::RM; ++i) {
+        if (m + i >= q.a.rows) continue;
+#pragma unroll
+        for (int j = 0; j < T::RN; ++j)
+            if (n + j < q.b.rows) q.c[(m + i) * q.ldc + n + j] = acc[i][j];
+    }
+}
+
+template <typename T, bool A_KMAJOR, bool B_KMAJOR, bool VEC, bool SEGMENTS>
+__global__ void __launch_bounds__(T::kThreads) k_products(const __grid_constant__ ProductList list) {
+    __shared__ __align__(16) typename T::Smem sm;
+    dependency_wait();
+    launch_dependents();
+    int which = 0;
+    while (which + 1 < list.n && static_cast<int>(blockIdx.x) >= list.p[which + 1].tile0) ++which;
+    run_product<T, A_KMAJOR, B_KMAJOR, VEC, SEGMENTS>(sm, list.p[which], blockIdx.x - list.p[which].tile0);
 }
 
 // ---- emission head and its density ---------------------------------------------------------------------------------
@@ -183,24 +222,25 @@ __global__ void __launch_bounds__(kGemmThreads, 2) k_products(const __grid_const
 // means, then the log-variances, of workers 2t and 2t+1, so a thread holds both halves of its workers), and at once
 //   log N(x; m, exp(lv)) summed over the tile's workers -> part[tile column][row],
 //   d_head = [r inv | -1/2 + r^2 inv / 2],  r = x - m, inv = exp(-lv)                    (d_head: null = forward only).
-constexpr int kHeadWorkers = kTile / 2;
+constexpr int kHeadWorkers = LargeTile::TN / 2;
 
 template <bool VEC>
-__global__ void __launch_bounds__(kGemmThreads, 2) k_emission_density(const float* __restrict__ v, const float* __restrict__ W4,
-                                                                      const float* __restrict__ b4, const float* __restrict__ x,
-                                                                      int R, int N, int H, float* __restrict__ d_head,
-                                                                      float* __restrict__ part) {
-    __shared__ __align__(16) TileSmem sm;
+__global__ void __launch_bounds__(LargeTile::kThreads, 2) k_emission_density(const float* __restrict__ v, const float* __restrict__ W4,
+                                                                             const float* __restrict__ b4, const float* __restrict__ x,
+                                                                             int R, int N, int H, float* __restrict__ d_head,
+                                                                             float* __restrict__ part) {
+    using T = LargeTile;
+    __shared__ __align__(16) T::Smem sm;
     dependency_wait();
     launch_dependents();
-    const int head_tiles = (N + kHeadWorkers - 1) / kHeadWorkers;          // one-dimensional grid: rows reach 2^24
-    const int m0 = blockIdx.x / head_tiles * kTile, head_tile = blockIdx.x % head_tiles, j0 = head_tile * kHeadWorkers;
-    const Operand a{v, H, R, 0, 0};
-    const int tid = threadIdx.x, col = tid >> 2;                             // the column of B this thread loads
+    const int head_tiles = (N + kHeadWorkers - 1) / kHeadWorkers;            // one-dimensional grid: rows reach 2^24
+    const int m0 = blockIdx.x / head_tiles * T::TM, head_tile = blockIdx.x % head_tiles, j0 = head_tile * kHeadWorkers;
+    const Operand a{v, H, 0, R};
+    const int tid = threadIdx.x, col = tid / (T::TK / 4);                    // the column of B this thread loads
     const int worker = j0 + 2 * (col >> 2) + (col & 1), head = (col >> 1) & 1;
     const float* wrow = W4 + (static_cast<long long>(head) * N + (worker < N ? worker : 0)) * H;
-    const auto load_b = [&](int k0) {
-        const int k = k0 + (tid & 3) * 4;
+    const auto load_b = [&](int k0, int, int vec) {
+        const int k = k0 + vec % (T::TK / 4) * 4;
         if (worker >= N) return make_float4(0.f, 0.f, 0.f, 0.f);
         if (VEC && k + 3 < H) return *reinterpret_cast<const float4*>(wrow + k);
         float t[4];
@@ -208,9 +248,10 @@ __global__ void __launch_bounds__(kGemmThreads, 2) k_emission_density(const floa
         for (int i = 0; i < 4; ++i) t[i] = k + i < H ? wrow[k + i] : 0.f;
         return make_float4(t[0], t[1], t[2], t[3]);
     };
-    float acc[4][4] = {};
+    static_assert(T::kBVecs == 1, "one column of B per thread");
+    float acc[T::RM][T::RN] = {};
     float unused = 0.f;
-    tile_product<true, true, VEC, false>(sm, a, m0, 0, H, load_b, acc, unused);
+    tile_product<T, true, true, VEC, false, false>(sm, a, m0, H, 1, load_b, acc, unused);
     const int tx = tid & 15, ty = tid >> 4;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -236,205 +277,207 @@ __global__ void __launch_bounds__(kGemmThreads, 2) k_emission_density(const floa
     }
 }
 
-// elbo[b] = what the guide and the transition contributed + the emission densities of the window's rows: a warp per window
-__global__ void __launch_bounds__(128) k_elbo_finish(const float* __restrict__ part, int n_part, int R, int W, int B,
-                                                     const float* __restrict__ path, float* __restrict__ elbo) {
-    dependency_wait();
-    launch_dependents();
-    const int b = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (b >= B) return;
+// elbo[b] = what the guide and the transition contributed + the emission densities of the window's rows (one warp)
+__device__ __forceinline__ void window_elbo(const float* __restrict__ part, int n_part, int R, int W, int b,
+                                            const float* __restrict__ path, float* __restrict__ elbo, int lane) {
     float s = 0.f;
     for (int i = lane; i < n_part * W; i += 32) s += part[static_cast<long long>(i / W) * R + b * W + i % W];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) elbo[b] = path[b] + s;
 }
-
-// ---- the two RNNs --------------------------------------------------------------------------------------------------
-// h_t = relu(P_t + Wh h_{t -+ 1}) for kRnnRows windows and one direction per CTA, all steps.  A row of Wh is dotted with
-// the states by 8 lanes; every weight read serves the CTA's windows.  Wh sits in shared memory when it fits
-// (H <= 200), else it is streamed from L2 at every step (64 bytes per clock and SM: 2 us a step at H = 256, with 4 windows
-// about what their multiply-adds take).  States: [B][W + 1][H]; forward: slot 0 = a0, slot t + 1 = a_t;  backward:
-// slot t = b_t, slot W = b0 -- so "the state before" of row t is slot t (forward) or slot t + 1 (backward).
-constexpr int kRnnRows = 4, kRnnThreads = 512;
-constexpr int kRnnSmemH = 200;
-
-struct RnnArgs {
-    const float* proj;              // [parts][R][2H]: input projections, forward then backward, to be added over the parts
-    int n_parts;
-    long long part_stride;
-    const float *Wh[2], *bias[2], *init[2];
-    float* state[2];
-    int B, W, H;
-};
-
-inline size_t rnn_smem_bytes(int H, bool staged) {
-    return sizeof(float) * (2 * static_cast<size_t>(kRnnRows) * H + (staged ? static_cast<size_t>(H) * (H + 4) : 0));
+__global__ void __launch_bounds__(128) k_elbo_finish(const float* __restrict__ part, int n_part, int R, int W, int B,
+                                                     const float* __restrict__ path, float* __restrict__ elbo) {
+    dependency_wait();
+    launch_dependents();
+    const int b = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (b < B) window_elbo(part, n_part, R, W, b, path, elbo, threadIdx.x & 31);
 }
 
-template <bool VEC>
-__global__ void __launch_bounds__(kRnnThreads) k_rnn_forward(RnnArgs a, int staged) {
-    extern __shared__ __align__(16) float sm[];
-    const int H = a.H, W = a.W, dir = blockIdx.y, b0 = blockIdx.x * kRnnRows;
-    float* cur = sm;                                   // [kRnnRows][H]
-    float* next = sm + kRnnRows * H;
-    const float* Wh = a.Wh[dir];
-    int ldw = H;
-    if (staged) {                                      // rows padded by 4: four consecutive rows fall into different banks
-        float* sW = sm + 2 * kRnnRows * H;
-        ldw = H + 4;
-        for (int i = threadIdx.x; i < H * H; i += kRnnThreads) sW[(i / H) * ldw + i % H] = Wh[i];
-        Wh = sW;
+// ---- the two RNNs --------------------------------------------------------------------------------------------------
+// h_t = relu(P_t + Wh h_{t -+ 1}) for RW windows and one direction per cluster, all steps.  A CTA of the cluster owns
+// ceil(H / cluster) hidden units: their share of Wh sits in its shared memory for all steps (or, if not even eight CTAs can hold
+// it, passes through it in chunks of k at every step), one thread per unit runs the chains of the RW windows, and every
+// new value is written into the next-state buffers of all CTAs of the cluster; one cluster barrier per step.  What
+// bounds a step is shared-memory wavefronts: one per k and warp for the weights, RW / 4 for the states (H = 256: 2 CTAs, 128
+// threads each, about 1500 clocks with RW = 2).
+// States: [B][W + 1][H]; forward: slot 0 = a0, slot t + 1 = a_t;  backward: slot t = b_t, slot W = b0 -- so "the state
+// before" of row t is slot t (forward) or slot t + 1 (backward).
+struct RnnArgs {
+    const float* proj;              // [R][2H]: input projections, forward then backward
+    const float *Wh[2], *bias[2], *init[2];
+    float* state[2];
+    // backward pass
+    const float* g;                 // [R][H]: d ELBO / d h_t from the combiner, the same for both directions
+    float* d_pre[2];                // [R][H]
+    float* carry_out[2];            // [B][H]: gradient of the initial state, per window
+    int B, W, H;
+    int cluster, units;             // CTAs per cluster, units per CTA
+    int chunk;                      // k rows of the weights in shared memory at a time (H: all of them, loaded once)
+};
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void store_all(float* p, float v, int cluster) {
+    const uint32_t local = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+    for (int c = 0; c < cluster; ++c) {
+        uint32_t remote;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(c));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
     }
+}
+
+// Pitch of a window's state vector and of a weight row: both read without bank conflicts (rows of 16-byte chunks; the
+// transposing copy writes consecutive k, so the pitch of a weight row is odd).
+__host__ __device__ inline int rnn_state_pitch(int H) { return (H + 3) / 4 * 4; }
+__host__ __device__ inline int rnn_weight_pitch(int units) { return units | 1; }
+inline size_t rnn_smem_bytes(int H, int units, int chunk, int rw) {
+    return sizeof(float) * (2 * static_cast<size_t>(rw) * rnn_state_pitch(H) + static_cast<size_t>(chunk) * rnn_weight_pitch(units));
+}
+
+// acc[w] += sum_k sW[k][unit] x[w][k0 + k] for k < n, ascending: one chain per window
+template <int RW>
+__device__ __forceinline__ void rnn_chains(const float* sW, int pitch, const float* x, int xp, int n, float (&acc)[RW]) {
+    int k = 0;
+#pragma unroll 2
+    for (; k + 4 <= n; k += 4) {
+        float4 xv[RW];
+#pragma unroll
+        for (int w = 0; w < RW; ++w) xv[w] = *reinterpret_cast<const float4*>(x + w * xp + k);
+        const float w0 = sW[k * pitch], w1 = sW[(k + 1) * pitch], w2 = sW[(k + 2) * pitch], w3 = sW[(k + 3) * pitch];
+#pragma unroll
+        for (int w = 0; w < RW; ++w) acc[w] = fmaf(w3, xv[w].w, fmaf(w2, xv[w].z, fmaf(w1, xv[w].y, fmaf(w0, xv[w].x, acc[w]))));
+    }
+    for (; k < n; ++k)
+#pragma unroll
+        for (int w = 0; w < RW; ++w) acc[w] = fmaf(sW[k * pitch], x[w * xp + k], acc[w]);
+}
+
+template <int RW>
+__global__ void __launch_bounds__(256) k_rnn_forward(RnnArgs a) {
+    extern __shared__ __align__(16) float sm[];
+    const int H = a.H, W = a.W, xp = rnn_state_pitch(H), wp = rnn_weight_pitch(a.units), T = blockDim.x;
+    const int rank = static_cast<int>(cluster_rank()), dir = blockIdx.y, b0 = static_cast<int>(blockIdx.x) / a.cluster * RW;
+    const int u0 = rank * a.units, units = min(a.units, H - u0), tid = threadIdx.x;
+    float* cur = sm;                                   // [RW][xp]
+    float* next = sm + RW * xp;
+    float* sW = sm + 2 * RW * xp;                      // [chunk][wp]: sW[k][u] = Wh[u0 + u][k]
+    const float* Wh = a.Wh[dir] + static_cast<long long>(u0) * H;
+    const auto stage = [&](int k0, int n) {
+        for (int i = tid; i < units * n; i += T) sW[(i % n) * wp + i / n] = Wh[static_cast<long long>(i / n) * H + k0 + i % n];
+    };
+    if (a.chunk >= H) stage(0, H);                     // weights: no kernel of this step writes them
     dependency_wait();
     launch_dependents();
     float* state = a.state[dir];
-    for (int i = threadIdx.x; i < kRnnRows * H; i += kRnnThreads) {
-        const int rb = i / H, h = i % H;
+    for (int i = tid; i < RW * H; i += T) {
+        const int w = i / H, h = i % H;
         const float s = a.init[dir][h];
-        cur[i] = s;
-        if (b0 + rb < a.B) state[(static_cast<long long>(b0 + rb) * (W + 1) + (dir ? W : 0)) * H + h] = s;
+        cur[w * xp + h] = s;
+        if (rank == 0 && b0 + w < a.B) state[(static_cast<long long>(b0 + w) * (W + 1) + (dir ? W : 0)) * H + h] = s;
     }
-    __syncthreads();
-    const int part = threadIdx.x & 7, group = threadIdx.x >> 3;
+    cluster_sync();                                    // every CTA has started before anyone writes into it
+    const int h = u0 + tid;
+    const bool mine = tid < units;
+    const float bias = mine ? a.bias[dir][h] : 0.f;
     for (int s = 0; s < W; ++s) {
         const int t = dir ? W - 1 - s : s;
-        for (int h0 = group; h0 < ((H + 3) & ~3); h0 += kRnnThreads / 8) {        // a warp's four groups stay together
-            const int h = h0 < H ? h0 : H - 1;
-            float acc[kRnnRows] = {};
-            const float* wrow = Wh + static_cast<long long>(h) * ldw;
-            if (VEC) {
-#pragma unroll 4
-                for (int c = 4 * part; c < H; c += 32) {
-                    const float4 w = *reinterpret_cast<const float4*>(wrow + c);
+        float p[RW], acc[RW];
 #pragma unroll
-                    for (int rb = 0; rb < kRnnRows; ++rb) {
-                        const float4 x = *reinterpret_cast<const float4*>(cur + rb * H + c);
-                        acc[rb] = fmaf(w.x, x.x, fmaf(w.y, x.y, fmaf(w.z, x.z, fmaf(w.w, x.w, acc[rb]))));
-                    }
-                }
-            } else {
-                for (int c = part; c < H; c += 8) {
-                    const float w = wrow[c];
-#pragma unroll
-                    for (int rb = 0; rb < kRnnRows; ++rb) acc[rb] = fmaf(w, cur[rb * H + c], acc[rb]);
-                }
+        for (int w = 0; w < RW; ++w) {
+            acc[w] = 0.f;
+            p[w] = mine && b0 + w < a.B ? a.proj[(static_cast<long long>(b0 + w) * W + t) * 2 * H + dir * H + h] + bias : 0.f;
+        }
+        for (int k0 = 0; k0 < H; k0 += a.chunk) {
+            const int n = min(a.chunk, H - k0);
+            if (a.chunk < H) {
+                __syncthreads();
+                stage(k0, n);
+                __syncthreads();
             }
+            if (mine) rnn_chains<RW>(sW + tid, wp, cur + k0, xp, n, acc);
+        }
+        if (mine) {
 #pragma unroll
-            for (int rb = 0; rb < kRnnRows; ++rb) {
-                acc[rb] += __shfl_xor_sync(0xffffffffu, acc[rb], 1);
-                acc[rb] += __shfl_xor_sync(0xffffffffu, acc[rb], 2);
-                acc[rb] += __shfl_xor_sync(0xffffffffu, acc[rb], 4);
-            }
-            // lane `part` finishes window `part`
-            float mine = 0.f;
-#pragma unroll
-            for (int rb = 0; rb < kRnnRows; ++rb)
-                if (rb == part) mine = acc[rb];
-            if (part < kRnnRows && b0 + part < a.B && h0 < H) {
-                const long long r = static_cast<long long>(b0 + part) * W + t;
-                float p = a.bias[dir][h];
-                for (int k = 0; k < a.n_parts; ++k) p += a.proj[k * a.part_stride + r * 2 * H + dir * H + h];
-                const float v = fmaxf(mine + p, 0.f);
-                next[part * H + h] = v;
-                state[(static_cast<long long>(b0 + part) * (W + 1) + (dir ? t : t + 1)) * H + h] = v;
+            for (int w = 0; w < RW; ++w) {
+                const float v = fmaxf(acc[w] + p[w], 0.f);
+                store_all(next + w * xp + h, v, a.cluster);
+                if (b0 + w < a.B) state[(static_cast<long long>(b0 + w) * (W + 1) + (dir ? t : t + 1)) * H + h] = v;
             }
         }
-        __syncthreads();
+        cluster_sync();
         float* swap = cur; cur = next; next = swap;
     }
 }
 
-// Backwards through the same recurrences: d_pre_t = (g_t + carry) (h_t > 0), carry = d_pre_t Wh.  g_t = d ELBO / d h_t
-// from the combiner (the same for both directions).  A thread owns four columns of carry and every kSlices-th row of Wh.
-struct RnnBackArgs {
-    const float* g;                 // [R][H]
-    const float* state[2];
-    const float* Wh[2];
-    float* d_pre[2];                // [R][H]
-    float* carry_out[2];            // [B][H]: gradient of the initial state, per window
-    int B, W, H;
-};
-
-inline size_t rnn_back_smem_bytes(int H, bool staged) {
-    const size_t slices = kRnnThreads / ((H + 3) / 4) > 0 ? kRnnThreads / ((H + 3) / 4) : 1;
-    return sizeof(float) * (static_cast<size_t>(kRnnRows) * H * (2 + slices) + (staged ? static_cast<size_t>(H) * H : 0));
-}
-
-template <bool VEC>
-__global__ void __launch_bounds__(kRnnThreads) k_rnn_backward(RnnBackArgs a, int staged) {
+// Backwards through the same recurrences: d_pre_t = (g_t + carry) (h_t > 0), carry = d_pre_t Wh: a CTA owns columns of Wh.
+template <int RW>
+__global__ void __launch_bounds__(256) k_rnn_backward(RnnArgs a) {
     extern __shared__ __align__(16) float sm[];
-    const int H = a.H, W = a.W, dir = blockIdx.y, b0 = blockIdx.x * kRnnRows;
-    const int groups = (H + 3) / 4, slices = kRnnThreads / groups > 0 ? kRnnThreads / groups : 1;
-    float* dpre = sm;                                  // [H][kRnnRows]: one 16-byte read gives a unit's value in every window
-    float* carry = dpre + kRnnRows * H;                // [kRnnRows][H]
-    float* red = carry + kRnnRows * H;                 // [slices][kRnnRows][H]
-    const float* Wh = a.Wh[dir];
-    if (staged) {
-        float* sW = red + static_cast<size_t>(slices) * kRnnRows * H;
-        for (int i = threadIdx.x; i < H * H; i += kRnnThreads) sW[i] = Wh[i];
-        Wh = sW;
-    }
+    const int H = a.H, W = a.W, xp = rnn_state_pitch(H), wp = rnn_weight_pitch(a.units), T = blockDim.x;
+    const int rank = static_cast<int>(cluster_rank()), dir = blockIdx.y, b0 = static_cast<int>(blockIdx.x) / a.cluster * RW;
+    const int u0 = rank * a.units, units = min(a.units, H - u0), tid = threadIdx.x;
+    float* cur = sm;                                   // [RW][xp]: d_pre of this step, all units
+    float* next = sm + RW * xp;
+    float* sW = sm + 2 * RW * xp;                      // [chunk][wp]: sW[i][u] = Wh[i][u0 + u]
+    const float* Wh = a.Wh[dir] + u0;
+    const auto stage = [&](int k0, int n) {
+        for (int i = tid; i < units * n; i += T) sW[(i / units) * wp + i % units] = Wh[static_cast<long long>(k0 + i / units) * H + i % units];
+    };
+    if (a.chunk >= H) stage(0, H);
     dependency_wait();
     launch_dependents();
-    for (int i = threadIdx.x; i < kRnnRows * H; i += kRnnThreads) carry[i] = 0.f;
-    __syncthreads();
+    cluster_sync();
+    const int h = u0 + tid;
+    const bool mine = tid < units;
+    float carry[RW];
+#pragma unroll
+    for (int w = 0; w < RW; ++w) carry[w] = 0.f;
     for (int s = 0; s < W; ++s) {
         const int t = dir ? s : W - 1 - s;
-        for (int i = threadIdx.x; i < kRnnRows * H; i += kRnnThreads) {
-            const int rb = i / H, h = i % H;
-            float d = 0.f;
-            if (b0 + rb < a.B) {
-                const long long r = static_cast<long long>(b0 + rb) * W + t;
-                const float act = a.state[dir][(static_cast<long long>(b0 + rb) * (W + 1) + (dir ? t : t + 1)) * H + h];
-                d = act > 0.f ? a.g[r * H + h] + carry[i] : 0.f;
-                a.d_pre[dir][r * H + h] = d;
-            }
-            dpre[h * kRnnRows + rb] = d;
-        }
-        __syncthreads();
-        for (int w = threadIdx.x; w < groups * slices; w += kRnnThreads) {
-            const int c = (w % groups) * 4, slice = w / groups;
-            float acc[kRnnRows][4] = {};
-#pragma unroll 4
-            for (int i = slice; i < H; i += slices) {
-                float wv[4];
-                const float* p = Wh + static_cast<long long>(i) * H + c;
-                if (VEC) {
-                    const float4 q = *reinterpret_cast<const float4*>(p);
-                    wv[0] = q.x; wv[1] = q.y; wv[2] = q.z; wv[3] = q.w;
-                } else {
+        if (mine) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) wv[j] = c + j < H ? p[j] : 0.f;
+            for (int w = 0; w < RW; ++w) {
+                float d = 0.f;
+                if (b0 + w < a.B) {
+                    const long long r = static_cast<long long>(b0 + w) * W + t;
+                    const float act = a.state[dir][(static_cast<long long>(b0 + w) * (W + 1) + (dir ? t : t + 1)) * H + h];
+                    d = act > 0.f ? a.g[r * H + h] + carry[w] : 0.f;
+                    a.d_pre[dir][r * H + h] = d;
                 }
-                const float4 d4 = *reinterpret_cast<const float4*>(dpre + i * kRnnRows);
-                const float dv[kRnnRows] = {d4.x, d4.y, d4.z, d4.w};
-#pragma unroll
-                for (int rb = 0; rb < kRnnRows; ++rb)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[rb][j] = fmaf(dv[rb], wv[j], acc[rb][j]);
+                store_all(cur + w * xp + h, d, a.cluster);
+                carry[w] = 0.f;
             }
-#pragma unroll
-            for (int rb = 0; rb < kRnnRows; ++rb)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (c + j < H) red[(slice * kRnnRows + rb) * H + c + j] = acc[rb][j];
         }
-        __syncthreads();
-        for (int i = threadIdx.x; i < kRnnRows * H; i += kRnnThreads) {
-            float v = 0.f;
-            for (int k = 0; k < slices; ++k) v += red[k * kRnnRows * H + i];
-            carry[i] = v;
+        cluster_sync();
+        for (int k0 = 0; k0 < H; k0 += a.chunk) {
+            const int n = min(a.chunk, H - k0);
+            if (a.chunk < H) {
+                __syncthreads();
+                stage(k0, n);
+                __syncthreads();
+            }
+            if (mine) rnn_chains<RW>(sW + tid, wp, cur + k0, xp, n, carry);
         }
-        // the next step reads only the carry entries this thread has just written, and dpre, red are rewritten behind a barrier
-        __syncthreads();
+        // the other buffer is written next: its readers passed the cluster barrier of this step
+        float* swap = cur; cur = next; next = swap;
     }
-    for (int i = threadIdx.x; i < kRnnRows * H; i += kRnnThreads)
-        if (b0 + i / H < a.B) a.carry_out[dir][static_cast<long long>(b0 + i / H) * H + i % H] = carry[i];
+    if (mine)
+#pragma unroll
+        for (int w = 0; w < RW; ++w)
+            if (b0 + w < a.B) a.carry_out[dir][static_cast<long long>(b0 + w) * H + h] = carry[w];
+    cluster_sync();                                    // nobody leaves while others may still write into its buffers
 }
 
 // ---- the sampled path: guide, transition density, hidden layers -------------------------------------------------------
-// One CTA per window.  The small matrices sit in shared memory (rows padded to an odd length) when they fit.
+// One CTA per window.  The small matrices sit in shared memory (rows padded to an odd length) when they fit.  A latent
+// result is a chain over the H hidden units, one thread each (D to 3D of them): about 5 clocks per unit.
 constexpr int kPathThreads = 256;
 
 struct PathArgs {
@@ -447,35 +490,29 @@ struct PathArgs {
     float* dzt;                     // [R][D]: d log p(z_t | z_{t-1}) / d z_t
     float* path;                    // [B]: guide and transition part of the ELBO
     // backward
-    const float* dv_parts;          // [parts][R][H]: d_head W4, to be added over the parts
-    int n_parts;
-    long long part_stride;
+    const float* part;              // emission densities, see k_emission_density
+    int n_part;
+    float* elbo;
+    const float* dv_raw;            // [R][H]: d_head W4
     float *dv, *du, *dpc, *dh, *dmu, *dps;
     float* gz0;                     // [B][D]
     int B, W, D, H;
 };
 
-// out[o] = bias[o] + sum_i M[o][i] in[i] for o < O: a warp per output
-__device__ __forceinline__ void block_rows_dot(const float* M, int ld, const float* in, int O, int I, const float* bias, float* out) {
-    const int lane = threadIdx.x & 31;
-    for (int o = threadIdx.x >> 5; o < O; o += kPathThreads / 32) {
-        float s = 0.f;
-        for (int i = lane; i < I; i += 32) s = fmaf(M[o * ld + i], in[i], s);
-#pragma unroll
-        for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-        if (lane == 0) out[o] = s + (bias ? bias[o] : 0.f);
-    }
+// sum_i M[row][i] in[i], one chain from zero
+__device__ __forceinline__ float row_dot(const float* M, int ld, int row, const float* in, int n) {
+    const float* p = M + static_cast<long long>(row) * ld;
+    float s = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < n; ++i) s = fmaf(p[i], in[i], s);
+    return s;
 }
-// out[d] += sum_h M[h][d] in[h]: a warp per output
-__device__ __forceinline__ void block_cols_dot(const float* M, int ld, const float* in, int D, int H, float* out) {
-    const int lane = threadIdx.x & 31;
-    for (int d = threadIdx.x >> 5; d < D; d += kPathThreads / 32) {
-        float s = 0.f;
-        for (int h = lane; h < H; h += 32) s = fmaf(M[h * ld + d], in[h], s);
-#pragma unroll
-        for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
-        if (lane == 0) out[d] += s;
-    }
+// sum_i M[i][col] in[i], one chain from zero
+__device__ __forceinline__ float col_dot(const float* M, int ld, int col, const float* in, int n) {
+    float s = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < n; ++i) s = fmaf(M[static_cast<long long>(i) * ld + col], in[i], s);
+    return s;
 }
 
 struct PathWeights {
@@ -505,12 +542,6 @@ __device__ __forceinline__ PathWeights path_weights(const PathArgs& a, float* sm
     return w;
 }
 
-__device__ __forceinline__ float row_dot(const float* M, int ld, int row, const float* in, int n, float s) {
-    const float* p = M + static_cast<long long>(row) * ld;
-    for (int i = 0; i < n; ++i) s = fmaf(p[i], in[i], s);
-    return s;
-}
-
 __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int staged) {
     extern __shared__ __align__(16) float sm[];
     const int D = a.D, H = a.H, W = a.W, b = blockIdx.x, tid = threadIdx.x;
@@ -518,12 +549,12 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
     float* mu = z + D;               // [D]
     float* zp = mu + D;              // [D]
     float* hz = zp + D;              // [2D]
-    float* h = sm + 8 * D;           // [H]
+    float* h = sm + 8 * D;           // [2][H] (of 3)
     float* scal = h + 3 * H;         // [64]
     const PathWeights w = path_weights(a, scal + 64, staged);
-    for (int d = tid; d < D; d += kPathThreads) { z[d] = a.z0[d]; a.z[static_cast<long long>(b) * (W + 1) * D + d] = a.z0[d]; }
     dependency_wait();
     launch_dependents();
+    for (int d = tid; d < D; d += kPathThreads) { z[d] = a.z0[d]; a.z[static_cast<long long>(b) * (W + 1) * D + d] = a.z0[d]; }
     __syncthreads();
     float elbo = 0.f;                // of this thread's latent dimensions
     for (int t = 0; t < W; ++t) {
@@ -532,9 +563,9 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
         const float* sb = a.b + (static_cast<long long>(b) * (W + 1) + t) * H;
         // hidden layers that read z_{t-1}: the combiner and the transition's
         for (int i = tid; i < H; i += kPathThreads) {
-            const float c = tanhf(row_dot(w.Wz, w.ldd, i, z, D, a.bz[i]));
+            const float c = tanhf(row_dot(w.Wz, w.ldd, i, z, D) + a.bz[i]);
             const float o = (c + sa[i] + sb[i]) * (1.f / 3.f);
-            const float u = fmaxf(row_dot(w.W1, w.ldd, i, z, D, a.b1[i]), 0.f);
+            const float u = fmaxf(row_dot(w.W1, w.ldd, i, z, D) + a.b1[i], 0.f);
             a.comb[r * H + i] = c;
             a.hout[r * H + i] = o;
             a.u[r * H + i] = u;
@@ -542,11 +573,13 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
             h[H + i] = u;
         }
         __syncthreads();
-        block_rows_dot(w.Wmu, w.ldh, h, D, H, a.bmu, mu);
-        block_rows_dot(w.W2, w.ldh, h + H, 2 * D, H, a.b2, hz);
+        for (int o = tid; o < 3 * D; o += kPathThreads) {
+            if (o < D) mu[o] = row_dot(w.Wmu, w.ldh, o, h, H) + a.bmu[o];
+            else hz[o - D] = row_dot(w.W2, w.ldh, o - D, h + H, H) + a.b2[o - D];
+        }
         __syncthreads();
         for (int d = tid; d < D; d += kPathThreads) {
-            const float pre = row_dot(a.Wsig, D, d, mu, D, a.bsig[d]);
+            const float pre = row_dot(a.Wsig, D, d, mu, D) + a.bsig[d];
             const float sg = softplus_f(pre), e = a.eps[r * D + d], zt = fmaf(sg, e, mu[d]);
             a.mu[r * D + d] = mu[d];
             a.presig[r * D + d] = pre;
@@ -561,15 +594,15 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
         }
         __syncthreads();
         for (int i = tid; i < H; i += kPathThreads)
-            a.v[r * H + i] = fmaxf(row_dot(w.W3, w.ldd, i, zp, D, a.b3[i]), 0.f);
-        float* swap = z; z = zp; zp = swap;            // h and mu are rewritten behind the next barriers
+            a.v[r * H + i] = fmaxf(row_dot(w.W3, w.ldd, i, zp, D) + a.b3[i], 0.f);
+        float* swap = z; z = zp; zp = swap;            // h, mu and hz are rewritten behind the next barriers
     }
     // D <= 64: the sums sit in the first two warps
     if (tid < 64) scal[tid] = elbo;
     __syncthreads();
     if (tid == 0) {
         float s = 0.f;
-        for (int d = 0; d < (D < 64 ? D : 64); ++d) s += scal[d];
+        for (int d = 0; d < D; ++d) s += scal[d];
         a.path[b] = s;
     }
 }
@@ -588,27 +621,27 @@ __global__ void __launch_bounds__(kPathThreads) k_path_backward(PathArgs a, int 
     dependency_wait();
     launch_dependents();
     __syncthreads();
+    if (tid >= kPathThreads - 32) window_elbo(a.part, a.n_part, a.B * W, W, b, a.path, a.elbo, tid & 31);
     for (int t = W - 1; t >= 0; --t) {
         const long long r = static_cast<long long>(b) * W + t;
-        for (int d = tid; d < D; d += kPathThreads) { gz[d] = gzp[d] + a.dzt[r * D + d]; gzp[d] = 0.f; }
+        for (int d = tid; d < D; d += kPathThreads) gz[d] = gzp[d] + a.dzt[r * D + d];
         for (int d = tid; d < 2 * D; d += kPathThreads) dhz[d] = a.dhz[r * 2 * D + d];
         __syncthreads();
-        // hidden-layer gradients of the emission (its head's input gradient comes in parts) and of the transition
+        // hidden-layer gradients of the emission and of the transition
         for (int i = tid; i < H; i += kPathThreads) {
-            float dv = 0.f;
-            if (a.v[r * H + i] > 0.f)
-                for (int k = 0; k < a.n_parts; ++k) dv += a.dv_parts[k * a.part_stride + r * H + i];
-            float du = 0.f;
-            if (a.u[r * H + i] > 0.f)
-                for (int o = 0; o < 2 * D; ++o) du = fmaf(dhz[o], w.W2[o * w.ldh + i], du);
+            const float dv = a.v[r * H + i] > 0.f ? a.dv_raw[r * H + i] : 0.f;
+            const float du = a.u[r * H + i] > 0.f ? col_dot(w.W2, w.ldh, i, dhz, 2 * D) : 0.f;
             a.dv[r * H + i] = dv;
             a.du[r * H + i] = du;
             h[i] = dv;
             h[H + i] = du;
         }
         __syncthreads();
-        block_cols_dot(w.W3, w.ldd, h, D, H, gz);
-        block_cols_dot(w.W1, w.ldd, h + H, D, H, gzp);
+        // the two sums in different warps: each is a chain over H
+        for (int d = tid; d < 64 + D; d += kPathThreads) {
+            if (d < D) gz[d] = col_dot(w.W3, w.ldd, d, h, H) + gz[d];
+            else if (d >= 64) gzp[d - 64] = col_dot(w.W1, w.ldd, d - 64, h + H, H);
+        }
         __syncthreads();
         // guide: d_mu = g_z + Wsig^T d_pre_sig,  d_pre_sig = (g_z eps + 1 / sigma) sigmoid(pre_sig)
         for (int d = tid; d < D; d += kPathThreads) {
@@ -619,16 +652,13 @@ __global__ void __launch_bounds__(kPathThreads) k_path_backward(PathArgs a, int 
         }
         __syncthreads();
         for (int d = tid; d < D; d += kPathThreads) {
-            float s = gz[d];
-            for (int o = 0; o < D; ++o) s = fmaf(dps[o], a.Wsig[o * D + d], s);
+            const float s = col_dot(a.Wsig, D, d, dps, D) + gz[d];
             dmu[d] = s;
             a.dmu[r * D + d] = s;
         }
         __syncthreads();
         for (int i = tid; i < H; i += kPathThreads) {
-            float s = 0.f;
-            for (int d = 0; d < D; ++d) s = fmaf(dmu[d], w.Wmu[d * w.ldh + i], s);
-            s *= 1.f / 3.f;
+            const float s = col_dot(w.Wmu, w.ldh, i, dmu, D) * (1.f / 3.f);
             const float c = a.comb[r * H + i];
             a.dh[r * H + i] = s;
             const float p = s * (1.f - c * c);
@@ -636,7 +666,7 @@ __global__ void __launch_bounds__(kPathThreads) k_path_backward(PathArgs a, int 
             h[2 * H + i] = p;
         }
         __syncthreads();
-        block_cols_dot(w.Wz, w.ldd, h + 2 * H, D, H, gzp);
+        for (int d = tid; d < D; d += kPathThreads) gzp[d] = col_dot(w.Wz, w.ldd, d, h + 2 * H, H) + gzp[d];
         __syncthreads();
     }
     for (int d = tid; d < D; d += kPathThreads) a.gz0[static_cast<long long>(b) * D + d] = gzp[d];
