@@ -35,21 +35,19 @@ __device__ __forceinline__ float sigmoid_f(float v) { return 1.f / (1.f + expf(-
 // C[m][n] = sum_k A(m, k) B(n, k).  An operand is either "k-major" (element (m, k) at m*ld + k) or "m-major" (at k*ld + m),
 // so the three orientations a dense layer needs are X W^T, dY W and dY^T X.  With n_seg > 1 the product is a sum of n_seg
 // products over K, segment s at p + s * seg; the segments' sums are added in order.
-// Two tiles: 64 x 64 with 4 x 4 results per thread where there are enough of them to fill the GPU, 16 x 32 with 2 x 2
-// where there are not -- then the time is the chain's: about 8 clocks per k (64 windows of n1024: the projections have
-// K = 1024 and 40 large or 320 small tiles, the input gradient of the emission head K = 2048 and 20 or 160).
-// The next slab's global loads are in flight while the current one is multiplied.
+// Two tiles: 64 x 64 with 8 x 4 results per thread where there are enough of them to fill the GPU, 16 x 32 with 2 x 2
+// where there are not -- then the time is the chain's.  Slabs of TK k arrive by asynchronous copies, kSlabs in flight (a
+// slab is multiplied in a fraction of the time its copies take), and keep the operand's own orientation: k-major rows
+// are read four k at a time, m-major ones several m at a time, pitches chosen so that neither conflicts.
 template <int TM_, int TN_, int RM_, int RN_, int TK_> struct Tile {
     static constexpr int TM = TM_, TN = TN_, RM = RM_, RN = RN_, TK = TK_;
-    static constexpr int kThreads = (TM / RM) * (TN / RN);
-    static constexpr int kAVecs = TM * TK / 4 / kThreads, kBVecs = TN * TK / 4 / kThreads;    // float4 per thread and slab
-    struct Smem {
-        float a[2][TK][TM + 4];
-        float b[2][TK][TN + 4];
-    };
+    static constexpr int TX = TN / RN, TY = TM / RM, kThreads = TX * TY;
+    __host__ __device__ static constexpr int pitch(int t, bool k_major) { return (k_major ? TK : t) + 4; }
+    __host__ __device__ static constexpr int floats(int t, bool k_major) { return (k_major ? t : TK) * pitch(t, k_major); }
 };
-using LargeTile = Tile<64, 64, 4, 4, 16>;        // 256 threads
+using LargeTile = Tile<64, 64, 8, 4, 16>;        // 128 threads
 using SmallTile = Tile<16, 32, 2, 2, 32>;        // 128 threads
+constexpr int kSlabs = 4;
 
 struct Operand {
     const float* p;
@@ -65,101 +63,142 @@ struct Product {
     int tile0, tiles_n;  // first tile of this product in the launch, tiles per tile row
 };
 
-// Vector v of a T x TK slab: 4 values along the operand's contiguous dimension.
-template <int T, int TK, bool K_MAJOR, bool VEC>
-__device__ __forceinline__ float4 load_slab(const float* base, long long ld, int rows, int m0, int k0, int K, int v) {
-    float r[4] = {0.f, 0.f, 0.f, 0.f};
-    if (K_MAJOR) {
-        const int m = m0 + v / (TK / 4), k = k0 + v % (TK / 4) * 4;
-        if (m < rows) {
-            const float* p = base + m * ld + k;
-            if (VEC && k + 3 < K) return *reinterpret_cast<const float4*>(p);
+// Four consecutive values of an operand into shared memory, zero where they do not exist.
+template <bool VEC>
+__device__ __forceinline__ void copy4(uint32_t dst, const float* src, int valid) {
+    if (VEC) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid > 0 ? 16 : 0) : "memory");
+    } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (k + i < K) r[i] = p[i];
+        for (int i = 0; i < 4; ++i)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4 * i), "l"(i < valid ? src + i : src), "r"(i < valid ? 4 : 0) : "memory");
+    }
+}
+__device__ __forceinline__ void copy1(uint32_t dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ uint32_t smem_addr(const float* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// n consecutive floats, by all threads of the CTA
+__device__ __forceinline__ void copy_vector(float* dst, const float* src, int n) {
+    const uint32_t d = smem_addr(dst);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) copy1(d + 4 * i, src + i);
+}
+// rows x cols of a row-major matrix (pitch ld) to shared memory with another pitch, or transposed; a warp per row.  All
+// copies are in flight at once: loaded through registers the matrices took longer to arrive than the steps that use them.
+__device__ __forceinline__ void copy_matrix(float* dst, int pitch, const float* src, long long ld, int rows, int cols) {
+    for (int r = threadIdx.x >> 5; r < rows; r += blockDim.x >> 5) {
+        const uint32_t d = smem_addr(dst + r * pitch);
+        for (int c = threadIdx.x & 31; c < cols; c += 32) copy1(d + 4 * c, src + r * ld + c);
+    }
+}
+__device__ __forceinline__ void copy_matrix_transposed(float* dst, int pitch, const float* src, long long ld, int rows, int cols) {
+    for (int r = threadIdx.x >> 5; r < rows; r += blockDim.x >> 5) {
+        const uint32_t d = smem_addr(dst + r);
+        for (int c = threadIdx.x & 31; c < cols; c += 32) copy1(d + 4 * c * pitch, src + r * ld + c);
+    }
+}
+// One slab of an operand, T rows (m) x TK k.
+template <typename T, int ROWS, bool K_MAJOR, bool VEC>
+__device__ __forceinline__ void copy_slab(uint32_t dst, const float* base, long long ld, int rows, int m0, int k0, int K) {
+    constexpr int kVecs = ROWS * T::TK / 4, P = T::pitch(ROWS, K_MAJOR);
+#pragma unroll
+    for (int v = threadIdx.x; v < kVecs; v += T::kThreads) {
+        const int r = K_MAJOR ? v / (T::TK / 4) : v / (ROWS / 4), c = K_MAJOR ? v % (T::TK / 4) * 4 : v % (ROWS / 4) * 4;
+        const int m = m0 + (K_MAJOR ? r : c), k = k0 + (K_MAJOR ? c : r);
+        const int valid = K_MAJOR ? (m < rows ? K - k : 0) : (k < K ? rows - m : 0);
+        copy4<VEC>(dst + 4 * (r * P + c), valid > 0 ? base + (K_MAJOR ? m * ld + k : k * ld + m) : base, valid);
+    }
+}
+// r[i][q]: the thread's R values of four consecutive k.  k-major: rows at, at + STEP, ..; m-major: R consecutive from at * R.
+template <int R, int STEP, int PITCH, bool K_MAJOR>
+__device__ __forceinline__ void load_four_k(float (&r)[R][4], const float* slab, int at, int k) {
+    if (K_MAJOR) {
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const float4 q = *reinterpret_cast<const float4*>(slab + (at + i * STEP) * PITCH + k);
+            r[i][0] = q.x; r[i][1] = q.y; r[i][2] = q.z; r[i][3] = q.w;
         }
     } else {
-        const int k = k0 + v / (T / 4), m = m0 + v % (T / 4) * 4;
-        if (k < K) {
-            const float* p = base + k * ld + m;
-            if (VEC && m + 3 < rows) return *reinterpret_cast<const float4*>(p);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (m + i < rows) r[i] = p[i];
+        for (int q = 0; q < 4; ++q) {
+            const float* p = slab + (k + q) * PITCH + at * R;
+            if constexpr (R % 4 == 0) {
+#pragma unroll
+                for (int i = 0; i < R; i += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(p + i);
+                    r[i][q] = v.x; r[i + 1][q] = v.y; r[i + 2][q] = v.z; r[i + 3][q] = v.w;
+                }
+            } else {
+                const float2 v = *reinterpret_cast<const float2*>(p);
+                r[0][q] = v.x; r[1][q] = v.y;
+            }
         }
     }
-    return make_float4(r[0], r[1], r[2], r[3]);
 }
-template <int T, int TK, bool K_MAJOR>
-__device__ __forceinline__ void store_slab(float (*s)[T + 4], const float4& q, int v) {
-    if (K_MAJOR) {
-        const int m = v / (TK / 4), k = v % (TK / 4) * 4;
-        s[k][m] = q.x; s[k + 1][m] = q.y; s[k + 2][m] = q.z; s[k + 3][m] = q.w;
-    } else {
-        *reinterpret_cast<float4*>(&s[v / (T / 4)][v % (T / 4) * 4]) = q;
-    }
-}
-template <int R>
-__device__ __forceinline__ void load_regs(float (&r)[R], const float* p) {
-    if (R == 4) {
-        const float4 q = *reinterpret_cast<const float4*>(p);
-        r[0] = q.x; r[1] = q.y; r[2 % R] = q.z; r[3 % R] = q.w;
-    } else {
-        const float2 q = *reinterpret_cast<const float2*>(p);
-        r[0] = q.x; r[1] = q.y;
-    }
-}
+// Tile row (column) of a thread's i-th result.
+template <int R, int STEP, bool K_MAJOR>
+__device__ __forceinline__ int result_at(int at, int i) { return K_MAJOR ? at + i * STEP : at * R + i; }
 
-// acc[i][j] = sum over segments and k of A(m0 + .., k) B(n0 + .., k).  load_b(k0, s, v) supplies vector v of B's slab.
-template <typename T, bool A_KMAJOR, bool B_KMAJOR, bool VEC, bool SUMS, bool SEGMENTS, typename LoadB>
-__device__ __forceinline__ void tile_product(typename T::Smem& sm, const Operand& a, int m0, int K, int n_seg, LoadB load_b,
+template <typename T, bool A_KMAJOR, bool B_KMAJOR> struct Slabs {
+    static constexpr int kA = T::floats(T::TM, A_KMAJOR), kB = T::floats(T::TN, B_KMAJOR);
+    float f[kSlabs * (kA + kB)];
+};
+
+// acc[i][j] = sum over segments and k of A(m0 + .., k) B(n0 + .., k).  copy_b(dst, k0, s) requests B's slab.
+template <typename T, bool A_KMAJOR, bool B_KMAJOR, bool VEC, bool SUMS, bool SEGMENTS, typename CopyB>
+__device__ __forceinline__ void tile_product(Slabs<T, A_KMAJOR, B_KMAJOR>& sm, const Operand& a, int m0, int K, int n_seg, CopyB copy_b,
                                              float (&acc)[T::RM][T::RN], float& a_sum) {
-    const int tid = threadIdx.x, tx = tid % (T::TN / T::RN), ty = tid / (T::TN / T::RN);
-    float4 ra[T::kAVecs], rb[T::kBVecs];
-    const auto fetch = [&](int k0, int s) {
-#pragma unroll
-        for (int u = 0; u < T::kAVecs; ++u)
-            ra[u] = load_slab<T::TM, T::TK, A_KMAJOR, VEC>(a.p + (SEGMENTS ? s * a.seg : 0), a.ld, a.rows, m0, k0, K, tid + u * T::kThreads);
-#pragma unroll
-        for (int u = 0; u < T::kBVecs; ++u) rb[u] = load_b(k0, s, tid + u * T::kThreads);
+    using S = Slabs<T, A_KMAJOR, B_KMAJOR>;
+    const int tid = threadIdx.x, tx = tid % T::TX, ty = tid / T::TX;
+    const uint32_t smem = static_cast<uint32_t>(__cvta_generic_to_shared(sm.f));
+    const int per_seg = (K + T::TK - 1) / T::TK, slabs = per_seg * (SEGMENTS ? n_seg : 1);
+    int k_req = 0, s_req = 0, buf_req = 0;
+    const auto request = [&] {
+        if (s_req < (SEGMENTS ? n_seg : 1)) {
+            const uint32_t dst = smem + 4 * buf_req * (S::kA + S::kB);
+            copy_slab<T, T::TM, A_KMAJOR, VEC>(dst, a.p + (SEGMENTS ? s_req * a.seg : 0), a.ld, a.rows, m0, k_req, K);
+            copy_b(dst + 4 * S::kA, k_req, s_req);
+            k_req += T::TK;
+            if (k_req >= K) { k_req = 0; ++s_req; }
+            if (++buf_req == kSlabs) buf_req = 0;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
+#pragma unroll
+    for (int i = 0; i < kSlabs - 1; ++i) request();
     float total[T::RM][T::RN] = {};
-    fetch(0, 0);
-    int buf = 0, k0 = 0, s = 0;
-    while (true) {
+    int buf = 0, left = per_seg;
+    for (int it = 0; it < slabs; ++it) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSlabs - 2) : "memory");
+        __syncthreads();                 // the slab is there for everyone, and everyone has finished with the one before it
+        request();
+        const float* sa = sm.f + buf * (S::kA + S::kB);
+        const float* sb = sa + S::kA;
 #pragma unroll
-        for (int u = 0; u < T::kAVecs; ++u) store_slab<T::TM, T::TK, A_KMAJOR>(sm.a[buf], ra[u], tid + u * T::kThreads);
+        for (int k = 0; k < T::TK; k += 4) {
+            float x[T::RM][4], y[T::RN][4];
+            load_four_k<T::RM, T::TY, T::pitch(T::TM, A_KMAJOR), A_KMAJOR>(x, sa, ty, k);
+            load_four_k<T::RN, T::TX, T::pitch(T::TN, B_KMAJOR), B_KMAJOR>(y, sb, tx, k);
 #pragma unroll
-        for (int u = 0; u < T::kBVecs; ++u) store_slab<T::TN, T::TK, B_KMAJOR>(sm.b[buf], rb[u], tid + u * T::kThreads);
-        __syncthreads();                 // one barrier per slab: the buffer written next was read before this barrier
-        int k_next = k0 + T::TK, s_next = s;
-        if (k_next >= K) { k_next = 0; ++s_next; }
-        const bool more = SEGMENTS ? s_next < n_seg : s_next == 0;
-        if (more) fetch(k_next, s_next);
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int k = 0; k < T::TK; ++k) {
-            float x[T::RM], y[T::RN];
-            load_regs<T::RM>(x, &sm.a[buf][k][T::RM * ty]);
-            load_regs<T::RN>(y, &sm.b[buf][k][T::RN * tx]);
+                for (int i = 0; i < T::RM; ++i)
 #pragma unroll
-            for (int i = 0; i < T::RM; ++i)
-#pragma unroll
-                for (int j = 0; j < T::RN; ++j) acc[i][j] = fmaf(x[i], y[j], acc[i][j]);
+                    for (int j = 0; j < T::RN; ++j) acc[i][j] = fmaf(x[i][q], y[j][q], acc[i][j]);
         }
         if (SUMS && tid < T::TM) {
 #pragma unroll
-            for (int k = 0; k < T::TK; ++k) a_sum += sm.a[buf][k][tid];
+            for (int k = 0; k < T::TK; ++k) a_sum += sa[k * T::pitch(T::TM, false) + tid];
         }
-        if (SEGMENTS && s_next != s) {
+        if (SEGMENTS && --left == 0) {
+            left = per_seg;
 #pragma unroll
             for (int i = 0; i < T::RM; ++i)
 #pragma unroll
                 for (int j = 0; j < T::RN; ++j) { total[i][j] += acc[i][j]; acc[i][j] = 0.f; }
         }
-        if (!more) break;
-        k0 = k_next;
-        s = s_next;
-        buf ^= 1;
+        if (++buf == kSlabs) buf = 0;
     }
     if (SEGMENTS) {
 #pragma unroll
@@ -176,7 +215,7 @@ struct ProductList {
 };
 
 template <typename T, bool A_KMAJOR, bool B_KMAJOR, bool VEC, bool SEGMENTS>
-__device__ __forceinline__ void run_product(typename T::Smem& sm, const Product& q, int tile) {
+__device__ __forceinline__ void run_product(Slabs<T, A_KMAJOR, B_KMAJOR>& sm, const Product& q, int tile) {
     const int m0 = tile / q.tiles_n * T::TM, n0 = tile % q.tiles_n * T::TN;
     float a_sum = 0.f;
     if (q.b.rows == 0) {                       // sums only
@@ -188,28 +227,31 @@ __device__ __forceinline__ void run_product(typename T::Smem& sm, const Product&
         return;
     }
     float acc[T::RM][T::RN] = {};
-    const auto load_b = [&](int k0, int s, int v) {
-        return load_slab<T::TN, T::TK, B_KMAJOR, VEC>(q.b.p + (SEGMENTS ? s * q.b.seg : 0), q.b.ld, q.b.rows, n0, k0, q.K, v);
+    const auto copy_b = [&](uint32_t dst, int k0, int s) {
+        copy_slab<T, T::TN, B_KMAJOR, VEC>(dst, q.b.p + (SEGMENTS ? s * q.b.seg : 0), q.b.ld, q.b.rows, n0, k0, q.K);
     };
     if (SEGMENTS && q.a_sums && n0 == 0) {
-        tile_product<T, A_KMAJOR, B_KMAJOR, VEC, true, SEGMENTS>(sm, q.a, m0, q.K, q.n_seg, load_b, acc, a_sum);
+        tile_product<T, A_KMAJOR, B_KMAJOR, VEC, true, SEGMENTS>(sm, q.a, m0, q.K, q.n_seg, copy_b, acc, a_sum);
         if (threadIdx.x < T::TM && m0 + static_cast<int>(threadIdx.x) < q.a.rows) q.a_sums[m0 + threadIdx.x] = a_sum;
     } else {
-        tile_product<T, A_KMAJOR, B_KMAJOR, VEC, false, SEGMENTS>(sm, q.a, m0, q.K, q.n_seg, load_b, acc, a_sum);
+        tile_product<T, A_KMAJOR, B_KMAJOR, VEC, false, SEGMENTS>(sm, q.a, m0, q.K, q.n_seg, copy_b, acc, a_sum);
     }
-    const int m = m0 + T::RM * static_cast<int>(threadIdx.x / (T::TN / T::RN)), n = n0 + T::RN * static_cast<int>(threadIdx.x % (T::TN / T::RN));
+    const int tx = threadIdx.x % T::TX, ty = threadIdx.x / T::TX;
 #pragma unroll
     for (int i = 0; i < T::RM; ++i) {
-        if (m + i >= q.a.rows) continue;
+        const int m = m0 + result_at<T::RM, T::TY, A_KMAJOR>(ty, i);
+        if (m >= q.a.rows) continue;
 #pragma unroll
-        for (int j = 0; j < T::RN; ++j)
-            if (n + j < q.b.rows) q.c[(m + i) * q.ldc + n + j] = acc[i][j];
+        for (int j = 0; j < T::RN; ++j) {
+            const int n = n0 + result_at<T::RN, T::TX, B_KMAJOR>(tx, j);
+            if (n < q.b.rows) q.c[m * q.ldc + n] = acc[i][j];
+        }
     }
 }
 
 template <typename T, bool A_KMAJOR, bool B_KMAJOR, bool VEC, bool SEGMENTS>
 __global__ void __launch_bounds__(T::kThreads) k_products(const __grid_constant__ ProductList list) {
-    __shared__ __align__(16) typename T::Smem sm;
+    __shared__ __align__(16) Slabs<T, A_KMAJOR, B_KMAJOR> sm;
     dependency_wait();
     launch_dependents();
     int which = 0;
@@ -218,49 +260,46 @@ __global__ void __launch_bounds__(T::kThreads) k_products(const __grid_constant_
 }
 
 // ---- emission head and its density ---------------------------------------------------------------------------------
-// head = v W4^T + b4 for 64 rows x 32 workers (32 means and 32 log-variances: the tile's columns 4t .. 4t+3 are the
-// means, then the log-variances, of workers 2t and 2t+1, so a thread holds both halves of its workers), and at once
+// head = v W4^T + b4 for 64 rows x 32 workers: the tile's columns are the means of its workers, then their log-variances,
+// so a thread (columns tx, tx + 16, tx + 32, tx + 48) holds both halves of two workers, and at once
 //   log N(x; m, exp(lv)) summed over the tile's workers -> part[tile column][row],
 //   d_head = [r inv | -1/2 + r^2 inv / 2],  r = x - m, inv = exp(-lv)                    (d_head: null = forward only).
 constexpr int kHeadWorkers = LargeTile::TN / 2;
 
 template <bool VEC>
-__global__ void __launch_bounds__(LargeTile::kThreads, 2) k_emission_density(const float* __restrict__ v, const float* __restrict__ W4,
+__global__ void __launch_bounds__(LargeTile::kThreads) k_emission_density(const float* __restrict__ v, const float* __restrict__ W4,
                                                                              const float* __restrict__ b4, const float* __restrict__ x,
                                                                              int R, int N, int H, float* __restrict__ d_head,
                                                                              float* __restrict__ part) {
     using T = LargeTile;
-    __shared__ __align__(16) T::Smem sm;
+    __shared__ __align__(16) Slabs<T, true, true> sm;
     dependency_wait();
     launch_dependents();
     const int head_tiles = (N + kHeadWorkers - 1) / kHeadWorkers;            // one-dimensional grid: rows reach 2^24
     const int m0 = blockIdx.x / head_tiles * T::TM, head_tile = blockIdx.x % head_tiles, j0 = head_tile * kHeadWorkers;
     const Operand a{v, H, 0, R};
-    const int tid = threadIdx.x, col = tid / (T::TK / 4);                    // the column of B this thread loads
-    const int worker = j0 + 2 * (col >> 2) + (col & 1), head = (col >> 1) & 1;
-    const float* wrow = W4 + (static_cast<long long>(head) * N + (worker < N ? worker : 0)) * H;
-    const auto load_b = [&](int k0, int, int vec) {
-        const int k = k0 + vec % (T::TK / 4) * 4;
-        if (worker >= N) return make_float4(0.f, 0.f, 0.f, 0.f);
-        if (VEC && k + 3 < H) return *reinterpret_cast<const float4*>(wrow + k);
-        float t[4];
+    const auto copy_b = [&](uint32_t dst, int k0, int) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) t[i] = k + i < H ? wrow[k + i] : 0.f;
-        return make_float4(t[0], t[1], t[2], t[3]);
+        for (int u = threadIdx.x; u < T::TN * T::TK / 4; u += T::kThreads) {
+            const int col = u / (T::TK / 4), k = k0 + u % (T::TK / 4) * 4;
+            const int worker = j0 + col % kHeadWorkers, head = col / kHeadWorkers, valid = worker < N ? H - k : 0;
+            copy4<VEC>(dst + 4 * (col * T::pitch(T::TN, true) + u % (T::TK / 4) * 4),
+                       valid > 0 ? W4 + (static_cast<long long>(head) * N + worker) * H + k : W4, valid);
+        }
     };
-    static_assert(T::kBVecs == 1, "one column of B per thread");
     float acc[T::RM][T::RN] = {};
     float unused = 0.f;
-    tile_product<T, true, true, VEC, false, false>(sm, a, m0, H, 1, load_b, acc, unused);
-    const int tx = tid & 15, ty = tid >> 4;
+    tile_product<T, true, true, VEC, false, false>(sm, a, m0, H, 1, copy_b, acc, unused);
+    static_assert(T::RN == 4 && 2 * T::TX == kHeadWorkers && T::TX == 16, "columns 0, 1 of a thread are means, 2, 3 their log-variances");
+    const int tx = threadIdx.x % T::TX, ty = threadIdx.x / T::TX;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = m0 + 4 * ty + i;
+    for (int i = 0; i < T::RM; ++i) {
+        const int r = m0 + result_at<T::RM, T::TY, true>(ty, i);
         float s = 0.f;
         if (r < R) {
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                const int j = j0 + 2 * tx + c;
+                const int j = j0 + tx + T::TX * c;
                 if (j >= N) continue;
                 const float mean = acc[i][c] + b4[j], lv = acc[i][2 + c] + b4[N + j];
                 const float d = x[static_cast<long long>(r) * N + j] - mean, inv = expf(-lv);
@@ -370,7 +409,7 @@ __global__ void __launch_bounds__(256) k_rnn_forward(RnnArgs a) {
     float* sW = sm + 2 * RW * xp;                      // [chunk][wp]: sW[k][u] = Wh[u0 + u][k]
     const float* Wh = a.Wh[dir] + static_cast<long long>(u0) * H;
     const auto stage = [&](int k0, int n) {
-        for (int i = tid; i < units * n; i += T) sW[(i % n) * wp + i / n] = Wh[static_cast<long long>(i / n) * H + k0 + i % n];
+        copy_matrix_transposed(sW, wp, Wh + k0, H, units, n);
     };
     if (a.chunk >= H) stage(0, H);                     // weights: no kernel of this step writes them
     dependency_wait();
@@ -382,23 +421,32 @@ __global__ void __launch_bounds__(256) k_rnn_forward(RnnArgs a) {
         cur[w * xp + h] = s;
         if (rank == 0 && b0 + w < a.B) state[(static_cast<long long>(b0 + w) * (W + 1) + (dir ? W : 0)) * H + h] = s;
     }
+    copies_landed();
     cluster_sync();                                    // every CTA has started before anyone writes into it
     const int h = u0 + tid;
     const bool mine = tid < units;
     const float bias = mine ? a.bias[dir][h] : 0.f;
+    const auto projection = [&](int w, int s) {
+        return mine && b0 + w < a.B && s < W ? a.proj[(static_cast<long long>(b0 + w) * W + (dir ? W - 1 - s : s)) * 2 * H + dir * H + h] : 0.f;
+    };
+    float ahead[RW];                                   // the next step's projections are requested a step early
+#pragma unroll
+    for (int w = 0; w < RW; ++w) ahead[w] = projection(w, 0);
     for (int s = 0; s < W; ++s) {
         const int t = dir ? W - 1 - s : s;
         float p[RW], acc[RW];
 #pragma unroll
         for (int w = 0; w < RW; ++w) {
             acc[w] = 0.f;
-            p[w] = mine && b0 + w < a.B ? a.proj[(static_cast<long long>(b0 + w) * W + t) * 2 * H + dir * H + h] + bias : 0.f;
+            p[w] = ahead[w] + bias;
+            ahead[w] = projection(w, s + 1);
         }
         for (int k0 = 0; k0 < H; k0 += a.chunk) {
             const int n = min(a.chunk, H - k0);
             if (a.chunk < H) {
                 __syncthreads();
                 stage(k0, n);
+                copies_landed();
                 __syncthreads();
             }
             if (mine) rnn_chains<RW>(sW + tid, wp, cur + k0, xp, n, acc);
@@ -420,7 +468,7 @@ __global__ void __launch_bounds__(256) k_rnn_forward(RnnArgs a) {
 template <int RW>
 __global__ void __launch_bounds__(256) k_rnn_backward(RnnArgs a) {
     extern __shared__ __align__(16) float sm[];
-    const int H = a.H, W = a.W, xp = rnn_state_pitch(H), wp = rnn_weight_pitch(a.units), T = blockDim.x;
+    const int H = a.H, W = a.W, xp = rnn_state_pitch(H), wp = rnn_weight_pitch(a.units);
     const int rank = static_cast<int>(cluster_rank()), dir = blockIdx.y, b0 = static_cast<int>(blockIdx.x) / a.cluster * RW;
     const int u0 = rank * a.units, units = min(a.units, H - u0), tid = threadIdx.x;
     float* cur = sm;                                   // [RW][xp]: d_pre of this step, all units
@@ -428,39 +476,48 @@ __global__ void __launch_bounds__(256) k_rnn_backward(RnnArgs a) {
     float* sW = sm + 2 * RW * xp;                      // [chunk][wp]: sW[i][u] = Wh[i][u0 + u]
     const float* Wh = a.Wh[dir] + u0;
     const auto stage = [&](int k0, int n) {
-        for (int i = tid; i < units * n; i += T) sW[(i / units) * wp + i % units] = Wh[static_cast<long long>(k0 + i / units) * H + i % units];
+        copy_matrix(sW, wp, Wh + static_cast<long long>(k0) * H, H, n, units);
     };
     if (a.chunk >= H) stage(0, H);
     dependency_wait();
     launch_dependents();
+    copies_landed();
     cluster_sync();
     const int h = u0 + tid;
     const bool mine = tid < units;
     float carry[RW];
 #pragma unroll
     for (int w = 0; w < RW; ++w) carry[w] = 0.f;
+    float g[RW], act[RW];                              // of the coming step, requested a step early
+    const auto fetch = [&](int s) {
+        const int t = dir ? s : W - 1 - s;
+#pragma unroll
+        for (int w = 0; w < RW; ++w) {
+            const bool there = mine && b0 + w < a.B && s < W;
+            g[w] = there ? a.g[(static_cast<long long>(b0 + w) * W + t) * H + h] : 0.f;
+            act[w] = there ? a.state[dir][(static_cast<long long>(b0 + w) * (W + 1) + (dir ? t : t + 1)) * H + h] : 0.f;
+        }
+    };
+    fetch(0);
     for (int s = 0; s < W; ++s) {
         const int t = dir ? s : W - 1 - s;
         if (mine) {
 #pragma unroll
             for (int w = 0; w < RW; ++w) {
-                float d = 0.f;
-                if (b0 + w < a.B) {
-                    const long long r = static_cast<long long>(b0 + w) * W + t;
-                    const float act = a.state[dir][(static_cast<long long>(b0 + w) * (W + 1) + (dir ? t : t + 1)) * H + h];
-                    d = act > 0.f ? a.g[r * H + h] + carry[w] : 0.f;
-                    a.d_pre[dir][r * H + h] = d;
-                }
+                const float d = act[w] > 0.f ? g[w] + carry[w] : 0.f;
+                if (b0 + w < a.B) a.d_pre[dir][(static_cast<long long>(b0 + w) * W + t) * H + h] = d;
                 store_all(cur + w * xp + h, d, a.cluster);
                 carry[w] = 0.f;
             }
         }
         cluster_sync();
+        fetch(s + 1);
         for (int k0 = 0; k0 < H; k0 += a.chunk) {
             const int n = min(a.chunk, H - k0);
             if (a.chunk < H) {
                 __syncthreads();
                 stage(k0, n);
+                copies_landed();
                 __syncthreads();
             }
             if (mine) rnn_chains<RW>(sW + tid, wp, cur + k0, xp, n, carry);
@@ -503,14 +560,14 @@ struct PathArgs {
 __device__ __forceinline__ float row_dot(const float* M, int ld, int row, const float* in, int n) {
     const float* p = M + static_cast<long long>(row) * ld;
     float s = 0.f;
-#pragma unroll 8
+#pragma unroll 16
     for (int i = 0; i < n; ++i) s = fmaf(p[i], in[i], s);
     return s;
 }
 // sum_i M[i][col] in[i], one chain from zero
 __device__ __forceinline__ float col_dot(const float* M, int ld, int col, const float* in, int n) {
     float s = 0.f;
-#pragma unroll 8
+#pragma unroll 16
     for (int i = 0; i < n; ++i) s = fmaf(M[static_cast<long long>(i) * ld + col], in[i], s);
     return s;
 }
@@ -523,22 +580,25 @@ struct PathWeights {
 inline size_t path_weight_floats(int D, int H) {
     return 3 * static_cast<size_t>(H) * (D | 1) + 3 * static_cast<size_t>(D) * (H | 1);
 }
-inline size_t path_scratch_floats(int D, int H) { return 3 * static_cast<size_t>(H) + 8 * static_cast<size_t>(D) + 64; }
+// What a step reads from global memory is copied to shared memory a step early: 4 rows of H, 5 of D, twice.
+inline size_t path_scratch_floats(int D, int H) { return 11 * static_cast<size_t>(H) + 18 * static_cast<size_t>(D) + 64; }
 
-__device__ __forceinline__ float* stage_padded(float* dst, const float* src, int rows, int cols, int ld) {
-    for (int i = threadIdx.x; i < rows * cols; i += kPathThreads) dst[(i / cols) * ld + i % cols] = src[i];
-    return dst + rows * ld;
-}
 __device__ __forceinline__ PathWeights path_weights(const PathArgs& a, float* sm, int staged) {
     if (!staged) return PathWeights{a.Wz, a.W1, a.W3, a.Wmu, a.W2, a.D, a.H};
     PathWeights w;
     w.ldd = a.D | 1;
     w.ldh = a.H | 1;
-    w.Wz = sm; sm = stage_padded(sm, a.Wz, a.H, a.D, w.ldd);
-    w.W1 = sm; sm = stage_padded(sm, a.W1, a.H, a.D, w.ldd);
-    w.W3 = sm; sm = stage_padded(sm, a.W3, a.H, a.D, w.ldd);
-    w.Wmu = sm; sm = stage_padded(sm, a.Wmu, a.D, a.H, w.ldh);
-    w.W2 = sm; stage_padded(sm, a.W2, 2 * a.D, a.H, w.ldh);
+    const auto put = [&](const float* src, int rows, int cols, int ld) {
+        float* dst = sm;
+        copy_matrix(dst, ld, src, cols, rows, cols);
+        sm += rows * ld;
+        return dst;
+    };
+    w.Wz = put(a.Wz, a.H, a.D, w.ldd);
+    w.W1 = put(a.W1, a.H, a.D, w.ldd);
+    w.W3 = put(a.W3, a.H, a.D, w.ldd);
+    w.Wmu = put(a.Wmu, a.D, a.H, w.ldh);
+    w.W2 = put(a.W2, 2 * a.D, a.H, w.ldh);
     return w;
 }
 
@@ -551,16 +611,28 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
     float* hz = zp + D;              // [2D]
     float* h = sm + 8 * D;           // [2][H] (of 3)
     float* scal = h + 3 * H;         // [64]
-    const PathWeights w = path_weights(a, scal + 64, staged);
+    float* ahead = scal + 64;        // [2]: h_left, h_right (H each), eps (D)
+    const int ahead_n = 4 * H + 5 * D;
+    const PathWeights w = path_weights(a, ahead + 2 * ahead_n, staged);
     dependency_wait();
     launch_dependents();
+    const auto fetch = [&](int t) {
+        float* dst = ahead + (t & 1) * ahead_n;
+        copy_vector(dst, a.a + (static_cast<long long>(b) * (W + 1) + t + 1) * H, H);
+        copy_vector(dst + H, a.b + (static_cast<long long>(b) * (W + 1) + t) * H, H);
+        copy_vector(dst + 2 * H, a.eps + (static_cast<long long>(b) * W + t) * D, D);
+    };
+    fetch(0);
     for (int d = tid; d < D; d += kPathThreads) { z[d] = a.z0[d]; a.z[static_cast<long long>(b) * (W + 1) * D + d] = a.z0[d]; }
-    __syncthreads();
     float elbo = 0.f;                // of this thread's latent dimensions
     for (int t = 0; t < W; ++t) {
         const long long r = static_cast<long long>(b) * W + t;
-        const float* sa = a.a + (static_cast<long long>(b) * (W + 1) + t + 1) * H;
-        const float* sb = a.b + (static_cast<long long>(b) * (W + 1) + t) * H;
+        const float* sa = ahead + (t & 1) * ahead_n;
+        const float* sb = sa + H;
+        const float* eps = sb + H;
+        copies_landed();
+        __syncthreads();
+        if (t + 1 < W) fetch(t + 1);
         // hidden layers that read z_{t-1}: the combiner and the transition's
         for (int i = tid; i < H; i += kPathThreads) {
             const float c = tanhf(row_dot(w.Wz, w.ldd, i, z, D) + a.bz[i]);
@@ -580,7 +652,7 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
         __syncthreads();
         for (int d = tid; d < D; d += kPathThreads) {
             const float pre = row_dot(a.Wsig, D, d, mu, D) + a.bsig[d];
-            const float sg = softplus_f(pre), e = a.eps[r * D + d], zt = fmaf(sg, e, mu[d]);
+            const float sg = softplus_f(pre), e = eps[d], zt = fmaf(sg, e, mu[d]);
             a.mu[r * D + d] = mu[d];
             a.presig[r * D + d] = pre;
             a.z[(static_cast<long long>(b) * (W + 1) + t + 1) * D + d] = zt;
@@ -614,23 +686,39 @@ __global__ void __launch_bounds__(kPathThreads) k_path_backward(PathArgs a, int 
     float* gzp = gz + D;             // [D]   d ELBO / d z_{t-1}
     float* dmu = gzp + D;            // [D]
     float* dps = dmu + D;            // [D]
-    float* dhz = dps + D;            // [2D]
     float* h = sm + 8 * D;           // [3][H]: dv, du, dpc
-    const PathWeights w = path_weights(a, h + 3 * H + 64, staged);
+    float* ahead = h + 3 * H + 64;   // [2]: v, u, d_head W4, comb (H each), d transition head (2D), dzt, presig, eps (D each)
+    const int ahead_n = 4 * H + 5 * D;
+    const PathWeights w = path_weights(a, ahead + 2 * ahead_n, staged);
     for (int d = tid; d < D; d += kPathThreads) gzp[d] = 0.f;
     dependency_wait();
     launch_dependents();
-    __syncthreads();
+    const auto fetch = [&](int t) {
+        float* dst = ahead + (t & 1) * ahead_n;
+        const long long r = static_cast<long long>(b) * W + t;
+        copy_vector(dst, a.v + r * H, H);
+        copy_vector(dst + H, a.u + r * H, H);
+        copy_vector(dst + 2 * H, a.dv_raw + r * H, H);
+        copy_vector(dst + 3 * H, a.comb + r * H, H);
+        copy_vector(dst + 4 * H, a.dhz + r * 2 * D, 2 * D);
+        copy_vector(dst + 4 * H + 2 * D, a.dzt + r * D, D);
+        copy_vector(dst + 4 * H + 3 * D, a.presig + r * D, D);
+        copy_vector(dst + 4 * H + 4 * D, a.eps + r * D, D);
+    };
+    fetch(W - 1);
     if (tid >= kPathThreads - 32) window_elbo(a.part, a.n_part, a.B * W, W, b, a.path, a.elbo, tid & 31);
     for (int t = W - 1; t >= 0; --t) {
         const long long r = static_cast<long long>(b) * W + t;
-        for (int d = tid; d < D; d += kPathThreads) gz[d] = gzp[d] + a.dzt[r * D + d];
-        for (int d = tid; d < 2 * D; d += kPathThreads) dhz[d] = a.dhz[r * 2 * D + d];
+        const float* v = ahead + (t & 1) * ahead_n;
+        const float *u = v + H, *dv_raw = u + H, *comb = dv_raw + H, *dhz = comb + H, *dzt = dhz + 2 * D, *presig = dzt + D, *eps = presig + D;
+        copies_landed();
         __syncthreads();
+        if (t > 0) fetch(t - 1);
+        for (int d = tid; d < D; d += kPathThreads) gz[d] = gzp[d] + dzt[d];
         // hidden-layer gradients of the emission and of the transition
         for (int i = tid; i < H; i += kPathThreads) {
-            const float dv = a.v[r * H + i] > 0.f ? a.dv_raw[r * H + i] : 0.f;
-            const float du = a.u[r * H + i] > 0.f ? col_dot(w.W2, w.ldh, i, dhz, 2 * D) : 0.f;
+            const float dv = v[i] > 0.f ? dv_raw[i] : 0.f;
+            const float du = u[i] > 0.f ? col_dot(w.W2, w.ldh, i, dhz, 2 * D) : 0.f;
             a.dv[r * H + i] = dv;
             a.du[r * H + i] = du;
             h[i] = dv;
@@ -645,8 +733,8 @@ __global__ void __launch_bounds__(kPathThreads) k_path_backward(PathArgs a, int 
         __syncthreads();
         // guide: d_mu = g_z + Wsig^T d_pre_sig,  d_pre_sig = (g_z eps + 1 / sigma) sigmoid(pre_sig)
         for (int d = tid; d < D; d += kPathThreads) {
-            const float pre = a.presig[r * D + d];
-            const float p = (gz[d] * a.eps[r * D + d] + 1.f / softplus_f(pre)) * sigmoid_f(pre);
+            const float pre = presig[d];
+            const float p = fmaf(gz[d], eps[d], 1.f / softplus_f(pre)) * sigmoid_f(pre);
             dps[d] = p;
             a.dps[r * D + d] = p;
         }
@@ -659,7 +747,7 @@ __global__ void __launch_bounds__(kPathThreads) k_path_backward(PathArgs a, int 
         __syncthreads();
         for (int i = tid; i < H; i += kPathThreads) {
             const float s = col_dot(w.Wmu, w.ldh, i, dmu, D) * (1.f / 3.f);
-            const float c = a.comb[r * H + i];
+            const float c = comb[i];
             a.dh[r * H + i] = s;
             const float p = s * (1.f - c * c);
             a.dpc[r * H + i] = p;
