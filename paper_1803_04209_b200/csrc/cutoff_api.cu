@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -1794,6 +1795,46 @@ int cutoff_debug_sort_values(cutoff_ctx* c, const float* rows, int64_t n_rows, i
     return rc;
 }
 
+// Device memory for the duration of one call that has no context: taken from and returned to a memory pool of the
+// library's own, in the order of the call's stream, so calls on other threads and streams do not meet in it.  The pool keeps at
+// most kPoolKeeps bytes between calls (what exceeds that goes back to the driver at the next synchronisation; the
+// rest when another allocation of the process needs it): cudaMalloc and cudaFree took 1 to 10 ms per call, the kernels 60 us.
+namespace {
+constexpr uint64_t kPoolKeeps = 64ull << 20;
+constexpr int kPoolDevices = 64;
+
+cudaMemPool_t scratch_pool(int device) {
+    static std::mutex lock;
+    static cudaMemPool_t pools[kPoolDevices] = {};
+    if (device < 0 || device >= kPoolDevices) return nullptr;
+    std::lock_guard<std::mutex> hold(lock);
+    if (!pools[device]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+        uint64_t keep = kPoolKeeps;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        pools[device] = pool;
+    }
+    return pools[device];
+}
+
+struct Scratch {
+    void* p = nullptr;
+    cudaStream_t stream;
+    Scratch(int device, cudaStream_t s, size_t bytes) : stream(s) {
+        cudaMemPool_t pool = bytes ? scratch_pool(device) : nullptr;
+        if (pool && cudaMallocFromPoolAsync(&p, bytes, pool, s) != cudaSuccess) { cudaGetLastError(); p = nullptr; }
+    }
+    ~Scratch() { if (p) cudaFreeAsync(p, stream); }
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+};
+}  // namespace
+
 // ---- evaluation of cutoff rules on recorded run-times ------------------------------------------------------
 
 int cutoff_eval_trace(int device, const float* trace, int64_t n_steps, int32_t n, int32_t ld, const int32_t* cutoffs,
@@ -1806,36 +1847,37 @@ int cutoff_eval_trace(int device, const float* trace, int64_t n_steps, int32_t n
     DeviceGuard guard(device);
     CU_CHECK(none, guard.err);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaDeviceProp prop;
-    CU_CHECK(none, cudaGetDeviceProperties(&prop, device));
-    float* d_sorted = nullptr;         // the sorted rows, kept only when the static cutoff is asked for
-    double* d_total = nullptr;
-    if (static_c) {
-        if (cudaMalloc(&d_sorted, sizeof(float) * static_cast<size_t>(n_steps) * n) != cudaSuccess) return CUTOFF_ERR_NOMEM;
-        if (cudaMalloc(&d_total, sizeof(double)) != cudaSuccess) { cudaFree(d_sorted); return CUTOFF_ERR_NOMEM; }
-    }
+    int sms = 0;
+    CU_CHECK(none, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+    // scratch only for the static cutoff: the sorted rows and the columns' totals
+    Scratch scratch(device, s, static_c ? sizeof(double) * n + sizeof(float) * static_cast<size_t>(n_steps) * n : 0);
+    if (static_c && !scratch.p) return CUTOFF_ERR_NOMEM;
+    double* d_totals = static_cast<double*>(scratch.p);
+    float* d_sorted = static_c ? reinterpret_cast<float*>(d_totals + n) : nullptr;
     const int P = next_pow2(n) < 32 ? 32 : next_pow2(n);
-    const int cap = 8 * prop.multiProcessorCount;
-    const int64_t want_w = ceil_div64(n_steps, kSortWarps);
-    const int grid_w = static_cast<int>(want_w < cap ? want_w : cap);
+    const int cap = 8 * sms;
+    const int64_t want_w = ceil_div64(n_steps, kEvalWarps);
+    const int grid_w = static_cast<int>(want_w < 2 * cap ? want_w : 2 * cap);
     const int grid_c = static_cast<int>(n_steps < cap ? n_steps : cap);
 #define EVAL_ARGS trace, n_steps, n, ld, cutoffs, n_rules, best_c, best, all, achieved, step_time, d_sorted
     switch (P) {
-        case 32: k_eval_trace_warp<1><<<grid_w, kSortWarps * 32, 0, s>>>(EVAL_ARGS); break;
-        case 64: k_eval_trace_warp<2><<<grid_w, kSortWarps * 32, 0, s>>>(EVAL_ARGS); break;
-        case 128: k_eval_trace_warp<4><<<grid_w, kSortWarps * 32, 0, s>>>(EVAL_ARGS); break;
-        case 256: k_eval_trace_warp<8><<<grid_w, kSortWarps * 32, 0, s>>>(EVAL_ARGS); break;
-        case 512: k_eval_trace_warp<16><<<grid_w, kSortWarps * 32, 0, s>>>(EVAL_ARGS); break;
-        case 1024: k_eval_trace_warp<32><<<grid_w, kSortWarps * 32, 0, s>>>(EVAL_ARGS); break;
+        case 32: k_eval_trace_warp<1><<<grid_w, kEvalWarps * 32, 0, s>>>(EVAL_ARGS); break;
+        case 64: k_eval_trace_warp<2><<<grid_w, kEvalWarps * 32, 0, s>>>(EVAL_ARGS); break;
+        case 128: k_eval_trace_warp<4><<<grid_w, kEvalWarps * 32, 0, s>>>(EVAL_ARGS); break;
+        case 256: k_eval_trace_warp<8><<<grid_w, kEvalWarps * 32, 0, s>>>(EVAL_ARGS); break;
+        case 512: k_eval_trace_warp<16><<<grid_w, kEvalWarps * 32, 0, s>>>(EVAL_ARGS); break;
+        case 1024: k_eval_trace_warp<32><<<grid_w, kEvalWarps * 32, 0, s>>>(EVAL_ARGS); break;
         case 2048: k_eval_trace_cta<2><<<grid_c, 64, 0, s>>>(EVAL_ARGS); break;
         default: k_eval_trace_cta<4><<<grid_c, 128, 0, s>>>(EVAL_ARGS); break;
     }
 #undef EVAL_ARGS
-    if (static_c) k_best_static<<<1, kStaticThreads, 0, s>>>(d_sorted, n_steps, n, static_c, d_total);
+    if (static_c) {
+        launch_dependent(k_static_totals, dim3(ceil_div(n, 32)), dim3(32 * kStaticSlices), 0, s, d_sorted, n_steps, n, d_totals);
+        launch_dependent(k_best_static, dim3(1), dim3(1024), 0, s, d_totals, n, static_c);
+    }
+    const cudaError_t launched = cudaGetLastError();
     const cudaError_t err = cudaStreamSynchronize(s);
-    cudaFree(d_sorted);
-    cudaFree(d_total);
-    return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? CUTOFF_OK : CUTOFF_ERR_CUDA;
+    return err == cudaSuccess && launched == cudaSuccess ? CUTOFF_OK : CUTOFF_ERR_CUDA;
 }
 
 int cutoff_order_baseline(int device, const float* trace, int64_t n_steps, int32_t n, int32_t ld, int32_t* cutoffs_out,
@@ -1846,18 +1888,19 @@ int cutoff_order_baseline(int device, const float* trace, int64_t n_steps, int32
     DeviceGuard guard(device);
     CU_CHECK(none, guard.err);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    double* d_work = nullptr;          // [T] sums / means, [T] sums of squares / deviations, [n] normal quantiles
-    if (cudaMalloc(&d_work, sizeof(double) * (2 * static_cast<size_t>(n_steps) + n)) != cudaSuccess) return CUTOFF_ERR_NOMEM;
-    double* d1 = d_work;
-    double* d2 = d_work + n_steps;
-    double* dq = d_work + 2 * n_steps;
-    k_step_moments<<<static_cast<unsigned>(n_steps), kMomentThreads, 0, s>>>(trace, n_steps, n, ld, d1, d2);
-    k_running_moments<<<1, 32, 0, s>>>(n_steps, n, d1, d2);
-    k_elfving_quantiles<<<ceil_div(n, 256), 256, 0, s>>>(n, dq);
-    k_order_cutoffs<<<static_cast<unsigned>(ceil_div64(n_steps, 8)), 256, 0, s>>>(n_steps, n, d1, d2, dq, cutoffs_out);
+    // [T] sums / means, [T] sums of squares / deviations, [n] normal quantiles
+    Scratch scratch(device, s, sizeof(double) * (2 * static_cast<size_t>(n_steps) + n));
+    if (!scratch.p) return CUTOFF_ERR_NOMEM;
+    double* d1 = static_cast<double*>(scratch.p);
+    double* d2 = d1 + n_steps;
+    double* dq = d1 + 2 * n_steps;
+    const unsigned step_ctas = static_cast<unsigned>(ceil_div64(n_steps, kMomentWarps));
+    k_step_moments<<<step_ctas + ceil_div(n, kMomentWarps * 32), kMomentWarps * 32, 0, s>>>(trace, n_steps, n, ld, d1, d2, dq, step_ctas);
+    launch_dependent(k_running_moments, dim3(1), dim3(1024), 0, s, n_steps, n, d1, d2);
+    launch_dependent(k_order_cutoffs, dim3(static_cast<unsigned>(ceil_div64(n_steps, 8))), dim3(256), 0, s, n_steps, n, d1, d2, dq, cutoffs_out);
+    const cudaError_t launched = cudaGetLastError();
     const cudaError_t err = cudaStreamSynchronize(s);
-    cudaFree(d_work);
-    return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? CUTOFF_OK : CUTOFF_ERR_CUDA;
+    return err == cudaSuccess && launched == cudaSuccess ? CUTOFF_OK : CUTOFF_ERR_CUDA;
 }
 
 // ---- learning the model: ELBO, gradient, Adam -------------------------------------------------------------------

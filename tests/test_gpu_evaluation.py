@@ -80,3 +80,46 @@ def test_eval_trace_rejects_bad_arguments():
     assert lib.cutoff_eval_trace(0, t.data_ptr(), 3, 4097, 4097, None, 0, oi.data_ptr(), o.data_ptr(), o.data_ptr(), None, None, None, None) == binding.ERR_BAD_ARG
     assert lib.cutoff_eval_trace(0, t.data_ptr(), 3, 8, 8, None, 1, oi.data_ptr(), o.data_ptr(), o.data_ptr(), None, None, None, None) == binding.ERR_BAD_ARG
     assert lib.cutoff_order_baseline(0, t.data_ptr(), 0, 8, 8, oi.data_ptr(), None) == binding.ERR_BAD_ARG
+
+
+# running moments are scanned 1024 steps at a time, a warp at a time; the moments kernel takes 8 steps per CTA
+@pytest.mark.parametrize("N,T", [(24, 1), (7, 33), (5, 1024), (5, 1025), (6, 2100)])
+def test_order_baseline_over_long_traces(N, T):
+    import torch
+    trace = _trace(N, T, seed=N + 3 * T)
+    got = binding.order_baseline(torch.from_numpy(trace).cuda()).cpu().numpy()
+    x = trace.astype(np.float64)
+    s1, s2 = np.cumsum(x.sum(1)), np.cumsum((x * x).sum(1))
+    assert got[0] == N
+    for t in range(1, T):
+        mu, n = s1[t - 1] / (t * N), t * N
+        e = E.elfving_expected(N, float(mu), float(np.sqrt(max(s2[t - 1] / n - mu * mu, 0.0))))
+        want = E.cutoff_from_expected(e)
+        # moments differ by the order of a sum in double: 1e-12 of the throughput at most
+        assert got[t] == want or abs(got[t] / e[got[t] - 1] - want / e[want - 1]) <= 1e-9 * abs(want / e[want - 1]), t
+
+
+def test_calls_from_several_threads_and_streams_do_not_share_scratch():
+    import threading
+    import torch
+    cases = [(_trace(N, T, seed=N), torch.cuda.Stream()) for N, T in ((40, 300), (700, 80), (1500, 20), (64, 500))]
+    wrong = []
+
+    def work(trace, stream):
+        dev = torch.from_numpy(trace).cuda()
+        torch.cuda.synchronize()
+        want_c, want_order = E.best_static_cutoff(trace), None
+        with torch.cuda.stream(stream):
+            for _ in range(5):
+                c = int(binding.eval_trace(dev, None, stream=stream.cuda_stream)["static_c"].item())
+                order = binding.order_baseline(dev, stream=stream.cuda_stream).cpu().numpy()
+                want_order = order if want_order is None else want_order
+                if c != want_c or not np.array_equal(order, want_order):
+                    wrong.append((trace.shape, c, want_c))
+
+    threads = [threading.Thread(target=work, args=c) for c in cases]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
