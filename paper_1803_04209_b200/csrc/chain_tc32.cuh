@@ -114,7 +114,6 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
         sb1[i] = a.b1[i];
         sb3[i] = a.b3[i];
     }
-    for (int i = threadIdx.x; i < W * H; i += kChainTcThreads) slr[i] = (a.hlr[i] + a.hlr[W * H + i]) * (1.0f / 3.0f);
     for (int i = threadIdx.x; i < 1024; i += kChainTcThreads) sWsig[i] = a.Wsig[i];
     if (threadIdx.x < 32) {
         sbmu[threadIdx.x] = a.bmu[threadIdx.x];
@@ -153,6 +152,9 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
                      ::"r"(smem_u32(const_cast<uint32_t*>(tmem_slot))), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    dependency_wait();            // up to here: weights.  The encoder's states and the device state are earlier kernels'
+    launch_dependents();
+    for (int i = threadIdx.x; i < W * H; i += kChainTcThreads) slr[i] = (a.hlr[i] + a.hlr[W * H + i]) * (1.0f / 3.0f);
     if (LITERAL) fence_proxy_async();                             // the Ws tile was written with ordinary stores
     tc_fence_before();
     __syncthreads();

@@ -26,6 +26,12 @@ struct DevState {
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// The device state as the host will see it, written straight into pinned host memory by one thread (no copy behind the
+// kernel): visible to the host once the stream has been waited for.
+__device__ __forceinline__ void publish_state(const DevState* st, DevState* host) {
+    if (host) *host = *st;
+}
+
 constexpr int kErrBadValue = 1;
 constexpr int kErrTimeout = 2;
 constexpr int kErrNoFinisher = 4;   // a censored push in which every worker was censored

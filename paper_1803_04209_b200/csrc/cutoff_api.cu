@@ -58,8 +58,7 @@ struct cutoff_ctx {
 
     float* d_ring = nullptr;        // [W][N]
     float* d_stage = nullptr;       // [N] landing buffer for host pushes
-    uint8_t* d_mask = nullptr;      // [N] censoring mask of the push in progress
-    uint8_t* h_mask = nullptr;      // pinned [N]
+    uint8_t* h_mask = nullptr;      // pinned [N]: censoring mask of the push in progress
     bool draws_valid = false;       // d_x holds every predictive draw of the last decision (needed for imputation)
     DevState* d_state = nullptr;
     float* d_proj = nullptr;        // [2][W slots][H] raw input projections of the ring's vectors, kept up to date by every push
@@ -72,8 +71,6 @@ struct cutoff_ctx {
     bool want_std = false;
     bool have_std = false;
     double* d_sums = nullptr;       // [N]
-    float* d_E = nullptr;           // [N]
-    float* d_omega = nullptr;       // [N]
 
     CUtensorMap map_v{};            // TMA view of d_v   [alloc_rows][H]
     CUtensorMap map_w4{};           // TMA view of W4    [2N][H]
@@ -95,8 +92,11 @@ struct cutoff_ctx {
     bool chain_tcl32 = false;       // the same for D = 32, H <= 512 (weights staged phase by phase)
     float* d_chain_image = nullptr; // swizzled tf32 operand tiles of the chain
 
-    float* h_stage = nullptr;       // pinned [N]
-    DevState* h_state = nullptr;    // pinned
+    // pinned host memory that kernels read and write directly (one address on both sides)
+    float* h_stage = nullptr;       // [N] run-times of a host push
+    DevState* h_state = nullptr;    // the device state as of the last push or decision
+    float* h_E = nullptr;           // [N] expected order statistics of the last decision
+    float* h_omega = nullptr;       // [N] throughput per cutoff
 
     uint32_t pushes = 0;            // host mirror of DevState::push_count
     bool pending = false;           // a decision is enqueued and not yet fetched
@@ -112,7 +112,7 @@ struct cutoff_ctx {
 
     cudaGraph_t graph = nullptr;            // captured push + decision (CUTOFF_FLAG_GRAPH)
     cudaGraphExec_t graph_exec = nullptr;
-    cudaGraph_t graph_dev = nullptr;        // the same without the host-to-device copy (cutoff_step_device)
+    cudaGraph_t graph_dev = nullptr;        // the same from the device's landing buffer (cutoff_step_device)
     cudaGraphExec_t graph_dev_exec = nullptr;
     int graph_kernels = 0;                  // kernels one replay launches
     bool decided_once = false;              // a decision has run outside capture (function attributes are set)
@@ -233,12 +233,14 @@ int next_pow2(int n) {
 
 void free_all(cutoff_ctx* c) {
     cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_M);
-    cudaFree(c->d_blob); cudaFree(c->d_WT); cudaFree(c->d_WhR); cudaFree(c->d_chain_image); cudaFree(c->d_mask);
+    cudaFree(c->d_blob); cudaFree(c->d_WT); cudaFree(c->d_WhR); cudaFree(c->d_chain_image);
     if (c->h_mask) cudaFreeHost(c->h_mask); cudaFree(c->d_ring); cudaFree(c->d_stage);
     cudaFree(c->d_state); cudaFree(c->d_proj); cudaFree(c->d_hlr); cudaFree(c->d_v); cudaFree(c->d_x);
-    cudaFree(c->d_partial); cudaFree(c->d_std); cudaFree(c->d_sums); cudaFree(c->d_E); cudaFree(c->d_omega);
+    cudaFree(c->d_partial); cudaFree(c->d_std); cudaFree(c->d_sums);
     if (c->h_stage) cudaFreeHost(c->h_stage);
     if (c->h_state) cudaFreeHost(c->h_state);
+    if (c->h_E) cudaFreeHost(c->h_E);
+    if (c->h_omega) cudaFreeHost(c->h_omega);
     if (c->owns_stream && c->stream) cudaStreamDestroy(c->stream);
     if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
     if (c->graph) cudaGraphDestroy(c->graph);
@@ -360,11 +362,11 @@ void launch_chain_t(cutoff_ctx* c, uint32_t sample_base, int count, size_t smem)
         const int batch = 32 / ChainShape<D>::G * ChainShape<D>::SPL;
         const int batches = ceil_div(count, batch);
         const int grid = batches < c->sm_count ? batches : c->sm_count;
-        k_chain_resident<D><<<grid, kChainResidentThreads, resident, c->stream>>>(c->m, c->d_hlr, c->d_state, key,
-                                                                                sample_base, count, round_v, c->d_v);
+        launch_dependent(k_chain_resident<D>, dim3(grid), dim3(kChainResidentThreads), resident, c->stream, c->m, c->d_hlr, c->d_state, key,
+                         sample_base, count, round_v, c->d_v);
     } else {
-        k_chain<D><<<ceil_div(count, ChainShape<D>::kSamplesPerCta), ChainShape<D>::kThreads, smem, c->stream>>>(
-            c->m, c->d_hlr, c->d_state, key, sample_base, count, round_v, c->d_v);
+        launch_dependent(k_chain<D>, dim3(ceil_div(count, ChainShape<D>::kSamplesPerCta)), dim3(ChainShape<D>::kThreads), smem, c->stream,
+                         c->m, c->d_hlr, c->d_state, key, sample_base, count, round_v, c->d_v);
     }
 }
 
@@ -403,8 +405,8 @@ void launch_chain_tc32(cutoff_ctx* c, uint32_t sample_base, int count) {
     a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.round_v = 1; a.v_out = c->d_v;
     const int tiles = ceil_div(count, 128);
     const int grid = tiles < c->sm_count ? tiles : c->sm_count;
-    if (c->chain_tcl32) tc::k_chain_tc32<true><<<grid, tc::kChainTcThreads, tc::chain_tc32_smem_bytes(c->H, c->W, true), c->stream>>>(a);
-    else tc::k_chain_tc32<false><<<grid, tc::kChainTcThreads, tc::chain_tc32_smem_bytes(c->H, c->W), c->stream>>>(a);
+    if (c->chain_tcl32) launch_dependent(tc::k_chain_tc32<true>, dim3(grid), dim3(tc::kChainTcThreads), tc::chain_tc32_smem_bytes(c->H, c->W, true), c->stream, a);
+    else launch_dependent(tc::k_chain_tc32<false>, dim3(grid), dim3(tc::kChainTcThreads), tc::chain_tc32_smem_bytes(c->H, c->W), c->stream, a);
     c->launches += 1;
 }
 
@@ -412,8 +414,8 @@ template <int D>
 void launch_chain_literal_t(cutoff_ctx* c, uint32_t sample_base, int count) {
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     const size_t smem = chain_smem_floats(c->D, c->H, c->W) * sizeof(float);
-    k_chain_literal<D><<<ceil_div(count, ChainShape<D>::kSamplesPerCta), ChainShape<D>::kThreads, smem, c->stream>>>(
-        c->m, c->lit, c->d_hlr, c->d_state, key, sample_base, count, c->use_tc ? 1 : 0, c->d_v);
+    launch_dependent(k_chain_literal<D>, dim3(ceil_div(count, ChainShape<D>::kSamplesPerCta)), dim3(ChainShape<D>::kThreads), smem, c->stream,
+                     c->m, c->lit, c->d_hlr, c->d_state, key, sample_base, count, c->use_tc ? 1 : 0, c->d_v);
 }
 
 void launch_chain(cutoff_ctx* c, uint32_t sample_base, int count) {
@@ -495,7 +497,7 @@ void launch_emission_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
 void launch_gemm_relu_tc(cutoff_ctx* c, const CUtensorMap& map_a, const CUtensorMap& map_b, const tc::GemmTcArgs& a) {
     const int tiles = ceil_div(a.Nout, tc::kGemmBN) * ceil_div(a.M, tc::kBM);
     const int grid = tiles < c->sm_count ? tiles : c->sm_count;
-    tc::k_gemm_relu_tc<<<grid, tc::kThreads, tc::kSmemBytes, c->stream>>>(map_a, map_b, a);
+    launch_dependent(tc::k_gemm_relu_tc, dim3(grid), dim3(tc::kThreads), tc::kSmemBytes, c->stream, map_a, map_b, a);
     c->launches += 1;
 }
 
@@ -512,8 +514,8 @@ void launch_emission_literal(cutoff_ctx* c, uint32_t sample_base, int count) {
         e.bias_mean = l.bi2; e.bias_scale = l.bj2; e.x = c->d_x; e.st = c->d_state; e.key = key;
         e.sample_base = sample_base; e.count = count; e.N = c->N; e.H = c->H; e.ldx = c->ldx;
         const int tiles = ceil_div(c->N, tc::kBW) * ceil_div(count, tc::kBM);
-        tc::k_emit_dual_tc<<<tiles < c->sm_count ? tiles : c->sm_count, tc::kThreads, tc::kDualSmemBytes, c->stream>>>(
-            c->map_v, c->map_r, c->map_wi2, c->map_wj2, e);
+        launch_dependent(tc::k_emit_dual_tc, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kThreads), tc::kDualSmemBytes, c->stream,
+                         c->map_v, c->map_r, c->map_wi2, c->map_wj2, e);
         c->launches += 1;
         return;
     }
@@ -521,13 +523,13 @@ void launch_emission_literal(cutoff_ctx* c, uint32_t sample_base, int count) {
     a.st = c->d_state; a.key = key; a.sample_base = sample_base; a.M = count;
     a.A = c->d_v; a.lda = c->H; a.B = l.Wi2; a.ldb = c->H; a.bias = l.bi2; a.out = c->d_I; a.ld_out = c->ldx;
     a.Nout = c->N; a.K = c->H;
-    k_gemm_fma<kEpiAffine><<<dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), kEmitThreads, 0, c->stream>>>(a);
+    launch_dependent(k_gemm_fma<kEpiAffine>, dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), dim3(kEmitThreads), 0, c->stream, a);
     a.A = c->d_I; a.lda = c->ldx; a.B = l.Wj1; a.ldb = l.ldn; a.bias = l.bj1; a.out = c->d_r; a.ld_out = c->H;
     a.Nout = c->H; a.K = c->ldx;                                   // the padding columns of both operands are zero
-    k_gemm_fma<kEpiRelu><<<dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), kEmitThreads, 0, c->stream>>>(a);
+    launch_dependent(k_gemm_fma<kEpiRelu>, dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), dim3(kEmitThreads), 0, c->stream, a);
     a.A = c->d_r; a.lda = c->H; a.B = l.Wj2; a.ldb = c->H; a.bias = l.bj2; a.add = c->d_I; a.out = c->d_x; a.ld_out = c->ldx;
     a.Nout = c->N; a.K = c->H;
-    k_gemm_fma<kEpiScaleNoise><<<dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), kEmitThreads, 0, c->stream>>>(a);
+    launch_dependent(k_gemm_fma<kEpiScaleNoise>, dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), dim3(kEmitThreads), 0, c->stream, a);
     c->launches += 3;
 }
 
@@ -536,20 +538,20 @@ void launch_emission(cutoff_ctx* c, uint32_t sample_base, int count) {
     if (c->use_tc) { launch_emission_tc(c, sample_base, count); return; }
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     dim3 grid(ceil_div(c->N, kEmitTN), ceil_div(count, kEmitTM));
-    k_emit_fma<<<grid, kEmitThreads, 0, c->stream>>>(c->m, c->d_v, c->d_state, key, sample_base, count, c->d_x, c->ldx);
+    launch_dependent(k_emit_fma, grid, dim3(kEmitThreads), 0, c->stream, c->m, c->d_v, c->d_state, key, sample_base, count, c->d_x, c->ldx);
     c->launches += 1;
 }
 
 template <int HQ>
 void launch_rnn_resident(cutoff_ctx* c) {
     const size_t smem = enc_rnn_resident_smem_floats(c->H, c->W) * sizeof(float);
-    k_enc_rnn_resident<HQ><<<2, 16 * HQ, smem, c->stream>>>(c->m, c->d_WhR, c->d_proj, c->d_state, c->d_hlr);
+    launch_dependent(k_enc_rnn_resident<HQ>, dim3(2), dim3(16 * HQ), smem, c->stream, c->m, c->d_WhR, c->d_proj, c->d_state, c->d_hlr);
 }
 
 // Input projections: of the newest vector after a push, of every slot when the ring or the weights changed.
 void launch_projection(cutoff_ctx* c, bool newest_only) {
-    dim3 grid(ceil_div(c->H, kProjWarps), 2);
-    k_enc_proj<<<grid, kProjWarps * 32, 0, c->stream>>>(c->m, c->d_ring, c->d_state, newest_only ? 1 : 0, c->d_proj);
+    launch_dependent(c->N % 4 == 0 ? k_enc_proj<true> : k_enc_proj<false>, dim3(ceil_div(c->H, kProjRows), 2), dim3(kProjThreads), 0, c->stream,
+                     c->m, c->d_ring, c->d_state, newest_only ? 1 : 0, c->d_proj);
     c->launches += 1;
 }
 
@@ -570,9 +572,9 @@ void launch_encoder(cutoff_ctx* c) {
     else if (c->H == 64 && resident_smem <= 200 * 1024) launch_rnn_resident<16>(c);
     else if (c->H == 128 && resident_smem <= 200 * 1024) launch_rnn_resident<32>(c);
     else if (c->H >= 256 && c->H % 32 == 0 && c->H <= 1024 && cluster_smem <= 200 * 1024)
-        k_enc_rnn_cluster<<<2 * kRnnClusterSize, c->H, cluster_smem, c->stream>>>(c->m, c->d_proj, c->d_state, c->d_hlr);
+        launch_dependent(k_enc_rnn_cluster, dim3(2 * kRnnClusterSize), dim3(c->H), cluster_smem, c->stream, c->m, c->d_proj, c->d_state, c->d_hlr);
     else
-        k_enc_rnn<<<2, kRnnThreads, 2 * c->H * sizeof(float), c->stream>>>(c->m, c->d_proj, c->d_state, c->d_hlr);
+        launch_dependent(k_enc_rnn, dim3(2), dim3(kRnnThreads), 2 * c->H * sizeof(float), c->stream, c->m, c->d_proj, c->d_state, c->d_hlr);
     c->launches += 1;
 }
 
@@ -611,13 +613,12 @@ int enqueue_decision(cutoff_ctx* c, bool decide = true) {
     const int64_t total = c->cfg.total_samples > 0 ? c->cfg.total_samples : c->S;
     launch_dependent(k_colsum_decide, dim3(ceil_div(c->N, 32)), dim3(kColsumThreads), 0, c->stream,
                      c->d_partial, c->n_chunks * c->sort_grid, c->N, c->d_sums, 1.0 / static_cast<double>(total), c->d_state,
-                     c->d_E, c->d_omega, c->want_std ? c->d_partial + static_cast<size_t>(kPartialRows) * c->N : nullptr,
-                     c->d_std, decide ? 1 : 0);
+                     c->h_E, c->h_omega, c->want_std ? c->d_partial + static_cast<size_t>(kPartialRows) * c->N : nullptr,
+                     c->d_std, decide ? 1 : 0, c->h_state);
     c->have_std = c->want_std;
     c->launches += 1;
     if (timed) cudaEventRecord(c->ev[5][0], c->stream);
     c->timed_chunks = timed ? c->n_chunks : 0;
-    CU_CHECK(c, cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CU_CHECK(c, cudaGetLastError());
     return CUTOFF_OK;
 }
@@ -831,7 +832,6 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     if (c->chain_tcl32) CREATE_CHECK(cudaMalloc(&c->d_chain_image, sizeof(float) * tc::chain_tc32_image_floats(c->H, true)));
     CREATE_CHECK(cudaMalloc(&c->d_ring, sizeof(float) * c->W * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_stage, sizeof(float) * c->N));
-    CREATE_CHECK(cudaMalloc(&c->d_mask, c->N));
     CREATE_CHECK(cudaMallocHost(&c->h_mask, c->N));
     CREATE_CHECK(cudaMalloc(&c->d_state, sizeof(DevState)));
     CREATE_CHECK(cudaMalloc(&c->d_proj, sizeof(float) * 2 * c->W * c->H));
@@ -841,8 +841,6 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     CREATE_CHECK(cudaMalloc(&c->d_partial, sizeof(float) * 2 * static_cast<size_t>(kPartialRows) * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_std, sizeof(float) * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_sums, sizeof(double) * c->N));
-    CREATE_CHECK(cudaMalloc(&c->d_E, sizeof(float) * c->N));
-    CREATE_CHECK(cudaMalloc(&c->d_omega, sizeof(float) * c->N));
     if (c->use_tc) {
         int rc = make_tile_map(c, &c->map_v, c->d_v, static_cast<uint64_t>(c->alloc_rows), static_cast<uint64_t>(c->H));
         if (!rc && c->literal)
@@ -869,6 +867,8 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     }
     CREATE_CHECK(cudaMallocHost(&c->h_stage, sizeof(float) * c->N));
     CREATE_CHECK(cudaMallocHost(&c->h_state, sizeof(DevState)));
+    CREATE_CHECK(cudaMallocHost(&c->h_E, sizeof(float) * c->N));
+    CREATE_CHECK(cudaMallocHost(&c->h_omega, sizeof(float) * c->N));
     CREATE_CHECK(cudaMemsetAsync(c->d_state, 0, sizeof(DevState), c->stream));
     CREATE_CHECK(cudaMemsetAsync(c->d_ring, 0, sizeof(float) * c->W * c->N, c->stream));
     CREATE_CHECK(cudaStreamSynchronize(c->stream));
@@ -1093,9 +1093,13 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
     return CUTOFF_OK;
 }
 
-static int push_common(cutoff_ctx* c, const float* dev_src) {
-    k_push<<<1, kPushThreads, 0, c->stream>>>(dev_src, c->d_ring, c->d_state, c->N, c->W);
+static void launch_push(cutoff_ctx* c, const float* src) {
+    launch_dependent(k_push, dim3(1), dim3(kPushThreads), 0, c->stream, src, c->d_ring, c->d_state, c->N, c->W, c->h_state);
     c->launches += 1;
+}
+
+static int push_common(cutoff_ctx* c, const float* src) {
+    launch_push(c, src);
     if (c->weights_loaded && !c->proj_stale) launch_projection(c, true);     // else every slot is redone before the next decision
     CU_CHECK(c, cudaGetLastError());
     c->pushes += 1;
@@ -1115,7 +1119,8 @@ static int push_censored(cutoff_ctx* c, const float* runtimes_sec, int on_device
     if (!c->draws_valid) return CUTOFF_ERR_STATE;          // no decision yet whose draws could be used
     if (c->cfg.sample_offset != 0 || (c->cfg.total_samples > 0 && c->cfg.total_samples != c->S))
         return CUTOFF_ERR_UNSUPPORTED;                      // a context that holds only part of the draws
-    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    const float* src = runtimes_sec;
+    const uint8_t* mask = censored;
     if (!on_device) {
         int finished = 0;
         for (int j = 0; j < c->N; ++j) {
@@ -1127,19 +1132,15 @@ static int push_censored(cutoff_ctx* c, const float* runtimes_sec, int on_device
         CU_CHECK(c, cudaStreamSynchronize(c->stream));     // the landing buffers may still be in use
         for (int j = 0; j < c->N; ++j) c->h_stage[j] = censored[j] ? 1.0f : runtimes_sec[j];
         std::memcpy(c->h_mask, censored, c->N);
-        CU_CHECK(c, cudaMemcpyAsync(c->d_stage, c->h_stage, sizeof(float) * c->N, kind, c->stream));
-        CU_CHECK(c, cudaMemcpyAsync(c->d_mask, c->h_mask, c->N, kind, c->stream));
-    } else {
-        CU_CHECK(c, cudaMemcpyAsync(c->d_stage, runtimes_sec, sizeof(float) * c->N, kind, c->stream));
-        CU_CHECK(c, cudaMemcpyAsync(c->d_mask, censored, c->N, kind, c->stream));
+        src = c->h_stage;
+        mask = c->h_mask;
     }
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
-    k_impute<<<1, kImputeThreads, 0, c->stream>>>(c->d_stage, c->d_mask, c->d_x, c->ldx, c->S, c->N, c->d_state, key);
+    k_impute<<<1, kImputeThreads, 0, c->stream>>>(src, mask, c->d_stage, c->d_x, c->ldx, c->S, c->N, c->d_state, key);
     c->launches += 1;
     c->draws_valid = false;                                 // one step's draws serve one push
     int rc = push_common(c, c->d_stage);
     if (rc) return rc;
-    CU_CHECK(c, cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CU_CHECK(c, cudaStreamSynchronize(c->stream));
     if (c->h_state->error_flags & (kErrBadValue | kErrNoFinisher)) {
         c->pushes = c->h_state->push_count;
@@ -1159,12 +1160,10 @@ int cutoff_push(cutoff_ctx* c, const float* runtimes_sec, int on_device, const u
             if (!(runtimes_sec[j] > 0.0f) || !std::isfinite(runtimes_sec[j])) return CUTOFF_ERR_BAD_VALUE;
         CU_CHECK(c, cudaStreamSynchronize(c->stream));       // the landing buffer may still be in use
         std::memcpy(c->h_stage, runtimes_sec, sizeof(float) * c->N);
-        CU_CHECK(c, cudaMemcpyAsync(c->d_stage, c->h_stage, sizeof(float) * c->N, cudaMemcpyHostToDevice, c->stream));
-        return push_common(c, c->d_stage);
+        return push_common(c, c->h_stage);
     }
     const int rc = push_common(c, runtimes_sec);
     if (rc) return rc;
-    CU_CHECK(c, cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CU_CHECK(c, cudaStreamSynchronize(c->stream));
     if (c->h_state->error_flags & kErrBadValue) {
         // the kernel left the window untouched; clear the flag and undo the host-side count
@@ -1226,16 +1225,14 @@ int cutoff_predict(cutoff_ctx* c, int32_t* c_out) {
     return cutoff_fetch(c, c_out);
 }
 
-// Capture "land the staged run-times, push, decide, read back the state" once; replays need no
+// Capture "push, decide" once, the run-times read from the pinned landing buffer or from the one on the device; replays need no
 // changing argument because the window position, the normaliser and the decision counter live
 // in device memory.
-static int build_graph(cutoff_ctx* c, bool with_host_copy) {
+static int build_graph(cutoff_ctx* c, bool from_host) {
     refresh_projections(c);                        // not part of the graph: replays only project the vector they push
     const int64_t launches_before = c->launches;
     CU_CHECK(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-    if (with_host_copy) cudaMemcpyAsync(c->d_stage, c->h_stage, sizeof(float) * c->N, cudaMemcpyHostToDevice, c->stream);
-    k_push<<<1, kPushThreads, 0, c->stream>>>(c->d_stage, c->d_ring, c->d_state, c->N, c->W);
-    c->launches += 1;
+    launch_push(c, from_host ? c->h_stage : c->d_stage);
     launch_projection(c, true);
     const bool timing = c->timing;
     c->timing = false;
@@ -1251,7 +1248,7 @@ static int build_graph(cutoff_ctx* c, bool with_host_copy) {
         cudaGetLastError();
         return CUTOFF_ERR_CUDA;
     }
-    if (with_host_copy) {
+    if (from_host) {
         c->graph = g;
         CU_CHECK(c, cudaGraphInstantiate(&c->graph_exec, c->graph, 0));
     } else {
@@ -1338,10 +1335,9 @@ int cutoff_get_stats(cutoff_ctx* c, float* e_out, float* omega_out) {
     if (!c->have_result) return CUTOFF_ERR_STATE;
     DeviceGuard guard(c->cfg.device);
     CU_CHECK(c, guard.err);
-    if (e_out) CU_CHECK(c, cudaMemcpyAsync(e_out, c->d_E, sizeof(float) * c->N, cudaMemcpyDeviceToHost, c->stream));
-    if (omega_out)
-        CU_CHECK(c, cudaMemcpyAsync(omega_out, c->d_omega, sizeof(float) * c->N, cudaMemcpyDeviceToHost, c->stream));
-    CU_CHECK(c, cudaStreamSynchronize(c->stream));
+    if (c->pending || c->partial_pending) CU_CHECK(c, cudaStreamSynchronize(c->stream));   // a later decision is writing them
+    if (e_out) std::memcpy(e_out, c->h_E, sizeof(float) * c->N);
+    if (omega_out) std::memcpy(omega_out, c->h_omega, sizeof(float) * c->N);
     return CUTOFF_OK;
 }
 
@@ -1374,9 +1370,8 @@ int cutoff_decide_from_sums(cutoff_ctx* c, const double* sums, int32_t* c_out) {
     CU_CHECK(c, cudaMemcpyAsync(c->d_sums, sums, sizeof(double) * c->N, cudaMemcpyHostToDevice, c->stream));
     const int64_t total = c->cfg.total_samples > 0 ? c->cfg.total_samples : c->S;
     k_decide<<<1, kDecideThreads, 0, c->stream>>>(c->d_sums, c->N, 1.0 / static_cast<double>(total), c->d_state, 0,
-                                                  c->d_E, c->d_omega);
+                                                  c->h_E, c->h_omega, c->h_state);
     c->launches += 1;
-    CU_CHECK(c, cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CU_CHECK(c, cudaStreamSynchronize(c->stream));
     c->have_result = true;
     *c_out = c->h_state->c_star;
@@ -1412,9 +1407,8 @@ int cutoff_decide_from_device_sums(cutoff_ctx* c, const double* sums_device, int
     const int64_t total = c->cfg.total_samples > 0 ? c->cfg.total_samples : c->S;
     // the decision counter moves on here if the sums came from cutoff_predict_partial_async (which left it alone)
     k_decide<<<1, kDecideThreads, 0, c->stream>>>(c->d_sums, c->N, 1.0 / static_cast<double>(total), c->d_state,
-                                                  c->partial_pending ? 1 : 0, c->d_E, c->d_omega);
+                                                  c->partial_pending ? 1 : 0, c->h_E, c->h_omega, c->h_state);
     c->launches += 1;
-    CU_CHECK(c, cudaMemcpyAsync(c->h_state, c->d_state, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     CU_CHECK(c, cudaStreamSynchronize(c->stream));
     if (c->h_state->error_flags & kErrBadValue) {
         // a bad asynchronous push came before this decision: as cutoff_fetch reports it

@@ -127,6 +127,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    dependency_wait();            // the operands and the device state are an earlier kernel's
+    launch_dependents();
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------------------------------------------------
@@ -359,6 +361,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    dependency_wait();            // the operands and the device state are an earlier kernel's
+    launch_dependents();
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------------------------------------------------

@@ -98,8 +98,6 @@ __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain_literal(Model
     const int H = m.H, W = m.W;
     const int g = threadIdx.x % G;
     const int k0 = (blockIdx.x * (ChainShape<D>::kThreads / G) + threadIdx.x / G) * SPL;
-    const ChainNoise nz{key, st->step, sample_base + static_cast<uint32_t>(k0)};
-
     {   // guide
         float* sWzT = sm;
         float* sWmu = sWzT + H * D;
@@ -110,8 +108,11 @@ __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain_literal(Model
         stage_vector4(sWmu, m.Wmu, H * D);
         stage_vector4(sWsig, m.Wsig, D * D);
         stage_vector4(sbz, m.bz, H);
+        dependency_wait();        // up to here: weights
+        launch_dependents();
         for (int i = threadIdx.x; i < W * H; i += blockDim.x) shl[i] = hlr[i] + hlr[W * H + i];
     }
+    const ChainNoise nz{key, st->step, sample_base + static_cast<uint32_t>(k0)};
     __syncthreads();
     float z[SPL][D];
 #pragma unroll
@@ -213,6 +214,8 @@ __global__ void __launch_bounds__(kEmitThreads) k_gemm_fma(GemmFmaArgs a) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
     const int lr = tid >> 2, lc = (tid & 3) * 4;
+    dependency_wait();
+    launch_dependents();
     for (int kk = 0; kk < a.K; kk += kEmitTK) {
         float4 av = make_float4(0.f, 0.f, 0.f, 0.f), bv = av;
         if (kk + lc < a.K) {

@@ -10,45 +10,63 @@ namespace cutoff {
 // push: obs <- obs U r_w for one whole step (Algorithm 1), plus the normaliser of Section 3.1.3
 // (twice the mean of the first fixed-lag window).  One CTA; the sum is a fixed-order tree.
 // ---------------------------------------------------------------------------------------------
-constexpr int kPushThreads = 256;
+constexpr int kPushThreads = 1024, kPushPer = 4;             // N <= 4096: every run-time is read once, into a register
 
+// src may be pinned host memory (read over the bus: one round trip, less than a copy and the launch behind it).
 __global__ void __launch_bounds__(kPushThreads) k_push(const float* __restrict__ src, float* __restrict__ ring,
-                                                       DevState* st, int N, int W) {
-    __shared__ double red[kPushThreads];
-    const int tid = threadIdx.x;
+                                                       DevState* st, int N, int W, DevState* host_state) {
+    __shared__ double red[kPushThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    dependency_wait();
+    launch_dependents();
+    float v[kPushPer];
+#pragma unroll
+    for (int i = 0; i < kPushPer; ++i) v[i] = tid + i * kPushThreads < N ? src[tid + i * kPushThreads] : 1.0f;
     const uint32_t pushes = st->push_count;
-    double s = 0.0;
     int bad = 0;
-    for (int j = tid; j < N; j += kPushThreads) {
-        const float v = src[j];
-        if (!(v > 0.0f) || !isfinite(v)) bad = 1;
-        s += static_cast<double>(v);
-    }
+#pragma unroll
+    for (int i = 0; i < kPushPer; ++i)
+        if (!(v[i] > 0.0f) || !isfinite(v[i])) bad = 1;
     if (tid == 0 && (st->error_flags & kErrNoFinisher)) bad = 1;   // raised by the imputation that precedes this push
     bad = __syncthreads_or(bad);
     if (bad) {
-        if (tid == 0) st->error_flags |= kErrBadValue;
+        if (tid == 0) {
+            st->error_flags |= kErrBadValue;
+            publish_state(st, host_state);
+        }
         return;
     }
-    red[tid] = s;
-    __syncthreads();
-    for (int half = kPushThreads / 2; half > 0; half >>= 1) {
-        if (tid < half) red[tid] += red[tid + half];
-        __syncthreads();
-    }
     float* dst = ring + static_cast<size_t>(pushes % W) * N;
-    for (int j = tid; j < N; j += kPushThreads) dst[j] = src[j];
-    if (tid == 0) {
-        if (pushes < static_cast<uint32_t>(W)) {
-            const double total = st->norm_sum + red[0];
-            st->norm_sum = total;
-            if (pushes + 1 == static_cast<uint32_t>(W)) {
-                const double scale = 2.0 * total / (static_cast<double>(N) * W);
-                st->scale = static_cast<float>(scale);
-                st->inv_scale = static_cast<float>(1.0 / scale);
+#pragma unroll
+    for (int i = 0; i < kPushPer; ++i)
+        if (tid + i * kPushThreads < N) dst[tid + i * kPushThreads] = v[i];
+    if (pushes < static_cast<uint32_t>(W)) {           // the normaliser is still being formed
+        double s = 0.0;
+#pragma unroll
+        for (int i = 0; i < kPushPer; ++i)
+            if (tid + i * kPushThreads < N) s += static_cast<double>(v[i]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) red[warp] = s;
+        __syncthreads();
+        if (warp == 0) {
+            s = red[lane];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            if (lane == 0) {
+                const double total = st->norm_sum + s;
+                st->norm_sum = total;
+                if (pushes + 1 == static_cast<uint32_t>(W)) {
+                    const double scale = 2.0 * total / (static_cast<double>(N) * W);
+                    st->scale = static_cast<float>(scale);
+                    st->inv_scale = static_cast<float>(1.0 / scale);
+                }
             }
         }
+    }
+    if (tid == 0) {
         st->push_count = pushes + 1;
+        publish_state(st, host_state);
     }
 }
 
@@ -64,27 +82,31 @@ __global__ void __launch_bounds__(kPushThreads) k_push(const float* __restrict__
 constexpr int kImputeThreads = 1024;
 constexpr uint32_t kStreamImpute = 0x300u;
 
-__global__ void __launch_bounds__(kImputeThreads) k_impute(float* __restrict__ stage, const uint8_t* __restrict__ censored,
-                                                            const float* __restrict__ x, int ldx, int S, int N,
+// src and censored may be pinned host memory; stage receives the completed vector.  Draws above the threshold are rare, so a
+// column is mostly read to its end: kImputeAhead blocks of 32 draws are in flight at a time.
+constexpr int kImputeAhead = 8;
+
+__global__ void __launch_bounds__(kImputeThreads) k_impute(const float* __restrict__ src, const uint8_t* __restrict__ censored,
+                                                            float* __restrict__ stage, const float* __restrict__ x, int ldx, int S, int N,
                                                             DevState* __restrict__ st, NoiseKey key) {
     __shared__ float red[kImputeThreads / 32];
-    __shared__ float s_threshold;
+    __shared__ uint8_t mask[4096];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float m = -INFINITY;
-    for (int j = threadIdx.x; j < N; j += kImputeThreads)
-        if (!censored[j]) m = fmaxf(m, stage[j]);
+    for (int j = threadIdx.x; j < N; j += kImputeThreads) {
+        const uint8_t c = censored[j];
+        const float v = src[j];
+        mask[j] = c;
+        if (!c) { m = fmaxf(m, v); stage[j] = v; }
+    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     if (lane == 0) red[warp] = m;
     __syncthreads();
-    if (warp == 0) {
-        m = red[lane];
+    m = red[lane];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        if (lane == 0) s_threshold = m;
-    }
-    __syncthreads();
-    const float threshold = s_threshold;
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    const float threshold = m;
     if (!(threshold > -INFINITY)) {
         // nobody finished, so there is no cutoff time to truncate at: flag the vector; the push kernel that
         // follows sees the flag and leaves the window untouched
@@ -93,23 +115,33 @@ __global__ void __launch_bounds__(kImputeThreads) k_impute(float* __restrict__ s
     }
     const float scale = st->scale;
     const uint32_t step = st->step;
-    for (int j = warp; j < N; j += kImputeThreads / 32) {
-        if (!censored[j]) continue;
+    int turn = 0;                                       // censored workers go to the warps in turn
+    for (int j = 0; j < N; ++j) {
+        if (!mask[j]) continue;
+        if ((turn++ & (kImputeThreads / 32 - 1)) != warp) continue;
         const uint32_t start = philox4x32_10(static_cast<uint32_t>(j), 0u, kStreamImpute, step, key.seed_lo, key.seed_hi).x %
                                static_cast<uint32_t>(S);
         float value = threshold;
-        for (int base = 0; base < S; base += 32) {
-            const int i = base + lane;
-            float v = -INFINITY;
-            if (i < S) {
-                uint32_t k = start + static_cast<uint32_t>(i);
-                if (k >= static_cast<uint32_t>(S)) k -= static_cast<uint32_t>(S);
-                v = x[static_cast<size_t>(k) * ldx + j] * scale;
+        bool found = false;
+        for (int base = 0; base < S && !found; base += 32 * kImputeAhead) {
+            float v[kImputeAhead];
+#pragma unroll
+            for (int u = 0; u < kImputeAhead; ++u) {
+                const int i = base + 32 * u + lane;
+                v[u] = -INFINITY;
+                if (i < S) {
+                    uint32_t k = start + static_cast<uint32_t>(i);
+                    if (k >= static_cast<uint32_t>(S)) k -= static_cast<uint32_t>(S);
+                    v[u] = x[static_cast<size_t>(k) * ldx + j] * scale;
+                }
             }
-            const uint32_t hit = __ballot_sync(0xffffffffu, v > threshold);
-            if (hit) {
-                value = __shfl_sync(0xffffffffu, v, __ffs(hit) - 1);
-                break;
+#pragma unroll
+            for (int u = 0; u < kImputeAhead; ++u) {
+                const uint32_t hit = __ballot_sync(0xffffffffu, v[u] > threshold);
+                if (hit && !found) {
+                    value = __shfl_sync(0xffffffffu, v[u], __ffs(hit) - 1);
+                    found = true;
+                }
             }
         }
         if (lane == 0) stage[j] = value;
@@ -120,65 +152,61 @@ __global__ void __launch_bounds__(kImputeThreads) k_impute(float* __restrict__ s
 // Encoder, part 1: input projections of both RNNs, cached per ring slot,
 //   R[dir][slot][i] = sum_j Wx_dir[i][j] * x_slot[j]          (raw seconds: the normaliser is applied by part 2,
 //                                                              so a slot's projection never has to be redone)
-// One warp per hidden unit i; the weight row is read once for all slots of the launch.
+// Four warps per hidden unit, a quarter of the workers each; the weight row is read once for all slots of the launch, into
+// registers, before the kernel waits for the push in front of it.  (One warp per row with its loads behind the wait: 20 us for
+// N = 2175, whose rows are not aligned, and for N = 4096, H = 512; 5 us for N = 1024.)
 // newest_only = 1: only the slot of the vector pushed last (launched after every push);
 // newest_only = 0: every slot (after the ring or the weights were replaced).  Both run the same
 // arithmetic per slot, so a cached projection equals a recomputed one bit for bit.
 // ---------------------------------------------------------------------------------------------
-constexpr int kProjWarps = 8;
-constexpr int kProjChunk = 8;
+constexpr int kProjRows = 2, kProjSplit = 4, kProjThreads = kProjRows * kProjSplit * 32;
+constexpr int kProjPer = 4096 / kProjSplit / 32;              // columns per lane at most
 
-__global__ void __launch_bounds__(kProjWarps * 32) k_enc_proj(ModelDev m, const float* __restrict__ ring,
-                                                               const DevState* __restrict__ st, int newest_only,
-                                                               float* __restrict__ proj /*[2][W slots][H]*/) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = blockIdx.x * kProjWarps + warp;
-    const int dir = blockIdx.y;
-    if (i >= m.H) return;
-    const float* Wx = (dir ? m.Wxb : m.Wxf) + static_cast<size_t>(i) * m.N;
+template <bool VEC>          // VEC: N is a multiple of 4, rows and ring slots start on 16 bytes
+__device__ __forceinline__ void load_quarter(const float* __restrict__ row, int c0, int c1, int lane, float (&v)[kProjPer]) {
+    if (VEC) {
+#pragma unroll
+        for (int i = 0; i < kProjPer; i += 4) {
+            const int c = c0 + i * 32 + 4 * lane;
+            const float4 q = c < c1 ? *reinterpret_cast<const float4*>(row + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[i] = q.x; v[i + 1] = q.y; v[i + 2] = q.z; v[i + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kProjPer; ++i) {
+            const int c = c0 + i * 32 + lane;
+            v[i] = c < c1 ? row[c] : 0.f;
+        }
+    }
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(kProjThreads) k_enc_proj(ModelDev m, const float* __restrict__ ring,
+                                                            const DevState* __restrict__ st, int newest_only,
+                                                            float* __restrict__ proj /*[2][W slots][H]*/) {
+    __shared__ float red[kProjRows][kProjSplit];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, part = warp % kProjSplit, r = warp / kProjSplit;
+    const int i = blockIdx.x * kProjRows + r, dir = blockIdx.y;
+    const int len = (m.N + 4 * kProjSplit - 1) / (4 * kProjSplit) * 4, c0 = part * len, c1 = min(c0 + len, m.N);
+    float w[kProjPer], x[kProjPer];
+    load_quarter<VEC>((dir ? m.Wxb : m.Wxf) + static_cast<size_t>(min(i, m.H - 1)) * m.N, c0, c1, lane, w);
+    dependency_wait();
+    launch_dependents();
     const int slot_first = newest_only ? static_cast<int>((st->push_count + m.W - 1) % m.W) : 0;
     const int n_slots = newest_only ? 1 : m.W;
-    for (int s0 = 0; s0 < n_slots; s0 += kProjChunk) {
-        float acc[kProjChunk];
-        const float* row[kProjChunk];
+    for (int s = 0; s < n_slots; ++s) {
+        load_quarter<VEC>(ring + static_cast<size_t>(slot_first + s) * m.N, c0, c1, lane, x);
+        float acc[4] = {};
 #pragma unroll
-        for (int tt = 0; tt < kProjChunk; ++tt) {
-            acc[tt] = 0.0f;
-            row[tt] = ring + static_cast<size_t>(slot_first + min(s0 + tt, n_slots - 1)) * m.N;
-        }
-        if ((m.N & 3) == 0) {
-            // 16-byte loads, four independent iterations in flight
-#pragma unroll 4
-            for (int j = 4 * lane; j < m.N; j += 128) {
-                const float4 w = *reinterpret_cast<const float4*>(Wx + j);
+        for (int k = 0; k < kProjPer; ++k) acc[k & 3] = fmaf(w[k], x[k], acc[k & 3]);
+        float v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
 #pragma unroll
-                for (int tt = 0; tt < kProjChunk; ++tt) {
-                    if (s0 + tt >= n_slots) break;          // uniform: one slot after a push
-                    const float4 xv = *reinterpret_cast<const float4*>(row[tt] + j);
-                    acc[tt] = fmaf(w.x, xv.x, acc[tt]);
-                    acc[tt] = fmaf(w.y, xv.y, acc[tt]);
-                    acc[tt] = fmaf(w.z, xv.z, acc[tt]);
-                    acc[tt] = fmaf(w.w, xv.w, acc[tt]);
-                }
-            }
-        } else {
-            for (int j = lane; j < m.N; j += 32) {
-                const float w = Wx[j];
-#pragma unroll
-                for (int tt = 0; tt < kProjChunk; ++tt) {
-                    if (s0 + tt >= n_slots) break;
-                    acc[tt] = fmaf(w, row[tt][j], acc[tt]);
-                }
-            }
-        }
-#pragma unroll
-        for (int tt = 0; tt < kProjChunk; ++tt) {
-            float v = acc[tt];
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-            if (lane == 0 && s0 + tt < n_slots)
-                proj[(static_cast<size_t>(dir) * m.W + slot_first + s0 + tt) * m.H + i] = v;
-        }
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (lane == 0) red[r][part] = v;
+        __syncthreads();
+        if (part == 0 && lane == 0 && i < m.H)
+            proj[(static_cast<size_t>(dir) * m.W + slot_first + s) * m.H + i] = (red[r][0] + red[r][1]) + (red[r][2] + red[r][3]);
+        __syncthreads();
     }
 }
 
@@ -208,6 +236,8 @@ __global__ void __launch_bounds__(kRnnThreads) k_enc_rnn(ModelDev m, const float
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float* Wh = dir ? m.Whb : m.Whf;
     const float* init = dir ? m.b0 : m.a0;
+    dependency_wait();
+    launch_dependents();
     const uint32_t pushes = st->push_count;
     const float inv_scale = st->inv_scale;
     for (int i = threadIdx.x; i < m.H; i += kRnnThreads) state[i] = init[i];
@@ -260,12 +290,14 @@ __global__ void __launch_bounds__(16 * HQ) k_enc_rnn_resident(ModelDev m, const 
         const float4 v = Wh[static_cast<size_t>(j4) * T + t];
         w[4 * j4 + 0] = v.x; w[4 * j4 + 1] = v.y; w[4 * j4 + 2] = v.z; w[4 * j4 + 3] = v.w;
     }
+    if (t < H) state[(t / HQ) * PAD + (t % HQ)] = init[t];
+    dependency_wait();            // up to here: weights.  The projections and the device state are earlier kernels'
+    launch_dependents();
     {
         const uint32_t pushes = dev_state->push_count;
         const float inv_scale = dev_state->inv_scale;
         for (int idx = t; idx < m.W * H; idx += T) sproj[idx] = window_projection(m, proj, dir, idx / H, idx % H, pushes, inv_scale);
     }
-    if (t < H) state[(t / HQ) * PAD + (t % HQ)] = init[t];
     __syncthreads();
     int cur = 0;
     for (int s = 0; s < m.W; ++s) {
@@ -314,7 +346,6 @@ __global__ void __cluster_dims__(kRnnClusterSize, 1, 1) __launch_bounds__(1024)
 k_enc_rnn_cluster(ModelDev m, const float* __restrict__ proj, const DevState* __restrict__ dev_state,
                   float* __restrict__ hlr /*[2][W][H]*/) {
     extern __shared__ __align__(16) float sm_rc[];
-    launch_dependents();      // the chain kernel may set itself up on the SMs this kernel leaves free
     const int H = m.H, W = m.W, R = H / kRnnClusterSize, ldw = H + 8;
     float* sW = sm_rc;                         // [R][ldw]  rows rank*R .. of the recurrence matrix
     float* state = sW + static_cast<size_t>(R) * ldw;      // [2][H]
@@ -341,6 +372,8 @@ k_enc_rnn_cluster(ModelDev m, const float* __restrict__ proj, const DevState* __
         }
     }
     for (int k = threadIdx.x; k < H; k += blockDim.x) state[k] = init[k];
+    dependency_wait();            // up to here: weights.  The projections and the device state are earlier kernels'
+    launch_dependents();          // the chain kernel may set itself up on the SMs this kernel leaves free
     {
         const uint32_t pushes = dev_state->push_count;
         const float inv_scale = dev_state->inv_scale;
@@ -628,7 +661,6 @@ __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain(ModelDev m, c
     const int H = m.H, W = m.W;
     const int g = threadIdx.x % G;
     const int k0 = (blockIdx.x * (ChainShape<D>::kThreads / G) + threadIdx.x / G) * SPL;      // first sample of the lane
-    const ChainNoise nz{key, st->step, sample_base + static_cast<uint32_t>(k0)};
 
     float* sWzT = sm;                   // [D][H]
     float* sWmu = sWzT + H * D;         // [D][H]
@@ -639,6 +671,9 @@ __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain(ModelDev m, c
     stage_vector4(sWmu, m.Wmu, H * D);
     stage_vector4(sWsig, m.Wsig, D * D);
     stage_vector4(sbz, m.bz, H);
+    dependency_wait();            // up to here: weights
+    launch_dependents();
+    const ChainNoise nz{key, st->step, sample_base + static_cast<uint32_t>(k0)};
     for (int i = threadIdx.x; i < W * H; i += blockDim.x) shl[i] = hlr[i] + hlr[W * H + i];
     __syncthreads();
     float z[SPL][D];
@@ -704,6 +739,8 @@ k_chain_resident(ModelDev m, const float* __restrict__ hlr, const DevState* __re
     stage_vector4(sbz, m.bz, H);
     stage_vector4(sb1, m.b1, H);
     stage_vector4(sb3, m.b3, H);
+    dependency_wait();            // up to here: weights
+    launch_dependents();
     for (int i = threadIdx.x; i < W * H; i += kChainResidentThreads) shl[i] = hlr[i] + hlr[W * H + i];
     __syncthreads();
 
@@ -750,6 +787,8 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit_fma(ModelDev m, const flo
         for (int b = 0; b < 4; ++b) acc_m[a][b] = acc_l[a][b] = 0.0f;
 
     const int lr = tid >> 2, lc = (tid & 3) * 4;
+    dependency_wait();
+    launch_dependents();
     for (int kk = 0; kk < H; kk += kEmitTK) {
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), bm = a, bl = a;
         if (kk + lc < H) {

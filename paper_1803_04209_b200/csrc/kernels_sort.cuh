@@ -393,11 +393,12 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_sum_tma(const float* _
 // ---------------------------------------------------------------------------------------------
 // Decision: E_j = s * sums_j / S (seconds), Omega(c) = c / E_c (minus infinity where E_c <= 0),
 // c* = the largest c attaining the maximum; c* = N and code 2 if no c is admissible.
-// Executed by one whole CTA of THREADS threads.  Advances the decision counter when asked to.
+// Executed by one whole CTA of THREADS threads.  Advances the decision counter when asked to.  e_out, omega_out and host_state are
+// pinned host memory: the results are where cutoff_get_stats and cutoff_fetch read them when the stream has been waited for.
 // ---------------------------------------------------------------------------------------------
 template <int THREADS>
 __device__ __forceinline__ void decide_block(const double* sums, int N, double inv_samples, DevState* st, int advance,
-                                             float* __restrict__ e_out, float* __restrict__ omega_out) {
+                                             float* __restrict__ e_out, float* __restrict__ omega_out, DevState* host_state) {
     __shared__ double best_val[THREADS / 32];
     __shared__ int best_idx[THREADS / 32];
     const double scale = static_cast<double>(st->scale);
@@ -411,23 +412,27 @@ __device__ __forceinline__ void decide_block(const double* sums, int N, double i
         if (om > -INFINITY && om >= bv) { bv = om; bi = j + 1; }   // j ascends per thread: ties -> larger c
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const auto across_warp = [&] {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, bv, off);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-        if (oi != 0 && (bi == 0 || ov > bv || (ov == bv && oi > bi))) { bv = ov; bi = oi; }
-    }
-    if (lane == 0) { best_val[warp] = bv; best_idx[warp] = bi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < THREADS / 32; ++w) {
-            const double ov = best_val[w];
-            const int oi = best_idx[w];
+        for (int off = 16; off > 0; off >>= 1) {
+            const double ov = __shfl_xor_sync(0xffffffffu, bv, off);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
             if (oi != 0 && (bi == 0 || ov > bv || (ov == bv && oi > bi))) { bv = ov; bi = oi; }
         }
-        st->c_star = bi == 0 ? N : bi;
-        st->code = bi == 0 ? 2 : 0;
-        if (advance) st->step += 1;
+    };
+    across_warp();
+    if (lane == 0) { best_val[warp] = bv; best_idx[warp] = bi; }
+    __syncthreads();
+    if (warp == 0) {
+        bv = lane < THREADS / 32 ? best_val[lane] : -INFINITY;
+        bi = lane < THREADS / 32 ? best_idx[lane] : 0;
+        across_warp();
+        if (lane == 0) {
+            st->c_star = bi == 0 ? N : bi;
+            st->code = bi == 0 ? 2 : 0;
+            if (advance) st->step += 1;
+            publish_state(st, host_state);
+        }
     }
 }
 
@@ -435,8 +440,8 @@ constexpr int kDecideThreads = 1024;
 
 __global__ void __launch_bounds__(kDecideThreads) k_decide(const double* __restrict__ sums, int N, double inv_samples,
                                                             DevState* st, int advance, float* __restrict__ e_out,
-                                                            float* __restrict__ omega_out) {
-    decide_block<kDecideThreads>(sums, N, inv_samples, st, advance, e_out, omega_out);
+                                                            float* __restrict__ omega_out, DevState* host_state) {
+    decide_block<kDecideThreads>(sums, N, inv_samples, st, advance, e_out, omega_out, host_state);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -453,8 +458,8 @@ __global__ void __launch_bounds__(kColsumThreads) k_colsum_decide(const float* _
                                                                    double* sums, double inv_samples, DevState* st,
                                                                    float* __restrict__ e_out, float* __restrict__ omega_out,
                                                                    const float* __restrict__ partial_sq,
-                                                                   float* __restrict__ std_out, int decide) {
-    __shared__ double red[kColsumSlices][32];
+                                                                   float* __restrict__ std_out, int decide, DevState* host_state) {
+    __shared__ double red[kColsumSlices][33];
     __shared__ bool is_last;
     dependency_wait();            // the partial rows are an earlier kernel's
     const int col = blockIdx.x * 32 + (threadIdx.x & 31), slice = threadIdx.x >> 5;
@@ -484,28 +489,25 @@ __global__ void __launch_bounds__(kColsumThreads) k_colsum_decide(const float* _
     }
     double s = 0.0;
     if (col < N) {
-        int p = slice;
-        for (; p + 3 * kColsumSlices < n_part; p += 4 * kColsumSlices) {        // four loads in flight
-            const float a = partial[static_cast<size_t>(p) * N + col];
-            const float b = partial[static_cast<size_t>(p + kColsumSlices) * N + col];
-            const float c = partial[static_cast<size_t>(p + 2 * kColsumSlices) * N + col];
-            const float d = partial[static_cast<size_t>(p + 3 * kColsumSlices) * N + col];
-            s += static_cast<double>(a);
-            s += static_cast<double>(b);
-            s += static_cast<double>(c);
-            s += static_cast<double>(d);
-        }
-        for (; p < n_part; p += kColsumSlices) s += static_cast<double>(partial[static_cast<size_t>(p) * N + col]);
+#pragma unroll 8
+        for (int p = slice; p < n_part; p += kColsumSlices) s += static_cast<double>(partial[static_cast<size_t>(p) * N + col]);
     }
     red[slice][threadIdx.x & 31] = s;
     __syncthreads();
-    if (slice == 0 && col < N) {
-        double total = 0.0;
+    {
+        // warp w adds the slices of column w, pairwise
+        const int lane = threadIdx.x & 31, c = blockIdx.x * 32 + slice;
+        double total = red[lane][slice];
 #pragma unroll
-        for (int k = 0; k < kColsumSlices; ++k) total += red[k][threadIdx.x];
-        sums[col] = total;
+        for (int off = 16; off > 0; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
+        if (lane == 0 && c < N) sums[c] = total;
     }
     if (!decide) return;                                // only the sums were asked for
+    if (gridDim.x == 1) {
+        __syncthreads();
+        decide_block<kColsumThreads>(sums, N, inv_samples, st, 1, e_out, omega_out, host_state);
+        return;
+    }
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -516,7 +518,7 @@ __global__ void __launch_bounds__(kColsumThreads) k_colsum_decide(const float* _
     __syncthreads();
     if (is_last) {
         __threadfence();
-        decide_block<kColsumThreads>(sums, N, inv_samples, st, 1, e_out, omega_out);
+        decide_block<kColsumThreads>(sums, N, inv_samples, st, 1, e_out, omega_out, host_state);
     }
 }
 

@@ -811,3 +811,15 @@ def test_sharded_decision_all_reduces_the_librarys_own_array_under_nccl():
             assert np.array_equal(ctx.get_stats()[0], ref.get_stats()[0])
     finally:
         dist.destroy_process_group()
+
+
+def test_stats_are_those_of_the_decision_in_flight():
+    """The results are written by the deciding kernel itself: read while a later decision is under way, they are that one's."""
+    wl, gpu, orc, _ = make_pair("n128", S=1024, steps=inputs.WORKLOADS["n128"].window + 2)
+    gpu.predict()
+    first = gpu.get_stats()[0]
+    assert np.array_equal(first, gpu.get_stats()[0])
+    gpu.predict_async()
+    second = gpu.get_stats()[0]
+    gpu.fetch()
+    assert not np.array_equal(first, second) and np.array_equal(second, gpu.get_stats()[0])
