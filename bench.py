@@ -608,14 +608,14 @@ def main():
     })
 
     # The emission output layer on the tensor cores is bound by its operand stream from L2 into shared memory
-    # (per 128 x 128 output tile the 128 hidden vectors and the 256 weight rows, 4 * H bytes each).
+    # (per 128 x 128 output tile the 128 hidden vectors and the 256 weight rows, 2 * H bytes each).
     # Set it against the rate the library measures for exactly those copies on this GPU: weights from a matrix of a
     # few MB that every SM re-reads, hidden vectors from one of tens of MB.
     if wl.precision and not literal and not args.no_measure_alu_peak:
         from paper_1803_04209_b200 import binding as _b
         op_rates = _b.measure_operand_stream(local_rank)
         n_tiles = -(-wl.S // 128) * -(-wl.N // 128)
-        k_bytes = -(-wl.H // 32) * 128                               # bytes of one operand row (K blocks of 32 floats)
+        k_bytes = -(-wl.H // 64) * 128                               # bytes of one operand row (K blocks of 64 halves)
         bytes_w, bytes_v = n_tiles * 256 * k_bytes, n_tiles * 128 * k_bytes
         t_stream = bytes_w / (op_rates["weights_2mb"] * 1e9) + bytes_v / (op_rates["hidden_64mb"] * 1e9)
         roofline["emission_stream"] = {

@@ -18,7 +18,8 @@
 // next A operand.  In the literal variant the proposal's result is combined with the gate and the linear map
 // (computed by the epilogue threads from the latent tile) into G, relu(G) then takes the place of the latent
 // tile and one more small product with Ws gives the scale.
-// The last layer's hidden vector (v, or u) goes to global memory for the emission output GEMMs.
+// The last layer's hidden vector (v, or u) goes to global memory as halves for the emission output GEMMs (half_operand.cuh),
+// its scale from the largest |latent| of the sample.
 //
 // All weight operands live in shared memory for the whole kernel: the host prepares their
 // swizzled image once, the CTA copies it in at start.  Latent rows are 128 bytes wide (32 tf32)
@@ -51,8 +52,8 @@ struct ChainTcArgs {
     DevState* st;
     NoiseKey key;
     uint32_t sample_base;
-    int count, H, W, round_v;   // round_v: round v to tf32 (compact; u of the literal variant always is)
-    float* v_out;               // [count][H]
+    int count, H, W;
+    HalfRows v_out;             // v (literal: u), rounded to tf32 and scaled
 };
 
 inline size_t chain_tc_image_floats(int H, bool literal = false) {
@@ -104,6 +105,28 @@ __device__ __forceinline__ float4 ld_shared_v4(uint32_t addr) {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
     return v;
+}
+
+__device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+// The largest |latent| of a thread's dimensions, into the hidden-chunk buffer: all its chunks have been multiplied by now,
+// and the next one is written when every warp has begun the next tile, that is, finished the last layer, which reads it.
+template <int N>
+__device__ __forceinline__ void put_largest(uint32_t addr, const float (&z)[N]) {
+    float m = 0.0f;
+#pragma unroll
+    for (int c = 0; c < N; ++c) m = fmaxf(m, fabsf(z[c]));
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(m) : "memory");
+}
+
+// 16 consecutive halves: the two 16-byte halves of one sector.
+__device__ __forceinline__ void store8(__half* p, const uint32_t (&w)[8]) {
+    *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4*>(p + 8) = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
 // One of the two tiles a CTA has in flight: its shared-memory operands, TMEM columns and barriers,
@@ -334,6 +357,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
         const int hb_chunk = 4 * (cg & 1);                                        // its first 16-byte chunk in a row
         float gate_own[2][4], lin_own[2][4], G_own[2][4];     // literal: per tile in flight, latent dimensions 4cg..4cg+3
         bool ok = true;
+        float v_scale[2] = {1.0f, 1.0f};                                          // per tile in flight: of its last layer's row
         for (int t0 = blockIdx.x; ok && t0 < n_tiles; t0 += 2 * gridDim.x) {
             slot[0].tile = t0;
             slot[1].tile = t0 + static_cast<int>(gridDim.x) < n_tiles ? t0 + static_cast<int>(gridDim.x) : -1;
@@ -361,6 +385,14 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                             if (!ok) continue;
                             ++sl.np;
                             tc_fence_after();
+                            if (ph == ph_last) {                   // the four column groups' largest |latent| of this sample
+                                float zm = 0.0f, inv;
+#pragma unroll
+                                for (int gg = 0; gg < 4; ++gg) zm = fmaxf(zm, ld_shared_f32(sl.t_hb + (gg * 128 + row) * 4));
+                                half_scale(1.01f * fmaf(a.v_out.slope, zm, a.v_out.offset), v_scale[s], inv);
+                                const int k = sl.tile * 128 + row;
+                                if (cg == 0 && k < a.count) a.v_out.inv_scale[k] = inv;
+                            }
                         }
                         const int col0 = c * 64 + cg * 16;
                         uint32_t acc[16];
@@ -406,12 +438,10 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                         } else {
                             const int k = sl.tile * 128 + row;
                             if (k < a.count) {
-                                if (LITERAL || a.round_v) {
+                                uint32_t w[8];
 #pragma unroll
-                                    for (int i = 0; i < 16; ++i) h[i] = tf32_rna(h[i]);
-                                }
-                                store8(a.v_out + static_cast<size_t>(k) * H + col0, h);          // whole 32-byte sectors
-                                store8(a.v_out + static_cast<size_t>(k) * H + col0 + 8, h + 8);
+                                for (int i = 0; i < 8; ++i) w[i] = pack_half2(tf32_rna(h[2 * i]) * v_scale[s], tf32_rna(h[2 * i + 1]) * v_scale[s]);
+                                store8(a.v_out.p + static_cast<size_t>(k) * a.v_out.ld + col0, w);      // one whole 32-byte sector
                             }
                         }
                     }
@@ -506,6 +536,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                             }
                         }
                     }
+                    if (!LITERAL && ph == W) put_largest(sl.t_hb + (cg * 128 + row) * 4, z_own);
                     if (store_z) {
                         st_shared_v4(sl.t_z + sw128(row, cg), tf32_rna(z_own[0]), tf32_rna(z_own[1]), tf32_rna(z_own[2]), tf32_rna(z_own[3]));
                         fence_proxy_async();
@@ -538,6 +569,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                             if (gg == cg) pre = __uint_as_float(res_bits[4 * gg + c]);
                         z_own[c] = fmaf(softplus_fast(pre + sbs[4 * cg + c]), eps[c], G_own[s][c]);
                     }
+                    put_largest(sl.t_hb + (cg * 128 + row) * 4, z_own);
                     st_shared_v4(sl.t_z + sw128(row, cg), tf32_rna(z_own[0]), tf32_rna(z_own[1]), tf32_rna(z_own[2]), tf32_rna(z_own[3]));
                     fence_proxy_async();
                     tc_fence_before();

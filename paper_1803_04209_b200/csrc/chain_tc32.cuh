@@ -39,8 +39,8 @@ struct ChainTc32Args {
     DevState* st;
     NoiseKey key;
     uint32_t sample_base;
-    int count, H, W, round_v;
-    float* v_out;               // [count][H]
+    int count, H, W;
+    HalfRows v_out;             // v (literal: u), rounded to tf32 and scaled
 };
 
 inline size_t chain_tc32_image_floats(int H, bool literal = false) {
@@ -283,6 +283,14 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
                 }
                 const float* bias = ph < W ? sbzs : (ph == W ? sb1 : (ph == W + 1 ? sb3 : sbi1));
                 const float* lr = slr + (ph < W ? ph : 0) * H;
+                float v_scale = 1.0f;
+                if (ph == ph_last) {                                   // the four column groups' largest |latent| of this sample
+                    float zm = 0.0f, inv;
+#pragma unroll
+                    for (int gg = 0; gg < 4; ++gg) zm = fmaxf(zm, ld_shared_f32(t_hb + (gg * 128 + row) * 4));
+                    half_scale(1.01f * fmaf(a.v_out.slope, zm, a.v_out.offset), v_scale, inv);
+                    if (cg == 0 && k < a.count) a.v_out.inv_scale[k] = inv;
+                }
                 for (int c = 0; c < n_chunks; ++c) {
                     const int col0 = c * 32 + cg * 8;
                     uint32_t acc[8];
@@ -324,11 +332,10 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
                         if (lane == 0) mbar_arrive(bar_h + 8 * b);
                         ++nu;
                     } else if (k < a.count) {
-                        if (a.round_v) {
+                        uint32_t w[4];
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) h[i] = tf32_rna(h[i]);
-                        }
-                        store8(a.v_out + static_cast<size_t>(k) * H + col0, h);          // one whole 32-byte sector
+                        for (int i = 0; i < 4; ++i) w[i] = pack_half2(tf32_rna(h[2 * i]) * v_scale, tf32_rna(h[2 * i + 1]) * v_scale);
+                        *reinterpret_cast<uint4*>(a.v_out.p + static_cast<size_t>(k) * a.v_out.ld + col0) = make_uint4(w[0], w[1], w[2], w[3]);
                     }
                 }
                 if (!ok || ph == ph_last) continue;
@@ -434,6 +441,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
                     for (int c = 0; c < 8; ++c)
                         z_own[c] = fmaf(softplus_fast(__uint_as_float(res[c]) + sbs[8 * cg + c]), eps[c], G_own[c]);
                 }
+                if (ph + 1 == ph_last) put_largest(t_hb + (cg * 128 + row) * 4, z_own);
                 st_shared_v4(t_z + sw128(row, 2 * cg), tf32_rna(z_own[0]), tf32_rna(z_own[1]), tf32_rna(z_own[2]), tf32_rna(z_own[3]));
                 st_shared_v4(t_z + sw128(row, 2 * cg + 1), tf32_rna(z_own[4]), tf32_rna(z_own[5]), tf32_rna(z_own[6]), tf32_rna(z_own[7]));
                 fence_proxy_async();

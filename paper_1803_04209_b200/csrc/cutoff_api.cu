@@ -64,7 +64,15 @@ struct cutoff_ctx {
     float* d_proj = nullptr;        // [2][W slots][H] raw input projections of the ring's vectors, kept up to date by every push
     bool proj_stale = true;         // the ring or the weights were replaced: recompute every slot before the next decision
     float* d_hlr = nullptr;         // [2][W][H]
-    float* d_v = nullptr;           // [chunk_rows][H]
+    float* d_v = nullptr;           // [chunk_rows][H]; fp32 path only
+    // tensor-core path: operands of the emission products as halves, row pitch ldh, with inverse scales per row
+    int ldh = 0;                    // H rounded up to 8 (rows start on 16 bytes)
+    __half* d_v16 = nullptr;        // [alloc_rows][ldh] v (literal: u)
+    float* d_v_inv = nullptr;       // [alloc_rows]
+    __half* d_w16 = nullptr;        // weights: W4 [2N][ldh]; literal: Wi2 [N], Wj2 [N], M [H] rows
+    float* d_w_inv = nullptr;       // their inverse scales
+    float v_slope = 0.0f, v_offset = 0.0f;   // bound of v's (u's) entries: slope * largest |latent| + offset
+    float r_slope = 0.0f, r_offset = 0.0f;   // literal: of r's entries, from the largest |u|
     float* d_x = nullptr;           // [chunk_rows][ldx]
     float* d_partial = nullptr;     // [n_chunks * sort_grid][N]; a second block of kPartialRows rows holds sums of squares
     float* d_std = nullptr;         // [N] spread of each order statistic (when asked for)
@@ -78,9 +86,11 @@ struct cutoff_ctx {
     bool literal = false;           // the networks as Section 3.1.3 prints them (CUTOFF_FLAG_LITERAL)
     LiteralDev lit{};
     float* d_I = nullptr;           // [alloc_rows][ldx]  emission mean I (padding columns stay zero); fp32 path only
-    float* d_r = nullptr;           // [alloc_rows][H]    hidden layer of the emission scale
+    float* d_r = nullptr;           // [alloc_rows][H]    hidden layer of the emission scale; fp32 path only
+    __half* d_r16 = nullptr;        // [alloc_rows][ldh]  the same as an operand; tensor-core path
+    float* d_r_inv = nullptr;       // [alloc_rows]
     float* d_Wj1p = nullptr;        // [H][ldx]           Wj1 with rows padded with zeros to ldx; fp32 path only
-    float* d_M = nullptr;           // [H][H] then [H]    M = Wj1 Wi2 and b' = Wj1 bi2 + bj1 (tensor-core path: Wj1 I + bj1 = M u + b')
+    float* d_Mb = nullptr;          // [H]                b' = Wj1 bi2 + bj1 (tensor-core path: Wj1 I + bj1 = M u + b' with M = Wj1 Wi2)
     CUtensorMap map_r{};            // TMA view of d_r [alloc_rows][H]
     CUtensorMap map_wi2{}, map_M{}, map_wj2{};
     bool use_tc = false;            // emission output layer on tensor cores
@@ -208,6 +218,32 @@ void put_second_layer(float* tiles, const float* w, size_t out_rows, size_t H, s
             for (size_t jj = 0; jj < 32; ++jj) tiles[kb * block_rows * 32 + swz(o, jj)] = host_tf32(w[o * H + kb * 32 + jj]);
 }
 
+// A weight matrix [rows][cols], already rounded to at most 11 significant bits, as halves with a power of two per row.
+void half_rows(const float* w, size_t rows, size_t cols, size_t ld, __half* out, float* inv) {
+    for (size_t r = 0; r < rows; ++r) {
+        float big = 0.0f;
+        for (size_t k = 0; k < cols; ++k) big = std::fmax(big, std::fabs(w[r * cols + k]));
+        uint32_t bits;
+        std::memcpy(&bits, &big, 4);
+        const int e = big > 0.0f ? half_exponent(bits) : 0;
+        for (size_t k = 0; k < ld; ++k) out[r * ld + k] = __float2half_rn(k < cols ? std::ldexp(w[r * cols + k], e) : 0.0f);
+        inv[r] = std::ldexp(1.0f, -e);
+    }
+}
+
+// |A x + b| <= slope * max |x| + offset, from the matrix as the tensor cores see it (rounded up a little)
+void layer_bound(const float* w, const float* b, size_t rows, size_t cols, float& slope, float& offset) {
+    double l1 = 0.0, mb = 0.0;
+    for (size_t r = 0; r < rows; ++r) {
+        double s = 0.0;
+        for (size_t k = 0; k < cols; ++k) s += std::fabs(static_cast<double>(w[r * cols + k]));
+        l1 = std::fmax(l1, s);
+        mb = std::fmax(mb, std::fabs(static_cast<double>(b[r])));
+    }
+    slope = static_cast<float>(l1 * 1.001);
+    offset = static_cast<float>(mb * 1.001);
+}
+
 // Launch `kernel` so that it may begin while the kernel before it in the stream is still running (programmatic
 // dependent launch): the kernel itself waits, by dependency_wait(), before it touches that kernel's results.
 template <typename... KArgs, typename... Args>
@@ -232,7 +268,8 @@ int next_pow2(int n) {
 }
 
 void free_all(cutoff_ctx* c) {
-    cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_M);
+    cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_Mb);
+    cudaFree(c->d_v16); cudaFree(c->d_v_inv); cudaFree(c->d_w16); cudaFree(c->d_w_inv); cudaFree(c->d_r16); cudaFree(c->d_r_inv);
     cudaFree(c->d_blob); cudaFree(c->d_WT); cudaFree(c->d_WhR); cudaFree(c->d_chain_image);
     if (c->h_mask) cudaFreeHost(c->h_mask); cudaFree(c->d_ring); cudaFree(c->d_stage);
     cudaFree(c->d_state); cudaFree(c->d_proj); cudaFree(c->d_hlr); cudaFree(c->d_v); cudaFree(c->d_x);
@@ -352,10 +389,12 @@ int launch_sort(cutoff_ctx* c, int count, float* partial) {
     return CUTOFF_OK;
 }
 
+HalfRows half_v(const cutoff_ctx* c) { return HalfRows{c->d_v16, c->d_v_inv, c->ldh, c->v_slope, c->v_offset}; }
+ChainOut chain_out(const cutoff_ctx* c) { return ChainOut{c->use_tc ? nullptr : c->d_v, half_v(c)}; }
+
 template <int D>
 void launch_chain_t(cutoff_ctx* c, uint32_t sample_base, int count, size_t smem) {
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
-    const int round_v = c->cfg.precision != CUTOFF_PRECISION_FP32;
     const size_t resident = chain_resident_smem_floats(c->D, c->H, c->W) * sizeof(float);
     if (resident <= 200 * 1024) {
         // all weights fit: one persistent CTA per SM, as many as there are warp batches to hand out
@@ -363,10 +402,10 @@ void launch_chain_t(cutoff_ctx* c, uint32_t sample_base, int count, size_t smem)
         const int batches = ceil_div(count, batch);
         const int grid = batches < c->sm_count ? batches : c->sm_count;
         launch_dependent(k_chain_resident<D>, dim3(grid), dim3(kChainResidentThreads), resident, c->stream, c->m, c->d_hlr, c->d_state, key,
-                         sample_base, count, round_v, c->d_v);
+                         sample_base, count, chain_out(c));
     } else {
         launch_dependent(k_chain<D>, dim3(ceil_div(count, ChainShape<D>::kSamplesPerCta)), dim3(ChainShape<D>::kThreads), smem, c->stream,
-                         c->m, c->d_hlr, c->d_state, key, sample_base, count, round_v, c->d_v);
+                         c->m, c->d_hlr, c->d_state, key, sample_base, count, chain_out(c));
     }
 }
 
@@ -382,7 +421,7 @@ void launch_chain_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
     }
     a.hlr = c->d_hlr; a.st = c->d_state;
     a.key = NoiseKey{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
-    a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.round_v = 1; a.v_out = c->d_v;
+    a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.v_out = half_v(c);
     const int tiles = ceil_div(count, 128);
     const int grid = tiles < c->sm_count ? tiles : c->sm_count;
     if (c->chain_tcl) launch_dependent(tc::k_chain_tc<true>, dim3(grid), dim3(tc::kChainTcThreads), tc::chain_tc_smem_bytes(c->H, c->W, true), c->stream, a);
@@ -402,7 +441,7 @@ void launch_chain_tc32(cutoff_ctx* c, uint32_t sample_base, int count) {
     }
     a.hlr = c->d_hlr; a.st = c->d_state;
     a.key = NoiseKey{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
-    a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.round_v = 1; a.v_out = c->d_v;
+    a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.v_out = half_v(c);
     const int tiles = ceil_div(count, 128);
     const int grid = tiles < c->sm_count ? tiles : c->sm_count;
     if (c->chain_tcl32) launch_dependent(tc::k_chain_tc32<true>, dim3(grid), dim3(tc::kChainTcThreads), tc::chain_tc32_smem_bytes(c->H, c->W, true), c->stream, a);
@@ -415,7 +454,7 @@ void launch_chain_literal_t(cutoff_ctx* c, uint32_t sample_base, int count) {
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     const size_t smem = chain_smem_floats(c->D, c->H, c->W) * sizeof(float);
     launch_dependent(k_chain_literal<D>, dim3(ceil_div(count, ChainShape<D>::kSamplesPerCta)), dim3(ChainShape<D>::kThreads), smem, c->stream,
-                     c->m, c->lit, c->d_hlr, c->d_state, key, sample_base, count, c->use_tc ? 1 : 0, c->d_v);
+                     c->m, c->lit, c->d_hlr, c->d_state, key, sample_base, count, chain_out(c));
 }
 
 void launch_chain(cutoff_ctx* c, uint32_t sample_base, int count) {
@@ -443,9 +482,10 @@ void launch_chain(cutoff_ctx* c, uint32_t sample_base, int count) {
     c->launches += 1;
 }
 
-// 2-D fp32 tensor map over a row-major [rows][cols] matrix, boxes of 128 rows x 32 columns
+// 2-D tensor map over a row-major [rows][cols] matrix of floats or halves, boxes of 128 rows x 128 bytes
 // (one 128-byte-swizzled K-major operand tile).  The driver entry point is looked up at run time.
-int make_tile_map(cutoff_ctx* c, CUtensorMap* map, const float* base, uint64_t rows, uint64_t cols, uint64_t ld = 0) {
+template <typename T>
+int make_tile_map(cutoff_ctx* c, CUtensorMap* map, const T* base, uint64_t rows, uint64_t cols, uint64_t ld = 0) {
     typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -461,10 +501,10 @@ int make_tile_map(cutoff_ctx* c, CUtensorMap* map, const float* base, uint64_t r
         encode = reinterpret_cast<EncodeFn>(fn);
     }
     const cuuint64_t dims[2] = {cols, rows};
-    const cuuint64_t strides[1] = {(ld ? ld : cols) * sizeof(float)};
-    const cuuint32_t box[2] = {tc::kBK, tc::kBM};
+    const cuuint64_t strides[1] = {(ld ? ld : cols) * sizeof(T)};
+    const cuuint32_t box[2] = {128 / sizeof(T), tc::kBM};
     const cuuint32_t elem[2] = {1, 1};
-    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box,
+    const CUresult r = encode(map, sizeof(T) == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<T*>(base), dims, strides, box,
                               elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
@@ -476,7 +516,7 @@ int make_tile_map(cutoff_ctx* c, CUtensorMap* map, const float* base, uint64_t r
 
 void launch_emission_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
     tc::EmitArgs a;
-    a.b4 = c->m.b4; a.x = c->d_x; a.st = c->d_state;
+    a.b4 = c->m.b4; a.v_inv = c->d_v_inv; a.w_inv = c->d_w_inv; a.x = c->d_x; a.st = c->d_state;
     a.key = NoiseKey{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     a.sample_base = sample_base; a.count = count; a.N = c->N; a.H = c->H; a.ldx = c->ldx;
     if (c->pair_emission && c->pair_clusters > 0 && count > tc::kBM) {
@@ -507,11 +547,13 @@ void launch_emission_literal(cutoff_ctx* c, uint32_t sample_base, int count) {
     if (c->use_tc) {
         // r = relu(M u + b') with M = Wj1 Wi2 (I is affine in u), then x = (Wi2 u + bi2) + softplus(Wj2 r + bj2) * eps
         tc::GemmTcArgs a{};
-        a.st = c->d_state; a.M = count; a.bias = c->d_M + static_cast<size_t>(c->H) * c->H; a.out = c->d_r;
-        a.ld_out = c->H; a.Nout = c->H; a.K = c->H;
+        a.st = c->d_state; a.M = count; a.bias = c->d_Mb; a.a_inv = c->d_v_inv; a.b_inv = c->d_w_inv + 2 * c->N;
+        a.out = HalfRows{c->d_r16, c->d_r_inv, c->ldh, c->r_slope, c->r_offset};
+        a.Nout = c->H; a.K = c->H;
         launch_gemm_relu_tc(c, c->map_v, c->map_M, a);
         tc::EmitDualArgs e;
-        e.bias_mean = l.bi2; e.bias_scale = l.bj2; e.x = c->d_x; e.st = c->d_state; e.key = key;
+        e.bias_mean = l.bi2; e.bias_scale = l.bj2; e.u_inv = c->d_v_inv; e.r_inv = c->d_r_inv;
+        e.wi_inv = c->d_w_inv; e.wj_inv = c->d_w_inv + c->N; e.x = c->d_x; e.st = c->d_state; e.key = key;
         e.sample_base = sample_base; e.count = count; e.N = c->N; e.H = c->H; e.ldx = c->ldx;
         const int tiles = ceil_div(c->N, tc::kBW) * ceil_div(count, tc::kBM);
         launch_dependent(tc::k_emit_dual_tc, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kThreads), tc::kDualSmemBytes, c->stream,
@@ -765,6 +807,7 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     c->cfg = *cfg;
     c->N = cfg->n_workers; c->D = cfg->latent_dim; c->H = cfg->hidden; c->W = cfg->lag + 1; c->S = cfg->n_samples;
     c->ldx = (c->N + 7) & ~7;
+    c->ldh = (c->H + 7) & ~7;
     c->P = next_pow2(c->N) < 32 ? 32 : next_pow2(c->N);
     c->stream = static_cast<cudaStream_t>(cfg->stream);
     c->literal = (cfg->flags & CUTOFF_FLAG_LITERAL) != 0;
@@ -815,10 +858,12 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     CREATE_CHECK(cudaMalloc(&c->d_blob, blob_floats * sizeof(float)));
     CREATE_CHECK(cudaMalloc(&c->d_WT, sizeof(float) * 4 * c->H * c->D));
     if (c->literal) {
-        CREATE_CHECK(cudaMalloc(&c->d_r, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->H));
         if (c->use_tc) {
-            CREATE_CHECK(cudaMalloc(&c->d_M, sizeof(float) * (static_cast<size_t>(c->H) * c->H + c->H)));
+            CREATE_CHECK(cudaMalloc(&c->d_r16, sizeof(__half) * static_cast<size_t>(c->alloc_rows) * c->ldh));
+            CREATE_CHECK(cudaMalloc(&c->d_r_inv, sizeof(float) * c->alloc_rows));
+            CREATE_CHECK(cudaMalloc(&c->d_Mb, sizeof(float) * c->H));
         } else {
+            CREATE_CHECK(cudaMalloc(&c->d_r, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->H));
             CREATE_CHECK(cudaMalloc(&c->d_I, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->ldx));
             CREATE_CHECK(cudaMalloc(&c->d_Wj1p, sizeof(float) * static_cast<size_t>(c->H) * c->ldx));
             // the padding columns of I are never written and must read as zero
@@ -836,17 +881,28 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     CREATE_CHECK(cudaMalloc(&c->d_state, sizeof(DevState)));
     CREATE_CHECK(cudaMalloc(&c->d_proj, sizeof(float) * 2 * c->W * c->H));
     CREATE_CHECK(cudaMalloc(&c->d_hlr, sizeof(float) * 2 * c->W * c->H));
-    CREATE_CHECK(cudaMalloc(&c->d_v, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->H));
+    if (c->use_tc) {
+        const size_t w_rows = 2 * static_cast<size_t>(c->N) + (c->literal ? c->H : 0);
+        CREATE_CHECK(cudaMalloc(&c->d_v16, sizeof(__half) * static_cast<size_t>(c->alloc_rows) * c->ldh));
+        CREATE_CHECK(cudaMalloc(&c->d_v_inv, sizeof(float) * c->alloc_rows));
+        CREATE_CHECK(cudaMalloc(&c->d_w16, sizeof(__half) * w_rows * c->ldh));
+        CREATE_CHECK(cudaMalloc(&c->d_w_inv, sizeof(float) * w_rows));
+    } else {
+        CREATE_CHECK(cudaMalloc(&c->d_v, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->H));
+    }
     CREATE_CHECK(cudaMalloc(&c->d_x, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->ldx));
     CREATE_CHECK(cudaMalloc(&c->d_partial, sizeof(float) * 2 * static_cast<size_t>(kPartialRows) * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_std, sizeof(float) * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_sums, sizeof(double) * c->N));
     if (c->use_tc) {
-        int rc = make_tile_map(c, &c->map_v, c->d_v, static_cast<uint64_t>(c->alloc_rows), static_cast<uint64_t>(c->H));
-        if (!rc && c->literal)
-            rc = make_tile_map(c, &c->map_M, c->d_M, static_cast<uint64_t>(c->H), static_cast<uint64_t>(c->H));
-        if (!rc && c->literal)
-            rc = make_tile_map(c, &c->map_r, c->d_r, static_cast<uint64_t>(c->alloc_rows), static_cast<uint64_t>(c->H));
+        const uint64_t rows = static_cast<uint64_t>(c->alloc_rows), H = static_cast<uint64_t>(c->H), N = static_cast<uint64_t>(c->N);
+        const uint64_t ld = static_cast<uint64_t>(c->ldh);
+        int rc = make_tile_map(c, &c->map_v, c->d_v16, rows, H, ld);
+        if (!rc && !c->literal) rc = make_tile_map(c, &c->map_w4, c->d_w16, 2 * N, H, ld);
+        if (!rc && c->literal) rc = make_tile_map(c, &c->map_r, c->d_r16, rows, H, ld);
+        if (!rc && c->literal) rc = make_tile_map(c, &c->map_wi2, c->d_w16, N, H, ld);
+        if (!rc && c->literal) rc = make_tile_map(c, &c->map_wj2, c->d_w16 + N * ld, N, H, ld);
+        if (!rc && c->literal) rc = make_tile_map(c, &c->map_M, c->d_w16 + 2 * N * ld, H, H, ld);
         if (rc) return fail(rc);
     }
     CREATE_CHECK(set_kernel_attributes(c));
@@ -935,6 +991,19 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         }
     }
     CU_CHECK(c, cudaMemcpy(c->d_blob, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice));
+    std::vector<__half> w16(c->use_tc ? (2 * static_cast<size_t>(c->N) + (c->literal ? c->H : 0)) * c->ldh : 0);
+    std::vector<float> w_inv(c->use_tc ? 2 * static_cast<size_t>(c->N) + (c->literal ? c->H : 0) : 0);
+    if (c->use_tc) {
+        const size_t N = c->N, H = c->H, D = c->D, ld = c->ldh;
+        if (c->literal) {
+            half_rows(host.data() + off[29], N, H, ld, w16.data(), w_inv.data());                         // Wi2
+            half_rows(host.data() + off[33], N, H, ld, w16.data() + N * ld, w_inv.data() + N);            // Wj2
+        } else {
+            half_rows(host.data() + off[21], 2 * N, H, ld, w16.data(), w_inv.data());                     // W4
+        }
+        const size_t first = c->literal ? 27 : 19;                                                       // Wi1 or W3, and its bias
+        layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, c->v_slope, c->v_offset);
+    }
     // transposed copies [D][H] of the latent-to-hidden matrices for the per-sample chain
     const size_t D = c->D, H = c->H;
     const int n_transposed = c->literal ? 4 : 3;
@@ -1035,7 +1104,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
             const float* wi2 = host.data() + off[29];    // [N][H]
             const float* bi2 = host.data() + off[30];
             const float* bj1 = host.data() + off[32];
-            std::vector<float> mb(H * H + H);
+            std::vector<float> big_m(H * H), mb(H);
             std::vector<double> acc(H);
             for (size_t i = 0; i < H; ++i) {
                 std::fill(acc.begin(), acc.end(), 0.0);
@@ -1046,17 +1115,14 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                     for (size_t j = 0; j < H; ++j) acc[j] += w * row[j];
                     bacc += w * bi2[k];
                 }
-                for (size_t j = 0; j < H; ++j) {
-                    float f = static_cast<float>(acc[j]);
-                    uint32_t u;
-                    std::memcpy(&u, &f, 4);
-                    u = (u + 0x1000u) & 0xFFFFE000u;
-                    std::memcpy(&f, &u, 4);
-                    mb[i * H + j] = f;
-                }
-                mb[H * H + i] = static_cast<float>(bacc);
+                for (size_t j = 0; j < H; ++j) big_m[i * H + j] = host_tf32(static_cast<float>(acc[j]));
+                mb[i] = static_cast<float>(bacc);
             }
-            CU_CHECK(c, cudaMemcpy(c->d_M, mb.data(), mb.size() * sizeof(float), cudaMemcpyHostToDevice));
+            half_rows(big_m.data(), H, H, c->ldh, w16.data() + 2 * N * c->ldh, w_inv.data() + 2 * N);
+            layer_bound(big_m.data(), mb.data(), H, H, c->r_slope, c->r_offset);
+            CU_CHECK(c, cudaMemcpy(c->d_Mb, mb.data(), mb.size() * sizeof(float), cudaMemcpyHostToDevice));
+            CU_CHECK(c, cudaMemcpy(c->d_w16, w16.data(), w16.size() * sizeof(__half), cudaMemcpyHostToDevice));
+            CU_CHECK(c, cudaMemcpy(c->d_w_inv, w_inv.data(), w_inv.size() * sizeof(float), cudaMemcpyHostToDevice));
         } else {
             // Wj1 [H][N] with rows padded with zeros to ldx floats (rows then start on 32 bytes for any N)
             std::vector<float> wj1p(H * static_cast<size_t>(c->ldx), 0.0f);
@@ -1073,11 +1139,6 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         l.Wj1 = c->d_Wj1p; l.bj1 = b + off[32]; l.ldn = c->ldx;
         l.Wj2 = b + off[33]; l.bj2 = b + off[34];
         m.W1T = m.b1 = m.W2 = m.b2 = m.W3T = m.b3 = m.W4 = m.b4 = nullptr;
-        if (c->use_tc) {
-            int rc = make_tile_map(c, &c->map_wi2, l.Wi2, static_cast<uint64_t>(c->N), static_cast<uint64_t>(c->H));
-            if (!rc) rc = make_tile_map(c, &c->map_wj2, l.Wj2, static_cast<uint64_t>(c->N), static_cast<uint64_t>(c->H));
-            if (rc) return rc;
-        }
         c->weights_loaded = true;
         c->proj_stale = true;
         return CUTOFF_OK;
@@ -1085,8 +1146,8 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
     m.W1T = c->d_WT + H * D; m.b1 = b + off[16]; m.W2 = b + off[17]; m.b2 = b + off[18];
     m.W3T = c->d_WT + 2 * H * D; m.b3 = b + off[20]; m.W4 = b + off[21]; m.b4 = b + off[22];
     if (c->use_tc) {
-        const int rc = make_tile_map(c, &c->map_w4, m.W4, 2ull * c->N, static_cast<uint64_t>(c->H));
-        if (rc) return rc;
+        CU_CHECK(c, cudaMemcpy(c->d_w16, w16.data(), w16.size() * sizeof(__half), cudaMemcpyHostToDevice));
+        CU_CHECK(c, cudaMemcpy(c->d_w_inv, w_inv.data(), w_inv.size() * sizeof(float), cudaMemcpyHostToDevice));
     }
     c->weights_loaded = true;
     c->proj_stale = true;

@@ -3,13 +3,17 @@
 //
 // One persistent CTA per SM walks over output tiles of 128 samples x 128 workers.  A tile is one
 // accumulator of 128 TMEM lanes (samples) x 256 fp32 columns (128 means, then 128 log-variances),
-// filled by UMMA instructions of shape M=128, N=256, K=8 in kind::tf32.  Operands arrive by TMA
+// filled by UMMA instructions of shape M=128, N=256, K=16 in kind::f16: the operands are tf32 (or bf16) values stored as
+// halves with a power of two per row taken out (half_operand.cuh), which the epilogue multiplies back.  Operands arrive by TMA
 // (plain, per-CTA loads) into a 4-stage ring of 128-byte-swizzled K-major tiles; the accumulator
 // is double-buffered (2 x 256 of the 512 TMEM columns) so that the epilogue of one tile runs
 // while the next tile is multiplied.
 //
 // Warp roles: warp 0 issues TMA loads, warp 1 owns TMEM and issues the MMAs, warps 2..17 are the
 // epilogue (warp w reads TMEM lanes 32*(w%4).., the 32 workers of column group (w-2)/4).
+//
+// What bounds it: as four-byte operands it was the stream L2 -> shared memory, 384 KB per tile (N = 1024, S = 65536: 0.148 ms); as
+// halves the stream and the tensor time halve and the epilogue sets the pace, about 150 instructions per four draws.
 //
 // Every wait on an mbarrier is bounded: after about two seconds it records kErrTimeout in the
 // device state, raises a CTA-wide abort flag and the kernel winds down (outstanding copies are
@@ -19,6 +23,7 @@
 
 #include "async.cuh"
 #include "common.cuh"
+#include "half_operand.cuh"
 #include "rng.cuh"
 
 namespace cutoff {
@@ -28,20 +33,21 @@ using namespace cutoff::async;
 
 constexpr int kBM = 128;                 // samples per tile (TMEM lanes)
 constexpr int kBW = 128;                 // workers per tile
-constexpr int kBK = 32;                  // tf32 elements per 128-byte swizzle row
+constexpr int kBK = 64;                  // halves per 128-byte swizzle row
 constexpr int kStages = 4;
-constexpr int kABytes = kBM * kBK * 4;           // 16 KB
-constexpr int kBBytes = 2 * kBW * kBK * 4;       // 32 KB: mean rows, then log-variance rows
+constexpr int kABytes = kBM * kBK * 2;           // 16 KB
+constexpr int kBBytes = 2 * kBW * kBK * 2;       // 32 KB: mean rows, then log-variance rows
 constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = (2 + kEpiWarps) * 32;
 constexpr int kTmemCols = 512;
 constexpr int kAccCols = 2 * kBW;                // 256 columns per accumulator
-constexpr int kBiasBytes = kEpiWarps * 64 * 4;   // per epilogue warp: 32 mean + 32 log-variance biases of its columns
+constexpr int kBiasBytes = kEpiWarps * 128 * 4;  // per epilogue warp: biases of its 32 + 32 columns, then their inverse scales
 constexpr size_t kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kBiasBytes;
 
-// instruction descriptor: D = f32, A = B = tf32, both K-major, N = 256, M = 128
-constexpr uint32_t kInstrDesc = (1u << 4) | (2u << 7) | (2u << 10) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
+// instruction descriptor: D = f32, A = B = f16, both K-major, N columns, M rows
+constexpr uint32_t instr_desc_f16(uint32_t n, uint32_t m) { return (1u << 4) | ((n >> 3) << 17) | ((m >> 4) << 24); }
+constexpr uint32_t kInstrDesc = instr_desc_f16(256, 128);
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
     asm volatile(
@@ -66,6 +72,13 @@ __device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t a_desc, uint
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.u32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
@@ -108,6 +121,8 @@ __device__ __forceinline__ void store8(float* p, const float* v) {
 
 struct EmitArgs {
     const float* b4;        // [2N]
+    const float* v_inv;     // [count] inverse scales of the samples' hidden vectors
+    const float* w_inv;     // [2N] inverse scales of the rows of W4
     float* x;               // [count][ldx]
     DevState* st;
     NoiseKey key;
@@ -115,67 +130,67 @@ struct EmitArgs {
     int count, N, H, ldx;
 };
 
-// Epilogue of one 128 x 128 output tile for one warp: read its 32 lanes x 32 (+32) accumulator columns, hand the
-// accumulator back, add the biases, draw the noise and store x = mean + exp(logvar / 2) * eps.
-// bias_s: this warp's 32 mean biases, then its 32 log-variance biases, in shared memory (zero beyond worker N).
-__device__ __forceinline__ void emit_epilogue_tile(const EmitArgs& a, uint32_t tmem_base, uint32_t acc, int q, int cg,
-                                                   int lane, int m0, int w0, uint32_t step, uint32_t bar_acc_empty,
-                                                   const float* bias_s) {
-    const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32;
-    const int row = m0 + q * 32 + lane;
-    const bool row_ok = row < a.count;
-    const uint32_t sample = a.sample_base + static_cast<uint32_t>(row);
+// Epilogue of one 128 x 128 output tile for one warp: 32 samples (its TMEM lanes) x 32 workers, eight workers at a time.
+// The noise of the eight is drawn while their accumulators are on their way from tensor memory, without a branch between
+// the two generator calls: the generator is a chain of ten dependent rounds, and one call after the other, behind the loads,
+// left the issue slots 54 % empty (N = 1024, S = 65536: 0.165 ms with half-precision operands).
+// finish(first 8 columns' words, second 8 columns' words, 8 normals, column of the warp, 8 results): the variant's own arithmetic.
+template <typename Finish>
+__device__ __forceinline__ void noise_epilogue_tile(float* __restrict__ x, int ldx, int N, bool row_ok, int row, uint32_t sample, NoiseKey key,
+                                                    uint32_t step, uint32_t taddr, int jw0, int lane, uint32_t bar_acc_empty, Finish finish) {
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        uint32_t mean_bits[16], logvar_bits[16];
-        tmem_ld16(taddr + 16 * half, mean_bits);
-        tmem_ld16(taddr + kBW + 16 * half, logvar_bits);
+    for (int c8 = 0; c8 < 32; c8 += 8) {
+        uint32_t lo[8], hi[8];
+        tmem_ld8(taddr + c8, lo);
+        tmem_ld8(taddr + kBW + c8, hi);
+        const int jw = jw0 + c8;
+        float eps[8], out[8];
+        normal4_fast(static_cast<uint32_t>(jw >> 2), sample, kStreamEmission, step, key.seed_lo, key.seed_hi, eps);
+        normal4_fast(static_cast<uint32_t>(jw >> 2) + 1u, sample, kStreamEmission, step, key.seed_lo, key.seed_hi, eps + 4);
         tmem_ld_wait();
-        if (half == 1) {
+        if (c8 == 24) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_acc_empty + 8 * acc);    // accumulator is free again
+            if (lane == 0) mbar_arrive(bar_acc_empty);              // accumulator is free again
         }
-        const int jw = w0 + cg * 32 + 16 * half;
-        if (row_ok && jw < a.N) {
-            float* dst = a.x + static_cast<size_t>(row) * a.ldx + jw;
-            float out[16];
+        finish(lo, hi, eps, c8, out);
+        if (!row_ok || jw >= N) continue;
+        // whole sectors (the row pitch is a multiple of 8 floats), 16-byte or scalar stores on the ragged edge
+        float* dst = x + static_cast<size_t>(row) * ldx + jw;
+        if (jw + 7 < N) {
+            store8(dst, out);
+        } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int j = jw + 4 * i;
-                if (j >= a.N) continue;
-                float eps[4];
-                normal4_fast(static_cast<uint32_t>(j >> 2), sample, kStreamEmission, step, a.key.seed_lo,
-                             a.key.seed_hi, eps);
-                const float4 bm = *reinterpret_cast<const float4*>(bias_s + 16 * half + 4 * i);
-                const float4 bl = *reinterpret_cast<const float4*>(bias_s + 32 + 16 * half + 4 * i);
-                const float bmv[4] = {bm.x, bm.y, bm.z, bm.w}, blv[4] = {bl.x, bl.y, bl.z, bl.w};
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    out[4 * i + c] = fmaf(exp_half_fast(__uint_as_float(logvar_bits[4 * i + c]) + blv[c]), eps[c],
-                                          __uint_as_float(mean_bits[4 * i + c]) + bmv[c]);
-            }
-            // a thread owns 16 consecutive workers of its sample: two 32-byte stores (whole sectors; the row pitch
-            // is a multiple of 8 floats), 16-byte or scalar stores on the ragged edge
-#pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                if (jw + 8 * p + 7 < a.N) {
-                    store8(dst + 8 * p, out + 8 * p);
-                    continue;
-                }
-#pragma unroll
-                for (int i = 2 * p; i < 2 * p + 2; ++i) {
-                    const int ji = jw + 4 * i;
-                    if (ji + 3 < a.N) {
-                        *reinterpret_cast<float4*>(dst + 4 * i) =
-                            make_float4(out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
-                    } else {
-                        for (int c = 0; c < 4 && ji + c < a.N; ++c) dst[4 * i + c] = out[4 * i + c];
-                    }
-                }
-            }
+            for (int i = 0; i < 8; ++i)
+                if (jw + i < N) dst[i] = out[i];
         }
     }
+}
+
+__device__ __forceinline__ void load8(float (&r)[8], const float* p) {
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+    r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w; r[4] = b.x; r[5] = b.y; r[6] = b.z; r[7] = b.w;
+}
+
+// x = mean + exp(logvar / 2) * eps.  bias_s: this warp's 32 mean biases, then its 32 log-variance biases, then the inverse scales
+// of the same columns, in shared memory (zero beyond worker N).  v_inv: inverse scale of this thread's sample.
+__device__ __forceinline__ void emit_epilogue_tile(const EmitArgs& a, uint32_t tmem_base, uint32_t acc, int q, int cg,
+                                                   int lane, int m0, int w0, uint32_t step, uint32_t bar_acc_empty,
+                                                   const float* bias_s, float v_inv) {
+    const int row = m0 + q * 32 + lane;
+    noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, step,
+                        tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32, w0 + cg * 32, lane, bar_acc_empty + 8 * acc,
+                        [&](const uint32_t (&mean)[8], const uint32_t (&logvar)[8], const float (&eps)[8], int c8, float (&out)[8]) {
+        float bm[8], bl[8], sm[8], sl[8];
+        load8(bm, bias_s + c8);
+        load8(bl, bias_s + 32 + c8);
+        load8(sm, bias_s + 64 + c8);
+        load8(sl, bias_s + 96 + c8);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            out[c] = fmaf(exp_half_fast(fmaf(__uint_as_float(logvar[c]) * v_inv, sl[c], bl[c])), eps[c],
+                          fmaf(__uint_as_float(mean[c]) * v_inv, sm[c], bm[c]));
+    });
 }
 
 __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__ CUtensorMap map_v,
@@ -275,8 +290,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
                     const uint64_t a_desc = make_smem_desc(a_addr);
                     const uint64_t b_desc = make_smem_desc(a_addr + kABytes);
 #pragma unroll
-                    for (int k = 0; k < kBK / 8; ++k)          // 8 tf32 = 32 bytes per instruction
-                        umma_tf32(d_tmem, a_desc + 2 * k, b_desc + 2 * k, kInstrDesc, (kb | k) != 0);
+                    for (int k = 0; k < kBK / 16; ++k)         // 16 halves = 32 bytes per instruction
+                        umma_f16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, kInstrDesc, (kb | k) != 0);
                     umma_commit(bar_empty + 8 * stage);         // frees the stage when these MMAs are done
                     if (kb == k_blocks - 1) umma_commit(bar_acc_full + 8 * acc);
                 }
@@ -297,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
         // ---------------- epilogue ---------------------------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
         const uint32_t step = a.st->step;
-        float* bias_s = bias_all + (warp - 2) * 64;
+        float* bias_s = bias_all + (warp - 2) * 128;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -307,16 +322,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
                 const int j = w0 + cg * 32 + lane;
                 const float bm = j < a.N ? __ldg(a.b4 + j) : 0.f;
                 const float bl = j < a.N ? __ldg(a.b4 + a.N + j) : 0.f;
+                const float sm = j < a.N ? __ldg(a.w_inv + j) : 0.f;
+                const float sl = j < a.N ? __ldg(a.w_inv + a.N + j) : 0.f;
                 __syncwarp();                           // the previous tile's readers are done
                 bias_s[lane] = bm;
                 bias_s[32 + lane] = bl;
+                bias_s[64 + lane] = sm;
+                bias_s[96 + lane] = sl;
                 __syncwarp();
                 w_staged = w0;
             }
+            const int row = m0 + q * 32 + lane;
+            const float v_inv = row < a.count ? a.v_inv[row] : 0.f;      // on its way while the accumulator is waited for
             ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
-            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s);
+            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s, v_inv);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }

@@ -1,4 +1,4 @@
-// The emission output layer of emit_tc.cuh on pairs of SMs: one UMMA of shape M=256, N=256, K=8
+// The emission output layer of emit_tc.cuh on pairs of SMs: one UMMA of shape M=256, N=256, K=16
 // (tcgen05.mma.cta_group::2) spans a cluster of two CTAs.  Opt-in (option "pair_emission").
 //
 // The one-SM kernel streams 48 KB of operands from L2 into shared memory per K block for every 128 x 128 output
@@ -27,11 +27,10 @@ namespace cutoff {
 namespace tc {
 
 constexpr int kStages2 = 3;
-constexpr int kStageK2 = 2;                               // K blocks (of 32) per stage
-constexpr int kStage2Bytes = kStageK2 * (kABytes + kBBytes / 2);   // 64 KB: per K block 128 hidden vectors x 32 and this CTA's 128 weight rows x 32
+constexpr int kStageK2 = 2;                               // K blocks (of 64) per stage
+constexpr int kStage2Bytes = kStageK2 * (kABytes + kBBytes / 2);   // 64 KB: per K block 128 hidden vectors x 64 and this CTA's 128 weight rows x 64
 constexpr size_t kSmem2Bytes = kStages2 * kStage2Bytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kBiasBytes;
-// instruction descriptor: D = f32, A = B = tf32, both K-major, N = 256, M = 256 (two CTAs x 128)
-constexpr uint32_t kInstrDesc2 = (1u << 4) | (2u << 7) | (2u << 10) | ((256u >> 3) << 17) | ((256u >> 4) << 24);
+constexpr uint32_t kInstrDesc2 = instr_desc_f16(256, 256);        // M = 256: two CTAs x 128
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;
@@ -58,12 +57,12 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void umma_tf32_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+__device__ __forceinline__ void umma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                                uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.u32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 // arrive (once the pair's MMAs issued so far are done) on the barrier at this offset in the CTAs of `cta_mask`
@@ -185,8 +184,8 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
                         const uint64_t a_desc = make_smem_desc(a_addr);
                         const uint64_t b_desc = make_smem_desc(a_addr + kABytes);
 #pragma unroll
-                        for (int k = 0; k < kBK / 8; ++k)
-                            umma_tf32_pair(d_tmem, a_desc + 2 * k, b_desc + 2 * k, kInstrDesc2, (kb | j | k) != 0);
+                        for (int k = 0; k < kBK / 16; ++k)
+                            umma_f16_pair(d_tmem, a_desc + 2 * k, b_desc + 2 * k, kInstrDesc2, (kb | j | k) != 0);
                     }
                     umma_commit_pair(bar_empty + 8 * stage);          // frees the stage in both CTAs
                     if (kb + kStageK2 >= k_blocks) umma_commit_pair(bar_acc_full + 8 * acc);
@@ -207,7 +206,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
         // ---------------- epilogue (both CTAs): this CTA's 128 samples ---------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
         const uint32_t step = a.st->step;
-        float* bias_s = bias_all + (warp - 2) * 64;
+        float* bias_s = bias_all + (warp - 2) * 128;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -217,16 +216,22 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
                 const int j = w0 + cg * 32 + lane;
                 const float bm = j < a.N ? __ldg(a.b4 + j) : 0.f;
                 const float bl = j < a.N ? __ldg(a.b4 + a.N + j) : 0.f;
+                const float sm = j < a.N ? __ldg(a.w_inv + j) : 0.f;
+                const float sl = j < a.N ? __ldg(a.w_inv + a.N + j) : 0.f;
                 __syncwarp();
                 bias_s[lane] = bm;
                 bias_s[32 + lane] = bl;
+                bias_s[64 + lane] = sm;
+                bias_s[96 + lane] = sl;
                 __syncwarp();
                 w_staged = w0;
             }
+            const int row = m0 + q * 32 + lane;
+            const float v_inv = row < a.count ? a.v_inv[row] : 0.f;
             ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
-            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s);
+            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s, v_inv);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }

@@ -1,4 +1,5 @@
-// The emission of the literal model variant (Section 3.1.3) on the 5th-generation tensor cores (tcgen05, kind::tf32):
+// The emission of the literal model variant (Section 3.1.3) on the 5th-generation tensor cores (tcgen05), operands as in
+// half_operand.cuh:
 //   I = Wi2 u + bi2        r = relu(Wj1 I + bj1)        x = I + softplus(Wj2 r + bj2) * eps,      u = Wi1 z' + bi1.
 // I = MLP_2(z, Identity, Identity) is affine in u, so the hidden layer of the scale does not need I:
 //   Wj1 I + bj1 = (Wj1 Wi2) u + (Wj1 bi2 + bj1) = M u + b',
@@ -8,8 +9,8 @@
 //
 // k_gemm_relu_tc has the pipeline of the emission kernel of emit_tc.cuh: one persistent CTA per SM walks over output
 // tiles of 128 rows x 256 columns; a tile is one accumulator of 128 TMEM lanes x 256 fp32 columns,
-// filled by UMMA instructions of shape M=128, N=256, K=8; operands arrive by plain per-CTA TMA loads
-// (boxes of 128 rows x 32 tf32, 128-byte swizzle; rows or columns outside the matrices read as zero)
+// filled by UMMA instructions of shape M=128, N=256, K=16; operands arrive by plain per-CTA TMA loads
+// (boxes of 128 rows x 64 halves, 128-byte swizzle; rows or columns outside the matrices read as zero)
 // into a 4-stage ring; the accumulator is double-buffered.  Warp 0 loads, warp 1 issues the MMAs,
 // warps 2..17 are the epilogue (warp w reads TMEM lanes 32*(w%4).. and the columns
 // 32*cg .. 32*cg+31 and 128+32*cg .. 128+32*cg+31 of the tile, cg = (w-2)/4).
@@ -26,17 +27,22 @@ constexpr int kGemmBN = 256;              // output columns per tile
 
 struct GemmTcArgs {
     const float* bias;      // [Nout]
-    float* out;             // [M][ld_out]: relu(A B^T + bias), rounded to tf32 (it is the next product's operand)
+    const float* a_inv;     // [M] inverse scales of the rows of A
+    const float* b_inv;     // [Nout] inverse scales of the rows of B
+    HalfRows out;           // relu(A B^T + bias), rounded to tf32 and scaled: the next product's operand.  Its bound per row
+                            // follows from A's, whose entries are below 2^15 times their inverse scale
     DevState* st;
-    int M, Nout, K, ld_out;
+    int M, Nout, K;
 };
 
 __device__ __forceinline__ void gemm_epilogue_tile(const GemmTcArgs& a, uint32_t tmem_base, uint32_t acc, int q, int cg,
-                                                   int lane, int m0, int w0, uint32_t bar_acc_empty, const float* bias_s) {
+                                                   int lane, int m0, int w0, uint32_t bar_acc_empty, const float* bias_s, float a_inv) {
     const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32;
     const int row = m0 + q * 32 + lane;
     const bool row_ok = row < a.M;
-    const bool wide_store = (a.ld_out & 7) == 0;
+    float scale, inv;
+    half_scale(1.01f * fmaf(a.out.slope, 32768.0f * a_inv, a.out.offset), scale, inv);
+    if (row_ok && w0 == 0 && cg == 0) a.out.inv_scale[row] = inv;
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
         uint32_t bits[2][16];
@@ -52,33 +58,25 @@ __device__ __forceinline__ void gemm_epilogue_tile(const GemmTcArgs& a, uint32_t
         for (int part = 0; part < 2; ++part) {
             const int jw = w0 + 128 * part + cg * 32 + 16 * half;
             if (!row_ok || jw >= a.Nout) continue;
-            float* dst = a.out + static_cast<size_t>(row) * a.ld_out + jw;
-            float out[16];
+            uint32_t out[8];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float4 bv = *reinterpret_cast<const float4*>(bias_s + 32 * part + 16 * half + 4 * i);
-                const float b[4] = {bv.x, bv.y, bv.z, bv.w};
+                const float4 sv = *reinterpret_cast<const float4*>(bias_s + 64 + 32 * part + 16 * half + 4 * i);
+                const float b[4] = {bv.x, bv.y, bv.z, bv.w}, sc[4] = {sv.x, sv.y, sv.z, sv.w};
+                float v[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    out[4 * i + c] = round_tf32(fmaxf(__uint_as_float(bits[part][4 * i + c]) + b[c], 0.0f));
+                    v[c] = scale * round_tf32(fmaxf(fmaf(__uint_as_float(bits[part][4 * i + c]) * a_inv, sc[c], b[c]), 0.0f));
+                out[2 * i] = pack_half2(v[0], v[1]);
+                out[2 * i + 1] = pack_half2(v[2], v[3]);
             }
+            // rows are a multiple of 8 halves long, the pitch too: whole 16-byte chunks, the last of them short on the ragged edge
+            __half* dst = a.out.p + static_cast<size_t>(row) * a.out.ld + jw;
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                if (wide_store && jw + 8 * p + 7 < a.Nout) {
-                    store8(dst + 8 * p, out + 8 * p);
-                    continue;
-                }
-#pragma unroll
-                for (int i = 2 * p; i < 2 * p + 2; ++i) {
-                    const int ji = jw + 4 * i;
-                    if (ji + 3 < a.Nout) {
-                        *reinterpret_cast<float4*>(dst + 4 * i) =
-                            make_float4(out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
-                    } else {
-                        for (int c = 0; c < 4 && ji + c < a.Nout; ++c) dst[4 * i + c] = out[4 * i + c];
-                    }
-                }
-            }
+            for (int p = 0; p < 2; ++p)
+                if (jw + 8 * p < a.out.ld)
+                    *reinterpret_cast<uint4*>(dst + 8 * p) = make_uint4(out[4 * p], out[4 * p + 1], out[4 * p + 2], out[4 * p + 3]);
         }
     }
 }
@@ -180,8 +178,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
                     const uint64_t a_desc = make_smem_desc(a_addr);
                     const uint64_t b_desc = make_smem_desc(a_addr + kABytes);
 #pragma unroll
-                    for (int k = 0; k < kBK / 8; ++k)          // 8 tf32 = 32 bytes per instruction
-                        umma_tf32(d_tmem, a_desc + 2 * k, b_desc + 2 * k, kInstrDesc, (kb | k) != 0);
+                    for (int k = 0; k < kBK / 16; ++k)          // 16 halves = 32 bytes per instruction
+                        umma_f16(d_tmem, a_desc + 2 * k, b_desc + 2 * k, kInstrDesc, (kb | k) != 0);
                     umma_commit(bar_empty + 8 * stage);         // frees the stage when these MMAs are done
                     if (kb == k_blocks - 1) umma_commit(bar_acc_full + 8 * acc);
                 }
@@ -201,7 +199,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
     } else {
         // ---------------- epilogue ---------------------------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
-        float* bias_s = bias_all + (warp - 2) * 64;
+        float* bias_s = bias_all + (warp - 2) * 128;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -211,16 +209,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
                 const int j = w0 + cg * 32 + lane;
                 const float b_lo = j < a.Nout ? __ldg(a.bias + j) : 0.f;
                 const float b_hi = j + 128 < a.Nout ? __ldg(a.bias + j + 128) : 0.f;
+                const float s_lo = j < a.Nout ? __ldg(a.b_inv + j) : 0.f;
+                const float s_hi = j + 128 < a.Nout ? __ldg(a.b_inv + j + 128) : 0.f;
                 __syncwarp();                           // the previous tile's readers are done
                 bias_s[lane] = b_lo;
                 bias_s[32 + lane] = b_hi;
+                bias_s[64 + lane] = s_lo;
+                bias_s[96 + lane] = s_hi;
                 __syncwarp();
                 w_staged = w0;
             }
+            const int row = m0 + q * 32 + lane;
+            const float a_inv = row < a.M ? a.a_inv[row] : 1.f;
             ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
-            gemm_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s);
+            gemm_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s, a_inv);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }
@@ -244,11 +248,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
 constexpr int kDualStages = 3;
 constexpr int kDualStageBytes = 4 * kABytes;             // 64 KB
 constexpr size_t kDualSmemBytes = kDualStages * kDualStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kBiasBytes;
-constexpr uint32_t kDualInstrDesc = (1u << 4) | (2u << 7) | (2u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);   // N = 128
+constexpr uint32_t kDualInstrDesc = instr_desc_f16(128, 128);
 
 struct EmitDualArgs {
     const float* bias_mean;     // bi2 [N]
     const float* bias_scale;    // bj2 [N]
+    const float *u_inv, *r_inv; // [count] inverse scales of the samples' rows of u and r
+    const float *wi_inv, *wj_inv;   // [N] inverse scales of the rows of Wi2 and Wj2
     float* x;                   // [count][ldx]
     DevState* st;
     NoiseKey key;
@@ -256,65 +262,26 @@ struct EmitDualArgs {
     int count, N, H, ldx;
 };
 
+// x = I + softplus(scale) * eps
 __device__ __forceinline__ void dual_epilogue_tile(const EmitDualArgs& a, uint32_t tmem_base, uint32_t acc, int q, int cg,
                                                    int lane, int m0, int w0, uint32_t step, uint32_t bar_acc_empty,
-                                                   const float* bias_s) {
-    const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32;
+                                                   const float* bias_s, float u_inv, float r_inv) {
     const int row = m0 + q * 32 + lane;
-    const bool row_ok = row < a.count;
-    const uint32_t sample = a.sample_base + static_cast<uint32_t>(row);
+    noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, step,
+                        tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32, w0 + cg * 32, lane, bar_acc_empty + 8 * acc,
+                        [&](const uint32_t (&mean)[8], const uint32_t (&scale)[8], const float (&eps)[8], int c8, float (&out)[8]) {
+        float bm[8], bs[8], im[8], is[8];
+        load8(bm, bias_s + c8);
+        load8(bs, bias_s + 32 + c8);
+        load8(im, bias_s + 64 + c8);
+        load8(is, bias_s + 96 + c8);
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        uint32_t mean_bits[16], scale_bits[16];
-        tmem_ld16(taddr + 16 * half, mean_bits);
-        tmem_ld16(taddr + kBW + 16 * half, scale_bits);
-        tmem_ld_wait();
-        if (half == 1) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_acc_empty + 8 * acc);    // accumulator is free again
-        }
-        const int jw = w0 + cg * 32 + 16 * half;
-        if (row_ok && jw < a.N) {
-            float* dst = a.x + static_cast<size_t>(row) * a.ldx + jw;
-            float out[16];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int j = jw + 4 * i;
-                if (j >= a.N) continue;
-                float eps[4];
-                normal4_fast(static_cast<uint32_t>(j >> 2), sample, kStreamEmission, step, a.key.seed_lo,
-                             a.key.seed_hi, eps);
-                const float4 bm = *reinterpret_cast<const float4*>(bias_s + 16 * half + 4 * i);
-                const float4 bs = *reinterpret_cast<const float4*>(bias_s + 32 + 16 * half + 4 * i);
-                const float bmv[4] = {bm.x, bm.y, bm.z, bm.w}, bsv[4] = {bs.x, bs.y, bs.z, bs.w};
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    out[4 * i + c] = fmaf(softplus_fast(__uint_as_float(scale_bits[4 * i + c]) + bsv[c]), eps[c],
-                                          __uint_as_float(mean_bits[4 * i + c]) + bmv[c]);
-            }
-#pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                if (jw + 8 * p + 7 < a.N) {
-                    store8(dst + 8 * p, out + 8 * p);
-                    continue;
-                }
-#pragma unroll
-                for (int i = 2 * p; i < 2 * p + 2; ++i) {
-                    const int ji = jw + 4 * i;
-                    if (ji + 3 < a.N) {
-                        *reinterpret_cast<float4*>(dst + 4 * i) =
-                            make_float4(out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
-                    } else {
-                        for (int c = 0; c < 4 && ji + c < a.N; ++c) dst[4 * i + c] = out[4 * i + c];
-                    }
-                }
-            }
-        }
-    }
+        for (int c = 0; c < 8; ++c)
+            out[c] = fmaf(softplus_fast(fmaf(__uint_as_float(scale[c]) * r_inv, is[c], bs[c])), eps[c],
+                          fmaf(__uint_as_float(mean[c]) * u_inv, im[c], bm[c]));
+    });
 }
 
-// map_u, map_r: [rows][H] activations; map_wi2, map_wj2: [N][H] weights; boxes of 128 rows x 32 columns.
 __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_constant__ CUtensorMap map_u,
                                                                const __grid_constant__ CUtensorMap map_r,
                                                                const __grid_constant__ CUtensorMap map_wi2,
@@ -414,9 +381,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
                     const uint64_t u_desc = make_smem_desc(s_addr), r_desc = make_smem_desc(s_addr + kABytes);
                     const uint64_t wi_desc = make_smem_desc(s_addr + 2 * kABytes), wj_desc = make_smem_desc(s_addr + 3 * kABytes);
 #pragma unroll
-                    for (int k = 0; k < kBK / 8; ++k) {
-                        umma_tf32(d_tmem, u_desc + 2 * k, wi_desc + 2 * k, kDualInstrDesc, (kb | k) != 0);          // I
-                        umma_tf32(d_tmem + kBW, r_desc + 2 * k, wj_desc + 2 * k, kDualInstrDesc, (kb | k) != 0);    // scale
+                    for (int k = 0; k < kBK / 16; ++k) {
+                        umma_f16(d_tmem, u_desc + 2 * k, wi_desc + 2 * k, kDualInstrDesc, (kb | k) != 0);          // I
+                        umma_f16(d_tmem + kBW, r_desc + 2 * k, wj_desc + 2 * k, kDualInstrDesc, (kb | k) != 0);    // scale
                     }
                     umma_commit(bar_empty + 8 * stage);
                     if (kb == k_blocks - 1) umma_commit(bar_acc_full + 8 * acc);
@@ -437,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
         // ---------------- epilogue ---------------------------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
         const uint32_t step = a.st->step;
-        float* bias_s = bias_all + (warp - 2) * 64;
+        float* bias_s = bias_all + (warp - 2) * 128;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -447,16 +414,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
                 const int j = w0 + cg * 32 + lane;
                 const float bm = j < a.N ? __ldg(a.bias_mean + j) : 0.f;
                 const float bs = j < a.N ? __ldg(a.bias_scale + j) : 0.f;
+                const float im = j < a.N ? __ldg(a.wi_inv + j) : 0.f;
+                const float is = j < a.N ? __ldg(a.wj_inv + j) : 0.f;
                 __syncwarp();
                 bias_s[lane] = bm;
                 bias_s[32 + lane] = bs;
+                bias_s[64 + lane] = im;
+                bias_s[96 + lane] = is;
                 __syncwarp();
                 w_staged = w0;
             }
+            const int row = m0 + q * 32 + lane;
+            const float u_inv = row < a.count ? a.u_inv[row] : 0.f, r_inv = row < a.count ? a.r_inv[row] : 0.f;
             ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
-            dual_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s);
+            dual_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s, u_inv, r_inv);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }

@@ -1,0 +1,46 @@
+// Operands of the emission products in half precision, losing nothing.
+//
+// A value rounded to tf32 (or bf16) has at most 11 significant bits, which is what a half-precision number holds, so
+// the only thing that keeps a tf32 operand from being stored in two bytes is its exponent.  Every row of an operand --
+// a sample's hidden vector, a worker's weights -- is therefore multiplied by a power of two that brings its bound to
+// [2^14, 2^15), and the product's row and column are divided by the two powers of two again (exactly) when the
+// accumulator is read.  The products and their fp32 accumulation are those of tf32 operands; only an entry smaller than 2^-29
+// of its row's bound lands among the half-precision subnormals and is rounded, by at most 2^-40 of the bound, 2^16 below
+// what the fp32 accumulation itself rounds away.  Half-precision operands take half the bytes from L2 to shared memory
+// and half the tensor-core time.
+#pragma once
+#include <cstdint>
+#include <cuda_fp16.h>
+
+namespace cutoff {
+
+// 2^e and 2^-e with bound * 2^e in [2^14, 2^15) (bounds from 2^-86 to 2^114; beyond that the nearest such exponent).
+__host__ __device__ inline int half_exponent(uint32_t bound_bits) {
+    const int ex = static_cast<int>((bound_bits >> 23) & 0xffu) - 127, e = 14 - ex;
+    return e > 100 ? 100 : (e < -100 ? -100 : e);
+}
+__host__ __device__ inline uint32_t pow2_bits(int e) { return static_cast<uint32_t>(127 + e) << 23; }
+
+__device__ __forceinline__ void half_scale(float bound, float& scale, float& inv_scale) {
+    const int e = half_exponent(__float_as_uint(bound));
+    scale = __uint_as_float(pow2_bits(e));
+    inv_scale = __uint_as_float(pow2_bits(-e));
+}
+
+// Two values as one word of two halves (the first in the low half).
+__device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
+// A hidden vector as the emission products read it: halves with a row pitch of whole 16 bytes, one inverse scale per row,
+// and the bound of a row's entries, |entry| <= slope * (largest |input|) + offset.
+struct HalfRows {
+    __half* p;              // [rows][ld]
+    float* inv_scale;       // [rows]
+    int ld;
+    float slope, offset;
+};
+
+}  // namespace cutoff

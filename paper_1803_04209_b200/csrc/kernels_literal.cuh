@@ -66,24 +66,6 @@ __device__ __forceinline__ void relu_mlp2_partial(const float* sAT, const float*
     }
 }
 
-// First layer of the emission mean, u = Wi1 z + bi1 (no activation), written for the samples that exist.
-template <int D>
-__device__ __forceinline__ void literal_emission_first(const float* sWi1T, const float* sbi1, int H, int g,
-                                                       const float (&z)[ChainShape<D>::SPL][D], int k0, int count,
-                                                       int round_u, float* __restrict__ u_out) {
-    constexpr int G = ChainShape<D>::G, SPL = ChainShape<D>::SPL;
-    for (int i0 = 4 * g; i0 < H; i0 += 4 * G) {
-        float hid[SPL][4];
-        hidden_block<D, SPL>(sWi1T, sbi1, H, i0, z, hid);
-#pragma unroll
-        for (int s = 0; s < SPL; ++s) {
-            float4 o = make_float4(hid[s][0], hid[s][1], hid[s][2], hid[s][3]);
-            if (round_u) { o.x = round_tf32(o.x); o.y = round_tf32(o.y); o.z = round_tf32(o.z); o.w = round_tf32(o.w); }
-            if (k0 + s < count) *reinterpret_cast<float4*>(u_out + static_cast<size_t>(k0 + s) * H + i0) = o;
-        }
-    }
-}
-
 // Per-sample chain of the literal variant: guide steps over the window, gated transition, first emission layer.
 // Same work split as k_chain (G = D/4 lanes per group of SPL samples); the weights of each phase are staged in
 // shared memory one phase after the other: guide | gate | proposal | linear map, scale and first emission layer.
@@ -91,8 +73,7 @@ template <int D>
 __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain_literal(ModelDev m, LiteralDev lit,
                                                                            const float* __restrict__ hlr,
                                                                            const DevState* __restrict__ st, NoiseKey key,
-                                                                           uint32_t sample_base, int count, int round_u,
-                                                                           float* __restrict__ u_out /*[count][H]*/) {
+                                                                           uint32_t sample_base, int count, ChainOut out) {
     constexpr int G = ChainShape<D>::G, SPL = ChainShape<D>::SPL;
     extern __shared__ __align__(16) float sm[];
     const int H = m.H, W = m.W;
@@ -176,7 +157,7 @@ __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain_literal(Model
         for (int c = 0; c < 4; ++c) z_own[c] = fmaf(softplusf(scale_own[c]), eps[c], G_own[c]);
         group_allgather<G, D>(z_own, z[s]);
     }
-    literal_emission_first<D>(sWi1T, sbi1, H, g, z, k0, count, round_u, u_out);
+    chain_last_layer<D, false>(sWi1T, sbi1, H, g, z, k0, count, out);        // u = Wi1 z' + bi1: no activation
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -2,6 +2,7 @@
 // fp32 FMA version of the emission output layer.
 #pragma once
 #include "common.cuh"
+#include "half_operand.cuh"
 #include "rng.cuh"
 
 namespace cutoff {
@@ -629,23 +630,52 @@ __device__ __forceinline__ void chain_transition(const ModelDev& m, const float*
     }
 }
 
-// Emission hidden layer: v = relu(W3 z + b3), written for the samples k0 .. k0+SPL-1 that exist.
+// Where the chain's last layer goes: floats (fp32 emission), or halves scaled per sample (tensor-core emission).
+struct ChainOut {
+    float* v;               // [count][H], or null
+    HalfRows half;          // used when v is null: values are rounded to tf32 first
+};
+
+// Four entries i0 .. i0 + 3 of a sample's row, and (lane 0 of the group) the row's inverse scale.
 template <int D>
-__device__ __forceinline__ void chain_emission_hidden(const ModelDev& m, const float* sW3T, const float* sb3, int g,
-                                                      const float (&z)[ChainShape<D>::SPL][D], int k0, int count,
-                                                      int round_v, float* __restrict__ v_out) {
+__device__ __forceinline__ void store_hidden(const ChainOut& out, int k, int H, int i0, const float (&h)[4], float scale) {
+    if (out.v) {
+        *reinterpret_cast<float4*>(out.v + static_cast<size_t>(k) * H + i0) = make_float4(h[0], h[1], h[2], h[3]);
+    } else {
+        *reinterpret_cast<uint2*>(out.half.p + static_cast<size_t>(k) * out.half.ld + i0) =
+            make_uint2(pack_half2(round_tf32(h[0]) * scale, round_tf32(h[1]) * scale), pack_half2(round_tf32(h[2]) * scale, round_tf32(h[3]) * scale));
+    }
+}
+template <int D>
+__device__ __forceinline__ float hidden_scale(const ChainOut& out, int k, bool exists, int g, const float (&z)[D]) {
+    if (out.v) return 1.0f;
+    float zm = 0.0f, scale, inv;
+#pragma unroll
+    for (int d = 0; d < D; ++d) zm = fmaxf(zm, fabsf(z[d]));
+    half_scale(1.01f * fmaf(out.half.slope, zm, out.half.offset), scale, inv);
+    if (g == 0 && exists) out.half.inv_scale[k] = inv;
+    return scale;
+}
+
+// Last layer, act(A z + b) with the ReLU of the emission's hidden layer or none (literal: u), for the samples k0 .. k0+SPL-1
+// that exist.
+template <int D, bool RELU>
+__device__ __forceinline__ void chain_last_layer(const float* sAT, const float* sbias, int H, int g,
+                                                 const float (&z)[ChainShape<D>::SPL][D], int k0, int count, const ChainOut& out) {
     constexpr int G = ChainShape<D>::G, SPL = ChainShape<D>::SPL;
-    const int H = m.H;
+    float scale[SPL];
+#pragma unroll
+    for (int s = 0; s < SPL; ++s) scale[s] = hidden_scale<D>(out, k0 + s, k0 + s < count, g, z[s]);
     for (int i0 = 4 * g; i0 < H; i0 += 4 * G) {
         float hid[SPL][4];
-        hidden_block<D, SPL>(sW3T, sb3, H, i0, z, hid);
+        hidden_block<D, SPL>(sAT, sbias, H, i0, z, hid);
 #pragma unroll
         for (int s = 0; s < SPL; ++s) {
-            float4 o;
-            o.x = fmaxf(hid[s][0], 0.0f); o.y = fmaxf(hid[s][1], 0.0f);
-            o.z = fmaxf(hid[s][2], 0.0f); o.w = fmaxf(hid[s][3], 0.0f);
-            if (round_v) { o.x = round_tf32(o.x); o.y = round_tf32(o.y); o.z = round_tf32(o.z); o.w = round_tf32(o.w); }
-            if (k0 + s < count) *reinterpret_cast<float4*>(v_out + static_cast<size_t>(k0 + s) * H + i0) = o;
+            if (RELU) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) hid[s][c] = fmaxf(hid[s][c], 0.0f);
+            }
+            if (k0 + s < count) store_hidden<D>(out, k0 + s, H, i0, hid[s], scale[s]);
         }
     }
 }
@@ -654,8 +684,7 @@ __device__ __forceinline__ void chain_emission_hidden(const ModelDev& m, const f
 template <int D>
 __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain(ModelDev m, const float* __restrict__ hlr,
                                                           const DevState* __restrict__ st, NoiseKey key,
-                                                          uint32_t sample_base, int count, int round_v,
-                                                          float* __restrict__ v_out /*[count][H]*/) {
+                                                          uint32_t sample_base, int count, ChainOut out) {
     constexpr int G = ChainShape<D>::G, SPL = ChainShape<D>::SPL;
     extern __shared__ __align__(16) float sm[];
     const int H = m.H, W = m.W;
@@ -699,7 +728,7 @@ __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain(ModelDev m, c
     stage_vector4(sW3T, m.W3T, H * D);
     stage_vector4(sb3, m.b3, H);
     __syncthreads();
-    chain_emission_hidden<D>(m, sW3T, sb3, g, z, k0, count, round_v, v_out);
+    chain_last_layer<D, true>(sW3T, sb3, H, g, z, k0, count, out);
 }
 
 // Variant 2: every weight of the chain resident in shared memory, one persistent CTA per SM.
@@ -715,7 +744,7 @@ inline size_t chain_resident_smem_floats(int D, int H, int W) {
 template <int D>
 __global__ void __launch_bounds__(kChainResidentThreads, 1)
 k_chain_resident(ModelDev m, const float* __restrict__ hlr, const DevState* __restrict__ st, NoiseKey key,
-                 uint32_t sample_base, int count, int round_v, float* __restrict__ v_out /*[count][H]*/) {
+                 uint32_t sample_base, int count, ChainOut out) {
     constexpr int G = ChainShape<D>::G, SPL = ChainShape<D>::SPL;
     constexpr int kBatch = 32 / G * SPL;                // samples per warp and pass
     extern __shared__ __align__(16) float sm[];
@@ -759,7 +788,7 @@ k_chain_resident(ModelDev m, const float* __restrict__ hlr, const DevState* __re
             for (int d = 0; d < D; ++d) z[s][d] = m.z0[d];
         chain_guide<D>(m, sWzT, sWmu, sWsig, sbz, shl, g, nz, z);
         chain_transition<D>(m, sW1T, sW2, sb1, g, nz, z);
-        chain_emission_hidden<D>(m, sW3T, sb3, g, z, k0, count, round_v, v_out);
+        chain_last_layer<D, true>(sW3T, sb3, H, g, z, k0, count, out);
     }
 }
 
