@@ -42,7 +42,8 @@ constexpr int kEpiWarps = 16;
 constexpr int kThreads = (2 + kEpiWarps) * 32;
 constexpr int kTmemCols = 512;
 constexpr int kAccCols = 2 * kBW;                // 256 columns per accumulator
-constexpr int kBiasBytes = kEpiWarps * 128 * 4;  // per epilogue warp: biases of its 32 + 32 columns, then their inverse scales
+constexpr int kTableFloats = 128 + 32;           // per epilogue warp: biases of its 32 + 32 columns, their inverse scales, and the
+constexpr int kBiasBytes = kEpiWarps * kTableFloats * 4;   // generator's part of its 8 groups of four workers
 constexpr size_t kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kBiasBytes;
 
 // instruction descriptor: D = f32, A = B = f16, both K-major, N columns, M rows
@@ -137,7 +138,9 @@ struct EmitArgs {
 // finish(first 8 columns' words, second 8 columns' words, 8 normals, column of the warp, 8 results): the variant's own arithmetic.
 template <typename Finish>
 __device__ __forceinline__ void noise_epilogue_tile(float* __restrict__ x, int ldx, int N, bool row_ok, int row, uint32_t sample, NoiseKey key,
-                                                    uint32_t step, uint32_t taddr, int jw0, int lane, uint32_t bar_acc_empty, Finish finish) {
+                                                    const float* table, uint32_t taddr, int jw0, int lane, uint32_t bar_acc_empty, Finish finish) {
+    const PhiloxRow noise = philox_row(sample, kStreamEmission, key.seed_lo);
+    const uint4* columns = reinterpret_cast<const uint4*>(table + 128);
 #pragma unroll
     for (int c8 = 0; c8 < 32; c8 += 8) {
         uint32_t lo[8], hi[8];
@@ -145,8 +148,8 @@ __device__ __forceinline__ void noise_epilogue_tile(float* __restrict__ x, int l
         tmem_ld8(taddr + kBW + c8, hi);
         const int jw = jw0 + c8;
         float eps[8], out[8];
-        normal4_fast(static_cast<uint32_t>(jw >> 2), sample, kStreamEmission, step, key.seed_lo, key.seed_hi, eps);
-        normal4_fast(static_cast<uint32_t>(jw >> 2) + 1u, sample, kStreamEmission, step, key.seed_lo, key.seed_hi, eps + 4);
+        normal4_row_column_fast(noise, columns[c8 / 4], key.seed_lo, key.seed_hi, eps);
+        normal4_row_column_fast(noise, columns[c8 / 4 + 1], key.seed_lo, key.seed_hi, eps + 4);
         tmem_ld_wait();
         if (c8 == 24) {
             tc_fence_before();
@@ -167,6 +170,12 @@ __device__ __forceinline__ void noise_epilogue_tile(float* __restrict__ x, int l
     }
 }
 
+// The generator's column words of a warp's 32 workers from j0 on (j0 a multiple of 32): lanes 0 .. 7.
+__device__ __forceinline__ void put_noise_columns(float* table, int j0, int lane, uint32_t step, NoiseKey key) {
+    if (lane < 8)
+        reinterpret_cast<uint4*>(table + 128)[lane] = philox_column(static_cast<uint32_t>((j0 >> 2) + lane), kStreamEmission, step, key.seed_lo, key.seed_hi);
+}
+
 __device__ __forceinline__ void load8(float (&r)[8], const float* p) {
     const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
     r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w; r[4] = b.x; r[5] = b.y; r[6] = b.z; r[7] = b.w;
@@ -175,10 +184,10 @@ __device__ __forceinline__ void load8(float (&r)[8], const float* p) {
 // x = mean + exp(logvar / 2) * eps.  bias_s: this warp's 32 mean biases, then its 32 log-variance biases, then the inverse scales
 // of the same columns, in shared memory (zero beyond worker N).  v_inv: inverse scale of this thread's sample.
 __device__ __forceinline__ void emit_epilogue_tile(const EmitArgs& a, uint32_t tmem_base, uint32_t acc, int q, int cg,
-                                                   int lane, int m0, int w0, uint32_t step, uint32_t bar_acc_empty,
+                                                   int lane, int m0, int w0, uint32_t bar_acc_empty,
                                                    const float* bias_s, float v_inv) {
     const int row = m0 + q * 32 + lane;
-    noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, step,
+    noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, bias_s,
                         tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32, w0 + cg * 32, lane, bar_acc_empty + 8 * acc,
                         [&](const uint32_t (&mean)[8], const uint32_t (&logvar)[8], const float (&eps)[8], int c8, float (&out)[8]) {
         float bm[8], bl[8], sm[8], sl[8];
@@ -312,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
         // ---------------- epilogue ---------------------------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
         const uint32_t step = a.st->step;
-        float* bias_s = bias_all + (warp - 2) * 128;
+        float* bias_s = bias_all + (warp - 2) * kTableFloats;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -329,6 +338,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
                 bias_s[32 + lane] = bl;
                 bias_s[64 + lane] = sm;
                 bias_s[96 + lane] = sl;
+                put_noise_columns(bias_s, w0 + cg * 32, lane, step, a.key);
                 __syncwarp();
                 w_staged = w0;
             }
@@ -337,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
             ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
-            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s, v_inv);
+            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s, v_inv);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }

@@ -206,7 +206,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
         // ---------------- epilogue (both CTAs): this CTA's 128 samples ---------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
         const uint32_t step = a.st->step;
-        float* bias_s = bias_all + (warp - 2) * 128;
+        float* bias_s = bias_all + (warp - 2) * kTableFloats;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -223,6 +223,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
                 bias_s[32 + lane] = bl;
                 bias_s[64 + lane] = sm;
                 bias_s[96 + lane] = sl;
+                put_noise_columns(bias_s, w0 + cg * 32, lane, step, a.key);
                 __syncwarp();
                 w_staged = w0;
             }
@@ -231,7 +232,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
             ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
-            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s, v_inv);
+            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s, v_inv);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
     } else {
         // ---------------- epilogue ---------------------------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
-        float* bias_s = bias_all + (warp - 2) * 128;
+        float* bias_s = bias_all + (warp - 2) * kTableFloats;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -264,10 +264,10 @@ struct EmitDualArgs {
 
 // x = I + softplus(scale) * eps
 __device__ __forceinline__ void dual_epilogue_tile(const EmitDualArgs& a, uint32_t tmem_base, uint32_t acc, int q, int cg,
-                                                   int lane, int m0, int w0, uint32_t step, uint32_t bar_acc_empty,
+                                                   int lane, int m0, int w0, uint32_t bar_acc_empty,
                                                    const float* bias_s, float u_inv, float r_inv) {
     const int row = m0 + q * 32 + lane;
-    noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, step,
+    noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, bias_s,
                         tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32, w0 + cg * 32, lane, bar_acc_empty + 8 * acc,
                         [&](const uint32_t (&mean)[8], const uint32_t (&scale)[8], const float (&eps)[8], int c8, float (&out)[8]) {
         float bm[8], bs[8], im[8], is[8];
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
         // ---------------- epilogue ---------------------------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
         const uint32_t step = a.st->step;
-        float* bias_s = bias_all + (warp - 2) * 128;
+        float* bias_s = bias_all + (warp - 2) * kTableFloats;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -421,6 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
                 bias_s[32 + lane] = bs;
                 bias_s[64 + lane] = im;
                 bias_s[96 + lane] = is;
+                put_noise_columns(bias_s, w0 + cg * 32, lane, step, a.key);
                 __syncwarp();
                 w_staged = w0;
             }
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
             ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
-            dual_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, step, bar_acc_empty, bias_s, u_inv, r_inv);
+            dual_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s, u_inv, r_inv);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }

@@ -37,6 +37,47 @@ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint3
     return Philox4{c0, c1, c2, c3};
 }
 
+// The same ten rounds for a whole matrix of draws (rows = samples, columns = groups of four elements) of one stream and
+// decision: of the first three rounds only one multiplication depends on both, so the others are done once per column and
+// once per row.  Half the key reaches the first round through `row`; the words that come out are those of philox4x32_10.
+struct PhiloxRow {
+    uint32_t hi, lo;
+};
+__device__ __forceinline__ PhiloxRow philox_row(uint32_t sample, uint32_t stream, uint32_t k0) {
+    const uint32_t first = static_cast<uint32_t>((0xCD9E8D57ull * stream) >> 32) ^ sample ^ k0;
+    const unsigned long long p = 0xD2511F53ull * first;
+    return PhiloxRow{static_cast<uint32_t>(p >> 32), static_cast<uint32_t>(p)};
+}
+__device__ __forceinline__ uint4 philox_column(uint32_t q, uint32_t stream, uint32_t step, uint32_t k0, uint32_t k1) {
+    constexpr unsigned long long kMulA = 0xD2511F53u, kMulB = 0xCD9E8D57u;
+    constexpr uint32_t kWeylA = 0x9E3779B9u, kWeylB = 0xBB67AE85u;
+    const unsigned long long a1 = kMulA * q, b1 = kMulB * stream;
+    const unsigned long long b2 = kMulB * (static_cast<uint32_t>(a1 >> 32) ^ step ^ k1);
+    const unsigned long long a3 = kMulA * (static_cast<uint32_t>(b2 >> 32) ^ static_cast<uint32_t>(b1) ^ (k0 + kWeylA));
+    return make_uint4(static_cast<uint32_t>(a1) ^ (k1 + kWeylB), static_cast<uint32_t>(b2) ^ (k0 + 2 * kWeylA),
+                      static_cast<uint32_t>(a3 >> 32) ^ (k1 + 2 * kWeylB), static_cast<uint32_t>(a3));
+}
+__device__ __forceinline__ Philox4 philox_row_column(const PhiloxRow& row, const uint4& col, uint32_t k0, uint32_t k1) {
+    constexpr uint32_t kMulA = 0xD2511F53u, kMulB = 0xCD9E8D57u;
+    constexpr uint32_t kWeylA = 0x9E3779B9u, kWeylB = 0xBB67AE85u;
+    const unsigned long long b3 = static_cast<unsigned long long>(kMulB) * (row.hi ^ col.x);
+    uint32_t c0 = static_cast<uint32_t>(b3 >> 32) ^ col.y, c1 = static_cast<uint32_t>(b3), c2 = row.lo ^ col.z, c3 = col.w;
+    k0 += 3 * kWeylA;
+    k1 += 3 * kWeylB;
+#pragma unroll
+    for (int round = 3; round < 10; ++round) {
+        const unsigned long long prod_a = static_cast<unsigned long long>(kMulA) * c0;
+        const unsigned long long prod_b = static_cast<unsigned long long>(kMulB) * c2;
+        c0 = static_cast<uint32_t>(prod_b >> 32) ^ c1 ^ k0;
+        c1 = static_cast<uint32_t>(prod_b);
+        c2 = static_cast<uint32_t>(prod_a >> 32) ^ c3 ^ k1;
+        c3 = static_cast<uint32_t>(prod_a);
+        k0 += kWeylA;
+        k1 += kWeylB;
+    }
+    return Philox4{c0, c1, c2, c3};
+}
+
 __device__ __forceinline__ void box_muller(uint32_t r_a, uint32_t r_b, float& e_cos, float& e_sin) {
     const float u1 = static_cast<float>((r_a >> 8) + 1u) * 0x1p-24f;
     const float two_u2 = static_cast<float>(r_b >> 8) * 0x1p-23f;
@@ -55,7 +96,7 @@ __device__ __forceinline__ void box_muller(uint32_t r_a, uint32_t r_b, float& e_
 __device__ __forceinline__ void box_muller_fast(uint32_t r_a, uint32_t r_b, float& e_cos, float& e_sin) {
     const float u1 = static_cast<float>((r_a >> 8) + 1u) * 0x1p-24f;
     const float angle = static_cast<float>(static_cast<int32_t>(r_b) >> 8) * (6.283185307179586f * 0x1p-24f);
-    const float r2 = fmaxf(-1.3862943611198906f * __log2f(u1), 0.0f);     // -2 ln u1
+    const float r2 = fabsf(-1.3862943611198906f * __log2f(u1));           // -2 ln u1 (the absolute value costs nothing)
     float radius;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(radius) : "f"(r2));
     e_cos = radius * __cosf(angle);
@@ -79,6 +120,18 @@ __device__ __forceinline__ void normal4(uint32_t q, uint32_t sample, uint32_t st
 __device__ __forceinline__ void normal4_fast(uint32_t q, uint32_t sample, uint32_t stream, uint32_t step,
                                              uint32_t seed_lo, uint32_t seed_hi, float out[4]) {
     const Philox4 r = philox4x32_10(q, sample, stream, step, seed_lo, seed_hi);
+    box_muller_fast(r.x, r.y, out[0], out[1]);
+    box_muller_fast(r.z, r.w, out[2], out[3]);
+}
+
+// Four standard normals of one row and column of a matrix of draws.
+__device__ __forceinline__ void normal4_row_column(const PhiloxRow& row, const uint4& col, uint32_t seed_lo, uint32_t seed_hi, float out[4]) {
+    const Philox4 r = philox_row_column(row, col, seed_lo, seed_hi);
+    box_muller(r.x, r.y, out[0], out[1]);
+    box_muller(r.z, r.w, out[2], out[3]);
+}
+__device__ __forceinline__ void normal4_row_column_fast(const PhiloxRow& row, const uint4& col, uint32_t seed_lo, uint32_t seed_hi, float out[4]) {
+    const Philox4 r = philox_row_column(row, col, seed_lo, seed_hi);
     box_muller_fast(r.x, r.y, out[0], out[1]);
     box_muller_fast(r.z, r.w, out[2], out[3]);
 }
