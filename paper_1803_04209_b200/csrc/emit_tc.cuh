@@ -120,6 +120,9 @@ __device__ __forceinline__ void store8(float* p, const float* v) {
                  ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
 }
 
+// Tiles of CTA b of the grid: first_tile(b) .. first_tile(b + 1) - 1, as equal as they can be.
+__device__ __forceinline__ int first_tile(unsigned b, int total) { return static_cast<int>(static_cast<unsigned long long>(total) * b / gridDim.x); }
+
 struct EmitArgs {
     const float* b4;        // [2N]
     const float* v_inv;     // [count] inverse scales of the samples' hidden vectors
@@ -220,7 +223,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles_w = ceil_div(a.N, kBW);
     const int n_tiles_m = ceil_div(a.count, kBM);
-    const int total_tiles = n_tiles_w * n_tiles_m;
+    // consecutive tiles, samples first: a CTA stays with its workers, whose biases and generator words are staged once or twice
+    const int tile_begin = first_tile(blockIdx.x, n_tiles_w * n_tiles_m), tile_end = first_tile(blockIdx.x + 1, n_tiles_w * n_tiles_m);
     const int k_blocks = ceil_div(a.H, kBK);
 
     if (threadIdx.x == 0) {
@@ -254,8 +258,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
         uint32_t stage = 0, phase = 0;
         uint32_t armed_mask = 0, parity_mask = 0;      // per stage: armed at least once / parity of its last phase
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const int m0 = (t / n_tiles_w) * kBM, w0 = (t % n_tiles_w) * kBW;
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
+            const int m0 = (t % n_tiles_m) * kBM, w0 = (t / n_tiles_m) * kBW;
             for (int kb = 0; kb < k_blocks; ++kb) {
                 ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, a.st);
                 if (!ok) break;
@@ -285,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
         // ---------------- MMA issuer -------------------------------------------------------------
         uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
             ok = mbar_wait(bar_acc_empty + 8 * acc, acc_phase ^ 1u, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
@@ -325,8 +329,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const int m0 = (t / n_tiles_w) * kBM, w0 = (t % n_tiles_w) * kBW;
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
+            const int m0 = (t % n_tiles_m) * kBM, w0 = (t / n_tiles_m) * kBW;
             if (w0 != w_staged) {                       // biases of this warp's 32 workers, read once per worker tile
                 const int j = w0 + cg * 32 + lane;
                 const float bm = j < a.N ? __ldg(a.b4 + j) : 0.f;

@@ -99,7 +99,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles_w = ceil_div(a.Nout, kGemmBN);
     const int n_tiles_m = ceil_div(a.M, kBM);
-    const int total_tiles = n_tiles_w * n_tiles_m;
+    // consecutive tiles, samples first: a CTA stays with its workers, whose biases and generator words are staged once or twice
+    const int tile_begin = first_tile(blockIdx.x, n_tiles_w * n_tiles_m), tile_end = first_tile(blockIdx.x + 1, n_tiles_w * n_tiles_m);
     const int k_blocks = ceil_div(a.K, kBK);
 
     if (threadIdx.x == 0) {
@@ -133,8 +134,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
         uint32_t stage = 0, phase = 0;
         uint32_t armed_mask = 0, parity_mask = 0;      // per stage: armed at least once / parity of its last phase
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const int m0 = (t / n_tiles_w) * kBM, w0 = (t % n_tiles_w) * kGemmBN;
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
+            const int m0 = (t % n_tiles_m) * kBM, w0 = (t / n_tiles_m) * kGemmBN;
             for (int kb = 0; kb < k_blocks; ++kb) {
                 ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, a.st);
                 if (!ok) break;
@@ -164,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
         // ---------------- MMA issuer -------------------------------------------------------------
         uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
             ok = mbar_wait(bar_acc_empty + 8 * acc, acc_phase ^ 1u, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
@@ -203,8 +204,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const int m0 = (t / n_tiles_w) * kBM, w0 = (t % n_tiles_w) * kGemmBN;
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
+            const int m0 = (t % n_tiles_m) * kBM, w0 = (t / n_tiles_m) * kGemmBN;
             if (w0 != w_staged) {                       // biases of this warp's 2 x 32 columns, read once per column tile
                 const int j = w0 + cg * 32 + lane;
                 const float b_lo = j < a.Nout ? __ldg(a.bias + j) : 0.f;
@@ -302,7 +303,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles_w = ceil_div(a.N, kBW);
     const int n_tiles_m = ceil_div(a.count, kBM);
-    const int total_tiles = n_tiles_w * n_tiles_m;
+    // consecutive tiles, samples first: a CTA stays with its workers, whose biases and generator words are staged once or twice
+    const int tile_begin = first_tile(blockIdx.x, n_tiles_w * n_tiles_m), tile_end = first_tile(blockIdx.x + 1, n_tiles_w * n_tiles_m);
     const int k_blocks = ceil_div(a.H, kBK);
 
     if (threadIdx.x == 0) {
@@ -336,8 +338,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
         uint32_t stage = 0, phase = 0;
         uint32_t armed_mask = 0, parity_mask = 0;
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const int m0 = (t / n_tiles_w) * kBM, w0 = (t % n_tiles_w) * kBW;
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
+            const int m0 = (t % n_tiles_m) * kBM, w0 = (t / n_tiles_m) * kBW;
             for (int kb = 0; kb < k_blocks; ++kb) {
                 ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, a.st);
                 if (!ok) break;
@@ -367,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
         // ---------------- MMA issuer -------------------------------------------------------------
         uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
             ok = mbar_wait(bar_acc_empty + 8 * acc, acc_phase ^ 1u, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
@@ -408,8 +410,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const int m0 = (t / n_tiles_w) * kBM, w0 = (t % n_tiles_w) * kBW;
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
+            const int m0 = (t % n_tiles_m) * kBM, w0 = (t / n_tiles_m) * kBW;
             if (w0 != w_staged) {                       // biases of this warp's 32 workers, read once per worker tile
                 const int j = w0 + cg * 32 + lane;
                 const float bm = j < a.N ? __ldg(a.bias_mean + j) : 0.f;
