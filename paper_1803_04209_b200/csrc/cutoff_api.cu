@@ -523,13 +523,13 @@ void launch_emission_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
         // pairs of SMs share a weight tile: 256 samples x 128 workers per cluster and tile
         const int pair_tiles = ceil_div(c->N, tc::kBW) * ceil_div(count, 2 * tc::kBM);
         const int clusters = pair_tiles < c->pair_clusters ? pair_tiles : c->pair_clusters;
-        tc::k_emit_tc2<<<2 * clusters, tc::kNoiseThreads, tc::kSmem2Bytes, c->stream>>>(c->map_v, c->map_w4, a);
+        tc::k_emit_tc2<<<2 * clusters, tc::kThreads, tc::kSmem2Bytes, c->stream>>>(c->map_v, c->map_w4, a);
         c->launches += 1;
         return;
     }
     const int tiles = ceil_div(c->N, tc::kBW) * ceil_div(count, tc::kBM);
     const int grid = tiles < c->sm_count ? tiles : c->sm_count;
-    launch_dependent(tc::k_emit_tc, dim3(grid), dim3(tc::kNoiseThreads), tc::kSmemBytes, c->stream, c->map_v, c->map_w4, a);
+    launch_dependent(tc::k_emit_tc, dim3(grid), dim3(tc::kThreads), tc::kSmemBytes, c->stream, c->map_v, c->map_w4, a);
     c->launches += 1;
 }
 
@@ -556,7 +556,7 @@ void launch_emission_literal(cutoff_ctx* c, uint32_t sample_base, int count) {
         e.wi_inv = c->d_w_inv; e.wj_inv = c->d_w_inv + c->N; e.x = c->d_x; e.st = c->d_state; e.key = key;
         e.sample_base = sample_base; e.count = count; e.N = c->N; e.H = c->H; e.ldx = c->ldx;
         const int tiles = ceil_div(c->N, tc::kBW) * ceil_div(count, tc::kBM);
-        launch_dependent(tc::k_emit_dual_tc, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kNoiseThreads), tc::kDualSmemBytes, c->stream,
+        launch_dependent(tc::k_emit_dual_tc, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kThreads), tc::kDualSmemBytes, c->stream,
                          c->map_v, c->map_r, c->map_wi2, c->map_wj2, e);
         c->launches += 1;
         return;
@@ -910,7 +910,7 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
         // how many two-CTA clusters of the two-SM emission kernel the GPU can hold at once
         cudaLaunchConfig_t lc{};
         lc.gridDim = dim3(2 * c->sm_count);
-        lc.blockDim = dim3(tc::kNoiseThreads);
+        lc.blockDim = dim3(tc::kThreads);
         lc.dynamicSmemBytes = tc::kSmem2Bytes;
         cudaLaunchAttribute at{};
         at.id = cudaLaunchAttributeClusterDimension;

@@ -9,8 +9,8 @@
 // is double-buffered (2 x 256 of the 512 TMEM columns) so that the epilogue of one tile runs
 // while the next tile is multiplied.
 //
-// Warp roles: warp 0 issues TMA loads, warp 1 owns TMEM and issues the MMAs, warps 2..29 are the epilogue: a tile is 16 items of
-// eight workers for each quarter of its samples (TMEM lanes 32*(w%4)..), which the seven warps of a quarter take in turn.
+// Warp roles: warp 0 issues TMA loads, warp 1 owns TMEM and issues the MMAs, warps 2..17 are the
+// epilogue (warp w reads TMEM lanes 32*(w%4).., the 32 workers of column group (w-2)/4).
 //
 // What bounds it: as four-byte operands it was the stream L2 -> shared memory, 384 KB per tile (N = 1024, S = 65536: 0.148 ms); as
 // halves the stream and the tensor time halve and the epilogue sets the pace, about 150 instructions per four draws.
@@ -42,14 +42,9 @@ constexpr int kEpiWarps = 16;
 constexpr int kThreads = (2 + kEpiWarps) * 32;
 constexpr int kTmemCols = 512;
 constexpr int kAccCols = 2 * kBW;                // 256 columns per accumulator
-constexpr int kBiasBytes = kEpiWarps * 128 * 4;  // per epilogue warp: biases of its 32 + 32 columns, then their inverse scales
-constexpr size_t kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kBiasBytes;   // (the noise tables are smaller than the biases)
-
-// The kernels whose epilogue draws the noise.  28 epilogue warps of 64 registers: a draw is a chain of dependent instructions, and the
-// issue slots are filled by other warps' chains (16 warps of 96 registers: 55 % of the slots).
-constexpr int kNoiseWarps = 28, kNoiseThreads = (2 + kNoiseWarps) * 32;
-constexpr int kItemsPerTile = 64;                // 16 groups of eight workers x 4 quarters of the samples
-constexpr int kTableFloats = 4 * kBW + kBW;      // of a tile's 128 workers: two biases, two inverse scales, the generator's column words
+constexpr int kTableFloats = 128 + 32;           // per epilogue warp: biases of its 32 + 32 columns, their inverse scales, and the
+constexpr int kBiasBytes = kEpiWarps * kTableFloats * 4;   // generator's part of its 8 groups of four workers
+constexpr size_t kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kBiasBytes;
 
 // instruction descriptor: D = f32, A = B = f16, both K-major, N columns, M rows
 constexpr uint32_t instr_desc_f16(uint32_t n, uint32_t m) { return (1u << 4) | ((n >> 3) << 17) | ((m >> 4) << 24); }
@@ -139,109 +134,78 @@ struct EmitArgs {
     int count, N, H, ldx;
 };
 
+// Epilogue of one 128 x 128 output tile for one warp: 32 samples (its TMEM lanes) x 32 workers, eight workers at a time.
+// The noise of the eight is drawn while their accumulators are on their way from tensor memory, without a branch between
+// the two generator calls: the generator is a chain of ten dependent rounds, and one call after the other, behind the loads,
+// left the issue slots 54 % empty (N = 1024, S = 65536: 0.165 ms with half-precision operands).
+// finish(first 8 columns' words, second 8 columns' words, 8 normals, column of the warp, 8 results): the variant's own arithmetic.
+template <typename Finish>
+__device__ __forceinline__ void noise_epilogue_tile(float* __restrict__ x, int ldx, int N, bool row_ok, int row, uint32_t sample, NoiseKey key,
+                                                    const float* table, uint32_t taddr, int jw0, int lane, uint32_t bar_acc_empty, Finish finish) {
+    const PhiloxRow noise = philox_row(sample, kStreamEmission, key.seed_lo);
+    const uint4* columns = reinterpret_cast<const uint4*>(table + 128);
+#pragma unroll
+    for (int c8 = 0; c8 < 32; c8 += 8) {
+        uint32_t lo[8], hi[8];
+        tmem_ld8(taddr + c8, lo);
+        tmem_ld8(taddr + kBW + c8, hi);
+        const int jw = jw0 + c8;
+        float eps[8], out[8];
+        normal4_row_column_fast(noise, columns[c8 / 4], key.seed_lo, key.seed_hi, eps);
+        normal4_row_column_fast(noise, columns[c8 / 4 + 1], key.seed_lo, key.seed_hi, eps + 4);
+        tmem_ld_wait();
+        if (c8 == 24) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_acc_empty);              // accumulator is free again
+        }
+        finish(lo, hi, eps, c8, out);
+        if (!row_ok || jw >= N) continue;
+        // whole sectors (the row pitch is a multiple of 8 floats), 16-byte or scalar stores on the ragged edge
+        float* dst = x + static_cast<size_t>(row) * ldx + jw;
+        if (jw + 7 < N) {
+            store8(dst, out);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (jw + i < N) dst[i] = out[i];
+        }
+    }
+}
+
+// The generator's column words of a warp's 32 workers from j0 on (j0 a multiple of 32): lanes 0 .. 7.
+__device__ __forceinline__ void put_noise_columns(float* table, int j0, int lane, uint32_t step, NoiseKey key) {
+    if (lane < 8)
+        reinterpret_cast<uint4*>(table + 128)[lane] = philox_column(static_cast<uint32_t>((j0 >> 2) + lane), kStreamEmission, step, key.seed_lo, key.seed_hi);
+}
+
 __device__ __forceinline__ void load8(float (&r)[8], const float* p) {
     const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
     r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w; r[4] = b.x; r[5] = b.y; r[6] = b.z; r[7] = b.w;
 }
 
-// What the epilogue reads per worker, for the (at most two) blocks of 128 workers a CTA's tiles lie in: tables[i] for block
-// w_first + i.  A grid of consecutive tiles, samples first, crosses at most one border between blocks: there are at most 32 blocks.
-__device__ __forceinline__ void fill_noise_tables(float* tables, int w_first, int N, const float* bias_a, const float* bias_b,
-                                                  const float* inv_a, const float* inv_b, uint32_t step, NoiseKey key) {
-    for (int i = threadIdx.x; i < 2 * kBW; i += kNoiseThreads) {
-        float* t = tables + (i / kBW) * kTableFloats;
-        const int c = i % kBW, j = w_first * kBW + i;
-        t[c] = j < N ? bias_a[j] : 0.f;
-        t[kBW + c] = j < N ? bias_b[j] : 0.f;
-        t[2 * kBW + c] = j < N ? inv_a[j] : 0.f;
-        t[3 * kBW + c] = j < N ? inv_b[j] : 0.f;
-        if (c % 4 == 0)
-            reinterpret_cast<uint4*>(t + 4 * kBW)[c / 4] = philox_column(static_cast<uint32_t>(j >> 2), kStreamEmission, step, key.seed_lo, key.seed_hi);
-    }
+// x = mean + exp(logvar / 2) * eps.  bias_s: this warp's 32 mean biases, then its 32 log-variance biases, then the inverse scales
+// of the same columns, in shared memory (zero beyond worker N).  v_inv: inverse scale of this thread's sample.
+__device__ __forceinline__ void emit_epilogue_tile(const EmitArgs& a, uint32_t tmem_base, uint32_t acc, int q, int cg,
+                                                   int lane, int m0, int w0, uint32_t bar_acc_empty,
+                                                   const float* bias_s, float v_inv) {
+    const int row = m0 + q * 32 + lane;
+    noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, bias_s,
+                        tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32, w0 + cg * 32, lane, bar_acc_empty + 8 * acc,
+                        [&](const uint32_t (&mean)[8], const uint32_t (&logvar)[8], const float (&eps)[8], int c8, float (&out)[8]) {
+        float bm[8], bl[8], sm[8], sl[8];
+        load8(bm, bias_s + c8);
+        load8(bl, bias_s + 32 + c8);
+        load8(sm, bias_s + 64 + c8);
+        load8(sl, bias_s + 96 + c8);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            out[c] = fmaf(exp_half_fast(fmaf(__uint_as_float(logvar[c]) * v_inv, sl[c], bl[c])), eps[c],
+                          fmaf(__uint_as_float(mean[c]) * v_inv, sm[c], bm[c]));
+    });
 }
 
-struct NoiseTiles {
-    float* x;               // [rows][ldx]
-    int ldx, N, count;
-    uint32_t sample_base;
-    NoiseKey key;
-    const float* tables;
-    int tile_begin, tile_end, n_tiles_m, w_first;
-    int row_stride, row_first;      // first sample of row tile m: m * row_stride + row_first
-    uint32_t tmem_base, bar_acc_full, bar_acc_empty;
-};
-
-// The epilogue of one warp over all tiles of its CTA: items of 32 samples (its TMEM lanes) x 8 workers.  The noise of an item is
-// drawn while its accumulators are on their way from tensor memory, without a branch between the two generator calls.
-// row_scales(row, exists) loads what a sample needs (asked for a tile ahead); finish(words a, words b, 8 normals, scales, table, column,
-// 8 results) is the variant's own arithmetic.
-template <typename Scales, typename RowScales, typename Finish>
-__device__ __forceinline__ void noise_epilogue(const NoiseTiles& n, int warp, int lane, volatile int* abort_flag, DevState* st,
-                                               RowScales row_scales, Finish finish) {
-    const int q = warp & 3;
-    const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
-    const auto row_of = [&](int t) { return (t % n.n_tiles_m) * n.row_stride + n.row_first + q * 32 + lane; };
-    int ti = -1, row = 0, w0 = 0;
-    const float* table = n.tables;
-    PhiloxRow noise{};
-    Scales scales{}, ahead = row_scales(row_of(n.tile_begin));
-    for (int item = (warp - 2) >> 2;; item += kNoiseWarps / 4) {
-        const int t = n.tile_begin + (item >> 4), c8 = (item & 15) * 8;
-        if (t >= n.tile_end) break;
-        if ((item >> 4) != ti) {
-            ti = item >> 4;
-            row = row_of(t);
-            const int wt = t / n.n_tiles_m;
-            w0 = wt * kBW;
-            table = n.tables + (wt - n.w_first) * kTableFloats;
-            scales = ahead;
-            ahead = row_scales(t + 1 < n.tile_end ? row_of(t + 1) : row);
-            noise = philox_row(n.sample_base + static_cast<uint32_t>(row), kStreamEmission, n.key.seed_lo);
-            if (!mbar_wait(n.bar_acc_full + 8 * (ti & 1), (ti >> 1) & 1, abort_flag, st)) return;
-            tc_fence_after();
-        }
-        const uint32_t taddr = n.tmem_base + lanes + (ti & 1) * kAccCols + c8;
-        uint32_t lo[8], hi[8];
-        tmem_ld8(taddr, lo);
-        tmem_ld8(taddr + kBW, hi);
-        const uint4* columns = reinterpret_cast<const uint4*>(table + 4 * kBW) + c8 / 4;
-        float eps[8], out[8];
-        normal4_row_column_fast(noise, columns[0], n.key.seed_lo, n.key.seed_hi, eps);
-        normal4_row_column_fast(noise, columns[1], n.key.seed_lo, n.key.seed_hi, eps + 4);
-        tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(n.bar_acc_empty + 8 * (ti & 1));     // one of the accumulator's 64 items is read
-        finish(lo, hi, eps, scales, table + c8, out);
-        const int jw = w0 + c8;
-        if (row >= n.count || jw >= n.N) continue;
-        // whole sectors (the row pitch is a multiple of 8 floats), scalar stores on the ragged edge
-        float* dst = n.x + static_cast<size_t>(row) * n.ldx + jw;
-        if (jw + 7 < n.N) {
-            store8(dst, out);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (jw + i < n.N) dst[i] = out[i];
-        }
-    }
-}
-
-// x = mean + exp(logvar / 2) * eps; the sample's inverse scale is v_inv.
-__device__ __forceinline__ void emit_finish(const uint32_t (&mean)[8], const uint32_t (&logvar)[8], const float (&eps)[8], float v_inv,
-                                            const float* table, float (&out)[8]) {
-    float b[8], s[8], sd[8];
-    load8(b, table + kBW);
-    load8(s, table + 3 * kBW);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) sd[c] = exp_half_fast(fmaf(__uint_as_float(logvar[c]) * v_inv, s[c], b[c]));
-    load8(b, table);
-    load8(s, table + 2 * kBW);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) out[c] = fmaf(sd[c], eps[c], fmaf(__uint_as_float(mean[c]) * v_inv, s[c], b[c]));
-}
-
-__global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_tc(const __grid_constant__ CUtensorMap map_v,
+__global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__ CUtensorMap map_v,
                                                           const __grid_constant__ CUtensorMap map_w4, EmitArgs a) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -254,7 +218,7 @@ __global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_tc(const __grid_const
     uint8_t* gen = smem_raw + (tiles - raw) + kStages * kStageBytes;
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + 8 * (2 * kStages + 5));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + 8 * (2 * kStages + 5) + 8);
-    float* tables = reinterpret_cast<float*>(gen + 256);
+    float* bias_all = reinterpret_cast<float*>(gen + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles_w = ceil_div(a.N, kBW);
@@ -270,7 +234,7 @@ __global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_tc(const __grid_const
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_acc_full + 8 * b, 1);
-            mbar_init(bar_acc_empty + 8 * b, kItemsPerTile);
+            mbar_init(bar_acc_empty + 8 * b, kEpiWarps);
         }
         mbar_init(bar_drain, 1);
         *abort_flag = 0;
@@ -288,9 +252,6 @@ __global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_tc(const __grid_const
     const uint32_t tmem_base = *tmem_slot;
     dependency_wait();            // the hidden vectors and the device state are an earlier kernel's
     launch_dependents();
-    const int w_first = tile_begin / n_tiles_m;
-    fill_noise_tables(tables, w_first, a.N, a.b4, a.b4 + a.N, a.w_inv, a.w_inv + a.N, a.st->step, a.key);
-    __syncthreads();
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------------------------------------------------
@@ -362,9 +323,37 @@ __global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_tc(const __grid_const
         __syncwarp();
     } else {
         // ---------------- epilogue ---------------------------------------------------------------
-        const NoiseTiles n{a.x, a.ldx, a.N, a.count, a.sample_base, a.key, tables, tile_begin, tile_end, n_tiles_m, w_first, kBM, 0,
-                           tmem_base, bar_acc_full, bar_acc_empty};
-        noise_epilogue<float>(n, warp, lane, abort_flag, a.st, [&](int row) { return row < a.count ? a.v_inv[row] : 0.f; }, emit_finish);
+        const int q = warp & 3, cg = (warp - 2) >> 2;
+        const uint32_t step = a.st->step;
+        float* bias_s = bias_all + (warp - 2) * kTableFloats;
+        int w_staged = -1;
+        uint32_t acc = 0, acc_phase = 0;
+        bool ok = true;
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
+            const int m0 = (t % n_tiles_m) * kBM, w0 = (t / n_tiles_m) * kBW;
+            if (w0 != w_staged) {                       // biases of this warp's 32 workers, read once per worker tile
+                const int j = w0 + cg * 32 + lane;
+                const float bm = j < a.N ? __ldg(a.b4 + j) : 0.f;
+                const float bl = j < a.N ? __ldg(a.b4 + a.N + j) : 0.f;
+                const float sm = j < a.N ? __ldg(a.w_inv + j) : 0.f;
+                const float sl = j < a.N ? __ldg(a.w_inv + a.N + j) : 0.f;
+                __syncwarp();                           // the previous tile's readers are done
+                bias_s[lane] = bm;
+                bias_s[32 + lane] = bl;
+                bias_s[64 + lane] = sm;
+                bias_s[96 + lane] = sl;
+                put_noise_columns(bias_s, w0 + cg * 32, lane, step, a.key);
+                __syncwarp();
+                w_staged = w0;
+            }
+            const int row = m0 + q * 32 + lane;
+            const float v_inv = row < a.count ? a.v_inv[row] : 0.f;      // on its way while the accumulator is waited for
+            ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
+            if (!ok) break;
+            tc_fence_after();
+            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s, v_inv);
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        }
     }
     tc_fence_before();
     __syncthreads();

@@ -11,7 +11,7 @@
 //
 // Roles per CTA: warp 0 loads its operands by TMA (plain per-CTA loads, not multicast; the loads of both CTAs are
 // counted on the leader's "stage full" barrier); warp 1 of the leader (cluster rank 0) issues the MMAs for the
-// pair, warp 1 of the peer tells the leader when the peer's epilogue has emptied an accumulator; warps 2..29 are the
+// pair, warp 1 of the peer tells the leader when the peer's epilogue has emptied an accumulator; warps 2..17 are the
 // epilogue.  The leader's tcgen05.commit arrives on the "stage free" and "accumulator ready" barriers of BOTH CTAs
 // (multicast of the arrive, not of data).  A stage holds two K blocks (64 KB), three stages: with one K block per
 // stage the hand-shake across the pair, not the operand stream, set the pace.  Tensor memory is allocated by each
@@ -72,7 +72,7 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t cta_mask
                  ::"r"(bar), "h"(cta_mask) : "memory");
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kNoiseThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_w4, EmitArgs a) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -86,15 +86,13 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
     uint8_t* gen = smem_raw + (tiles - raw) + kStages2 * kStage2Bytes;
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + 8 * (3 * kStages2 + 5));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + 8 * (3 * kStages2 + 5) + 8);
-    float* tables = reinterpret_cast<float*>(gen + 256);
+    float* bias_all = reinterpret_cast<float*>(gen + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();                          // 0: leader (issues the MMAs), 1: peer
     const int cluster_id = static_cast<int>(blockIdx.x >> 1), n_clusters = static_cast<int>(gridDim.x >> 1);
-    const int n_tiles_m = ceil_div(a.count, 2 * kBM), total_tiles = ceil_div(a.N, kBW) * n_tiles_m;   // a tile: 256 samples (128 per CTA) x 128 workers
-    const int tile_begin = static_cast<int>(static_cast<long long>(total_tiles) * cluster_id / n_clusters);     // consecutive, samples first
-    const int tile_end = static_cast<int>(static_cast<long long>(total_tiles) * (cluster_id + 1) / n_clusters);
-    const int w_first = tile_begin / n_tiles_m;
+    const int n_tiles_w = ceil_div(a.N, kBW);
+    const int total_tiles = n_tiles_w * ceil_div(a.count, 2 * kBM);   // a tile: 256 samples (128 per CTA) x 128 workers
     const int k_blocks = ceil_div(a.H, kBK);
 
     if (threadIdx.x == 0) {
@@ -105,7 +103,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_acc_full + 8 * b, 1);
-            mbar_init(bar_acc_empty + 8 * b, kItemsPerTile);          // this CTA's epilogue
+            mbar_init(bar_acc_empty + 8 * b, kEpiWarps);              // this CTA's epilogue warps
         }
         mbar_init(bar_drain, 1);
         *abort_flag = 0;
@@ -117,7 +115,6 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
                      ::"r"(smem_u32(const_cast<uint32_t*>(tmem_slot))), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    fill_noise_tables(tables, w_first, a.N, a.b4, a.b4 + a.N, a.w_inv, a.w_inv + a.N, a.st->step, a.key);
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();                   // the peer's barriers and tensor memory exist before anything reaches across
@@ -129,8 +126,8 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
         uint32_t stage = 0, phase = 0;
         const uint32_t leader_full = map_to_cta(bar_full, 0u);        // every load of the pair is counted on the leader's barriers
         bool ok = true;
-        for (int t = tile_begin; ok && t < tile_end; ++t) {
-            const int m0 = (t % n_tiles_m) * 2 * kBM + static_cast<int>(rank) * kBM, w0 = (t / n_tiles_m) * kBW;
+        for (int t = cluster_id; ok && t < total_tiles; t += n_clusters) {
+            const int m0 = (t / n_tiles_w) * 2 * kBM + static_cast<int>(rank) * kBM, w0 = (t % n_tiles_w) * kBW;
             const int b_row = rank == 0 ? w0 : a.N + w0;              // mean rows in the leader, log-variance rows in the peer
             for (int kb = 0; kb < k_blocks; kb += kStageK2) {
                 ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, abort_flag, a.st);
@@ -159,7 +156,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
         const uint32_t leader_peer_free = map_to_cta(bar_peer_full, 0u);
-        for (int t = tile_begin; ok && t < tile_end; ++t) {
+        for (int t = cluster_id; ok && t < total_tiles; t += n_clusters) {
             ok = mbar_wait(bar_acc_empty + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             if (lane == 0) mbar_arrive_cluster(leader_peer_free + 8 * acc);
@@ -170,7 +167,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
         // ---------------- leader: MMA issuer for the pair ---------------------------------------------------------
         uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int t = tile_begin; ok && t < tile_end; ++t) {
+        for (int t = cluster_id; ok && t < total_tiles; t += n_clusters) {
             ok = mbar_wait(bar_acc_empty + 8 * acc, acc_phase ^ 1u, abort_flag, a.st) &&
                  mbar_wait(bar_peer_full + 8 * acc, acc_phase ^ 1u, abort_flag, a.st);
             if (!ok) break;
@@ -207,9 +204,37 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
         __syncwarp();
     } else {
         // ---------------- epilogue (both CTAs): this CTA's 128 samples ---------------------------------------------
-        const NoiseTiles n{a.x, a.ldx, a.N, a.count, a.sample_base, a.key, tables, tile_begin, tile_end, n_tiles_m, w_first,
-                           2 * kBM, static_cast<int>(rank) * kBM, tmem_base, bar_acc_full, bar_acc_empty};
-        noise_epilogue<float>(n, warp, lane, abort_flag, a.st, [&](int row) { return row < a.count ? a.v_inv[row] : 0.f; }, emit_finish);
+        const int q = warp & 3, cg = (warp - 2) >> 2;
+        const uint32_t step = a.st->step;
+        float* bias_s = bias_all + (warp - 2) * kTableFloats;
+        int w_staged = -1;
+        uint32_t acc = 0, acc_phase = 0;
+        bool ok = true;
+        for (int t = cluster_id; ok && t < total_tiles; t += n_clusters) {
+            const int m0 = (t / n_tiles_w) * 2 * kBM + static_cast<int>(rank) * kBM, w0 = (t % n_tiles_w) * kBW;
+            if (w0 != w_staged) {
+                const int j = w0 + cg * 32 + lane;
+                const float bm = j < a.N ? __ldg(a.b4 + j) : 0.f;
+                const float bl = j < a.N ? __ldg(a.b4 + a.N + j) : 0.f;
+                const float sm = j < a.N ? __ldg(a.w_inv + j) : 0.f;
+                const float sl = j < a.N ? __ldg(a.w_inv + a.N + j) : 0.f;
+                __syncwarp();
+                bias_s[lane] = bm;
+                bias_s[32 + lane] = bl;
+                bias_s[64 + lane] = sm;
+                bias_s[96 + lane] = sl;
+                put_noise_columns(bias_s, w0 + cg * 32, lane, step, a.key);
+                __syncwarp();
+                w_staged = w0;
+            }
+            const int row = m0 + q * 32 + lane;
+            const float v_inv = row < a.count ? a.v_inv[row] : 0.f;
+            ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
+            if (!ok) break;
+            tc_fence_after();
+            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s, v_inv);
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        }
     }
     tc_fence_before();
     __syncthreads();

@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_relu_tc(const __grid_const
     } else {
         // ---------------- epilogue ---------------------------------------------------------------
         const int q = warp & 3, cg = (warp - 2) >> 2;
-        float* bias_s = bias_all + (warp - 2) * 128;
+        float* bias_s = bias_all + (warp - 2) * kTableFloats;
         int w_staged = -1;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
@@ -263,21 +263,27 @@ struct EmitDualArgs {
     int count, N, H, ldx;
 };
 
-// x = I + softplus(scale) * eps; the sample's inverse scales are those of u and r.
-__device__ __forceinline__ void dual_finish(const uint32_t (&mean)[8], const uint32_t (&scale)[8], const float (&eps)[8], float2 inv,
-                                            const float* table, float (&out)[8]) {
-    float b[8], s[8], sd[8];
-    load8(b, table + kBW);
-    load8(s, table + 3 * kBW);
+// x = I + softplus(scale) * eps
+__device__ __forceinline__ void dual_epilogue_tile(const EmitDualArgs& a, uint32_t tmem_base, uint32_t acc, int q, int cg,
+                                                   int lane, int m0, int w0, uint32_t bar_acc_empty,
+                                                   const float* bias_s, float u_inv, float r_inv) {
+    const int row = m0 + q * 32 + lane;
+    noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, bias_s,
+                        tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32, w0 + cg * 32, lane, bar_acc_empty + 8 * acc,
+                        [&](const uint32_t (&mean)[8], const uint32_t (&scale)[8], const float (&eps)[8], int c8, float (&out)[8]) {
+        float bm[8], bs[8], im[8], is[8];
+        load8(bm, bias_s + c8);
+        load8(bs, bias_s + 32 + c8);
+        load8(im, bias_s + 64 + c8);
+        load8(is, bias_s + 96 + c8);
 #pragma unroll
-    for (int c = 0; c < 8; ++c) sd[c] = softplus_fast(fmaf(__uint_as_float(scale[c]) * inv.y, s[c], b[c]));
-    load8(b, table);
-    load8(s, table + 2 * kBW);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) out[c] = fmaf(sd[c], eps[c], fmaf(__uint_as_float(mean[c]) * inv.x, s[c], b[c]));
+        for (int c = 0; c < 8; ++c)
+            out[c] = fmaf(softplus_fast(fmaf(__uint_as_float(scale[c]) * r_inv, is[c], bs[c])), eps[c],
+                          fmaf(__uint_as_float(mean[c]) * u_inv, im[c], bm[c]));
+    });
 }
 
-__global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_dual_tc(const __grid_constant__ CUtensorMap map_u,
+__global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_constant__ CUtensorMap map_u,
                                                                const __grid_constant__ CUtensorMap map_r,
                                                                const __grid_constant__ CUtensorMap map_wi2,
                                                                const __grid_constant__ CUtensorMap map_wj2, EmitDualArgs a) {
@@ -292,7 +298,7 @@ __global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_dual_tc(const __grid_
     uint8_t* gen = smem_raw + (tiles - raw) + kDualStages * kDualStageBytes;
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gen + 8 * (2 * kDualStages + 5));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + 8 * (2 * kDualStages + 5) + 8);
-    float* tables = reinterpret_cast<float*>(gen + 256);
+    float* bias_all = reinterpret_cast<float*>(gen + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles_w = ceil_div(a.N, kBW);
@@ -308,7 +314,7 @@ __global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_dual_tc(const __grid_
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_acc_full + 8 * b, 1);
-            mbar_init(bar_acc_empty + 8 * b, kItemsPerTile);
+            mbar_init(bar_acc_empty + 8 * b, kEpiWarps);
         }
         mbar_init(bar_drain, 1);
         *abort_flag = 0;
@@ -326,9 +332,6 @@ __global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_dual_tc(const __grid_
     const uint32_t tmem_base = *tmem_slot;
     dependency_wait();            // the operands and the device state are an earlier kernel's
     launch_dependents();
-    const int w_first = tile_begin / n_tiles_m;
-    fill_noise_tables(tables, w_first, a.N, a.bias_mean, a.bias_scale, a.wi_inv, a.wj_inv, a.st->step, a.key);
-    __syncthreads();
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------------------------------------------------
@@ -401,10 +404,37 @@ __global__ void __launch_bounds__(kNoiseThreads, 1) k_emit_dual_tc(const __grid_
         __syncwarp();
     } else {
         // ---------------- epilogue ---------------------------------------------------------------
-        const NoiseTiles n{a.x, a.ldx, a.N, a.count, a.sample_base, a.key, tables, tile_begin, tile_end, n_tiles_m, w_first, kBM, 0,
-                           tmem_base, bar_acc_full, bar_acc_empty};
-        noise_epilogue<float2>(n, warp, lane, abort_flag, a.st,
-                               [&](int row) { return row < a.count ? make_float2(a.u_inv[row], a.r_inv[row]) : make_float2(0.f, 0.f); }, dual_finish);
+        const int q = warp & 3, cg = (warp - 2) >> 2;
+        const uint32_t step = a.st->step;
+        float* bias_s = bias_all + (warp - 2) * kTableFloats;
+        int w_staged = -1;
+        uint32_t acc = 0, acc_phase = 0;
+        bool ok = true;
+        for (int t = tile_begin; ok && t < tile_end; ++t) {
+            const int m0 = (t % n_tiles_m) * kBM, w0 = (t / n_tiles_m) * kBW;
+            if (w0 != w_staged) {                       // biases of this warp's 32 workers, read once per worker tile
+                const int j = w0 + cg * 32 + lane;
+                const float bm = j < a.N ? __ldg(a.bias_mean + j) : 0.f;
+                const float bs = j < a.N ? __ldg(a.bias_scale + j) : 0.f;
+                const float im = j < a.N ? __ldg(a.wi_inv + j) : 0.f;
+                const float is = j < a.N ? __ldg(a.wj_inv + j) : 0.f;
+                __syncwarp();
+                bias_s[lane] = bm;
+                bias_s[32 + lane] = bs;
+                bias_s[64 + lane] = im;
+                bias_s[96 + lane] = is;
+                put_noise_columns(bias_s, w0 + cg * 32, lane, step, a.key);
+                __syncwarp();
+                w_staged = w0;
+            }
+            const int row = m0 + q * 32 + lane;
+            const float u_inv = row < a.count ? a.u_inv[row] : 0.f, r_inv = row < a.count ? a.r_inv[row] : 0.f;
+            ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
+            if (!ok) break;
+            tc_fence_after();
+            dual_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s, u_inv, r_inv);
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        }
     }
     tc_fence_before();
     __syncthreads();
