@@ -90,6 +90,7 @@ struct cutoff_ctx {
     __half* d_r16 = nullptr;        // [alloc_rows][ldh]  the same as an operand; tensor-core path
     float* d_r_inv = nullptr;       // [alloc_rows]
     float* d_Wj1p = nullptr;        // [H][ldx]           Wj1 with rows padded with zeros to ldx; fp32 path only
+    float* d_M = nullptr;           // [H][H]             M, before it becomes rows of d_w16
     float* d_Mb = nullptr;          // [H]                b' = Wj1 bi2 + bj1 (tensor-core path: Wj1 I + bj1 = M u + b' with M = Wj1 Wi2)
     CUtensorMap map_r{};            // TMA view of d_r [alloc_rows][H]
     CUtensorMap map_wi2{}, map_M{}, map_wj2{};
@@ -218,17 +219,10 @@ void put_second_layer(float* tiles, const float* w, size_t out_rows, size_t H, s
             for (size_t jj = 0; jj < 32; ++jj) tiles[kb * block_rows * 32 + swz(o, jj)] = host_tf32(w[o * H + kb * 32 + jj]);
 }
 
-// A weight matrix [rows][cols], already rounded to at most 11 significant bits, as halves with a power of two per row.
-void half_rows(const float* w, size_t rows, size_t cols, size_t ld, __half* out, float* inv) {
-    for (size_t r = 0; r < rows; ++r) {
-        float big = 0.0f;
-        for (size_t k = 0; k < cols; ++k) big = std::fmax(big, std::fabs(w[r * cols + k]));
-        uint32_t bits;
-        std::memcpy(&bits, &big, 4);
-        const int e = big > 0.0f ? half_exponent(bits) : 0;
-        for (size_t k = 0; k < ld; ++k) out[r * ld + k] = __float2half_rn(k < cols ? std::ldexp(w[r * cols + k], e) : 0.0f);
-        inv[r] = std::ldexp(1.0f, -e);
-    }
+// `rows` rows of weights w [rows][H] on the device, already rounded to at most 11 significant bits, into the half-precision
+// operand from its row `row0` on.
+void half_rows(cutoff_ctx* c, const float* w, int rows, int row0) {
+    k_half_rows<<<ceil_div(rows, 8), 256, 0, c->stream>>>(w, rows, c->H, c->ldh, c->d_w16 + static_cast<size_t>(row0) * c->ldh, c->d_w_inv + row0);
 }
 
 // |A x + b| <= slope * max |x| + offset, from the matrix as the tensor cores see it (rounded up a little)
@@ -268,7 +262,7 @@ int next_pow2(int n) {
 }
 
 void free_all(cutoff_ctx* c) {
-    cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_Mb);
+    cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_Mb); cudaFree(c->d_M);
     cudaFree(c->d_v16); cudaFree(c->d_v_inv); cudaFree(c->d_w16); cudaFree(c->d_w_inv); cudaFree(c->d_r16); cudaFree(c->d_r_inv);
     cudaFree(c->d_blob); cudaFree(c->d_WT); cudaFree(c->d_WhR); cudaFree(c->d_chain_image);
     if (c->h_mask) cudaFreeHost(c->h_mask); cudaFree(c->d_ring); cudaFree(c->d_stage);
@@ -556,7 +550,7 @@ void launch_emission_literal(cutoff_ctx* c, uint32_t sample_base, int count) {
         e.wi_inv = c->d_w_inv; e.wj_inv = c->d_w_inv + c->N; e.x = c->d_x; e.st = c->d_state; e.key = key;
         e.sample_base = sample_base; e.count = count; e.N = c->N; e.H = c->H; e.ldx = c->ldx;
         const int tiles = ceil_div(c->N, tc::kBW) * ceil_div(count, tc::kBM);
-        launch_dependent(tc::k_emit_dual_tc, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kThreads), tc::kDualSmemBytes, c->stream,
+        launch_dependent(tc::k_emit_dual_tc, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kThreads), tc::kSmemBytes, c->stream,
                          c->map_v, c->map_r, c->map_wi2, c->map_wj2, e);
         c->launches += 1;
         return;
@@ -757,7 +751,7 @@ cudaError_t set_kernel_attributes(const cutoff_ctx* c) {
     e = allow_smem(tc::k_emit_tc, tc::kSmemBytes);
     if (e == cudaSuccess) e = allow_smem(tc::k_emit_tc2, tc::kSmem2Bytes);
     if (e == cudaSuccess) e = allow_smem(tc::k_gemm_relu_tc, tc::kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(tc::k_emit_dual_tc, tc::kDualSmemBytes);
+    if (e == cudaSuccess) e = allow_smem(tc::k_emit_dual_tc, tc::kSmemBytes);
     if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<false>, 227 * 1024);
     if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<true>, 227 * 1024);
     if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc32<false>, 227 * 1024);
@@ -862,6 +856,7 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
             CREATE_CHECK(cudaMalloc(&c->d_r16, sizeof(__half) * static_cast<size_t>(c->alloc_rows) * c->ldh));
             CREATE_CHECK(cudaMalloc(&c->d_r_inv, sizeof(float) * c->alloc_rows));
             CREATE_CHECK(cudaMalloc(&c->d_Mb, sizeof(float) * c->H));
+            CREATE_CHECK(cudaMalloc(&c->d_M, sizeof(float) * c->H * c->H));
         } else {
             CREATE_CHECK(cudaMalloc(&c->d_r, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->H));
             CREATE_CHECK(cudaMalloc(&c->d_I, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->ldx));
@@ -991,16 +986,15 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         }
     }
     CU_CHECK(c, cudaMemcpy(c->d_blob, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice));
-    std::vector<__half> w16(c->use_tc ? (2 * static_cast<size_t>(c->N) + (c->literal ? c->H : 0)) * c->ldh : 0);
-    std::vector<float> w_inv(c->use_tc ? 2 * static_cast<size_t>(c->N) + (c->literal ? c->H : 0) : 0);
     if (c->use_tc) {
-        const size_t N = c->N, H = c->H, D = c->D, ld = c->ldh;
+        const int N = c->N, H = c->H, D = c->D;
         if (c->literal) {
-            half_rows(host.data() + off[29], N, H, ld, w16.data(), w_inv.data());                         // Wi2
-            half_rows(host.data() + off[33], N, H, ld, w16.data() + N * ld, w_inv.data() + N);            // Wj2
+            half_rows(c, c->d_blob + off[29], N, 0);                                                     // Wi2
+            half_rows(c, c->d_blob + off[33], N, N);                                                     // Wj2
         } else {
-            half_rows(host.data() + off[21], 2 * N, H, ld, w16.data(), w_inv.data());                     // W4
+            half_rows(c, c->d_blob + off[21], 2 * N, 0);                                                 // W4
         }
+        CU_CHECK(c, cudaGetLastError());
         const size_t first = c->literal ? 27 : 19;                                                       // Wi1 or W3, and its bias
         layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, c->v_slope, c->v_offset);
     }
@@ -1118,11 +1112,11 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                 for (size_t j = 0; j < H; ++j) big_m[i * H + j] = host_tf32(static_cast<float>(acc[j]));
                 mb[i] = static_cast<float>(bacc);
             }
-            half_rows(big_m.data(), H, H, c->ldh, w16.data() + 2 * N * c->ldh, w_inv.data() + 2 * N);
             layer_bound(big_m.data(), mb.data(), H, H, c->r_slope, c->r_offset);
             CU_CHECK(c, cudaMemcpy(c->d_Mb, mb.data(), mb.size() * sizeof(float), cudaMemcpyHostToDevice));
-            CU_CHECK(c, cudaMemcpy(c->d_w16, w16.data(), w16.size() * sizeof(__half), cudaMemcpyHostToDevice));
-            CU_CHECK(c, cudaMemcpy(c->d_w_inv, w_inv.data(), w_inv.size() * sizeof(float), cudaMemcpyHostToDevice));
+            CU_CHECK(c, cudaMemcpy(c->d_M, big_m.data(), big_m.size() * sizeof(float), cudaMemcpyHostToDevice));
+            half_rows(c, c->d_M, c->H, 2 * c->N);
+            CU_CHECK(c, cudaGetLastError());
         } else {
             // Wj1 [H][N] with rows padded with zeros to ldx floats (rows then start on 32 bytes for any N)
             std::vector<float> wj1p(H * static_cast<size_t>(c->ldx), 0.0f);
@@ -1145,10 +1139,6 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
     }
     m.W1T = c->d_WT + H * D; m.b1 = b + off[16]; m.W2 = b + off[17]; m.b2 = b + off[18];
     m.W3T = c->d_WT + 2 * H * D; m.b3 = b + off[20]; m.W4 = b + off[21]; m.b4 = b + off[22];
-    if (c->use_tc) {
-        CU_CHECK(c, cudaMemcpy(c->d_w16, w16.data(), w16.size() * sizeof(__half), cudaMemcpyHostToDevice));
-        CU_CHECK(c, cudaMemcpy(c->d_w_inv, w_inv.data(), w_inv.size() * sizeof(float), cudaMemcpyHostToDevice));
-    }
     c->weights_loaded = true;
     c->proj_stale = true;
     return CUTOFF_OK;

@@ -1,7 +1,7 @@
 // The emission output layer of emit_tc.cuh on pairs of SMs: one UMMA of shape M=256, N=256, K=16
 // (tcgen05.mma.cta_group::2) spans a cluster of two CTAs.  Opt-in (option "pair_emission").
 //
-// The one-SM kernel streams 48 KB of operands from L2 into shared memory per K block for every 128 x 128 output
+// Streamed, the one-SM kernel moves 48 KB of operands from L2 into shared memory per K block for every 128 x 128 output
 // tile (16 KB of hidden vectors, 32 KB of weights).  Here the two CTAs of a cluster take the same 128 workers for
 // two neighbouring blocks of 128 samples.  Each CTA loads its own 128 hidden vectors (A: the instruction reads
 // rows 0..127 from the leader's shared memory and rows 128..255 from its peer's) and only HALF of the weight tile
@@ -17,9 +17,9 @@
 // stage the hand-shake across the pair, not the operand stream, set the pace.  Tensor memory is allocated by each
 // CTA for itself (all 512 columns, so both start at column 0).  Every wait is bounded as in emit_tc.cuh.
 //
-// Measured at N=1024, S=65536: 0.177 ms against 0.148 ms of the one-SM kernel (0.235 ms with one K block per
-// stage); tensor pipe 27 % active.  The operand stream shrinks as planned (L2 throughput 41 % against 59 %), but
-// a K=8 tf32 instruction is short and every stage now costs a round trip between two SMs.  Hence opt-in.
+// Measured with four-byte operands, at N=1024, S=65536: 0.177 ms against 0.148 ms of the one-SM kernel (0.235 ms with one
+// K block per stage); tensor pipe 27 % active, L2 throughput 41 % against 59 %.  Since then the one-SM kernel keeps the weights
+// in shared memory, so that the half of the stream that this kernel saves is no longer streamed there.  Hence opt-in.
 #pragma once
 #include "emit_tc.cuh"
 
@@ -213,17 +213,8 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
         for (int t = cluster_id; ok && t < total_tiles; t += n_clusters) {
             const int m0 = (t / n_tiles_w) * 2 * kBM + static_cast<int>(rank) * kBM, w0 = (t % n_tiles_w) * kBW;
             if (w0 != w_staged) {
-                const int j = w0 + cg * 32 + lane;
-                const float bm = j < a.N ? __ldg(a.b4 + j) : 0.f;
-                const float bl = j < a.N ? __ldg(a.b4 + a.N + j) : 0.f;
-                const float sm = j < a.N ? __ldg(a.w_inv + j) : 0.f;
-                const float sl = j < a.N ? __ldg(a.w_inv + a.N + j) : 0.f;
                 __syncwarp();
-                bias_s[lane] = bm;
-                bias_s[32 + lane] = bl;
-                bias_s[64 + lane] = sm;
-                bias_s[96 + lane] = sl;
-                put_noise_columns(bias_s, w0 + cg * 32, lane, step, a.key);
+                stage_emission_tables(a, bias_s, w0 + cg * 32, lane, step);
                 __syncwarp();
                 w_staged = w0;
             }
@@ -232,7 +223,8 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
             ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, a.st);
             if (!ok) break;
             tc_fence_after();
-            emit_epilogue_tile(a, tmem_base, acc, q, cg, lane, m0, w0, bar_acc_empty, bias_s, v_inv);
+            emit_epilogue_tile(a, tmem_base + (static_cast<uint32_t>(q * 32) << 16) + acc * kAccCols + cg * 32, row, w0 + cg * 32, lane,
+                               bar_acc_empty + 8 * acc, bias_s, v_inv);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }

@@ -34,6 +34,21 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
     return r;
 }
 
+// Rows of `cols` weights into rows of `ld` halves with a power of two per row, one warp per row (when weights are loaded).
+// Entries from cols on are zeros.
+__global__ void k_half_rows(const float* __restrict__ w, int rows, int cols, int ld, __half* __restrict__ out, float* __restrict__ inv_scale) {
+    const int row = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (row >= rows) return;
+    const float* src = w + static_cast<size_t>(row) * cols;
+    uint32_t big = 0;                                       // bit pattern of the largest magnitude
+    for (int k = lane; k < cols; k += 32) big = max(big, __float_as_uint(src[k]) & 0x7fffffffu);
+    big = __reduce_max_sync(0xffffffffu, big);
+    const int e = big ? half_exponent(big) : 0;
+    const float scale = __uint_as_float(pow2_bits(e));
+    for (int k = lane; k < ld; k += 32) out[static_cast<size_t>(row) * ld + k] = __float2half_rn(k < cols ? src[k] * scale : 0.0f);
+    if (lane == 0) inv_scale[row] = __uint_as_float(pow2_bits(-e));
+}
+
 // A hidden vector as the emission products read it: halves with a row pitch of whole 16 bytes, one inverse scale per row,
 // and the bound of a row's entries, |entry| <= slope * (largest |input|) + offset.
 struct HalfRows {
