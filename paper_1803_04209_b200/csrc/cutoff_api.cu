@@ -90,6 +90,7 @@ struct cutoff_ctx {
     __half* d_r16 = nullptr;        // [alloc_rows][ldh]  the same as an operand; tensor-core path
     float* d_r_inv = nullptr;       // [alloc_rows]
     float* d_Wj1p = nullptr;        // [H][ldx]           Wj1 with rows padded with zeros to ldx; fp32 path only
+    float* d_W4T = nullptr;         // [H][2][ldx]        fp32 compact path: W4 with the columns of both heads contiguous
     float* d_M = nullptr;           // [H][H]             M, before it becomes rows of d_w16
     float* d_Mb = nullptr;          // [H]                b' = Wj1 bi2 + bj1 (tensor-core path: Wj1 I + bj1 = M u + b' with M = Wj1 Wi2)
     CUtensorMap map_r{};            // TMA view of d_r [alloc_rows][H]
@@ -225,6 +226,13 @@ void half_rows(cutoff_ctx* c, const float* w, int rows, int row0) {
     k_half_rows<<<ceil_div(rows, 8), 256, 0, c->stream>>>(w, rows, c->H, c->ldh, c->d_w16 + static_cast<size_t>(row0) * c->ldh, c->d_w_inv + row0);
 }
 
+// A copy from pageable memory that has arrived when this returns: cudaMemcpy may return while its last part is under way, and
+// the contexts' streams do not wait for the default stream.
+cudaError_t upload(void* dst, const void* src, size_t bytes) {
+    const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
+
 // |A x + b| <= slope * max |x| + offset, from the matrix as the tensor cores see it (rounded up a little)
 void layer_bound(const float* w, const float* b, size_t rows, size_t cols, float& slope, float& offset) {
     double l1 = 0.0, mb = 0.0;
@@ -262,7 +270,7 @@ int next_pow2(int n) {
 }
 
 void free_all(cutoff_ctx* c) {
-    cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_Mb); cudaFree(c->d_M);
+    cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_Mb); cudaFree(c->d_M); cudaFree(c->d_W4T);
     cudaFree(c->d_v16); cudaFree(c->d_v_inv); cudaFree(c->d_w16); cudaFree(c->d_w_inv); cudaFree(c->d_r16); cudaFree(c->d_r_inv);
     cudaFree(c->d_blob); cudaFree(c->d_WT); cudaFree(c->d_WhR); cudaFree(c->d_chain_image);
     if (c->h_mask) cudaFreeHost(c->h_mask); cudaFree(c->d_ring); cudaFree(c->d_stage);
@@ -559,13 +567,13 @@ void launch_emission_literal(cutoff_ctx* c, uint32_t sample_base, int count) {
     a.st = c->d_state; a.key = key; a.sample_base = sample_base; a.M = count;
     a.A = c->d_v; a.lda = c->H; a.B = l.Wi2; a.ldb = c->H; a.bias = l.bi2; a.out = c->d_I; a.ld_out = c->ldx;
     a.Nout = c->N; a.K = c->H;
-    launch_dependent(k_gemm_fma<kEpiAffine>, dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), dim3(kEmitThreads), 0, c->stream, a);
+    launch_dependent(k_gemm_fma<kEpiAffine>, dim3(ceil_div(a.Nout, kGemmTN), ceil_div(count, kGemmTM)), dim3(kGemmThreads), 0, c->stream, a);
     a.A = c->d_I; a.lda = c->ldx; a.B = l.Wj1; a.ldb = l.ldn; a.bias = l.bj1; a.out = c->d_r; a.ld_out = c->H;
     a.Nout = c->H; a.K = c->ldx;                                   // the padding columns of both operands are zero
-    launch_dependent(k_gemm_fma<kEpiRelu>, dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), dim3(kEmitThreads), 0, c->stream, a);
+    launch_dependent(k_gemm_fma<kEpiRelu>, dim3(ceil_div(a.Nout, kGemmTN), ceil_div(count, kGemmTM)), dim3(kGemmThreads), 0, c->stream, a);
     a.A = c->d_r; a.lda = c->H; a.B = l.Wj2; a.ldb = c->H; a.bias = l.bj2; a.add = c->d_I; a.out = c->d_x; a.ld_out = c->ldx;
     a.Nout = c->N; a.K = c->H;
-    launch_dependent(k_gemm_fma<kEpiScaleNoise>, dim3(ceil_div(a.Nout, kEmitTN), ceil_div(count, kEmitTM)), dim3(kEmitThreads), 0, c->stream, a);
+    launch_dependent(k_gemm_fma<kEpiScaleNoise>, dim3(ceil_div(a.Nout, kGemmTN), ceil_div(count, kGemmTM)), dim3(kGemmThreads), 0, c->stream, a);
     c->launches += 3;
 }
 
@@ -573,8 +581,15 @@ void launch_emission(cutoff_ctx* c, uint32_t sample_base, int count) {
     if (c->literal) { launch_emission_literal(c, sample_base, count); return; }
     if (c->use_tc) { launch_emission_tc(c, sample_base, count); return; }
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
-    dim3 grid(ceil_div(c->N, kEmitTN), ceil_div(count, kEmitTM));
-    launch_dependent(k_emit_fma, grid, dim3(kEmitThreads), 0, c->stream, c->m, c->d_v, c->d_state, key, sample_base, count, c->d_x, c->ldx);
+    // 32 samples per CTA read the weights four times less often than 8 do, but need enough samples to occupy the GPU: at N=158, S=2048
+    // (192 large tiles) the small ones take 10.3 us
+    const int worker_tiles = ceil_div(c->N, kEmitTN), large = worker_tiles * ceil_div(count, 32);
+    if (large >= 2 * c->sm_count)
+        launch_dependent(k_emit_fma<8>, dim3(large), dim3(kEmitThreads), 0, c->stream, c->m, c->d_v, c->d_W4T, c->ldx, c->d_state, key, sample_base, count,
+                         c->d_x, c->ldx);
+    else
+        launch_dependent(k_emit_fma<2>, dim3(worker_tiles * ceil_div(count, 8)), dim3(kEmitThreads), 0, c->stream, c->m, c->d_v, c->d_W4T, c->ldx, c->d_state,
+                         key, sample_base, count, c->d_x, c->ldx);
     c->launches += 1;
 }
 
@@ -884,6 +899,7 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
         CREATE_CHECK(cudaMalloc(&c->d_w_inv, sizeof(float) * w_rows));
     } else {
         CREATE_CHECK(cudaMalloc(&c->d_v, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->H));
+        if (!c->literal) CREATE_CHECK(cudaMalloc(&c->d_W4T, sizeof(float) * 2 * static_cast<size_t>(c->H) * c->ldx));
     }
     CREATE_CHECK(cudaMalloc(&c->d_x, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->ldx));
     CREATE_CHECK(cudaMalloc(&c->d_partial, sizeof(float) * 2 * static_cast<size_t>(kPartialRows) * c->N));
@@ -985,7 +1001,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
             }
         }
     }
-    CU_CHECK(c, cudaMemcpy(c->d_blob, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice));
+    CU_CHECK(c, upload(c->d_blob, host.data(), host.size() * sizeof(float)));
     if (c->use_tc) {
         const int N = c->N, H = c->H, D = c->D;
         if (c->literal) {
@@ -998,6 +1014,10 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         const size_t first = c->literal ? 27 : 19;                                                       // Wi1 or W3, and its bias
         layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, c->v_slope, c->v_offset);
     }
+    if (!c->use_tc && !c->literal) {
+        k_transpose_heads<<<dim3(ceil_div(c->ldx, 32), ceil_div(c->H, 32), 2), dim3(32, 8), 0, c->stream>>>(c->d_blob + off[21], c->N, c->H, c->ldx, c->d_W4T);
+        CU_CHECK(c, cudaGetLastError());
+    }
     // transposed copies [D][H] of the latent-to-hidden matrices for the per-sample chain
     const size_t D = c->D, H = c->H;
     const int n_transposed = c->literal ? 4 : 3;
@@ -1008,7 +1028,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         for (size_t i = 0; i < H; ++i)
             for (size_t d = 0; d < D; ++d) wT[t * H * D + d * H + i] = w[i * D + d];
     }
-    CU_CHECK(c, cudaMemcpy(c->d_WT, wT.data(), wT.size() * sizeof(float), cudaMemcpyHostToDevice));
+    CU_CHECK(c, upload(c->d_WT, wT.data(), wT.size() * sizeof(float)));
 
     if (H == 32 || H == 64 || H == 128) {
         // recurrence matrices regrouped per thread of k_enc_rnn_resident (the widths that kernel serves; the layout
@@ -1023,7 +1043,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                     for (size_t j = 0; j < HQ; ++j)
                         whr[dir * H * H + ((j / 4) * T + (4 * i + q)) * 4 + (j % 4)] = w[i * H + q * HQ + j];
         }
-        CU_CHECK(c, cudaMemcpy(c->d_WhR, whr.data(), whr.size() * sizeof(float), cudaMemcpyHostToDevice));
+        CU_CHECK(c, upload(c->d_WhR, whr.data(), whr.size() * sizeof(float)));
     }
     // Operand tiles of the tensor-core chain kernels as they will sit in shared memory: tf32 (nearest, ties away),
     // K-major rows of 32 values, 16-byte chunks XOR-swizzled with the row index modulo 8.
@@ -1079,7 +1099,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                 put_second_layer(img.data() + 5 * tile, wc + 32 * H, 32, H, 32);
             }
         }
-        CU_CHECK(c, cudaMemcpy(c->d_chain_image, img.data(), img.size() * sizeof(float), cudaMemcpyHostToDevice));
+        CU_CHECK(c, upload(c->d_chain_image, img.data(), img.size() * sizeof(float)));
     }
 
     ModelDev& m = c->m;
@@ -1113,8 +1133,8 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                 mb[i] = static_cast<float>(bacc);
             }
             layer_bound(big_m.data(), mb.data(), H, H, c->r_slope, c->r_offset);
-            CU_CHECK(c, cudaMemcpy(c->d_Mb, mb.data(), mb.size() * sizeof(float), cudaMemcpyHostToDevice));
-            CU_CHECK(c, cudaMemcpy(c->d_M, big_m.data(), big_m.size() * sizeof(float), cudaMemcpyHostToDevice));
+            CU_CHECK(c, upload(c->d_Mb, mb.data(), mb.size() * sizeof(float)));
+            CU_CHECK(c, upload(c->d_M, big_m.data(), big_m.size() * sizeof(float)));
             half_rows(c, c->d_M, c->H, 2 * c->N);
             CU_CHECK(c, cudaGetLastError());
         } else {
@@ -1122,7 +1142,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
             std::vector<float> wj1p(H * static_cast<size_t>(c->ldx), 0.0f);
             for (size_t i = 0; i < H; ++i)
                 std::memcpy(wj1p.data() + i * c->ldx, host.data() + off[31] + i * c->N, sizeof(float) * c->N);
-            CU_CHECK(c, cudaMemcpy(c->d_Wj1p, wj1p.data(), wj1p.size() * sizeof(float), cudaMemcpyHostToDevice));
+            CU_CHECK(c, upload(c->d_Wj1p, wj1p.data(), wj1p.size() * sizeof(float)));
         }
         LiteralDev& l = c->lit;
         l.Wg1T = c->d_WT + H * D; l.bg1 = b + off[16]; l.Wg2 = b + off[17]; l.bg2 = b + off[18];
@@ -1620,9 +1640,8 @@ int cutoff_restore_state(cutoff_ctx* c, const void* buf, size_t nbytes) {
     DeviceGuard guard(c->cfg.device);
     CU_CHECK(c, guard.err);
     CU_CHECK(c, cudaStreamSynchronize(c->stream));
-    CU_CHECK(c, cudaMemcpy(c->d_state, &s, sizeof(DevState), cudaMemcpyHostToDevice));
-    CU_CHECK(c, cudaMemcpy(c->d_ring, p + sizeof(hdr) + sizeof(DevState), sizeof(float) * c->W * c->N,
-                           cudaMemcpyHostToDevice));
+    CU_CHECK(c, upload(c->d_state, &s, sizeof(DevState)));
+    CU_CHECK(c, upload(c->d_ring, p + sizeof(hdr) + sizeof(DevState), sizeof(float) * c->W * c->N));
     c->pushes = s.push_count;
     c->pending = false;
     c->partial_pending = false;

@@ -183,12 +183,14 @@ struct GemmFmaArgs {
     uint32_t sample_base;
 };
 
+constexpr int kGemmTM = 64, kGemmTN = 64, kGemmTK = 16, kGemmThreads = 256;
+
 template <int EPI>
-__global__ void __launch_bounds__(kEmitThreads) k_gemm_fma(GemmFmaArgs a) {
-    __shared__ __align__(16) float As[kEmitTK][kEmitTM + 4];
-    __shared__ __align__(16) float Bs[kEmitTK][kEmitTN + 4];
+__global__ void __launch_bounds__(kGemmThreads) k_gemm_fma(GemmFmaArgs a) {
+    __shared__ __align__(16) float As[kGemmTK][kGemmTM + 4];
+    __shared__ __align__(16) float Bs[kGemmTK][kGemmTN + 4];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int row0 = blockIdx.y * kEmitTM, j0 = blockIdx.x * kEmitTN;
+    const int row0 = blockIdx.y * kGemmTM, j0 = blockIdx.x * kGemmTN;
     float acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(kEmitThreads) k_gemm_fma(GemmFmaArgs a) {
     const int lr = tid >> 2, lc = (tid & 3) * 4;
     dependency_wait();
     launch_dependents();
-    for (int kk = 0; kk < a.K; kk += kEmitTK) {
+    for (int kk = 0; kk < a.K; kk += kGemmTK) {
         float4 av = make_float4(0.f, 0.f, 0.f, 0.f), bv = av;
         if (kk + lc < a.K) {
             if (row0 + lr < a.M) av = *reinterpret_cast<const float4*>(a.A + static_cast<size_t>(row0 + lr) * a.lda + kk + lc);
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(kEmitThreads) k_gemm_fma(GemmFmaArgs a) {
         Bs[lc + 0][lr] = bv.x; Bs[lc + 1][lr] = bv.y; Bs[lc + 2][lr] = bv.z; Bs[lc + 3][lr] = bv.w;
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < kEmitTK; ++k) {
+        for (int k = 0; k < kGemmTK; ++k) {
             const float4 a4 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
             const float4 b4 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
             const float ar[4] = {a4.x, a4.y, a4.z, a4.w};

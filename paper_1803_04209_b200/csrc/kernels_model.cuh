@@ -4,6 +4,7 @@
 #include "common.cuh"
 #include "half_operand.cuh"
 #include "rng.cuh"
+#include "tile_product.cuh"
 
 namespace cutoff {
 
@@ -795,79 +796,141 @@ k_chain_resident(ModelDev m, const float* __restrict__ hlr, const DevState* __re
 // ---------------------------------------------------------------------------------------------
 // Emission output layer in fp32 FMA, with the noise drawn in the epilogue:
 //   [mean | logvar] = W4 v + b4,   x_j = mean_j + exp(logvar_j / 2) * eps_j.
-// 64 samples x 64 workers per CTA, 4 x 4 (x 2 heads) per thread.
+// 4 RM samples x 64 workers per CTA of 64 threads; a thread has RM samples x 4 consecutive workers, both heads, so that one
+// generator call serves its four draws.  What bounds it is the issue of instructions: 64 multiply-adds per thread and k went through
+// with 62 % of the slots taken.  Hence two columns per instruction (their sums are the same two chains), operands by asynchronous
+// copies, and the weights with their columns contiguous (k_transpose_heads), so that a pair of columns is a pair of registers.
+// N=128, H=128, S=16384: 50 us with 4 x 4 x 2 results per thread of 256 and copies through registers, 52 us with 8 x 8 and single
+// multiply-adds, 41 us as it is (multiply-adds alone, at the measured rate: 19 us; the draws' log, sin, cos and exp most of the rest).
+// RM = 8 where that makes two CTAs per SM, else RM = 2: N=16, S=1024: 7.0 -> 4.5 us.  The decisions: N=128 105 -> 101 us, N=16 39.5 -> 37.4 us.
 // ---------------------------------------------------------------------------------------------
-constexpr int kEmitTM = 64, kEmitTN = 64, kEmitTK = 16, kEmitThreads = 256;
+constexpr int kEmitThreads = 64, kEmitTN = 64, kEmitTK = 8, kEmitSlabs = 5;
+constexpr int kEmitPitchA = kEmitTK + 4, kEmitPitchB = 2 * kEmitTN + 4;
 
-__global__ void __launch_bounds__(kEmitThreads) k_emit_fma(ModelDev m, const float* __restrict__ v,
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+// Two fused multiply-adds in one instruction.
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+// W4 [2N][H] as [H][2][ldn], so that the columns of a slab are contiguous (when weights are loaded).
+__global__ void k_transpose_heads(const float* __restrict__ W4, int N, int H, int ldn, float* __restrict__ out) {
+    __shared__ float tile[32][33];
+    const int j0 = blockIdx.x * 32, k0 = blockIdx.y * 32, head = blockIdx.z;
+    for (int r = threadIdx.y; r < 32; r += 8)
+        tile[r][threadIdx.x] = j0 + r < N && k0 + threadIdx.x < H ? W4[(static_cast<size_t>(head) * N + j0 + r) * H + k0 + threadIdx.x] : 0.f;
+    __syncthreads();
+    for (int r = threadIdx.y; r < 32; r += 8)
+        if (k0 + r < H && j0 + threadIdx.x < ldn)
+            out[(static_cast<size_t>(k0 + r) * 2 + head) * ldn + j0 + threadIdx.x] = tile[threadIdx.x][r];
+}
+
+template <int RM>
+__global__ void __launch_bounds__(kEmitThreads, RM == 8 ? 7 : 8) k_emit_fma(ModelDev m, const float* __restrict__ v, const float* __restrict__ W4T, int ldn,
                                                             const DevState* __restrict__ st, NoiseKey key,
                                                             uint32_t sample_base, int count,
                                                             float* __restrict__ x, int ldx) {
-    __shared__ __align__(16) float As[kEmitTK][kEmitTM + 4];
-    __shared__ __align__(16) float Bm[kEmitTK][kEmitTN + 4];
-    __shared__ __align__(16) float Bl[kEmitTK][kEmitTN + 4];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int row0 = blockIdx.y * kEmitTM, j0 = blockIdx.x * kEmitTN;
-    const int H = m.H, N = m.N;
-    float acc_m[4][4], acc_l[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc_m[a][b] = acc_l[a][b] = 0.0f;
-
-    const int lr = tid >> 2, lc = (tid & 3) * 4;
+    constexpr int TM = 4 * RM, kFloats = TM * kEmitPitchA + kEmitTK * kEmitPitchB;
+    __shared__ __align__(16) float sm[kEmitSlabs * kFloats];
+    const int H = m.H, N = m.N, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int row_tiles = ceil_div(count, TM), row0 = static_cast<int>(blockIdx.x) % row_tiles * TM;
+    const int j0 = static_cast<int>(blockIdx.x) / row_tiles * kEmitTN, jbase = j0 + 4 * tx;
+    const uint32_t smem = fma32::smem_addr(sm);
+    // No launch_dependents here: the row sort after this kernel has a few CTAs per SM, and placed early they crowd on the SMs
+    // that happen to have room (N=128, S=16384: the decision 119 us with it, 101 us without).
     dependency_wait();
-    launch_dependents();
-    for (int kk = 0; kk < H; kk += kEmitTK) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), bm = a, bl = a;
-        if (kk + lc < H) {
-            if (row0 + lr < count) a = *reinterpret_cast<const float4*>(v + static_cast<size_t>(row0 + lr) * H + kk + lc);
-            if (j0 + lr < N) {
-                bm = *reinterpret_cast<const float4*>(m.W4 + static_cast<size_t>(j0 + lr) * H + kk + lc);
-                bl = *reinterpret_cast<const float4*>(m.W4 + static_cast<size_t>(N + j0 + lr) * H + kk + lc);
+    const int slabs = ceil_div(H, kEmitTK);
+    int k_req = 0, buf_req = 0;
+    const auto request = [&] {
+        if (k_req < H) {
+            const uint32_t dst = smem + 4 * buf_req * kFloats;
+#pragma unroll
+            for (int u = tid; u < TM * kEmitTK / 4; u += kEmitThreads) {
+                const int r = u / (kEmitTK / 4), k = k_req + u % (kEmitTK / 4) * 4, valid = row0 + r < count ? H - k : 0;
+                fma32::copy4<true>(dst + 4 * (r * kEmitPitchA + u % (kEmitTK / 4) * 4), valid > 0 ? v + static_cast<size_t>(row0 + r) * H + k : v, valid);
             }
+#pragma unroll
+            for (int u = tid; u < kEmitTK * kEmitTN / 2; u += kEmitThreads) {
+                const int kk = u / (kEmitTN / 2), c = u % (kEmitTN / 2) * 4, k = k_req + kk, j = j0 + c % kEmitTN, valid = k < H ? ldn - j : 0;
+                fma32::copy4<true>(dst + 4 * (TM * kEmitPitchA + kk * kEmitPitchB + c),
+                                   valid > 0 ? W4T + (static_cast<size_t>(k) * 2 + c / kEmitTN) * ldn + j : W4T, valid);
+            }
+            k_req += kEmitTK;
+            if (++buf_req == kEmitSlabs) buf_req = 0;
         }
-        As[lc + 0][lr] = a.x; As[lc + 1][lr] = a.y; As[lc + 2][lr] = a.z; As[lc + 3][lr] = a.w;
-        Bm[lc + 0][lr] = bm.x; Bm[lc + 1][lr] = bm.y; Bm[lc + 2][lr] = bm.z; Bm[lc + 3][lr] = bm.w;
-        Bl[lc + 0][lr] = bl.x; Bl[lc + 1][lr] = bl.y; Bl[lc + 2][lr] = bl.z; Bl[lc + 3][lr] = bl.w;
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
 #pragma unroll
-        for (int k = 0; k < kEmitTK; ++k) {
-            const float4 a4 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-            const float4 m4 = *reinterpret_cast<const float4*>(&Bm[k][tx * 4]);
-            const float4 l4 = *reinterpret_cast<const float4*>(&Bl[k][tx * 4]);
-            const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-            const float mv[4] = {m4.x, m4.y, m4.z, m4.w};
-            const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
+    for (int i = 0; i < kEmitSlabs - 1; ++i) request();
+    unsigned long long sums[RM][4] = {};                     // means of workers 0, 1 and 2, 3, then their log-variances
+    int buf = 0;
+    for (int it = 0; it < slabs; ++it) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kEmitSlabs - 2) : "memory");
+        __syncthreads();                                     // the slab is there for everyone, and everyone has finished with the one before it
+        request();
+        const float* sa = sm + buf * kFloats + ty * kEmitPitchA;
+        const float* sb = sm + buf * kFloats + TM * kEmitPitchA + 4 * tx;
 #pragma unroll
-            for (int a_ = 0; a_ < 4; ++a_)
+        for (int k = 0; k < kEmitTK; k += 4) {
+            float4 a[RM];
 #pragma unroll
-                for (int b_ = 0; b_ < 4; ++b_) {
-                    acc_m[a_][b_] = fmaf(av[a_], mv[b_], acc_m[a_][b_]);
-                    acc_l[a_][b_] = fmaf(av[a_], lv[b_], acc_l[a_][b_]);
+            for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const float4*>(sa + 4 * i * kEmitPitchA + k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const ulonglong2 mean = *reinterpret_cast<const ulonglong2*>(sb + (k + q) * kEmitPitchB);
+                const ulonglong2 logvar = *reinterpret_cast<const ulonglong2*>(sb + (k + q) * kEmitPitchB + kEmitTN);
+#pragma unroll
+                for (int i = 0; i < RM; ++i) {
+                    const float s = q == 0 ? a[i].x : q == 1 ? a[i].y : q == 2 ? a[i].z : a[i].w;
+                    const unsigned long long s2 = pack2(s, s);
+                    fma2(sums[i][0], s2, mean.x);
+                    fma2(sums[i][1], s2, mean.y);
+                    fma2(sums[i][2], s2, logvar.x);
+                    fma2(sums[i][3], s2, logvar.y);
                 }
-        }
-        __syncthreads();
-    }
-
-    const uint32_t step = st->step;
-    const int jbase = j0 + tx * 4;
-    if (jbase >= N) return;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int k = row0 + ty * 4 + s;
-        if (k >= count) continue;
-        float eps[4];
-        normal4(static_cast<uint32_t>(jbase >> 2), sample_base + static_cast<uint32_t>(k), kStreamEmission, step,
-                key.seed_lo, key.seed_hi, eps);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int j = jbase + c;
-            if (j < N) {
-                const float mean = acc_m[s][c] + m.b4[j];
-                const float logvar = acc_l[s][c] + m.b4[N + j];
-                x[static_cast<size_t>(k) * ldx + j] = fmaf(expf(0.5f * logvar), eps[c], mean);
             }
+        }
+        if (++buf == kEmitSlabs) buf = 0;
+    }
+    // The draws one row at a time, through shared memory (each thread its own results): unrolled, the generator and its
+    // logarithms and sines would be 30 KB of instructions, which a call that finds the caches cold fetches from memory.
+    __syncthreads();
+    ulonglong2* own = reinterpret_cast<ulonglong2*>(sm) + tid;
+#pragma unroll
+    for (int i = 0; i < RM; ++i) {
+        own[(2 * i) * kEmitThreads] = make_ulonglong2(sums[i][0], sums[i][1]);
+        own[(2 * i + 1) * kEmitThreads] = make_ulonglong2(sums[i][2], sums[i][3]);
+    }
+    static_assert(2 * RM * kEmitThreads * 4 <= kEmitSlabs * kFloats, "results fit where the slabs were");
+    if (jbase >= N) return;
+    const uint4 column = philox_column(static_cast<uint32_t>(jbase >> 2), kStreamEmission, st->step, key.seed_lo, key.seed_hi);
+    float b_mean[4], b_logvar[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        b_mean[c] = jbase + c < N ? m.b4[jbase + c] : 0.f;
+        b_logvar[c] = jbase + c < N ? m.b4[N + jbase + c] : 0.f;
+    }
+#pragma unroll 1
+    for (int i = 0; i < RM; ++i) {
+        const int k = row0 + ty + 4 * i;
+        if (k >= count) break;
+        float eps[4], mean[4], logvar[4], out[4];
+        normal4_row_column(philox_row(sample_base + static_cast<uint32_t>(k), kStreamEmission, key.seed_lo), column, key.seed_lo, key.seed_hi, eps);
+        *reinterpret_cast<float4*>(mean) = *reinterpret_cast<const float4*>(own + (2 * i) * kEmitThreads);
+        *reinterpret_cast<float4*>(logvar) = *reinterpret_cast<const float4*>(own + (2 * i + 1) * kEmitThreads);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) out[c] = fmaf(expf(0.5f * (logvar[c] + b_logvar[c])), eps[c], mean[c] + b_mean[c]);
+        float* dst = x + static_cast<size_t>(k) * ldx + jbase;               // the row pitch is a multiple of 8 floats
+        if (jbase + 3 < N) {
+            *reinterpret_cast<float4*>(dst) = make_float4(out[0], out[1], out[2], out[3]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (jbase + c < N) dst[c] = out[c];
         }
     }
 }
