@@ -793,6 +793,122 @@ k_chain_resident(ModelDev m, const float* __restrict__ hlr, const DevState* __re
     }
 }
 
+// Variant 3: D lanes per sample, one latent component each, for decisions with too few samples to occupy the GPU otherwise.
+// What bounds a small decision is the chain of a step -- D multiply-adds per hidden unit, H / (lanes per sample) hidden units, the sums
+// over the lanes -- with about one warp per scheduler to hide it: with D / 4 lanes and two samples per lane an SM had one warp at N=158, S=2048.
+// N=158, lag 20: 76 -> 23 us; N=16: 13 -> 7 us; N=2175, lag 20, S=1024 against the tensor-core chain on 8 SMs: 76 -> 32 us.  Every weight is
+// read from shared memory for one sample only, so with more than 16 warps per SM the kernels above are faster.
+// Drawing the noise of 16 steps at once into shared memory, off the chain, changed nothing (23 us).
+constexpr int kChainWideThreads = 512;
+
+// y[0 .. D-1] summed over the D lanes of a group: lane g ends with the total of component g (recursive halving, D - 1 shuffles).
+template <int D>
+__device__ __forceinline__ float group_reduce_scatter(float (&y)[D], int g) {
+#pragma unroll
+    for (int off = D / 2; off > 0; off >>= 1)
+#pragma unroll
+        for (int i = 0; i < off; ++i) {
+            const float keep = (g & off) ? y[i + off] : y[i], give = (g & off) ? y[i] : y[i + off];
+            y[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+    return y[0];
+}
+template <int D>
+__device__ __forceinline__ void group_broadcast(float own, float (&z)[D]) {
+#pragma unroll
+    for (int d = 0; d < D; ++d) z[d] = __shfl_sync(0xffffffffu, own, d, D);
+}
+// Element g of a sample's normals: its half of one Box-Muller pair.
+__device__ __forceinline__ float normal_element(int g, uint32_t sample, uint32_t stream, uint32_t step, const NoiseKey& key) {
+    const Philox4 r = philox4x32_10(static_cast<uint32_t>(g >> 2), sample, stream, step, key.seed_lo, key.seed_hi);
+    float c, s;
+    box_muller((g & 2) ? r.z : r.x, (g & 2) ? r.w : r.y, c, s);
+    return (g & 1) ? s : c;
+}
+
+template <int D>
+__global__ void __launch_bounds__(kChainWideThreads, 1)
+k_chain_wide(ModelDev m, const float* __restrict__ hlr, const DevState* __restrict__ st, NoiseKey key,
+             uint32_t sample_base, int count, ChainOut out) {
+    extern __shared__ __align__(16) float sm[];          // chain_resident_smem_floats
+    const int H = m.H, W = m.W;
+    float* sWzT = sm;                   // [D][H]
+    float* sWmu = sWzT + H * D;         // [D][H]
+    float* sW1T = sWmu + H * D;         // [D][H]
+    float* sW2 = sW1T + H * D;          // [2D][H]
+    float* sW3T = sW2 + 2 * H * D;      // [D][H]
+    float* sbz = sW3T + H * D;          // [H]
+    float* sb1 = sbz + H;               // [H]
+    float* sb3 = sb1 + H;               // [H]
+    float* shl = sb3 + H;               // [W][H]
+    float* sWsigT = shl + W * H;        // [D][D], transposed: a lane reads its row a column at a time
+    stage_vector4(sWzT, m.WzT, H * D);
+    stage_vector4(sWmu, m.Wmu, H * D);
+    stage_vector4(sW1T, m.W1T, H * D);
+    stage_vector4(sW2, m.W2, 2 * H * D);
+    stage_vector4(sW3T, m.W3T, H * D);
+    stage_vector4(sbz, m.bz, H);
+    stage_vector4(sb1, m.b1, H);
+    stage_vector4(sb3, m.b3, H);
+    for (int i = threadIdx.x; i < D * D; i += kChainWideThreads) sWsigT[(i % D) * D + i / D] = m.Wsig[i];
+    const int lane = threadIdx.x & 31, g = lane % D;
+    const float bmu = m.bmu[g], bsig = m.bsig[g], b2_mean = m.b2[g], b2_logvar = m.b2[D + g], z0 = m.z0[g];
+    dependency_wait();            // up to here: weights
+    launch_dependents();
+    for (int i = threadIdx.x; i < W * H; i += kChainWideThreads) shl[i] = hlr[i] + hlr[W * H + i];
+    __syncthreads();
+
+    const int n_batches = ceil_div(count, 32 / D);
+    const uint32_t step = st->step;
+    // consecutive batches go to different CTAs, so that a small decision still spreads over all SMs
+    for (int b = blockIdx.x + gridDim.x * (threadIdx.x >> 5); b < n_batches; b += gridDim.x * (kChainWideThreads / 32)) {
+        const int k = b * (32 / D) + lane / D;
+        const uint32_t sample = sample_base + static_cast<uint32_t>(k);
+        float z[1][D];
+        group_broadcast<D>(z0, z[0]);
+        for (int t = 0; t < W; ++t) {
+            const float eps = normal_element(g, sample, static_cast<uint32_t>(t), step, key);     // off the chain: nothing below feeds it
+            float mu[1][D] = {};
+            const float* hl = shl + t * H;
+            for (int i0 = 4 * g; i0 < H; i0 += 4 * D) {
+                float hid[1][4];
+                hidden_block<D, 1>(sWzT, sbz, H, i0, z, hid);
+                const float4 lr = lds4(hl + i0);
+                const float lrv[4] = {lr.x, lr.y, lr.z, lr.w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) hid[0][c] = (tanh_fast(hid[0][c]) + lrv[c]) * (1.0f / 3.0f);
+                output_block<D, 1>(sWmu, H, i0, hid, mu);
+            }
+            const float mu_own = group_reduce_scatter<D>(mu[0], g) + bmu;
+            group_broadcast<D>(mu_own, mu[0]);
+            float pre = bsig;
+#pragma unroll
+            for (int e = 0; e < D; ++e) pre = fmaf(sWsigT[e * D + g], mu[0][e], pre);
+            group_broadcast<D>(fmaf(softplusf(pre), eps, mu_own), z[0]);
+        }
+        const float eps = normal_element(g, sample, kStreamTransition, step, key);
+        float mean[1][D] = {}, logvar[1][D] = {};
+        for (int i0 = 4 * g; i0 < H; i0 += 4 * D) {
+            float hid[1][4];
+            hidden_block<D, 1>(sW1T, sb1, H, i0, z, hid);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) hid[0][c] = fmaxf(hid[0][c], 0.0f);
+            output_block<D, 1>(sW2, H, i0, hid, mean);
+            output_block<D, 1>(sW2 + D * H, H, i0, hid, logvar);
+        }
+        const float mean_own = group_reduce_scatter<D>(mean[0], g) + b2_mean, logvar_own = group_reduce_scatter<D>(logvar[0], g) + b2_logvar;
+        group_broadcast<D>(fmaf(expf(0.5f * logvar_own), eps, mean_own), z[0]);
+        const float scale = hidden_scale<D>(out, k, k < count, g, z[0]);
+        for (int i0 = 4 * g; i0 < H; i0 += 4 * D) {
+            float hid[1][4];
+            hidden_block<D, 1>(sW3T, sb3, H, i0, z, hid);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) hid[0][c] = fmaxf(hid[0][c], 0.0f);
+            if (k < count) store_hidden<D>(out, k, H, i0, hid[0], scale);
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------------------------
 // Emission output layer in fp32 FMA, with the noise drawn in the epilogue:
 //   [mean | logvar] = W4 v + b4,   x_j = mean_j + exp(logvar_j / 2) * eps_j.
