@@ -36,12 +36,7 @@ MINMAX_LANES_PER_SM = 64         # fp32 min / max lanes per SM per clock (ALU pi
 # DRAM bytes per launch of the dominant kernel, from the ncu capture summarised under profiles/ (valid for the
 # kernel as committed with that summary; set to None when the kernel changes): the sample matrix read once
 # (grows with S) plus the partial rows written (one per CTA: does not grow with S).
-NCU_TRAFFIC = {
-    ("n1024", "sort"): {"bytes_per_sample": 201400064 / 49152, "bytes_fixed": 4353792,
-                        "source": "profiles/ncu_full_n1024_s49152_chain_emit_sort.txt (S=49152, scaled by S)"},
-    ("n4096", "sort"): {"bytes_per_sample": 134251776 / 8192, "bytes_fixed": 8298752,
-                        "source": "profiles/ncu_full_n4096_s8192_sort.txt (S=8192, scaled by S)"},
-}
+NCU_TRAFFIC = {}
 PRECISION_NAMES = {0: "f32", 1: "tf32", 2: "tf32(bf16 weights)"}
 
 
@@ -63,6 +58,12 @@ def compare_exchanges(n_pow2: int) -> int:
         total += (n_pow2 // 2) * (k.bit_length() - 1)
         k *= 2
     return total
+
+
+def sorts_by_buckets(n: int, rows: int) -> bool:
+    """The library's rule: rows of more than 256 keys, and of more than 128 when there are many, are sorted by
+    distribution (each key read once, counted and placed in shared memory), the others by the network."""
+    return n > 256 or (n > 128 and rows >= 8192)
 
 
 def stage_work(wl, S, literal=False):
@@ -538,10 +539,17 @@ def main():
     rates = pipe_rates(local_rank, measure=not args.no_measure_alu_peak)
     lane_rate = lambda name: SM_COUNT * 32.0 * rates[name] * clock_mhz * 1e6          # lane-operations per second
     bf16 = peaks.get("bf16_tflops", 1590.0)
-    tensor_peak = 0.5 * bf16 * 1e12                      # tf32 runs at half the bf16 rate (nominal ratio)
-    tensor_src = ("measured bf16 burst x 0.5 (nominal tf32 : bf16 ratio)" if peaks else "fallback 1590 x 0.5")
+    tensor_peak = 0.5 * bf16 * 1e12                      # chain: tf32 runs at half the bf16 rate (nominal ratio)
+    half_peak = bf16 * 1e12                              # emission: tf32 values held as halves run at the f16 rate
+    tensor_src = ("measured bf16 burst (chain x 0.5: nominal tf32 : bf16 ratio)" if peaks else "fallback 1590 (chain x 0.5)")
+    hbm = peaks.get("hbm_gbs", 6650.0) * 1e9
+    by_buckets = sorts_by_buckets(wl.N, wl.S)
+    sort_bytes = 4 * wl.S * wl.N                         # the sample matrix, read once
     if kind == "tensor":
-        peak, unit, peak_src, bound = tensor_peak / 1e12, "TFLOP/s", tensor_src, "tensor"
+        peak, unit, peak_src, bound = half_peak / 1e12, "TFLOP/s", tensor_src, "tensor"
+    elif dominant == "sort" and by_buckets:
+        peak, unit, bound, amount = hbm / 1e12, "TB/s", "hbm", sort_bytes
+        peak_src = "measured copy bandwidth" if peaks else "fallback 6.65 TB/s"
     elif dominant == "sort":
         peak, unit, bound = lane_rate("minmax") / 1e12, "Tlane-op/s", "alu"
         peak_src = (f"{rates['source']}: {rates['minmax']:.3f} fp32 min/max warp-instructions per clock per SM x 32 lanes "
@@ -558,44 +566,49 @@ def main():
                 "algorithmic_per_launch": amount, "peak_source": peak_src,
                 "stage_ms": {k: round(v, 4) for k, v in stage_avg.items()}}
     # The path's model time: the slowest of the three resources the whole decision needs -- tensor cores (every
-    # product that runs on them), the plain ALUs (the sort's min/max at the measured min/max rate, plus the
-    # multiply-adds of whatever does not run on the tensor cores at the measured FMA rate), and the exchange of keys
-    # between threads (the network's cross-lane stages at the measured shuffle rate).  path_frac sets it against the
-    # measured time of a whole step; frac_vs_nlog2n sets the sort stage against the comparison-sort floor of
-    # N log2 N compare-exchanges per row instead of the network's own count.
+    # product that runs on them), the plain ALUs (the multiply-adds of whatever does not run on the tensor cores at the
+    # measured FMA rate; where the network sorts, its min/max at the measured min/max rate), and either the exchange of keys
+    # between threads (the network's cross-lane stages at the measured shuffle rate) or, where rows are sorted by
+    # distribution, the sample matrix written and read once through HBM.  path_frac sets it against the
+    # measured time of a whole step; frac_vs_nlog2n sets the sort stage against a comparison sort's N log2 N
+    # compare-exchanges per row at the min/max rate (a sort by distribution may exceed 1).
     p2 = 32
     while p2 < wl.N:
         p2 *= 2
     tensor_flops = sum(a for k, (kd, a) in work.items() if kd == "tensor")
+    t_tc = tensor_flops / half_peak
     chain_on_tensor = bool(wl.precision) and wl.D in (16, 32) and not (literal and wl.D == 32)
     if chain_on_tensor:
         tensor_flops += 2 * work["chain"][1]
+        t_tc += 2 * work["chain"][1] / tensor_peak
     fma_ops = sum(a for k, (kd, a) in work.items() if kd == "alu" and k not in ("sort", "chain")) + \
         (0 if chain_on_tensor else work["chain"][1])
-    minmax_ops = work["sort"][1]
+    minmax_ops = 0 if by_buckets else work["sort"][1]
     e_keys = min(32, p2 // 32)
     lane_bits = (p2 // e_keys).bit_length() - 1                    # cross-lane (and cross-warp) bits of a key's index
     xchg_stages = lane_bits * (lane_bits + 1) // 2                 # stages whose partners sit in another thread
-    xchg_ops = wl.S * p2 * xchg_stages                             # one key moved per lane per such stage
-    t_tc = tensor_flops / tensor_peak
+    xchg_ops = 0 if by_buckets else wl.S * p2 * xchg_stages        # one key moved per lane per such stage
     t_alu = minmax_ops / lane_rate("minmax") + fma_ops / lane_rate("fma")
     t_xchg = xchg_ops / lane_rate("shuffle")
-    t_model = max(t_tc, t_alu, t_xchg)
+    t_hbm = 2 * sort_bytes / hbm
+    t_model = max(t_tc, t_alu, t_xchg, t_hbm)
     # Stage by stage: each of the three large stages against the one unit its arithmetic runs on (tensor cores for the
-    # products that use them, the FMA rate for those that do not, the min/max rate for the sort), and their sum against
+    # products that use them, the FMA rate for those that do not; the sort against one read of the matrix or, where the
+    # network sorts, the min/max rate), and their sum against
     # the time the three take one after the other.  Looser than path_frac (it lets no stage overlap another), stricter
     # than the dominant kernel's own fraction.
     ideal = {
         "chain": 2 * work["chain"][1] / tensor_peak if chain_on_tensor else work["chain"][1] / lane_rate("fma"),
-        "emission": work["emission"][1] / (tensor_peak if work["emission"][0] == "tensor" else lane_rate("fma")),
-        "sort": minmax_ops / lane_rate("minmax"),
+        "emission": work["emission"][1] / (half_peak if work["emission"][0] == "tensor" else lane_rate("fma")),
+        "sort": sort_bytes / hbm if by_buckets else minmax_ops / lane_rate("minmax"),
     }
     big = ("chain", "emission", "sort")
     roofline.update({
         "stage_frac": {k: round(ideal[k] / (stage_avg[k] * 1e-3), 4) for k in big},
         "path_frac_sum": sum(ideal[k] for k in big) / (sum(stage_avg[k] for k in big) * 1e-3),
         "path_frac": t_model / (ms_per_step * 1e-3),
-        "path_model_ms": {"tensor": round(t_tc * 1e3, 4), "alu": round(t_alu * 1e3, 4), "exchange": round(t_xchg * 1e3, 4)},
+        "path_model_ms": {"tensor": round(t_tc * 1e3, 4), "alu": round(t_alu * 1e3, 4), "exchange": round(t_xchg * 1e3, 4),
+                          "hbm": round(t_hbm * 1e3, 4)},
         "path_model_sources": {
             "tensor": f"{tensor_flops:.4g} FLOP / ({tensor_src})",
             "alu": f"{minmax_ops:.4g} min/max + {fma_ops:.4g} multiply-adds (counted from the kernels' source) at the "
@@ -607,8 +620,8 @@ def main():
         "pipe_rates_source": rates["source"],
     })
 
-    # The emission output layer on the tensor cores is bound by its operand stream from L2 into shared memory
-    # (per 128 x 128 output tile the 128 hidden vectors and the 256 weight rows, 2 * H bytes each).
+    # The emission output layer's operand stream from L2 into shared memory (per 128 x 128 output tile the 128 hidden
+    # vectors, 2 * H bytes each, and, where they do not stay in shared memory, the 256 weight rows).
     # Set it against the rate the library measures for exactly those copies on this GPU: weights from a matrix of a
     # few MB that every SM re-reads, hidden vectors from one of tens of MB.
     if wl.precision and not literal and not args.no_measure_alu_peak:
@@ -616,7 +629,9 @@ def main():
         op_rates = _b.measure_operand_stream(local_rank)
         n_tiles = -(-wl.S // 128) * -(-wl.N // 128)
         k_bytes = -(-wl.H // 64) * 128                               # bytes of one operand row (K blocks of 64 halves)
-        bytes_w, bytes_v = n_tiles * 256 * k_bytes, n_tiles * 128 * k_bytes
+        # H <= 256: a CTA loads the weights of a block of workers once, and few CTAs work on two blocks
+        w_loads = min(n_tiles, SM_COUNT + -(-wl.N // 128)) if wl.H <= 256 else n_tiles
+        bytes_w, bytes_v = w_loads * 256 * k_bytes, n_tiles * 128 * k_bytes
         t_stream = bytes_w / (op_rates["weights_2mb"] * 1e9) + bytes_v / (op_rates["hidden_64mb"] * 1e9)
         roofline["emission_stream"] = {
             "bound": "l2 -> shared memory operand stream",

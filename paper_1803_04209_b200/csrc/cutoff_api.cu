@@ -1222,7 +1222,7 @@ static int push_censored(cutoff_ctx* c, const float* runtimes_sec, int on_device
         mask = c->h_mask;
     }
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
-    k_impute<<<1, kImputeThreads, 0, c->stream>>>(src, mask, c->d_stage, c->d_x, c->ldx, c->S, c->N, c->d_state, key);
+    k_impute<<<c->N < kImputeCtas ? c->N : kImputeCtas, kImputeThreads, 0, c->stream>>>(src, mask, c->d_stage, c->d_x, c->ldx, c->S, c->N, c->d_state, key);
     c->launches += 1;
     c->draws_valid = false;                                 // one step's draws serve one push
     int rc = push_common(c, c->d_stage);

@@ -79,9 +79,12 @@ __global__ void __launch_bounds__(kPushThreads) k_push(const float* __restrict__
 // matrix of the last decision.  The draws are iid, so the first one above the threshold, scanning
 // cyclically from a start that does not depend on their values (Philox word 0 of counter
 // (worker, 0, 0x300, decision number) modulo S), is an exact draw from the truncated distribution;
-// if there is none the threshold itself is used.  One CTA; a warp per censored worker.
+// if there is none the threshold itself is used.
+// A warp per censored worker, the workers j = b, b + CTAs, .. in CTA b.  A warp's load touches 32 rows, so what bounds one CTA is
+// its SM's load unit: N=158, S=2048 took 32 us in one CTA, 14 us in 16.  More CTAs would each read the run-times and the
+// mask over the bus for little (20 KB at N=4096).
 // ---------------------------------------------------------------------------------------------
-constexpr int kImputeThreads = 1024;
+constexpr int kImputeThreads = 512, kImputeCtas = 16;
 constexpr uint32_t kStreamImpute = 0x300u;
 
 // src and censored may be pinned host memory; stage receives the completed vector.  Draws above the threshold are rare, so a
@@ -92,35 +95,38 @@ __global__ void __launch_bounds__(kImputeThreads) k_impute(const float* __restri
                                                             float* __restrict__ stage, const float* __restrict__ x, int ldx, int S, int N,
                                                             DevState* __restrict__ st, NoiseKey key) {
     __shared__ float red[kImputeThreads / 32];
-    __shared__ uint8_t mask[4096];
+    __shared__ uint16_t mine[4096];                     // this CTA's censored workers, in any order
+    __shared__ int n_mine;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) n_mine = 0;
+    __syncthreads();
     float m = -INFINITY;
     for (int j = threadIdx.x; j < N; j += kImputeThreads) {
         const uint8_t c = censored[j];
         const float v = src[j];
-        mask[j] = c;
-        if (!c) { m = fmaxf(m, v); stage[j] = v; }
+        if (!c) m = fmaxf(m, v);
+        if (j % gridDim.x != blockIdx.x) continue;
+        if (c) mine[atomicAdd(&n_mine, 1)] = static_cast<uint16_t>(j);
+        else stage[j] = v;
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     if (lane == 0) red[warp] = m;
     __syncthreads();
-    m = red[lane];
+    m = red[lane % (kImputeThreads / 32)];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     const float threshold = m;
     if (!(threshold > -INFINITY)) {
         // nobody finished, so there is no cutoff time to truncate at: flag the vector; the push kernel that
         // follows sees the flag and leaves the window untouched
-        if (threadIdx.x == 0) st->error_flags |= kErrNoFinisher;
+        if (blockIdx.x == 0 && threadIdx.x == 0) st->error_flags |= kErrNoFinisher;
         return;
     }
     const float scale = st->scale;
     const uint32_t step = st->step;
-    int turn = 0;                                       // censored workers go to the warps in turn
-    for (int j = 0; j < N; ++j) {
-        if (!mask[j]) continue;
-        if ((turn++ & (kImputeThreads / 32 - 1)) != warp) continue;
+    for (int t = warp; t < n_mine; t += kImputeThreads / 32) {
+        const int j = mine[t];
         const uint32_t start = philox4x32_10(static_cast<uint32_t>(j), 0u, kStreamImpute, step, key.seed_lo, key.seed_hi).x %
                                static_cast<uint32_t>(S);
         float value = threshold;
