@@ -33,10 +33,13 @@ __device__ __forceinline__ float softplus_f(float v) { return v > 20.f ? v : log
 __device__ __forceinline__ float sigmoid_f(float v) { return 1.f / (1.f + expf(-v)); }
 
 // ---- tiled products (tile_product.cuh) ------------------------------------------------------------------------------
-// Two tiles: 64 x 64 with 8 x 4 results per thread where there are enough of them to fill the GPU, 16 x 32 with 2 x 2
-// where there are not -- then the time is the chain's.
+// Three tiles: 64 x 64 with 8 x 4 results per thread where there are several of them per SM, 32 x 64 with 4 x 4 where there would
+// be one or two (the emission head of 384 x 256 values, H=128: 12.1 -> 8.6 us; of 320 x 2048, H=256: 25 -> 20 us), and 16 x 32
+// with 2 x 2 where even those do not fill the GPU -- then the time is the chain's: 2048 steps of it take 41 us whatever the tile
+// (2 x 4 results per thread 51 us, 1 x 2 48 us, the next four k in registers ahead of time 43 us).
 using namespace fma32;
 using LargeTile = Tile<64, 64, 8, 4, 16>;        // 128 threads
+using MediumTile = Tile<32, 64, 4, 4, 16>;       // 128 threads
 using SmallTile = Tile<16, 32, 2, 2, 32>;        // 128 threads
 
 struct Product {
@@ -100,18 +103,17 @@ __global__ void __launch_bounds__(T::kThreads) k_products(const __grid_constant_
 }
 
 // ---- emission head and its density ---------------------------------------------------------------------------------
-// head = v W4^T + b4 for 64 rows x 32 workers: the tile's columns are the means of its workers, then their log-variances,
+// head = v W4^T + b4 for T::TM rows x 32 workers: the tile's columns are the means of its workers, then their log-variances,
 // so a thread (columns tx, tx + 16, tx + 32, tx + 48) holds both halves of two workers, and at once
 //   log N(x; m, exp(lv)) summed over the tile's workers -> part[tile column][row],
 //   d_head = [r inv | -1/2 + r^2 inv / 2],  r = x - m, inv = exp(-lv)                    (d_head: null = forward only).
 constexpr int kHeadWorkers = LargeTile::TN / 2;
 
-template <bool VEC>
-__global__ void __launch_bounds__(LargeTile::kThreads) k_emission_density(const float* __restrict__ v, const float* __restrict__ W4,
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(T::kThreads) k_emission_density(const float* __restrict__ v, const float* __restrict__ W4,
                                                                              const float* __restrict__ b4, const float* __restrict__ x,
                                                                              int R, int N, int H, float* __restrict__ d_head,
                                                                              float* __restrict__ part) {
-    using T = LargeTile;
     __shared__ __align__(16) Slabs<T, true, true> sm;
     dependency_wait();
     launch_dependents();

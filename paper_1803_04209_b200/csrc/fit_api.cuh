@@ -95,7 +95,7 @@ struct ProductBuilder {
 };
 
 // 64 x 64 tiles only where they fill the GPU: below that the small ones finish earlier.
-constexpr int kFillTiles = 148;
+constexpr int kFillTiles = 148, kManyTiles = 4 * kFillTiles;
 
 // One product per direction of a dense layer over all rows: C[a.rows][b.rows] = A B with B k-major (X W^T) or m-major (dY W).
 template <typename T, bool BK>
@@ -176,10 +176,14 @@ inline void elbo_grad(int N, int D, int H, int W, int B, const float* p, const f
     const size_t path_smem = staged ? path_full : path_scratch;
     launch(k_path_forward, dim3(B), kPathThreads, path_smem, stream, true, 1, a, staged);
     {
-        const dim3 grid(static_cast<unsigned>(head_tiles * tiles_of(R, LargeTile::TM)));
         float* dhx = back ? ws + o.dhx : nullptr;
-        launch(vec ? k_emission_density<true> : k_emission_density<false>, grid, LargeTile::kThreads, 0, stream, true, 1,
-               ws + o.v, w(iW4), w(ib4), xhat, R, N, H, dhx, ws + o.part);
+        const auto run = [&](auto tile) {
+            using T = decltype(tile);
+            launch(vec ? k_emission_density<T, true> : k_emission_density<T, false>, dim3(static_cast<unsigned>(head_tiles * tiles_of(R, T::TM))),
+                   T::kThreads, 0, stream, true, 1, ws + o.v, w(iW4), w(ib4), xhat, R, N, H, dhx, ws + o.part);
+        };
+        if (head_tiles * tiles_of(R, LargeTile::TM) >= kManyTiles) run(LargeTile{});
+        else run(MediumTile{});
     }
     if (!back) {
         launch(k_elbo_finish, dim3((B + 3) / 4), 128, 0, stream, true, 1, ws + o.part, head_tiles, R, W, B, ws + o.path, elbo);
@@ -196,27 +200,32 @@ inline void elbo_grad(int N, int D, int H, int W, int B, const float* p, const f
     {
         // every weight gradient d W = d_out^T in, one segment of B rows per step, and the biases as sums of d_out; the
         // largest first.  Descending steps, as the reverse pass reaches them; the backward RNN is reversed in ascending ones.
-        ProductBuilder<LargeTile> q;
-        const auto rows = [&](const float* base, int ld, bool ascending, int slots, int first) {      // of [B][slots][ld]
-            return Operand{base + static_cast<long long>(first + (ascending ? 0 : W - 1)) * ld, static_cast<long long>(slots) * ld, ascending ? ld : -ld, ld};
+        const auto run = [&](auto tile) {
+            ProductBuilder<decltype(tile)> q;
+            const auto rows = [&](const float* base, int ld, bool ascending, int slots, int first) {      // of [B][slots][ld]
+                return Operand{base + static_cast<long long>(first + (ascending ? 0 : W - 1)) * ld, static_cast<long long>(slots) * ld, ascending ? ld : -ld, ld};
+            };
+            const auto down = [&](long long off, int ld) { return rows(ws + off, ld, false, W, 0); };
+            const Operand none{nullptr, 0, 0, 0};
+            q.add(down(o.dhx, 2 * N), down(o.v, H), g(iW4), H, g(ib4), B, W);
+            q.add(down(o.dpf, H), rows(xhat, N, false, W, 0), g(iWxf), N, g(ibf), B, W);
+            q.add(rows(ws + o.dpb, H, true, W, 0), rows(xhat, N, true, W, 0), g(iWxb), N, g(ibb), B, W);
+            q.add(down(o.dpf, H), rows(ws + o.a, H, false, W + 1, 0), g(iWhf), H, nullptr, B, W);
+            q.add(rows(ws + o.dpb, H, true, W, 0), rows(ws + o.b, H, true, W + 1, 1), g(iWhb), H, nullptr, B, W);
+            q.add(down(o.dv, H), rows(ws + o.z, D, false, W + 1, 1), g(iW3), D, g(ib3), B, W);
+            q.add(down(o.du, H), rows(ws + o.z, D, false, W + 1, 0), g(iW1), D, g(ib1), B, W);
+            q.add(down(o.dpc, H), rows(ws + o.z, D, false, W + 1, 0), g(iWz), D, g(ibz), B, W);
+            q.add(down(o.dhz, 2 * D), down(o.u, H), g(iW2), H, g(ib2), B, W);
+            q.add(down(o.dmu, D), down(o.hout, H), g(iWmu), H, g(ibmu), B, W);
+            q.add(down(o.dps, D), down(o.mu, D), g(iWsig), D, g(ibsig), B, W);
+            q.add(Operand{ws + o.ca, H, 0, H}, none, nullptr, 0, g(ia0), B);
+            q.add(Operand{ws + o.cb, H, 0, H}, none, nullptr, 0, g(ib0), B);
+            q.add(Operand{ws + o.gz0, D, 0, D}, none, nullptr, 0, g(iz0), B);
+            q.template run<false, false, true>(vec, stream, true);
         };
-        const auto down = [&](long long off, int ld) { return rows(ws + off, ld, false, W, 0); };
-        const Operand none{nullptr, 0, 0, 0};
-        q.add(down(o.dhx, 2 * N), down(o.v, H), g(iW4), H, g(ib4), B, W);
-        q.add(down(o.dpf, H), rows(xhat, N, false, W, 0), g(iWxf), N, g(ibf), B, W);
-        q.add(rows(ws + o.dpb, H, true, W, 0), rows(xhat, N, true, W, 0), g(iWxb), N, g(ibb), B, W);
-        q.add(down(o.dpf, H), rows(ws + o.a, H, false, W + 1, 0), g(iWhf), H, nullptr, B, W);
-        q.add(rows(ws + o.dpb, H, true, W, 0), rows(ws + o.b, H, true, W + 1, 1), g(iWhb), H, nullptr, B, W);
-        q.add(down(o.dv, H), rows(ws + o.z, D, false, W + 1, 1), g(iW3), D, g(ib3), B, W);
-        q.add(down(o.du, H), rows(ws + o.z, D, false, W + 1, 0), g(iW1), D, g(ib1), B, W);
-        q.add(down(o.dpc, H), rows(ws + o.z, D, false, W + 1, 0), g(iWz), D, g(ibz), B, W);
-        q.add(down(o.dhz, 2 * D), down(o.u, H), g(iW2), H, g(ib2), B, W);
-        q.add(down(o.dmu, D), down(o.hout, H), g(iWmu), H, g(ibmu), B, W);
-        q.add(down(o.dps, D), down(o.mu, D), g(iWsig), D, g(ibsig), B, W);
-        q.add(Operand{ws + o.ca, H, 0, H}, none, nullptr, 0, g(ia0), B);
-        q.add(Operand{ws + o.cb, H, 0, H}, none, nullptr, 0, g(ib0), B);
-        q.add(Operand{ws + o.gz0, D, 0, D}, none, nullptr, 0, g(iz0), B);
-        q.run<false, false, true>(vec, stream, true);
+        // the head's gradient has the most tiles
+        if (tiles_of(2 * N, LargeTile::TM) * tiles_of(H, LargeTile::TN) >= kFillTiles) run(LargeTile{});
+        else run(MediumTile{});
     }
 }
 

@@ -164,9 +164,11 @@ def test_learning_calls_reject_bad_arguments():
 
 # where the kernels change their way: tiles of 64 rows, 64 columns or 32 workers and their remainders, dimensions that are
 # no multiple of 4 (scalar loads), recurrence matrices too wide for shared memory (H > 200), latent matrices too large for
-# it (D = 64), more windows than one CTA of the recurrences takes and not a multiple of it, a product split over K
+# it (D = 64), more windows than one CTA of the recurrences takes and not a multiple of it, a product over many k, enough
+# workers and rows for the tiles of 64 x 64 in the emission head and the weight gradients
 @pytest.mark.parametrize("N,D,H,lag,B", [(1, 1, 1, 0, 1), (32, 4, 64, 0, 64), (33, 4, 68, 1, 33), (65, 8, 200, 0, 5),
-                                          (31, 5, 201, 1, 6), (64, 64, 300, 1, 3), (600, 16, 204, 3, 9)])
+                                          (31, 5, 201, 1, 6), (64, 64, 300, 1, 3), (600, 16, 204, 3, 9),
+                                          (1250, 4, 260, 7, 150), (1250, 4, 258, 7, 150)])
 def test_step_at_the_edges_of_tiles_and_of_shared_memory(N, D, H, lag, B):
     """Bounds as above: an fp32 sum of n products errs by at most about n * 2^-24 of the sum of their magnitudes."""
     import torch
