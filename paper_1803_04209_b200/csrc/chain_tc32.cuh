@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
                     float zm = 0.0f, inv;
 #pragma unroll
                     for (int gg = 0; gg < 4; ++gg) zm = fmaxf(zm, ld_shared_f32(t_hb + (gg * 128 + row) * 4));
-                    half_scale(1.01f * fmaf(a.v_out.slope, zm, a.v_out.offset), v_scale, inv);
+                    half_scale(a.v_out, zm, v_scale, inv);
                     if (cg == 0 && k < a.count) a.v_out.inv_scale[k] = inv;
                 }
                 for (int c = 0; c < n_chunks; ++c) {

@@ -71,8 +71,7 @@ struct cutoff_ctx {
     float* d_v_inv = nullptr;       // [alloc_rows]
     __half* d_w16 = nullptr;        // weights: W4 [2N][ldh]; literal: Wi2 [N], Wj2 [N], M [H] rows
     float* d_w_inv = nullptr;       // their inverse scales
-    float v_slope = 0.0f, v_offset = 0.0f;   // bound of v's (u's) entries: slope * largest |latent| + offset
-    float r_slope = 0.0f, r_offset = 0.0f;   // literal: of r's entries, from the largest |u|
+    float* d_bound = nullptr;       // [4] bound of v's (u's) entries, slope * largest |latent| + offset; literal: of r's, from the largest |u|
     float* d_x = nullptr;           // [chunk_rows][ldx]
     float* d_partial = nullptr;     // [n_chunks * sort_grid][N]; a second block of kPartialRows rows holds sums of squares
     float* d_std = nullptr;         // [N] spread of each order statistic (when asked for)
@@ -235,7 +234,7 @@ cudaError_t upload(void* dst, const void* src, size_t bytes) {
 }
 
 // |A x + b| <= slope * max |x| + offset, from the matrix as the tensor cores see it (rounded up a little)
-void layer_bound(const float* w, const float* b, size_t rows, size_t cols, float& slope, float& offset) {
+void layer_bound(const float* w, const float* b, size_t rows, size_t cols, float (&bound)[2]) {
     double l1 = 0.0, mb = 0.0;
     for (size_t r = 0; r < rows; ++r) {
         double s = 0.0;
@@ -243,8 +242,8 @@ void layer_bound(const float* w, const float* b, size_t rows, size_t cols, float
         l1 = std::fmax(l1, s);
         mb = std::fmax(mb, std::fabs(static_cast<double>(b[r])));
     }
-    slope = static_cast<float>(l1 * 1.001);
-    offset = static_cast<float>(mb * 1.001);
+    bound[0] = static_cast<float>(l1 * 1.001);
+    bound[1] = static_cast<float>(mb * 1.001);
 }
 
 // Launch `kernel` so that it may begin while the kernel before it in the stream is still running (programmatic
@@ -272,7 +271,7 @@ int next_pow2(int n) {
 
 void free_all(cutoff_ctx* c) {
     cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_Mb); cudaFree(c->d_M); cudaFree(c->d_W4T);
-    cudaFree(c->d_v16); cudaFree(c->d_v_inv); cudaFree(c->d_w16); cudaFree(c->d_w_inv); cudaFree(c->d_r16); cudaFree(c->d_r_inv);
+    cudaFree(c->d_v16); cudaFree(c->d_v_inv); cudaFree(c->d_w16); cudaFree(c->d_w_inv); cudaFree(c->d_bound); cudaFree(c->d_r16); cudaFree(c->d_r_inv);
     cudaFree(c->d_blob); cudaFree(c->d_WT); cudaFree(c->d_WhR); cudaFree(c->d_chain_image);
     if (c->h_mask) cudaFreeHost(c->h_mask); cudaFree(c->d_ring); cudaFree(c->d_stage);
     cudaFree(c->d_state); cudaFree(c->d_proj); cudaFree(c->d_hlr); cudaFree(c->d_v); cudaFree(c->d_x);
@@ -392,7 +391,7 @@ int launch_sort(cutoff_ctx* c, int count, float* partial) {
     return CUTOFF_OK;
 }
 
-HalfRows half_v(const cutoff_ctx* c) { return HalfRows{c->d_v16, c->d_v_inv, c->ldh, c->v_slope, c->v_offset}; }
+HalfRows half_v(const cutoff_ctx* c) { return HalfRows{c->d_v16, c->d_v_inv, c->ldh, c->d_bound}; }
 ChainOut chain_out(const cutoff_ctx* c) { return ChainOut{c->use_tc ? nullptr : c->d_v, half_v(c)}; }
 
 template <int D>
@@ -555,7 +554,7 @@ void launch_emission_literal(cutoff_ctx* c, uint32_t sample_base, int count) {
         // r = relu(M u + b') with M = Wj1 Wi2 (I is affine in u), then x = (Wi2 u + bi2) + softplus(Wj2 r + bj2) * eps
         tc::GemmTcArgs a{};
         a.st = c->d_state; a.M = count; a.bias = c->d_Mb; a.a_inv = c->d_v_inv; a.b_inv = c->d_w_inv + 2 * c->N;
-        a.out = HalfRows{c->d_r16, c->d_r_inv, c->ldh, c->r_slope, c->r_offset};
+        a.out = HalfRows{c->d_r16, c->d_r_inv, c->ldh, c->d_bound + 2};
         a.Nout = c->H; a.K = c->H;
         launch_gemm_relu_tc(c, c->map_v, c->map_M, a);
         tc::EmitDualArgs e;
@@ -912,6 +911,7 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
         CREATE_CHECK(cudaMalloc(&c->d_v_inv, sizeof(float) * c->alloc_rows));
         CREATE_CHECK(cudaMalloc(&c->d_w16, sizeof(__half) * w_rows * c->ldh));
         CREATE_CHECK(cudaMalloc(&c->d_w_inv, sizeof(float) * w_rows));
+        CREATE_CHECK(cudaMalloc(&c->d_bound, 4 * sizeof(float)));
     } else {
         CREATE_CHECK(cudaMalloc(&c->d_v, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->H));
         if (!c->literal) CREATE_CHECK(cudaMalloc(&c->d_W4T, sizeof(float) * 2 * static_cast<size_t>(c->H) * c->ldx));
@@ -1027,7 +1027,9 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         }
         CU_CHECK(c, cudaGetLastError());
         const size_t first = c->literal ? 27 : 19;                                                       // Wi1 or W3, and its bias
-        layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, c->v_slope, c->v_offset);
+        float bound[2];
+        layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, bound);
+        CU_CHECK(c, upload(c->d_bound, bound, sizeof(bound)));
     }
     if (!c->use_tc && !c->literal) {
         k_transpose_heads<<<dim3(ceil_div(c->ldx, 32), ceil_div(c->H, 32), 2), dim3(32, 8), 0, c->stream>>>(c->d_blob + off[21], c->N, c->H, c->ldx, c->d_W4T);
@@ -1147,7 +1149,9 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                 for (size_t j = 0; j < H; ++j) big_m[i * H + j] = host_tf32(static_cast<float>(acc[j]));
                 mb[i] = static_cast<float>(bacc);
             }
-            layer_bound(big_m.data(), mb.data(), H, H, c->r_slope, c->r_offset);
+            float bound[2];
+            layer_bound(big_m.data(), mb.data(), H, H, bound);
+            CU_CHECK(c, upload(c->d_bound + 2, bound, sizeof(bound)));
             CU_CHECK(c, upload(c->d_Mb, mb.data(), mb.size() * sizeof(float)));
             CU_CHECK(c, upload(c->d_M, big_m.data(), big_m.size() * sizeof(float)));
             half_rows(c, c->d_M, c->H, 2 * c->N);

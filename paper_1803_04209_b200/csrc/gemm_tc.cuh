@@ -34,7 +34,7 @@ __device__ __forceinline__ void gemm_epilogue_tile(const GemmTcArgs& a, uint32_t
                                                    uint32_t bar_acc_empty, const float* bias_s, float a_inv) {
     const bool row_ok = row < a.M;
     float scale, inv;
-    half_scale(1.01f * fmaf(a.out.slope, 32768.0f * a_inv, a.out.offset), scale, inv);
+    half_scale(a.out, 32768.0f * a_inv, scale, inv);
     if (row_ok && w0 == 0 && cg == 0) a.out.inv_scale[row] = inv;
 #pragma unroll
     for (int half = 0; half < 2; ++half) {

@@ -50,12 +50,16 @@ __global__ void k_half_rows(const float* __restrict__ w, int rows, int cols, int
 }
 
 // A hidden vector as the emission products read it: halves with a row pitch of whole 16 bytes, one inverse scale per row,
-// and the bound of a row's entries, |entry| <= slope * (largest |input|) + offset.
+// and the bound of a row's entries, |entry| <= bound[0] * (largest |input|) + bound[1].  The bound follows from the weights, so it is
+// read from device memory: a captured graph outlives the weights it was captured with.
 struct HalfRows {
     __half* p;              // [rows][ld]
     float* inv_scale;       // [rows]
     int ld;
-    float slope, offset;
+    const float* bound;
 };
+__device__ __forceinline__ void half_scale(const HalfRows& rows, float largest_input, float& scale, float& inv_scale) {
+    half_scale(1.01f * fmaf(__ldg(rows.bound), largest_input, __ldg(rows.bound + 1)), scale, inv_scale);
+}
 
 }  // namespace cutoff

@@ -659,7 +659,7 @@ __device__ __forceinline__ float hidden_scale(const ChainOut& out, int k, bool e
     float zm = 0.0f, scale, inv;
 #pragma unroll
     for (int d = 0; d < D; ++d) zm = fmaxf(zm, fabsf(z[d]));
-    half_scale(1.01f * fmaf(out.half.slope, zm, out.half.offset), scale, inv);
+    half_scale(out.half, zm, scale, inv);
     if (g == 0 && exists) out.half.inv_scale[k] = inv;
     return scale;
 }

@@ -78,3 +78,28 @@ def test_powers_of_two_pass_through_exactly(N, D, H, S, prec, literal):
     if literal:                                          # M = Wj1 Wi2 would mix the rows
         quiet["Wj1"][:] = 0.0
     assert np.array_equal(samples(quiet, trace, D, H, lag, S, prec, literal), x0 * two)
+
+
+@pytest.mark.parametrize("N,D,H,S,literal", [(40, 16, 64, 2500, False), (40, 16, 64, 300, False), (40, 8, 64, 300, False), (40, 32, 64, 3000, False),
+                                             (40, 16, 64, 300, True)])
+def test_a_captured_graph_follows_reloaded_weights(N, D, H, S, literal):
+    # the bound a hidden vector is scaled by belongs to the weights, not to the graph: reloaded ones may be far larger
+    make = inputs.make_weights_literal if literal else inputs.make_weights
+    w = make(N, D, H, seed=1, fan_in_ref=32)
+    big = {k: t.copy() for k, t in w.items()}
+    hidden, out = (("Wi1", "bi1"), "Wi2") if literal else (("W3", "b3"), "W4")
+    for k in hidden:
+        big[k] *= np.float32(2.0 ** 24)
+    big[out] *= np.float32(2.0 ** -24)
+    trace = inputs.make_trace(N, 6, seed=2, sigma=0.25)
+    flags = binding.FLAG_LITERAL if literal else 0
+    stats = []
+    for graph in (binding.FLAG_GRAPH, 0):
+        gpu = binding.Cutoff(N, D, H, 1, S, precision=1, seed=77, flags=flags | graph)
+        gpu.load_weights(w)
+        for i, x in enumerate(trace):
+            if i == 4:
+                gpu.load_weights(big)
+            gpu.step(x)
+        stats.append(gpu.get_stats()[0])
+    assert np.all(np.isfinite(stats[0])) and np.array_equal(stats[0], stats[1])
