@@ -577,7 +577,8 @@ def main():
         p2 *= 2
     tensor_flops = sum(a for k, (kd, a) in work.items() if kd == "tensor")
     t_tc = tensor_flops / half_peak
-    chain_on_tensor = bool(wl.precision) and wl.D in (16, 32) and not (literal and wl.D == 32)
+    # a decision of few samples runs its chain on the FMA units, D lanes per sample
+    chain_on_tensor = bool(wl.precision) and wl.D in (16, 32) and (literal and wl.D == 16 or not literal and wl.S * world > 16 * SM_COUNT)
     if chain_on_tensor:
         tensor_flops += 2 * work["chain"][1]
         t_tc += 2 * work["chain"][1] / tensor_peak
