@@ -448,8 +448,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_tc(const __grid_constant__
     extern __shared__ uint8_t smem_raw[];
     const Operands<1> o{{&map_v}, {&map_w4, &map_w4}, {0, a.N}, kBW};
     const Pipeline p = open_pipeline(smem_raw, o, a.st, a.count, ceil_div(a.N, kBW), a.H);
+    // no launch_dependents: a row sort with several CTAs per SM would place them as the SMs come free, unevenly (N=4096, S=32768:
+    // 858 us per decision with it, 851 without; N=2175: 139.2 and 137.8; with one CTA per SM no difference)
     dependency_wait();            // the hidden vectors and the device state are an earlier kernel's
-    launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) {
         load_operands(p, o, lane);

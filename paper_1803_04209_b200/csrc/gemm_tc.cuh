@@ -149,8 +149,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_emit_dual_tc(const __grid_const
     extern __shared__ uint8_t smem_raw[];
     const Operands<2> o{{&map_u, &map_r}, {&map_wi2, &map_wj2}, {0, 0}, kBW};
     const Pipeline p = open_pipeline(smem_raw, o, a.st, a.count, ceil_div(a.N, kBW), a.H);
-    dependency_wait();            // the rows of u and r and the device state are an earlier kernel's
-    launch_dependents();
+    dependency_wait();            // the rows of u and r and the device state are an earlier kernel's (no launch_dependents: as in k_emit_tc)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) {
         load_operands(p, o, lane);
