@@ -97,7 +97,7 @@ struct cutoff_ctx {
     bool use_tc = false;            // emission output layer on tensor cores
     int pair_clusters = 0;          // clusters of two CTAs of the two-SM emission kernel that fit the GPU at once
     bool pair_emission = false;     // option "pair_emission": run the output layer on pairs of SMs (slower as measured; off)
-    bool chain_wide = false;        // compact chain with D lanes per sample: few samples
+    int chain_wide = 0;             // compact chain with D lanes per sample (few samples): samples per lane, 0 = another chain
     bool chain_tc = false;          // per-sample chain on tensor cores as well (D = 16, H in {64, 128, 192, 256})
     bool chain_tc32 = false;        // the same for D = 32, H <= 512 (weights staged phase by phase)
     bool chain_tcl = false;         // the literal variant's chain on tensor cores (D = 16, H in {64, 128, 192, 256})
@@ -399,9 +399,13 @@ void launch_chain_t(cutoff_ctx* c, uint32_t sample_base, int count, size_t smem)
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     const size_t resident = chain_resident_smem_floats(c->D, c->H, c->W) * sizeof(float);
     if (c->chain_wide) {
-        const int batches = ceil_div(count, 32 / D);
-        launch_dependent(k_chain_wide<D>, dim3(batches < c->sm_count ? batches : c->sm_count), dim3(kChainWideThreads), resident, c->stream, c->m, c->d_hlr,
-                         c->d_state, key, sample_base, count, chain_out(c));
+        const auto run = [&](auto* kernel, int spl) {
+            const int batches = ceil_div(count, 32 / D * spl);
+            launch_dependent(kernel, dim3(batches < c->sm_count ? batches : c->sm_count), dim3(kChainWideThreads), resident, c->stream, c->m, c->d_hlr,
+                             c->d_state, key, sample_base, count, chain_out(c));
+        };
+        if (c->chain_wide == 2) run(k_chain_wide<D, 2>, 2);
+        else run(k_chain_wide<D, 1>, 1);
     } else if (resident <= 200 * 1024) {
         // all weights fit: one persistent CTA per SM, as many as there are warp batches to hand out
         const int batch = 32 / ChainShape<D>::G * ChainShape<D>::SPL;
@@ -744,7 +748,8 @@ template <int D>
 cudaError_t allow_smem_chain() {
     cudaError_t e = allow_smem(k_chain<D>, 220 * 1024);
     if (e == cudaSuccess) e = allow_smem(k_chain_resident<D>, 220 * 1024);
-    if (e == cudaSuccess) e = allow_smem(k_chain_wide<D>, 220 * 1024);
+    if (e == cudaSuccess) e = allow_smem(k_chain_wide<D, 1>, 220 * 1024);
+    if (e == cudaSuccess) e = allow_smem(k_chain_wide<D, 2>, 220 * 1024);
     if (e == cudaSuccess) e = allow_smem(k_chain_literal<D>, 220 * 1024);
     return e;
 }
@@ -865,14 +870,18 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
                     (c->H <= 256 || (c->H - 256) % 16 == 0) && tc::chain_tc32_smem_bytes(c->H, c->W) <= 227 * 1024;
     c->chain_tcl32 = c->literal && c->use_tc && c->D == tc::kChain32D && c->H % 32 == 0 && c->H <= 512 &&
                      (c->H <= 256 || (c->H - 256) % 16 == 0) && tc::chain_tc32_smem_bytes(c->H, c->W, true) <= 227 * 1024;
-    // D lanes per sample pay while a decision's warps all run at once: up to 16 per SM where the alternative is the resident FMA kernel (H=64,
-    // lag 20: 4096 samples 28 us against 76; H=128, lag 2: 8192 samples 18 against 27, 16384 samples 31 against 29), up to 16
-    // samples per SM where it is a tensor-core chain, whose time hardly depends on the samples (D=16, H=128, lag 20: 2048 samples 43 us against 75;
-    // D=16, H=256, lag 4: 25 against 36, 4096 samples 41 against 35; D=32, H=128, lag 4: 29 against 45, 4096 samples 50 against 45).
+    // D lanes per sample pay for few samples.  Where the alternative is the resident FMA kernel: one sample per lane up to 12 warps per
+    // SM (H=64, lag 20: 4096 samples 28 us against 76; H=128, lag 2: 7000 samples 16.8 against 27), two up to 40 of those warps
+    // (9000 samples 16.7 against 19.8 with one and 27; 16384: 24 against 29; 20000: 32 against 39, lag 20: 95 against 110; 36000: 42
+    // against 41; D=16, H=128, lag 4: 4700 samples 23 against 27 with one and 39, 10000: 46 against 54; D=32 has no registers for
+    // two).  Where it is a tensor-core chain, whose time hardly depends on the samples, up to 16 samples per SM (D=16, H=128, lag 20:
+    // 2048 samples 43 us against 75; D=16, H=256, lag 4: 25 against 36, 4096 samples 41 against 35; D=32, H=128, lag 4: 29
+    // against 45, 4096 samples 50 against 45).
     const int64_t total = cfg->total_samples > 0 ? cfg->total_samples : c->S;       // the same for every shard of a decision, as its draws must be
     const int64_t few = 16 * static_cast<int64_t>(c->sm_count);
-    c->chain_wide = !c->literal && chain_resident_smem_floats(c->D, c->H, c->W) * sizeof(float) <= 200 * 1024 &&
-                    (c->chain_tc || c->chain_tc32 ? total <= few : total * c->D / 32 <= few);
+    const int64_t warps = total * c->D / 32;
+    if (!c->literal && chain_resident_smem_floats(c->D, c->H, c->W) * sizeof(float) <= 200 * 1024)
+        c->chain_wide = c->chain_tc || c->chain_tc32 ? total <= few : warps <= 3 * few / 4 ? 1 : warps <= 5 * few / 2 && c->D <= 16 ? 2 : warps <= few ? 1 : 0;
     if (c->chain_wide) c->chain_tc = c->chain_tc32 = false;
 
     size_t blob_floats = 0;

@@ -800,10 +800,11 @@ k_chain_resident(ModelDev m, const float* __restrict__ hlr, const DevState* __re
 }
 
 // Variant 3: D lanes per sample, one latent component each, for decisions with too few samples to occupy the GPU otherwise.
-// What bounds a small decision is the chain of a step -- D multiply-adds per hidden unit, H / (lanes per sample) hidden units, the sums
-// over the lanes -- with about one warp per scheduler to hide it: with D / 4 lanes and two samples per lane an SM had one warp at N=158, S=2048.
-// N=158, lag 20: 76 -> 23 us; N=16: 13 -> 7 us; N=2175, lag 20, S=1024 against the tensor-core chain on 8 SMs: 76 -> 32 us.  Every weight is
-// read from shared memory for one sample only, so with more than 16 warps per SM the kernels above are faster.
+// What bounds a small decision is the chain of a step -- D multiply-adds per hidden unit, H / (4 D) groups of hidden units per lane, the
+// sums over the lanes -- with about one warp per scheduler to hide it: with D / 4 lanes and two samples per lane an SM had one warp at
+// N=158, S=2048.  N=158, lag 20: 76 -> 23 us; N=16: 13 -> 7 us; N=2175, lag 20, S=1024 against the tensor-core chain on 8 SMs: 76 -> 32 us.
+// With more samples it is the reads of the weights from shared memory, one per lane and sample; SPL = 2 samples per lane
+// share them (N=128, S=16384: 31 us with one, 24 with two, 28.5 by the kernel above).
 // Drawing the noise of 16 steps at once into shared memory, off the chain, changed nothing (23 us).
 constexpr int kChainWideThreads = 512;
 
@@ -832,7 +833,7 @@ __device__ __forceinline__ float normal_element(int g, uint32_t sample, uint32_t
     return (g & 1) ? s : c;
 }
 
-template <int D>
+template <int D, int SPL>
 __global__ void __launch_bounds__(kChainWideThreads, 1)
 k_chain_wide(ModelDev m, const float* __restrict__ hlr, const DevState* __restrict__ st, NoiseKey key,
              uint32_t sample_base, int count, ChainOut out) {
@@ -864,53 +865,71 @@ k_chain_wide(ModelDev m, const float* __restrict__ hlr, const DevState* __restri
     for (int i = threadIdx.x; i < W * H; i += kChainWideThreads) shl[i] = hlr[i] + hlr[W * H + i];
     __syncthreads();
 
-    const int n_batches = ceil_div(count, 32 / D);
+    constexpr int kBatch = 32 / D * SPL;                 // samples per warp and pass
+    const int n_batches = ceil_div(count, kBatch);
     const uint32_t step = st->step;
     // consecutive batches go to different CTAs, so that a small decision still spreads over all SMs
     for (int b = blockIdx.x + gridDim.x * (threadIdx.x >> 5); b < n_batches; b += gridDim.x * (kChainWideThreads / 32)) {
-        const int k = b * (32 / D) + lane / D;
+        const int k = b * kBatch + lane / D * SPL;       // the lane's first sample
         const uint32_t sample = sample_base + static_cast<uint32_t>(k);
-        float z[1][D];
-        group_broadcast<D>(z0, z[0]);
+        float z[SPL][D];
+#pragma unroll
+        for (int s = 0; s < SPL; ++s) group_broadcast<D>(z0, z[s]);
         for (int t = 0; t < W; ++t) {
-            const float eps = normal_element(g, sample, static_cast<uint32_t>(t), step, key);     // off the chain: nothing below feeds it
-            float mu[1][D] = {};
+            float eps[SPL], mu[SPL][D] = {};
+#pragma unroll
+            for (int s = 0; s < SPL; ++s) eps[s] = normal_element(g, sample + s, static_cast<uint32_t>(t), step, key);     // off the chain: nothing below feeds it
             const float* hl = shl + t * H;
             for (int i0 = 4 * g; i0 < H; i0 += 4 * D) {
-                float hid[1][4];
-                hidden_block<D, 1>(sWzT, sbz, H, i0, z, hid);
+                float hid[SPL][4];
+                hidden_block<D, SPL>(sWzT, sbz, H, i0, z, hid);
                 const float4 lr = lds4(hl + i0);
                 const float lrv[4] = {lr.x, lr.y, lr.z, lr.w};
 #pragma unroll
-                for (int c = 0; c < 4; ++c) hid[0][c] = (tanh_fast(hid[0][c]) + lrv[c]) * (1.0f / 3.0f);
-                output_block<D, 1>(sWmu, H, i0, hid, mu);
+                for (int s = 0; s < SPL; ++s)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) hid[s][c] = (tanh_fast(hid[s][c]) + lrv[c]) * (1.0f / 3.0f);
+                output_block<D, SPL>(sWmu, H, i0, hid, mu);
             }
-            const float mu_own = group_reduce_scatter<D>(mu[0], g) + bmu;
-            group_broadcast<D>(mu_own, mu[0]);
-            float pre = bsig;
 #pragma unroll
-            for (int e = 0; e < D; ++e) pre = fmaf(sWsigT[e * D + g], mu[0][e], pre);
-            group_broadcast<D>(fmaf(softplusf(pre), eps, mu_own), z[0]);
+            for (int s = 0; s < SPL; ++s) {
+                const float mu_own = group_reduce_scatter<D>(mu[s], g) + bmu;
+                group_broadcast<D>(mu_own, mu[s]);
+                float pre = bsig;
+#pragma unroll
+                for (int e = 0; e < D; ++e) pre = fmaf(sWsigT[e * D + g], mu[s][e], pre);
+                group_broadcast<D>(fmaf(softplusf(pre), eps[s], mu_own), z[s]);
+            }
         }
-        const float eps = normal_element(g, sample, kStreamTransition, step, key);
-        float mean[1][D] = {}, logvar[1][D] = {};
-        for (int i0 = 4 * g; i0 < H; i0 += 4 * D) {
-            float hid[1][4];
-            hidden_block<D, 1>(sW1T, sb1, H, i0, z, hid);
+        float eps[SPL], mean[SPL][D] = {}, logvar[SPL][D] = {};
 #pragma unroll
-            for (int c = 0; c < 4; ++c) hid[0][c] = fmaxf(hid[0][c], 0.0f);
-            output_block<D, 1>(sW2, H, i0, hid, mean);
-            output_block<D, 1>(sW2 + D * H, H, i0, hid, logvar);
+        for (int s = 0; s < SPL; ++s) eps[s] = normal_element(g, sample + s, kStreamTransition, step, key);
+        for (int i0 = 4 * g; i0 < H; i0 += 4 * D) {
+            float hid[SPL][4];
+            hidden_block<D, SPL>(sW1T, sb1, H, i0, z, hid);
+#pragma unroll
+            for (int s = 0; s < SPL; ++s)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) hid[s][c] = fmaxf(hid[s][c], 0.0f);
+            output_block<D, SPL>(sW2, H, i0, hid, mean);
+            output_block<D, SPL>(sW2 + D * H, H, i0, hid, logvar);
         }
-        const float mean_own = group_reduce_scatter<D>(mean[0], g) + b2_mean, logvar_own = group_reduce_scatter<D>(logvar[0], g) + b2_logvar;
-        group_broadcast<D>(fmaf(expf(0.5f * logvar_own), eps, mean_own), z[0]);
-        const float scale = hidden_scale<D>(out, k, k < count, g, z[0]);
-        for (int i0 = 4 * g; i0 < H; i0 += 4 * D) {
-            float hid[1][4];
-            hidden_block<D, 1>(sW3T, sb3, H, i0, z, hid);
+        float scale[SPL];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) hid[0][c] = fmaxf(hid[0][c], 0.0f);
-            if (k < count) store_hidden<D>(out, k, H, i0, hid[0], scale);
+        for (int s = 0; s < SPL; ++s) {
+            const float mean_own = group_reduce_scatter<D>(mean[s], g) + b2_mean, logvar_own = group_reduce_scatter<D>(logvar[s], g) + b2_logvar;
+            group_broadcast<D>(fmaf(expf(0.5f * logvar_own), eps[s], mean_own), z[s]);
+            scale[s] = hidden_scale<D>(out, k + s, k + s < count, g, z[s]);
+        }
+        for (int i0 = 4 * g; i0 < H; i0 += 4 * D) {
+            float hid[SPL][4];
+            hidden_block<D, SPL>(sW3T, sb3, H, i0, z, hid);
+#pragma unroll
+            for (int s = 0; s < SPL; ++s) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) hid[s][c] = fmaxf(hid[s][c], 0.0f);
+                if (k + s < count) store_hidden<D>(out, k + s, H, i0, hid[s], scale[s]);
+            }
         }
     }
 }

@@ -17,10 +17,13 @@ def _lib():
 
 
 # every D; hidden widths with idle lanes (H < 4 D) and with a ragged last block; sample counts around a warp's 32 / D; windows of
-# one step and long ones; both precisions; the largest decision that takes this chain and the smallest that does not
+# one step and long ones; both precisions; one and two samples per lane; the largest decision that takes either form and the
+# smallest that does not (148 SMs)
 @pytest.mark.parametrize("N,D,H,lag,S,prec", [(5, 4, 4, 0, 1, 0), (17, 4, 36, 3, 9, 0), (9, 8, 8, 20, 5, 0), (40, 8, 72, 20, 131, 0), (33, 16, 48, 1, 3, 0),
                                               (64, 16, 256, 4, 77, 1), (20, 32, 32, 0, 2, 0), (50, 32, 160, 6, 65, 2), (16, 16, 64, 2, 2368, 1),
-                                              (16, 16, 64, 2, 2369, 1), (16, 8, 32, 2, 9472, 0), (16, 8, 32, 2, 9504, 0)])
+                                              (16, 16, 64, 2, 2369, 1), (16, 8, 32, 2, 7104, 0), (16, 8, 32, 2, 7109, 0),
+                                              (16, 8, 32, 2, 23680, 0), (16, 8, 32, 2, 23689, 0), (16, 4, 32, 1, 20001, 0),
+                                              (33, 16, 48, 1, 4001, 0), (16, 32, 32, 1, 1999, 0), (16, 32, 32, 1, 2400, 0)])
 def test_wide_chain_meets_the_oracle(N, D, H, lag, S, prec):
     w = inputs.make_weights(N, D, H, seed=N + D, fan_in_ref=32, bf16=(prec == 2))
     gpu = binding.Cutoff(N, D, H, lag, S, precision=prec, seed=3)
