@@ -106,7 +106,7 @@ struct cutoff_ctx {
 
     // pinned host memory that kernels read and write directly (one address on both sides)
     float* h_stage = nullptr;       // [N] run-times of a host push
-    DevState* h_state = nullptr;    // the device state as of the last push or decision
+    DevState* h_state = nullptr;    // the device state as of the last decision, or push that the host waited for
     float* h_E = nullptr;           // [N] expected order statistics of the last decision
     float* h_omega = nullptr;       // [N] throughput per cutoff
 
@@ -1192,13 +1192,15 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
     return CUTOFF_OK;
 }
 
-static void launch_push(cutoff_ctx* c, const float* src) {
-    launch_dependent(k_push, dim3(1), dim3(kPushThreads), 0, c->stream, src, c->d_ring, c->d_state, c->N, c->W, c->h_state);
+// With `report` the device state as the push leaves it goes to h_state, for a call that waits for the push.  The others leave h_state to
+// the decisions: one that is in flight reports its own state to cutoff_fetch, not what a push behind it found.
+static void launch_push(cutoff_ctx* c, const float* src, bool report) {
+    launch_dependent(k_push, dim3(1), dim3(kPushThreads), 0, c->stream, src, c->d_ring, c->d_state, c->N, c->W, report ? c->h_state : nullptr);
     c->launches += 1;
 }
 
-static int push_common(cutoff_ctx* c, const float* src) {
-    launch_push(c, src);
+static int push_common(cutoff_ctx* c, const float* src, bool report) {
+    launch_push(c, src, report);
     if (c->weights_loaded && !c->proj_stale) launch_projection(c, true);     // else every slot is redone before the next decision
     CU_CHECK(c, cudaGetLastError());
     c->pushes += 1;
@@ -1209,7 +1211,7 @@ int cutoff_push_async(cutoff_ctx* c, const float* runtimes_sec_device) {
     if (!c || !runtimes_sec_device) return CUTOFF_ERR_BAD_ARG;
     DeviceGuard guard(c->cfg.device);
     CU_CHECK(c, guard.err);
-    return push_common(c, runtimes_sec_device);
+    return push_common(c, runtimes_sec_device, false);
 }
 
 // Push with a censoring mask: land run-times and mask on the device, replace the censored entries by
@@ -1238,7 +1240,7 @@ static int push_censored(cutoff_ctx* c, const float* runtimes_sec, int on_device
     k_impute<<<c->N < kImputeCtas ? c->N : kImputeCtas, kImputeThreads, 0, c->stream>>>(src, mask, c->d_stage, c->d_x, c->ldx, c->S, c->N, c->d_state, key);
     c->launches += 1;
     c->draws_valid = false;                                 // one step's draws serve one push
-    int rc = push_common(c, c->d_stage);
+    int rc = push_common(c, c->d_stage, true);
     if (rc) return rc;
     CU_CHECK(c, cudaStreamSynchronize(c->stream));
     if (c->h_state->error_flags & (kErrBadValue | kErrNoFinisher)) {
@@ -1259,9 +1261,9 @@ int cutoff_push(cutoff_ctx* c, const float* runtimes_sec, int on_device, const u
             if (!(runtimes_sec[j] > 0.0f) || !std::isfinite(runtimes_sec[j])) return CUTOFF_ERR_BAD_VALUE;
         CU_CHECK(c, cudaStreamSynchronize(c->stream));       // the landing buffer may still be in use
         std::memcpy(c->h_stage, runtimes_sec, sizeof(float) * c->N);
-        return push_common(c, c->h_stage);
+        return push_common(c, c->h_stage, false);
     }
-    const int rc = push_common(c, runtimes_sec);
+    const int rc = push_common(c, runtimes_sec, true);
     if (rc) return rc;
     CU_CHECK(c, cudaStreamSynchronize(c->stream));
     if (c->h_state->error_flags & kErrBadValue) {
@@ -1331,7 +1333,7 @@ static int build_graph(cutoff_ctx* c, bool from_host) {
     refresh_projections(c);                        // not part of the graph: replays only project the vector they push
     const int64_t launches_before = c->launches;
     CU_CHECK(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-    launch_push(c, from_host ? c->h_stage : c->d_stage);
+    launch_push(c, from_host ? c->h_stage : c->d_stage, false);
     launch_projection(c, true);
     const bool timing = c->timing;
     c->timing = false;

@@ -14,7 +14,8 @@ namespace cutoff {
 // ---------------------------------------------------------------------------------------------
 constexpr int kPushThreads = 1024, kPushPer = 4;             // N <= 4096: every run-time is read once, into a register
 
-// src may be pinned host memory (read over the bus: one round trip, less than a copy and the launch behind it).
+// src may be pinned host memory (read over the bus: one round trip, less than a copy and the launch behind it).  host_state: null = do
+// not report.
 __global__ void __launch_bounds__(kPushThreads) k_push(const float* __restrict__ src, float* __restrict__ ring,
                                                        DevState* st, int N, int W, DevState* host_state) {
     __shared__ double red[kPushThreads / 32];
