@@ -106,6 +106,7 @@ struct cutoff_ctx {
 
     // pinned host memory that kernels read and write directly (one address on both sides)
     float* h_stage = nullptr;       // [N] run-times of a host push
+    bool stage_in_use = false;      // by a push that may not have been waited for
     DevState* h_state = nullptr;    // the device state as of the last decision, or push that the host waited for
     float* h_E = nullptr;           // [N] expected order statistics of the last decision
     float* h_omega = nullptr;       // [N] throughput per cutoff
@@ -1261,7 +1262,9 @@ int cutoff_push(cutoff_ctx* c, const float* runtimes_sec, int on_device, const u
             if (!(runtimes_sec[j] > 0.0f) || !std::isfinite(runtimes_sec[j])) return CUTOFF_ERR_BAD_VALUE;
         CU_CHECK(c, cudaStreamSynchronize(c->stream));       // the landing buffer may still be in use
         std::memcpy(c->h_stage, runtimes_sec, sizeof(float) * c->N);
-        return push_common(c, c->h_stage, false);
+        const int rc = push_common(c, c->h_stage, false);
+        c->stage_in_use = true;
+        return rc;
     }
     const int rc = push_common(c, runtimes_sec, true);
     if (rc) return rc;
@@ -1378,7 +1381,9 @@ int cutoff_step(cutoff_ctx* c, const float* runtimes_sec, int32_t* c_out) {
         const int rc = build_graph(c, true);
         if (rc) return rc;
     }
-    std::memcpy(c->h_stage, runtimes_sec, sizeof(float) * c->N);     // the stream is idle: every call ends synchronised
+    if (c->stage_in_use) CU_CHECK(c, cudaStreamSynchronize(c->stream));   // cutoff_push returns while its kernel has yet to read the buffer
+    c->stage_in_use = false;
+    std::memcpy(c->h_stage, runtimes_sec, sizeof(float) * c->N);
     refresh_projections(c);                        // after a restore or new weights; the replay then adds the new vector
     CU_CHECK(c, cudaGraphLaunch(c->graph_exec, c->stream));
     CU_CHECK(c, cudaStreamSynchronize(c->stream));

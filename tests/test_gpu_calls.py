@@ -46,3 +46,21 @@ def test_a_bad_push_behind_a_decision_does_not_take_the_decision_away(N, S):
     window = ctx.debug_window()                          # ... and never entered the window
     assert np.array_equal(window, inputs.make_trace(N, 7, seed=S, sigma=0.3)[:2])
     assert ctx.predict()[0] >= 0
+
+
+def test_a_host_push_keeps_its_run_times_when_a_replayed_step_follows():
+    # both land in one buffer on the host: the step may not fill it before the push's kernel has read it
+    N, lag = 4096, 3
+    ctx, trace = _running(N, 4, 32, lag, 64, flags=binding.FLAG_GRAPH)
+    lib, c = binding.load_library(), binding.C.c_int32(0)
+    ctx.predict()
+    ctx.step(trace[0])                                   # captured here
+    window = list(ctx.debug_window())
+    rng = np.random.default_rng(0)
+    for _ in range(200):
+        first, second = rng.uniform(0.5, 2.0, (2, N)).astype(np.float32)
+        a, b = first.ctypes.data, second.ctypes.data
+        push, step = lib.cutoff_push, lib.cutoff_step
+        assert push(ctx._h, a, 0, None) == 0 and step(ctx._h, b, binding.C.byref(c)) == 0
+        window = (window + [first, second])[-(lag + 1):]
+        assert np.array_equal(ctx.debug_window(), np.stack(window))
