@@ -223,14 +223,18 @@ __global__ void __launch_bounds__(1024) k_running_moments(int64_t T, int N, doub
     double before1 = 0.0, before2 = 0.0;
     for (int64_t t0 = 0; t0 < T; t0 += 1024) {
         const int64_t t = t0 + threadIdx.x;
-        const double s1 = t < T ? sum1[t] : 0.0, s2 = t < T ? sum2[t] : 0.0;
-        double a = s1, b = s2;
+        double a = t < T ? sum1[t] : 0.0, b = t < T ? sum2[t] : 0.0;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const double oa = __shfl_up_sync(0xffffffffu, a, off), ob = __shfl_up_sync(0xffffffffu, b, off);
             if (lane >= off) { a += oa; b += ob; }
         }
         if (lane == 31) { w1[warp] = a; w2[warp] = b; }
+        // what the lanes before this one have, and not its own sum minus its own value: that would leave the rounding of a far
+        // outlier in the moments of the very step that is to be decided without it
+        a = __shfl_up_sync(0xffffffffu, a, 1);
+        b = __shfl_up_sync(0xffffffffu, b, 1);
+        if (lane == 0) a = b = 0.0;
         __syncthreads();
         double pa = before1, pb = before2, all1 = before1, all2 = before2;
         for (int k = 0; k < 32; ++k) {
@@ -240,7 +244,7 @@ __global__ void __launch_bounds__(1024) k_running_moments(int64_t T, int N, doub
         }
         if (t < T) {
             const double count = static_cast<double>(t) * static_cast<double>(N);
-            const double sum_a = pa + (a - s1), sum_b = pb + (b - s2);
+            const double sum_a = pa + a, sum_b = pb + b;
             const double mu = t > 0 ? sum_a / count : 0.0;
             const double var = t > 0 ? sum_b / count - mu * mu : 0.0;
             sum1[t] = mu;

@@ -123,3 +123,20 @@ def test_calls_from_several_threads_and_streams_do_not_share_scratch():
     for t in threads:
         t.join()
     assert not wrong
+
+
+@pytest.mark.parametrize("N,T,outlier", [(24, 80, 1e15), (158, 40, 1e18), (5, 1100, 1e12)])
+def test_order_baseline_does_not_see_the_step_it_decides(N, T, outlier):
+    # a step's own run-times, however far out, must not reach its own moments, not even as a rounding error.  Moments are sums
+    # in double whose order differs between the two sides: 1e-12 of the throughput at most
+    import torch
+    trace = _trace(N, T, seed=N + T)
+    at = T - T // 4
+    trace[at] = np.float32(outlier)
+    got = binding.order_baseline(torch.from_numpy(trace).cuda()).cpu().numpy()
+    x = trace.astype(np.float64)
+    for t in range(1, at + 1):
+        mu = float(x[:t].mean())
+        e = E.elfving_expected(N, mu, float(np.sqrt(max(float((x[:t] * x[:t]).mean()) - mu * mu, 0.0))))
+        want = E.cutoff_from_expected(e)
+        assert got[t] == want or abs(got[t] / e[got[t] - 1] - want / e[want - 1]) <= 1e-9 * abs(want / e[want - 1]), t
