@@ -362,9 +362,10 @@ int cutoff_adam_step(int device, int64_t n, float* params, const float* grads, f
  *   x         device, n_rows x ldx floats, row-major; entries beyond n in a row are ignored
  *   n_rows    1 .. CUTOFF_STATIC_MAX_ROWS;   n  1 .. CUTOFF_STATIC_MAX_N;   ldx >= n
  *   sums      device, n doubles, overwritten
- * Accuracy: the rows go through in blocks of 131072; inside a block a warp adds at most 64 sorted rows in
- * single precision, everything above that is added in double, so the error of a sum does not grow with
- * n_rows beyond that of 64 single-precision additions (about 4e-6 relative to the largest partial sum).
+ * Accuracy: the rows go through in blocks of at most 131072; inside a block a warp adds at most 64 sorted rows
+ * in single precision.  Everything above that is added in double and rounded to single precision once per CTA,
+ * so the error of a sum does not grow with n_rows beyond that of 64 single-precision additions (about 4e-6
+ * relative to the largest partial sum).
  *   stream    cudaStream_t to run on (NULL = default stream); the call only enqueues work
  * The call performs no cudaMalloc, cudaFree or other allocating routine.  Its only scratch is a
  * fixed array of CUTOFF_STATIC_SCRATCH_BYTES that is part of the library image: every GPU that

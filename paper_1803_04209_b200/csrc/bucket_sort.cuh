@@ -359,7 +359,8 @@ __device__ __forceinline__ bool cta_bucket_sort(float (&v)[E], uint32_t row, flo
 constexpr int kBulk = 0;
 // Warps per SM the registers allow: two arrays of E (keys and sums) and about 60 more.  The variant that also sums squares
 // (SQ) keeps the same split of the rows, so that the means do not depend on it; its third array is spilled in part.
-template <int E> constexpr int kBucketWarps = E >= 24 ? 16 : 24;
+constexpr int kBucketFewestWarps = 16;
+template <int E> constexpr int kBucketWarps = E >= 24 ? kBucketFewestWarps : 24;
 
 template <int E> __host__ __device__ constexpr size_t bucket_warp_floats() { return 32 * (E + BucketShape<E>::kLaneWords); }
 template <int E> constexpr size_t bucket_smem_bytes() { return 128 + kBucketWarps<E> * (bucket_warp_floats<E>() * 4 + 8) + 16; }
@@ -372,12 +373,7 @@ __device__ __forceinline__ void store_partial_row(const float (&acc)[E], float* 
 #pragma unroll
     for (int r = 0; r < E; ++r) stage[warp * 32 * E + lane * E + r] = acc[r];
     __syncthreads();
-    for (int j = threadIdx.x; j < n; j += WARPS * 32) {
-        float s = 0.0f;
-#pragma unroll
-        for (int w = 0; w < WARPS; ++w) s += stage[w * 32 * E + j];
-        out[j] = s;
-    }
+    for (int j = threadIdx.x; j < n; j += WARPS * 32) out[j] = add_warps<WARPS>(stage, 32 * E, j);
 }
 
 template <int E, bool SQ, int COPY>

@@ -2131,16 +2131,18 @@ extern "C" int cutoff_sorted_row_sums_static(int device, const float* x, int64_t
     float* partial = g_static_partial_addr[device];
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int P = next_pow2(n) < 32 ? 32 : next_pow2(n);
-    // The rows go through in blocks of kStaticBlockRows: within a block a warp adds at most kStaticRowsPerWarp
-    // sorted rows in fp32, then the block's partial rows are added to `sums` in double.  The blocks run one after
-    // the other on the stream, so they can share the scratch array.
-    for (int64_t r0 = 0; r0 < n_rows; r0 += kStaticBlockRows) {
-        const int rows = static_cast<int>(n_rows - r0 < kStaticBlockRows ? n_rows - r0 : kStaticBlockRows);
+    // The rows go through in blocks: within a block a warp adds at most kStaticRowsPerWarp sorted rows in fp32 (the bucket sort has a
+    // CTA per SM, so its blocks are shorter on a GPU of less than 128 SMs), then the block's partial rows are added to `sums`
+    // in double.  The blocks run one after the other on the stream, so they can share the scratch array.
+    const int sms = g_static_sms[device];
+    const int64_t bucket_rows = static_cast<int64_t>(kStaticRowsPerWarp) * kBucketFewestWarps * (sms < kStaticParts ? sms : kStaticParts);
+    const int64_t block_rows = n > 128 && bucket_rows < kStaticBlockRows ? bucket_rows : kStaticBlockRows;
+    for (int64_t r0 = 0; r0 < n_rows; r0 += block_rows) {
+        const int rows = static_cast<int>(n_rows - r0 < block_rows ? n_rows - r0 : block_rows);
         const float* xb = x + static_cast<size_t>(r0) * ldx;
         // every CTA of the grid writes its whole partial row (zeros if it had no sample), and the
         // column sum reads exactly `grid` rows: stale contents of the shared array are never read
         int grid = 0;
-        const int sms = g_static_sms[device];
         if (by_buckets(n, rows)) {
             switch (keys_per_thread(n, 32)) {
                 case 8: grid = launch_static_bucket<8>(xb, ldx, n, rows, partial, s, sms); break;

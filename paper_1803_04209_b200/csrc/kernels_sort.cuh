@@ -234,10 +234,19 @@ __device__ __forceinline__ void cta_bitonic_sort(T (&v)[32], T* xch) {
 
 // ---------------------------------------------------------------------------------------------
 // Sort + accumulate, one warp per sample row, N <= 32*E.  Each warp keeps the running sum of its
-// sorted rows in registers; a CTA adds its warps in a fixed order and writes one partial row.
+// sorted rows in registers; a CTA adds its warps in a fixed order, in double, and writes one partial row.
 // The network sorts any arrangement, so rows are loaded coalesced (element r*32 + lane).
 // ---------------------------------------------------------------------------------------------
 constexpr int kSortWarps = 8;
+
+// Position j of the CTA's warps, whose sums stand in rows of `pitch` floats: added in double, rounded to single once.
+template <int WARPS>
+__device__ __forceinline__ float add_warps(const float* stage, int pitch, int j) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) s += static_cast<double>(stage[w * pitch + j]);
+    return static_cast<float>(s);
+}
 
 template <int E>
 __global__ void __launch_bounds__(kSortWarps * 32) k_sort_sum_warp(const float* __restrict__ x, int ldx, int N,
@@ -262,12 +271,8 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_sum_warp(const float* 
 #pragma unroll
     for (int r = 0; r < E; ++r) stage[warp][lane * E + r] = acc[r];
     __syncthreads();
-    for (int j = threadIdx.x; j < N; j += kSortWarps * 32) {
-        float s = 0.0f;
-#pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) s += stage[w][j];
-        partial[static_cast<size_t>(blockIdx.x) * N + j] = s;
-    }
+    for (int j = threadIdx.x; j < N; j += kSortWarps * 32)
+        partial[static_cast<size_t>(blockIdx.x) * N + j] = add_warps<kSortWarps>(&stage[0][0], 32 * E, j);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -370,23 +375,15 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_sum_tma(const float* _
 #pragma unroll
     for (int r = 0; r < E; ++r) stage[warp * 32 * E + lane * E + r] = acc[r];
     __syncthreads();
-    for (int j = threadIdx.x; j < N; j += kSortWarps * 32) {
-        float s = 0.0f;
-#pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) s += stage[w * 32 * E + j];
-        partial[static_cast<size_t>(blockIdx.x) * N + j] = s;
-    }
+    for (int j = threadIdx.x; j < N; j += kSortWarps * 32)
+        partial[static_cast<size_t>(blockIdx.x) * N + j] = add_warps<kSortWarps>(stage, 32 * E, j);
     if (SQ) {                                          // the same reduction for the sums of squares
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < E; ++r) stage[warp * 32 * E + lane * E + r] = acc_sq[SQ ? r : 0];
         __syncthreads();
-        for (int j = threadIdx.x; j < N; j += kSortWarps * 32) {
-            float s = 0.0f;
-#pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) s += stage[w * 32 * E + j];
-            partial_sq[static_cast<size_t>(blockIdx.x) * N + j] = s;
-        }
+        for (int j = threadIdx.x; j < N; j += kSortWarps * 32)
+            partial_sq[static_cast<size_t>(blockIdx.x) * N + j] = add_warps<kSortWarps>(stage, 32 * E, j);
     }
 }
 

@@ -117,3 +117,38 @@ def test_decision_sums_of_tied_and_clustered_draws(N, S):
     ctx.predict()
     _check(ctx.get_partial_sums(), draws)
     ctx.close()
+
+
+def _one_value_decision(N, S, v):
+    w = inputs.make_weights(N, 4, 32, seed=1, fan_in_ref=32)
+    w["W4"][:] = 0.0
+    w["b4"][:N] = v
+    w["b4"][N:] = -400.0                                  # every draw is v exactly
+    ctx = binding.Cutoff(N, 4, 32, 1, S, precision=0, seed=N)
+    ctx.load_weights(w)
+    for x in inputs.make_trace(N, 2, 7, sigma=0.3):
+        ctx.push(x)
+    ctx.predict()
+    sums = ctx.get_partial_sums()
+    ctx.close()
+    return sums
+
+
+# The warps of a CTA are added in double and rounded to single once: half a unit in the last place of the CTA's sum, 2^-24 relative.
+@pytest.mark.parametrize("N,S", [(130, 65536), (300, 65536), (700, 65536), (1024, 65536)])
+def test_the_warps_of_a_cta_are_added_in_double(N, S):
+    for v in (1 + 2.0 ** -18, 1 + 3 * 2.0 ** -18, 1 + 5 * 2.0 ** -17, 1.5 + 2.0 ** -18):
+        sums = _one_value_decision(N, S, np.float32(v))
+        assert np.all(np.abs(sums - S * v) <= 2.0 ** -24 * S * v), v
+
+
+@pytest.mark.parametrize("n", [130, 300, 700, 1024])
+def test_the_warps_of_a_cta_of_the_static_call_are_added_in_double(n):
+    import torch
+    sums = torch.empty(n, dtype=torch.float64, device="cuda")
+    for v in (1 + 2.0 ** -18, 1 + 3 * 2.0 ** -18, 1 + 5 * 2.0 ** -17):
+        x = torch.full((131072 + 70000, n + 1), v, dtype=torch.float32, device="cuda")
+        for rows, tolerance in ((65536, 2.0 ** -24), (x.shape[0], REL)):           # one block of rows; two, the first with chains beyond 32
+            for y in (x[:rows, :n], x.view(-1)[: rows * n].view(rows, n)):
+                binding.sorted_row_sums_static(y, sums, n=n)
+                assert np.all(np.abs(sums.cpu().numpy() - rows * v) <= tolerance * rows * v), (rows, v)
