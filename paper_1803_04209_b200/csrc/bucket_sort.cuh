@@ -458,24 +458,44 @@ k_bucket_sum_warp(const float* __restrict__ x, int ldx, int n, int count, float*
 
 // ---------------------------------------------------------------------------------------------
 // Sort + accumulate, four warps per row, 128 (E - 4) < N <= 128 E; otherwise as above, one partial row per CTA.
+// A thread's running sums go through at most kWideRun rows in registers, then into the thread's own totals: of the sums in shared
+// memory, of the squares (SQ: there is no room for both) at sq_totals [CTA][128 E].  One chain through all of a CTA's rows, twice
+// as long as with the eight CTAs per SM of a register sort, has twice its error (rms relative to the sum of magnitudes, N=4096:
+// S=32768 4.4e-9 against 2.2e-9, S=8192 2.3e-9 against 1.3e-9); runs of 8 rows 1.2e-9 and 1.7e-9, of 4 rows 1.1e-9 and 1.3e-9.  The
+// decision of N=4096, S=32768 takes 0.4 % longer for it (864 and 868 us); more CTAs instead would cost 10 us in the column sums.
 // ---------------------------------------------------------------------------------------------
 template <int E> constexpr int kBucketWideCtas = E >= 24 ? 4 : (E >= 16 ? 5 : 6);
+constexpr int kWideRun = 4;
 
 template <int E> constexpr size_t bucket_wide_smem_bytes() {
-    return 128 + (4096 + 128 * BucketShape<E>::kLaneWords) * 4 + 16 * 4 + 8 + 8;
+    return 128 + (4096 + 128 * BucketShape<E>::kLaneWords + 128 * E) * 4 + 16 * 4 + 8 + 8;
+}
+
+// The thread's entries of a CTA's totals: entry r at total[r * 128] (coalesced, free of conflicts).  What the addition rounds away
+// stays in the running sum (Dekker 1971), so that the totals add no error of their own.
+template <int E>
+__device__ __forceinline__ void add_to_totals(float* total, float (&acc)[E], bool first) {
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const float old = first ? 0.0f : total[r * 128], sum = old + acc[r];
+        total[r * 128] = sum;
+        acc[r] = fabsf(sum) < INFINITY ? acc[r] - (sum - old) : 0.0f;
+    }
 }
 
 template <int E, bool SQ>
 __global__ void __launch_bounds__(128, kBucketWideCtas<E>)
 k_bucket_sum_cta(const float* __restrict__ x, int ldx, int n, int count, float* __restrict__ partial,
-                 float* __restrict__ partial_sq, DevState* st) {
+                 float* __restrict__ partial_sq, float* __restrict__ sq_totals, DevState* st) {
     using namespace cutoff::async;
     extern __shared__ __align__(16) uint8_t sm_bucket[];
     constexpr int kCounters = 128 * BucketShape<E>::kLaneWords;
     float* data = reinterpret_cast<float*>(sm_bucket + (128u - (smem_u32(sm_bucket) & 127u)) % 128u);
     const int t = threadIdx.x;
     const uint32_t row_s = smem_u32(data), hist = row_s + 4096 * 4;
-    uint32_t* red = reinterpret_cast<uint32_t*>(data + 4096 + kCounters);
+    float* total = data + 4096 + kCounters + t;
+    uint32_t* red = reinterpret_cast<uint32_t*>(data + 4096 + kCounters + 128 * E);
+    float* total_sq = SQ ? sq_totals + static_cast<size_t>(blockIdx.x) * 128 * E + t : nullptr;
     const uint32_t bar = smem_u32(red + 16);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(red + 18);
     const uint32_t row_bytes = static_cast<uint32_t>(ldx) * 4u;
@@ -504,9 +524,9 @@ k_bucket_sum_cta(const float* __restrict__ x, int ldx, int n, int count, float* 
     const int row0 = blockIdx.x;
     if (row0 < count) request(row0);
     BucketMap map{};
-    uint32_t parity = 0;
-    for (int row = row0; row < count; row += gridDim.x, parity ^= 1u) {
-        const bool arrived = mbar_wait(bar, parity, abort_flag, st);
+    uint32_t done = 0;                                       // rows; the barrier's parity is that of their number
+    for (int row = row0; row < count; row += gridDim.x) {
+        const bool arrived = mbar_wait(bar, done & 1u, abort_flag, st);
         float v[E];
         if (!cta_bucket_sort<E>(v, row_s, data, hist, red, n, arrived, row == row0, map, [&] {
                 const int next = row + static_cast<int>(gridDim.x);
@@ -514,22 +534,27 @@ k_bucket_sum_cta(const float* __restrict__ x, int ldx, int n, int count, float* 
                 __syncthreads();
                 if (next < count) request(next);
             })) {
-            mbar_wait_quiet(bar, parity);
+            mbar_wait_quiet(bar, done & 1u);
             break;
         }
 #pragma unroll
         for (int r = 0; r < E; ++r) acc[r] += v[r];
-        if (SQ) {
+        if constexpr (SQ) {
 #pragma unroll
-            for (int r = 0; r < E; ++r) acc_sq[SQ ? r : 0] = fmaf(v[r], v[r], acc_sq[SQ ? r : 0]);
+            for (int r = 0; r < E; ++r) acc_sq[r] = fmaf(v[r], v[r], acc_sq[r]);
+        }
+        ++done;
+        if (done % kWideRun == 0) {
+            add_to_totals<E>(total, acc, done == kWideRun);
+            if constexpr (SQ) add_to_totals<E>(total_sq, acc_sq, done == kWideRun);
         }
     }
 #pragma unroll
     for (int r = 0; r < E; ++r) {
         const int j = t * E + r;
         if (j < n) {
-            partial[static_cast<size_t>(blockIdx.x) * n + j] = acc[r];
-            if (SQ) partial_sq[static_cast<size_t>(blockIdx.x) * n + j] = acc_sq[SQ ? r : 0];
+            partial[static_cast<size_t>(blockIdx.x) * n + j] = done < kWideRun ? acc[r] : total[r * 128] + acc[r];
+            if constexpr (SQ) partial_sq[static_cast<size_t>(blockIdx.x) * n + j] = done < kWideRun ? acc_sq[r] : total_sq[r * 128] + acc_sq[r];
         }
     }
 }

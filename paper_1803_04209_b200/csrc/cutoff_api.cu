@@ -75,6 +75,7 @@ struct cutoff_ctx {
     float* d_x = nullptr;           // [chunk_rows][ldx]
     float* d_partial = nullptr;     // [n_chunks * sort_grid][N]; a second block of kPartialRows rows holds sums of squares
     float* d_std = nullptr;         // [N] spread of each order statistic (when asked for)
+    float* d_sq_totals = nullptr;   // [CTA][128 E] for wide rows (when asked for)
     bool want_std = false;
     bool have_std = false;
     double* d_sums = nullptr;       // [N]
@@ -276,7 +277,7 @@ void free_all(cutoff_ctx* c) {
     cudaFree(c->d_blob); cudaFree(c->d_WT); cudaFree(c->d_WhR); cudaFree(c->d_chain_image);
     if (c->h_mask) cudaFreeHost(c->h_mask); cudaFree(c->d_ring); cudaFree(c->d_stage);
     cudaFree(c->d_state); cudaFree(c->d_proj); cudaFree(c->d_hlr); cudaFree(c->d_v); cudaFree(c->d_x);
-    cudaFree(c->d_partial); cudaFree(c->d_std); cudaFree(c->d_sums);
+    cudaFree(c->d_partial); cudaFree(c->d_sq_totals); cudaFree(c->d_std); cudaFree(c->d_sums);
     if (c->h_stage) cudaFreeHost(c->h_stage);
     if (c->h_state) cudaFreeHost(c->h_state);
     if (c->h_E) cudaFreeHost(c->h_E);
@@ -352,7 +353,7 @@ void launch_bucket_warp(cutoff_ctx* c, int count, float* partial) {
 template <int E, bool SQ>
 void launch_bucket_cta_sq(cutoff_ctx* c, int count, float* partial) {
     launch_dependent(k_bucket_sum_cta<E, SQ>, dim3(c->sort_grid), dim3(128), bucket_wide_smem_bytes<E>(), c->stream,
-                     c->d_x, c->ldx, c->N, count, partial, partial + static_cast<size_t>(kPartialRows) * c->N, c->d_state);
+                     c->d_x, c->ldx, c->N, count, partial, partial + static_cast<size_t>(kPartialRows) * c->N, c->d_sq_totals, c->d_state);
 }
 template <int E>
 void launch_bucket_cta(cutoff_ctx* c, int count, float* partial) {
@@ -1708,6 +1709,15 @@ int cutoff_set_option(cutoff_ctx* c, const char* name, int64_t value) {
         if (value != 0 && value != 1) return CUTOFF_ERR_BAD_ARG;
         if (value && c->cfg.total_samples > 0 && c->cfg.total_samples != c->S) return CUTOFF_ERR_UNSUPPORTED;
         if (c->graph_exec || c->graph_dev_exec) return CUTOFF_ERR_STATE;   // the captured graph has the other sort kernel in it
+        if (value && c->N > 1024 && !c->d_sq_totals) {
+            DeviceGuard guard(c->cfg.device);
+            CU_CHECK(c, guard.err);
+            const size_t ctas = static_cast<size_t>(c->sm_count) * bucket_wide_ctas(c->N);
+            if (cudaMalloc(&c->d_sq_totals, sizeof(float) * ctas * 128 * keys_per_thread(c->N, 128)) != cudaSuccess) {
+                cudaGetLastError();
+                return CUTOFF_ERR_NOMEM;
+            }
+        }
         c->want_std = value != 0;
         return CUTOFF_OK;
     }

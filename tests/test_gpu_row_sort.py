@@ -152,3 +152,38 @@ def test_the_warps_of_a_cta_of_the_static_call_are_added_in_double(n):
             for y in (x[:rows, :n], x.view(-1)[: rows * n].view(rows, n)):
                 binding.sorted_row_sums_static(y, sums, n=n)
                 assert np.all(np.abs(sums.cpu().numpy() - rows * v) <= tolerance * rows * v), (rows, v)
+
+
+# A thread of a wide decision adds 4 rows in single precision, then those to its totals, whose rounding is carried on: 4 copies of a
+# value of 21 bits add up without rounding, so all that is lost is the one rounding of a CTA's result.
+@pytest.mark.parametrize("N", [1025, 1537, 2049, 2561, 3073, 4096])
+def test_wide_decisions_keep_their_single_precision_sums_short(N):
+    for v in (1 + 2.0 ** -19, 1 + 3 * 2.0 ** -20):
+        sums = _one_value_decision(N, 32768, np.float32(v))
+        assert np.all(np.abs(sums - 32768 * v) <= 2.0 ** -24 * 32768 * v), v
+
+
+# rows per thread around multiples of the 4 that are added in registers, in one pass and in several; squares too
+@pytest.mark.parametrize("N,S,pass_rows", [(1100, 888 * 3, 0), (1100, 888 * 4, 0), (1100, 888 * 8, 0), (1700, 740 * 9 - 1, 0), (4096, 592 * 16, 0), (4096, 592 * 16 + 1, 0),
+                                           (2200, 20000, 0), (3000, 30000, 10000), (3500, 9000, 1024)])
+def test_wide_decisions_around_the_length_of_a_run(N, S, pass_rows):
+    got = []
+    for std in (0, 1):
+        ctx = binding.Cutoff(N, 4, 32, 1, S, precision=0, seed=N)
+        ctx.load_weights(inputs.make_weights(N, 4, 32, seed=N, fan_in_ref=32))
+        ctx.set_option("order_stat_std", std)
+        if pass_rows:
+            ctx.set_option("pass_rows", pass_rows)
+        for x in inputs.make_trace(N, 2, 7, sigma=0.3):
+            ctx.push(x)
+        want, size, squares = np.zeros(N), np.zeros(N), np.zeros(N)
+        for k in range(0, S if std else 0, 4096):
+            draws = np.sort(ctx.debug_samples(k, min(4096, S - k)), axis=1).astype(np.float64)
+            want, size, squares = want + draws.sum(axis=0), size + np.abs(draws).sum(axis=0), squares + (draws * draws).sum(axis=0)
+        ctx.predict()
+        got.append(ctx.get_partial_sums())
+    assert np.array_equal(got[0], got[1])                 # the sums do not depend on the squares
+    assert np.all(np.abs(got[1] - want) <= REL * size)
+    scale = float(ctx.get_stats()[0][-1]) * S / want[-1]
+    sd = np.sqrt(squares / S - (want / S) ** 2) * scale
+    assert np.all(np.abs(ctx.get_order_stat_std() - sd) <= 1e-5 + REL * squares / S * scale * scale / (2 * sd))
