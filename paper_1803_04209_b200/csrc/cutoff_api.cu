@@ -235,14 +235,15 @@ cudaError_t upload(void* dst, const void* src, size_t bytes) {
     return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
 }
 
-// |A x + b| <= slope * max |x| + offset, from the matrix as the tensor cores see it (rounded up a little)
-void layer_bound(const float* w, const float* b, size_t rows, size_t cols, float (&bound)[2]) {
+// |A x + b| <= slope * max |x| + offset, from the matrix as the tensor cores see it (rounded up a little); of a ReLU layer
+// relu(A x + b), where negative biases only lower the result
+void layer_bound(const float* w, const float* b, size_t rows, size_t cols, bool relu, float (&bound)[2]) {
     double l1 = 0.0, mb = 0.0;
     for (size_t r = 0; r < rows; ++r) {
         double s = 0.0;
         for (size_t k = 0; k < cols; ++k) s += std::fabs(static_cast<double>(w[r * cols + k]));
         l1 = std::fmax(l1, s);
-        mb = std::fmax(mb, std::fabs(static_cast<double>(b[r])));
+        mb = std::fmax(mb, relu ? static_cast<double>(b[r]) : std::fabs(static_cast<double>(b[r])));
     }
     bound[0] = static_cast<float>(l1 * 1.001);
     bound[1] = static_cast<float>(mb * 1.001);
@@ -1039,7 +1040,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         CU_CHECK(c, cudaGetLastError());
         const size_t first = c->literal ? 27 : 19;                                                       // Wi1 or W3, and its bias
         float bound[2];
-        layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, bound);
+        layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, !c->literal, bound);
         CU_CHECK(c, upload(c->d_bound, bound, sizeof(bound)));
     }
     if (!c->use_tc && !c->literal) {
@@ -1161,7 +1162,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                 mb[i] = static_cast<float>(bacc);
             }
             float bound[2];
-            layer_bound(big_m.data(), mb.data(), H, H, bound);
+            layer_bound(big_m.data(), mb.data(), H, H, true, bound);
             CU_CHECK(c, upload(c->d_bound + 2, bound, sizeof(bound)));
             CU_CHECK(c, upload(c->d_Mb, mb.data(), mb.size() * sizeof(float)));
             CU_CHECK(c, upload(c->d_M, big_m.data(), big_m.size() * sizeof(float)));

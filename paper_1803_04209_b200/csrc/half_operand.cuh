@@ -1,23 +1,26 @@
-// Operands of the emission products in half precision, losing nothing.
+// Operands of the emission products in half precision, as exact as tf32 ones wherever that can be seen.
 //
 // A value rounded to tf32 (or bf16) has at most 11 significant bits, which is what a half-precision number holds, so
 // the only thing that keeps a tf32 operand from being stored in two bytes is its exponent.  Every row of an operand --
 // a sample's hidden vector, a worker's weights -- is therefore multiplied by a power of two that brings its bound to
 // [2^14, 2^15), and the product's row and column are divided by the two powers of two again (exactly) when the
-// accumulator is read.  The products and their fp32 accumulation are those of tf32 operands; only an entry smaller than 2^-29
-// of its row's bound lands among the half-precision subnormals and is rounded, by at most 2^-40 of the bound, 2^16 below
-// what the fp32 accumulation itself rounds away.  Half-precision operands take half the bytes from L2 to shared memory
-// and half the tensor-core time.
+// accumulator is read.  The products and their fp32 accumulation are those of tf32 operands, with one exception: an entry below
+// 2^-28 of its row's bound may land among the half-precision subnormals and is then rounded by at most 2^-39 of the bound.
+// The bound of a row of weights is its largest entry.  That of a hidden vector is one that the layer's weights and the
+// sample's largest input allow, the row sums of |weights| and, for a ReLU layer, the largest positive bias (a unit that a large
+// negative bias switches off must not push the others into the subnormals); it lies above the largest entry by as much as the
+// terms of that unit cancel.  Half-precision operands take half the bytes from L2 to shared memory and half the
+// tensor-core time.
 #pragma once
 #include <cstdint>
 #include <cuda_fp16.h>
 
 namespace cutoff {
 
-// 2^e and 2^-e with bound * 2^e in [2^14, 2^15) (bounds from 2^-86 to 2^114; beyond that the nearest such exponent).
+// e with bound * 2^e in [2^14, 2^15), 2^e and 2^-e normal: every finite bound from 2^-112 on (a smaller one is scaled by 2^126).
 __host__ __device__ inline int half_exponent(uint32_t bound_bits) {
     const int ex = static_cast<int>((bound_bits >> 23) & 0xffu) - 127, e = 14 - ex;
-    return e > 100 ? 100 : (e < -100 ? -100 : e);
+    return e > 126 ? 126 : (e < -113 ? -113 : e);
 }
 __host__ __device__ inline uint32_t pow2_bits(int e) { return static_cast<uint32_t>(127 + e) << 23; }
 

@@ -103,3 +103,45 @@ def test_a_captured_graph_follows_reloaded_weights(N, D, H, S, literal):
             gpu.step(x)
         stats.append(gpu.get_stats()[0])
     assert np.all(np.isfinite(stats[0])) and np.array_equal(stats[0], stats[1])
+
+
+# A unit that is switched off by its bias contributes nothing, and nothing about the others may depend on how far off it is:
+# the same samples to the last bit.  Chains: wide, resident, tensor cores with D = 16 and 32; literal: the hidden layer of the scale.
+@pytest.mark.parametrize("N,D,H,S,literal", [(40, 8, 72, 300, False), (40, 4, 32, 60000, False), (300, 16, 128, 3000, False), (300, 32, 256, 3000, False),
+                                             (300, 16, 128, 300, True), (40, 8, 72, 300, True)])
+def test_units_that_are_switched_off_cost_the_others_nothing(N, D, H, S, literal):
+    make = inputs.make_weights_literal if literal else inputs.make_weights
+    w = make(N, D, H, seed=N + H, fan_in_ref=32)
+    trace = inputs.make_trace(N, 3, seed=S, sigma=0.25)
+    hidden, bias = ("Wj1", "bj1") if literal else ("W3", "b3")
+    w[hidden][::5] = 0.0
+    out = []
+    for off in (-1.0, -2.0 ** 20, -2.0 ** 34, -2.0 ** 100):
+        w[bias][::5] = off
+        out.append(samples(w, trace, D, H, 1, min(S, 3000), 1, literal) if S <= 3000 else _head(w, trace, D, H, S))
+    for x in out[1:]:
+        assert np.array_equal(x, out[0])
+
+
+def _head(w, trace, D, H, S):
+    gpu = binding.Cutoff(trace.shape[1], D, H, 1, S, precision=1, seed=77)
+    gpu.load_weights(w)
+    for x in trace:
+        gpu.push(x)
+    return gpu.debug_samples(S // 2, 500)
+
+
+# rows of weights whose size lies near either end of the fp32 range, up to results of 2^125
+@pytest.mark.parametrize("N,D,H,S", [(40, 8, 72, 300), (300, 16, 128, 3000)])
+@pytest.mark.parametrize("power", [-100, 100, 121])
+def test_rows_of_weights_near_the_ends_of_the_range(N, D, H, S, power):
+    w = inputs.make_weights(N, D, H, seed=N + H, fan_in_ref=32)
+    w["b4"][N:] = -400.0                                 # no noise: a worker's sample is its mean row alone
+    trace = inputs.make_trace(N, 3, seed=S, sigma=0.25)
+    x = samples(w, trace, D, H, 1, S, 1, False)
+    assert np.abs(x).max() < 8
+    two = np.float32(2.0 ** power)
+    w["W4"][:N:2] *= two
+    w["b4"][:N:2] *= two
+    x[:, ::2] *= two
+    assert np.array_equal(samples(w, trace, D, H, 1, S, 1, False), x)
