@@ -204,9 +204,13 @@ __device__ __forceinline__ void key_extremes(const float (&v)[E], int threads, i
 
 // Rows the map does not spread (ties, clusters far apart): the register network, on the keys as they stand in the row
 // buffer, put back in order.  A call of its own: the keys of the caller need not be kept in registers for it.
+// Such a row costs the counting, the scan and one more pass through shared memory than a kernel that only has the network.  32768
+// rows, all of them like that, against that kernel: 160 keys 59 and 56 us, 300 keys 107 and 90, 700 keys 185 and 170, 1024 keys 181 and
+// 173; of rows the map spreads 40 and 55, 46 and 92, 74 and 170, 92 and 173.  (Not counting the 15 rows after one that was not
+// spread took 57, 104, 181 and 176 us, but 1 to 3 % more where all are spread, and half as much again where a few are not.)
 template <int E>
 __device__ __noinline__ void warp_network_row(uint32_t row, int n, int lane) {
-    constexpr int EP = E <= 16 ? 16 : 32;
+    constexpr int EP = E <= 8 ? 8 : (E <= 16 ? 16 : 32);
     float v[EP];
 #pragma unroll
     for (int r = 0; r < EP; ++r) v[r] = r * 32 + lane < n ? lds_f32(row + (r * 32 + lane) * 4) : INFINITY;

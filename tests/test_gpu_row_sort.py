@@ -187,3 +187,16 @@ def test_wide_decisions_around_the_length_of_a_run(N, S, pass_rows):
     scale = float(ctx.get_stats()[0][-1]) * S / want[-1]
     sd = np.sqrt(squares / S - (want / S) ** 2) * scale
     assert np.all(np.abs(ctx.get_order_stat_std() - sd) <= 1e-5 + REL * squares / S * scale * scale / (2 * sd))
+@pytest.mark.parametrize("n,rows", [(160, 9000), (256, 9000), (300, 6000), (700, 6000), (1000, 6000)])
+def test_rows_that_change_between_spread_and_not(n, rows):
+    # a warp's rows take turns: ones the map spreads, ones it does not, and neighbours of another scale
+    import torch
+    rng = np.random.default_rng(n)
+    x = _rows("plain", rows, n, rng)
+    turn = rng.integers(0, 4, rows)
+    x[turn == 0] = np.float32(0.75)
+    x[turn == 1] *= np.float32(1e3)
+    x[rows // 2: rows // 2 + rows // 4] = np.float32(0.5)
+    sums = torch.empty(n, dtype=torch.float64, device="cuda")
+    binding.sorted_row_sums_static(torch.from_numpy(x).cuda(), sums)
+    _check(sums.cpu().numpy(), x)
