@@ -58,7 +58,6 @@ struct cutoff_ctx {
 
     float* d_ring = nullptr;        // [W][N]
     float* d_stage = nullptr;       // [N] landing buffer for host pushes
-    uint8_t* h_mask = nullptr;      // pinned [N]: censoring mask of the push in progress
     bool draws_valid = false;       // d_x holds every predictive draw of the last decision (needed for imputation)
     DevState* d_state = nullptr;
     float* d_proj = nullptr;        // [2][W slots][H] raw input projections of the ring's vectors, kept up to date by every push
@@ -105,7 +104,8 @@ struct cutoff_ctx {
     bool chain_tcl32 = false;       // the same for D = 32, H <= 512 (weights staged phase by phase)
     float* d_chain_image = nullptr; // swizzled tf32 operand tiles of the chain
 
-    // pinned host memory that kernels read and write directly (one address on both sides)
+    // pinned host memory that kernels read and write directly (one address on both sides); one block that begins with h_state
+    uint8_t* h_mask = nullptr;      // [N] censoring mask of the push in progress
     float* h_stage = nullptr;       // [N] run-times of a host push
     bool stage_in_use = false;      // by a push that may not have been waited for
     DevState* h_state = nullptr;    // the device state as of the last decision, or push that the host waited for
@@ -228,11 +228,10 @@ void half_rows(cutoff_ctx* c, const float* w, int rows, int row0) {
     k_half_rows<<<ceil_div(rows, 8), 256, 0, c->stream>>>(w, rows, c->H, c->ldh, c->d_w16 + static_cast<size_t>(row0) * c->ldh, c->d_w_inv + row0);
 }
 
-// A copy from pageable memory that has arrived when this returns: cudaMemcpy may return while its last part is under way, and
-// the contexts' streams do not wait for the default stream.
-cudaError_t upload(void* dst, const void* src, size_t bytes) {
-    const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
-    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+// A copy from pageable memory, taken from it when this returns, in the order of the context's stream: on the default stream the
+// context's kernels would not wait for it.
+cudaError_t upload(const cutoff_ctx* c, void* dst, const void* src, size_t bytes) {
+    return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream);
 }
 
 // |A x + b| <= slope * max |x| + offset, from the matrix as the tensor cores see it (rounded up a little); of a ReLU layer
@@ -276,13 +275,10 @@ void free_all(cutoff_ctx* c) {
     cudaFree(c->d_I); cudaFree(c->d_r); cudaFree(c->d_Wj1p); cudaFree(c->d_Mb); cudaFree(c->d_M); cudaFree(c->d_W4T);
     cudaFree(c->d_v16); cudaFree(c->d_v_inv); cudaFree(c->d_w16); cudaFree(c->d_w_inv); cudaFree(c->d_bound); cudaFree(c->d_r16); cudaFree(c->d_r_inv);
     cudaFree(c->d_blob); cudaFree(c->d_WT); cudaFree(c->d_WhR); cudaFree(c->d_chain_image);
-    if (c->h_mask) cudaFreeHost(c->h_mask); cudaFree(c->d_ring); cudaFree(c->d_stage);
+    cudaFree(c->d_ring); cudaFree(c->d_stage);
     cudaFree(c->d_state); cudaFree(c->d_proj); cudaFree(c->d_hlr); cudaFree(c->d_v); cudaFree(c->d_x);
     cudaFree(c->d_partial); cudaFree(c->d_sq_totals); cudaFree(c->d_std); cudaFree(c->d_sums);
-    if (c->h_stage) cudaFreeHost(c->h_stage);
-    if (c->h_state) cudaFreeHost(c->h_state);
-    if (c->h_E) cudaFreeHost(c->h_E);
-    if (c->h_omega) cudaFreeHost(c->h_omega);
+    if (c->h_state) cudaFreeHost(c->h_state);            // the whole pinned block
     if (c->owns_stream && c->stream) cudaStreamDestroy(c->stream);
     if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
     if (c->graph) cudaGraphDestroy(c->graph);
@@ -407,8 +403,12 @@ void launch_chain_t(cutoff_ctx* c, uint32_t sample_base, int count, size_t smem)
             launch_dependent(kernel, dim3(batches < c->sm_count ? batches : c->sm_count), dim3(kChainWideThreads), resident, c->stream, c->m, c->d_hlr,
                              c->d_state, key, sample_base, count, chain_out(c));
         };
-        if (c->chain_wide == 2) run(k_chain_wide<D, 2>, 2);
-        else run(k_chain_wide<D, 1>, 1);
+        bool two = false;
+        if constexpr (D <= 16) {
+            two = c->chain_wide == 2;
+            if (two) run(k_chain_wide<D, 2>, 2);
+        }
+        if (!two) run(k_chain_wide<D, 1>, 1);
     } else if (resident <= 200 * 1024) {
         // all weights fit: one persistent CTA per SM, as many as there are warp batches to hand out
         const int batch = 32 / ChainShape<D>::G * ChainShape<D>::SPL;
@@ -747,43 +747,46 @@ cudaError_t allow_smem_sort(int n) {
     }
 }
 
+// The per-sample chain that the context runs (launch_chain and launch_chain_t choose by the same fields).
 template <int D>
-cudaError_t allow_smem_chain() {
-    cudaError_t e = allow_smem(k_chain<D>, 220 * 1024);
-    if (e == cudaSuccess) e = allow_smem(k_chain_resident<D>, 220 * 1024);
-    if (e == cudaSuccess) e = allow_smem(k_chain_wide<D, 1>, 220 * 1024);
-    if (e == cudaSuccess) e = allow_smem(k_chain_wide<D, 2>, 220 * 1024);
-    if (e == cudaSuccess) e = allow_smem(k_chain_literal<D>, 220 * 1024);
-    return e;
+cudaError_t allow_smem_chain(const cutoff_ctx* c) {
+    if (c->literal) return allow_smem(k_chain_literal<D>, 220 * 1024);
+    if constexpr (D <= 16)
+        if (c->chain_wide == 2) return allow_smem(k_chain_wide<D, 2>, 220 * 1024);
+    if (c->chain_wide) return allow_smem(k_chain_wide<D, 1>, 220 * 1024);
+    if (chain_resident_smem_floats(c->D, c->H, c->W) * sizeof(float) <= 200 * 1024) return allow_smem(k_chain_resident<D>, 220 * 1024);
+    return allow_smem(k_chain<D>, 220 * 1024);
 }
 
+// Only for the kernels this context runs: each one is loaded by the driver when it is first named.
 cudaError_t set_kernel_attributes(const cutoff_ctx* c) {
-    cudaError_t e = cudaSuccess;
-    e = allow_smem_sort(c->N);
+    cudaError_t e = allow_smem_sort(c->N);
     if (e != cudaSuccess) return e;
-    switch (c->D) {
-        case 4: e = allow_smem_chain<4>(); break;
-        case 8: e = allow_smem_chain<8>(); break;
-        case 16: e = allow_smem_chain<16>(); break;
-        default: e = allow_smem_chain<32>(); break;
+    if (c->chain_tc) e = allow_smem(tc::k_chain_tc<false>, 227 * 1024);
+    else if (c->chain_tcl) e = allow_smem(tc::k_chain_tc<true>, 227 * 1024);
+    else if (c->chain_tc32) e = allow_smem(tc::k_chain_tc32<false>, 227 * 1024);
+    else if (c->chain_tcl32) e = allow_smem(tc::k_chain_tc32<true>, 227 * 1024);
+    else switch (c->D) {
+        case 4: e = allow_smem_chain<4>(c); break;
+        case 8: e = allow_smem_chain<8>(c); break;
+        case 16: e = allow_smem_chain<16>(c); break;
+        default: e = allow_smem_chain<32>(c); break;
     }
     if (e != cudaSuccess) return e;
     switch (c->H) {
         case 32: e = allow_smem(k_enc_rnn_resident<8>, 200 * 1024); break;
         case 64: e = allow_smem(k_enc_rnn_resident<16>, 200 * 1024); break;
         case 128: e = allow_smem(k_enc_rnn_resident<32>, 200 * 1024); break;
-        default: break;
+        default: if (c->H >= 256) e = allow_smem(k_enc_rnn_cluster, 200 * 1024);
     }
-    if (e == cudaSuccess) e = allow_smem(k_enc_rnn_cluster, 200 * 1024);
     if (e != cudaSuccess || !c->use_tc) return e;
-    e = allow_smem(tc::k_emit_tc, tc::kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(tc::k_emit_tc2, tc::kSmem2Bytes);
-    if (e == cudaSuccess) e = allow_smem(tc::k_gemm_relu_tc, tc::kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(tc::k_emit_dual_tc, tc::kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<false>, 227 * 1024);
-    if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<true>, 227 * 1024);
-    if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc32<false>, 227 * 1024);
-    if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc32<true>, 227 * 1024);
+    if (!c->literal) {
+        e = allow_smem(tc::k_emit_tc, tc::kSmemBytes);
+        if (e == cudaSuccess) e = allow_smem(tc::k_emit_tc2, tc::kSmem2Bytes);
+    } else {
+        e = allow_smem(tc::k_gemm_relu_tc, tc::kSmemBytes);
+        if (e == cudaSuccess) e = allow_smem(tc::k_emit_dual_tc, tc::kSmemBytes);
+    }
     return e;
 }
 
@@ -913,7 +916,6 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     if (c->chain_tcl32) CREATE_CHECK(cudaMalloc(&c->d_chain_image, sizeof(float) * tc::chain_tc32_image_floats(c->H, true)));
     CREATE_CHECK(cudaMalloc(&c->d_ring, sizeof(float) * c->W * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_stage, sizeof(float) * c->N));
-    CREATE_CHECK(cudaMallocHost(&c->h_mask, c->N));
     CREATE_CHECK(cudaMalloc(&c->d_state, sizeof(DevState)));
     CREATE_CHECK(cudaMalloc(&c->d_proj, sizeof(float) * 2 * c->W * c->H));
     CREATE_CHECK(cudaMalloc(&c->d_hlr, sizeof(float) * 2 * c->W * c->H));
@@ -959,10 +961,14 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
         if (cudaOccupancyMaxActiveClusters(&n, tc::k_emit_tc2, &lc) == cudaSuccess && n > 0) c->pair_clusters = n;
         else cudaGetLastError();
     }
-    CREATE_CHECK(cudaMallocHost(&c->h_stage, sizeof(float) * c->N));
-    CREATE_CHECK(cudaMallocHost(&c->h_state, sizeof(DevState)));
-    CREATE_CHECK(cudaMallocHost(&c->h_E, sizeof(float) * c->N));
-    CREATE_CHECK(cudaMallocHost(&c->h_omega, sizeof(float) * c->N));
+    // one pinned block: state | run-times | expected order statistics | throughputs | mask, each on a line of its own
+    const size_t line = 128, state_bytes = (sizeof(DevState) + line - 1) / line * line, row_bytes = (sizeof(float) * c->N + line - 1) / line * line;
+    CREATE_CHECK(cudaMallocHost(&c->h_state, state_bytes + 3 * row_bytes + c->N));
+    char* const pinned = reinterpret_cast<char*>(c->h_state) + state_bytes;
+    c->h_stage = reinterpret_cast<float*>(pinned);
+    c->h_E = reinterpret_cast<float*>(pinned + row_bytes);
+    c->h_omega = reinterpret_cast<float*>(pinned + 2 * row_bytes);
+    c->h_mask = reinterpret_cast<uint8_t*>(pinned + 3 * row_bytes);
     CREATE_CHECK(cudaMemsetAsync(c->d_state, 0, sizeof(DevState), c->stream));
     CREATE_CHECK(cudaMemsetAsync(c->d_ring, 0, sizeof(float) * c->W * c->N, c->stream));
     CREATE_CHECK(cudaStreamSynchronize(c->stream));
@@ -1028,7 +1034,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
             }
         }
     }
-    CU_CHECK(c, upload(c->d_blob, host.data(), host.size() * sizeof(float)));
+    CU_CHECK(c, upload(c, c->d_blob, host.data(), host.size() * sizeof(float)));
     if (c->use_tc) {
         const int N = c->N, H = c->H, D = c->D;
         if (c->literal) {
@@ -1041,7 +1047,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         const size_t first = c->literal ? 27 : 19;                                                       // Wi1 or W3, and its bias
         float bound[2];
         layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, !c->literal, bound);
-        CU_CHECK(c, upload(c->d_bound, bound, sizeof(bound)));
+        CU_CHECK(c, upload(c, c->d_bound, bound, sizeof(bound)));
     }
     if (!c->use_tc && !c->literal) {
         k_transpose_heads<<<dim3(ceil_div(c->ldx, 32), ceil_div(c->H, 32), 2), dim3(32, 8), 0, c->stream>>>(c->d_blob + off[21], c->N, c->H, c->ldx, c->d_W4T);
@@ -1057,7 +1063,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         for (size_t i = 0; i < H; ++i)
             for (size_t d = 0; d < D; ++d) wT[t * H * D + d * H + i] = w[i * D + d];
     }
-    CU_CHECK(c, upload(c->d_WT, wT.data(), wT.size() * sizeof(float)));
+    CU_CHECK(c, upload(c, c->d_WT, wT.data(), wT.size() * sizeof(float)));
 
     if (H == 32 || H == 64 || H == 128) {
         // recurrence matrices regrouped per thread of k_enc_rnn_resident (the widths that kernel serves; the layout
@@ -1072,7 +1078,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                     for (size_t j = 0; j < HQ; ++j)
                         whr[dir * H * H + ((j / 4) * T + (4 * i + q)) * 4 + (j % 4)] = w[i * H + q * HQ + j];
         }
-        CU_CHECK(c, upload(c->d_WhR, whr.data(), whr.size() * sizeof(float)));
+        CU_CHECK(c, upload(c, c->d_WhR, whr.data(), whr.size() * sizeof(float)));
     }
     // Operand tiles of the tensor-core chain kernels as they will sit in shared memory: tf32 (nearest, ties away),
     // K-major rows of 32 values, 16-byte chunks XOR-swizzled with the row index modulo 8.
@@ -1128,7 +1134,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
                 put_second_layer(img.data() + 5 * tile, wc + 32 * H, 32, H, 32);
             }
         }
-        CU_CHECK(c, upload(c->d_chain_image, img.data(), img.size() * sizeof(float)));
+        CU_CHECK(c, upload(c, c->d_chain_image, img.data(), img.size() * sizeof(float)));
     }
 
     ModelDev& m = c->m;
@@ -1163,9 +1169,9 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
             }
             float bound[2];
             layer_bound(big_m.data(), mb.data(), H, H, true, bound);
-            CU_CHECK(c, upload(c->d_bound + 2, bound, sizeof(bound)));
-            CU_CHECK(c, upload(c->d_Mb, mb.data(), mb.size() * sizeof(float)));
-            CU_CHECK(c, upload(c->d_M, big_m.data(), big_m.size() * sizeof(float)));
+            CU_CHECK(c, upload(c, c->d_bound + 2, bound, sizeof(bound)));
+            CU_CHECK(c, upload(c, c->d_Mb, mb.data(), mb.size() * sizeof(float)));
+            CU_CHECK(c, upload(c, c->d_M, big_m.data(), big_m.size() * sizeof(float)));
             half_rows(c, c->d_M, c->H, 2 * c->N);
             CU_CHECK(c, cudaGetLastError());
         } else {
@@ -1173,7 +1179,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
             std::vector<float> wj1p(H * static_cast<size_t>(c->ldx), 0.0f);
             for (size_t i = 0; i < H; ++i)
                 std::memcpy(wj1p.data() + i * c->ldx, host.data() + off[31] + i * c->N, sizeof(float) * c->N);
-            CU_CHECK(c, upload(c->d_Wj1p, wj1p.data(), wj1p.size() * sizeof(float)));
+            CU_CHECK(c, upload(c, c->d_Wj1p, wj1p.data(), wj1p.size() * sizeof(float)));
         }
         LiteralDev& l = c->lit;
         l.Wg1T = c->d_WT + H * D; l.bg1 = b + off[16]; l.Wg2 = b + off[17]; l.bg2 = b + off[18];
@@ -1677,8 +1683,8 @@ int cutoff_restore_state(cutoff_ctx* c, const void* buf, size_t nbytes) {
     DeviceGuard guard(c->cfg.device);
     CU_CHECK(c, guard.err);
     CU_CHECK(c, cudaStreamSynchronize(c->stream));
-    CU_CHECK(c, upload(c->d_state, &s, sizeof(DevState)));
-    CU_CHECK(c, upload(c->d_ring, p + sizeof(hdr) + sizeof(DevState), sizeof(float) * c->W * c->N));
+    CU_CHECK(c, upload(c, c->d_state, &s, sizeof(DevState)));
+    CU_CHECK(c, upload(c, c->d_ring, p + sizeof(hdr) + sizeof(DevState), sizeof(float) * c->W * c->N));
     c->pushes = s.push_count;
     c->pending = false;
     c->partial_pending = false;
