@@ -428,7 +428,7 @@ inline size_t path_weight_floats(int D, int H) {
 // What a step reads from global memory is copied to shared memory a step early: 4 rows of H, 5 of D, twice.
 inline size_t path_scratch_floats(int D, int H) { return 11 * static_cast<size_t>(H) + 18 * static_cast<size_t>(D) + 64; }
 
-__device__ __forceinline__ PathWeights path_weights(const PathArgs& a, float* sm, int staged) {
+__device__ __forceinline__ PathWeights path_weights(const PathArgs& a, float* sm, bool staged) {
     if (!staged) return PathWeights{a.Wz, a.W1, a.W3, a.Wmu, a.W2, a.D, a.H};
     PathWeights w;
     w.ldd = a.D | 1;
@@ -447,7 +447,13 @@ __device__ __forceinline__ PathWeights path_weights(const PathArgs& a, float* sm
     return w;
 }
 
-__global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int staged) {
+// Where the matrices do not fit, they pass through kPathBuffer floats of shared memory at every step, some rows (some columns of
+// W_mu and W_2) at a time.  With a thread per row reading its row from global memory instead, forward passes of five steps, N=64, D=64,
+// took: H=256, 300 windows 954 us (this way 541), H=512, 64 windows 770 us (552).
+constexpr int kPathBuffer = 16 * 1024;
+
+template <bool STAGED>
+__global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a) {
     extern __shared__ __align__(16) float sm[];
     const int D = a.D, H = a.H, W = a.W, b = blockIdx.x, tid = threadIdx.x;
     float* z = sm;                   // [D]
@@ -457,8 +463,15 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
     float* h = sm + 8 * D;           // [2][H] (of 3)
     float* scal = h + 3 * H;         // [64]
     float* ahead = scal + 64;        // [2]: h_left, h_right (H each), eps (D)
-    const int ahead_n = 4 * H + 5 * D;
-    const PathWeights w = path_weights(a, ahead + 2 * ahead_n, staged);
+    const int ahead_n = 4 * H + 5 * D, ldd = D | 1;
+    float* buffer = ahead + 2 * ahead_n;
+    PathWeights w{};
+    if constexpr (STAGED) {
+        w = path_weights(a, buffer, true);
+        // addresses of unknown space: in loads that it knows to be from shared memory the compiler puts the chains' loads between their
+        // multiply-adds (10 us more per five steps)
+        asm volatile("" : "+l"(w.Wz), "+l"(w.W1), "+l"(w.W3), "+l"(w.Wmu), "+l"(w.W2));
+    }
     dependency_wait();
     const auto fetch = [&](int t) {
         float* dst = ahead + (t & 1) * ahead_n;
@@ -478,20 +491,56 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
         __syncthreads();
         if (t + 1 < W) fetch(t + 1);
         // hidden layers that read z_{t-1}: the combiner and the transition's
-        for (int i = tid; i < H; i += kPathThreads) {
-            const float c = tanhf(row_dot(w.Wz, w.ldd, i, z, D) + a.bz[i]);
+        const auto hidden = [&](const float* Wz, const float* W1, int i, int row) {
+            const float c = tanhf(row_dot(Wz, ldd, row, z, D) + a.bz[i]);
             const float o = (c + sa[i] + sb[i]) * (1.f / 3.f);
-            const float u = fmaxf(row_dot(w.W1, w.ldd, i, z, D) + a.b1[i], 0.f);
+            const float u = fmaxf(row_dot(W1, ldd, row, z, D) + a.b1[i], 0.f);
             a.comb[r * H + i] = c;
             a.hout[r * H + i] = o;
             a.u[r * H + i] = u;
             h[i] = o;
             h[H + i] = u;
+        };
+        if constexpr (STAGED) {
+            for (int i = tid; i < H; i += kPathThreads) hidden(w.Wz, w.W1, i, i);
+        } else {
+            const int rows = kPathBuffer / (2 * ldd);
+            for (int r0 = 0; r0 < H; r0 += rows) {
+                const int n = min(rows, H - r0);
+                __syncthreads();
+                copy_matrix(buffer, ldd, a.Wz + static_cast<long long>(r0) * D, D, n, D);
+                copy_matrix(buffer + rows * ldd, ldd, a.W1 + static_cast<long long>(r0) * D, D, n, D);
+                copies_landed();
+                __syncthreads();
+                for (int i = tid; i < n; i += kPathThreads) hidden(buffer, buffer + rows * ldd, r0 + i, i);
+            }
         }
         __syncthreads();
-        for (int o = tid; o < 3 * D; o += kPathThreads) {
-            if (o < D) mu[o] = row_dot(w.Wmu, w.ldh, o, h, H) + a.bmu[o];
-            else hz[o - D] = row_dot(w.W2, w.ldh, o - D, h + H, H) + a.b2[o - D];
+        if constexpr (STAGED) {
+            for (int o = tid; o < 3 * D; o += kPathThreads) {
+                if (o < D) mu[o] = row_dot(w.Wmu, w.ldh, o, h, H) + a.bmu[o];
+                else hz[o - D] = row_dot(w.W2, w.ldh, o - D, h + H, H) + a.b2[o - D];
+            }
+        } else {
+            // D <= 64: a result per thread, its chain in pieces
+            const int cols = kPathBuffer / (3 * D) - 1, ld = cols | 1;
+            const float* in = tid < D ? h : h + H;
+            float s = 0.f;
+            for (int k0 = 0; k0 < H; k0 += cols) {
+                const int n = min(cols, H - k0);
+                __syncthreads();
+                copy_matrix(buffer, ld, a.Wmu + k0, H, D, n);
+                copy_matrix(buffer + D * ld, ld, a.W2 + k0, H, 2 * D, n);
+                copies_landed();
+                __syncthreads();
+                if (tid < 3 * D) {
+                    const float* p = buffer + tid * ld;
+#pragma unroll 16
+                    for (int k = 0; k < n; ++k) s = fmaf(p[k], in[k0 + k], s);
+                }
+            }
+            if (tid < D) mu[tid] = s + a.bmu[tid];
+            else if (tid < 3 * D) hz[tid - D] = s + a.b2[tid - D];
         }
         __syncthreads();
         for (int d = tid; d < D; d += kPathThreads) {
@@ -509,8 +558,22 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
             a.dhz[r * 2 * D + D + d] = -0.5f + 0.5f * rr * rr * inv;
         }
         __syncthreads();
-        for (int i = tid; i < H; i += kPathThreads)
-            a.v[r * H + i] = fmaxf(row_dot(w.W3, w.ldd, i, zp, D) + a.b3[i], 0.f);
+        const auto emission = [&](const float* W3, int i, int row) {
+            a.v[r * H + i] = fmaxf(row_dot(W3, ldd, row, zp, D) + a.b3[i], 0.f);
+        };
+        if constexpr (STAGED) {
+            for (int i = tid; i < H; i += kPathThreads) emission(w.W3, i, i);
+        } else {
+            const int rows = kPathBuffer / ldd;
+            for (int r0 = 0; r0 < H; r0 += rows) {
+                const int n = min(rows, H - r0);
+                __syncthreads();
+                copy_matrix(buffer, ldd, a.W3 + static_cast<long long>(r0) * D, D, n, D);
+                copies_landed();
+                __syncthreads();
+                for (int i = tid; i < n; i += kPathThreads) emission(buffer, r0 + i, i);
+            }
+        }
         float* swap = z; z = zp; zp = swap;            // h, mu and hz are rewritten behind the next barriers
     }
     // D <= 64: the sums sit in the first two warps
@@ -523,7 +586,7 @@ __global__ void __launch_bounds__(kPathThreads) k_path_forward(PathArgs a, int s
     }
 }
 
-__global__ void __launch_bounds__(kPathThreads) k_path_backward(PathArgs a, int staged) {
+__global__ void __launch_bounds__(kPathThreads) k_path_backward(PathArgs a, bool staged) {
     extern __shared__ __align__(16) float sm[];
     const int D = a.D, H = a.H, W = a.W, b = blockIdx.x, tid = threadIdx.x;
     float* gz = sm;                  // [D]   d ELBO / d z_t

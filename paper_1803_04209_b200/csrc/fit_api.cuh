@@ -172,9 +172,10 @@ inline void elbo_grad(int N, int D, int H, int W, int B, const float* p, const f
     a.gz0 = ws + o.gz0; a.B = B; a.W = W; a.D = D; a.H = H;
     const size_t path_scratch = path_scratch_floats(D, H) * sizeof(float);
     const size_t path_full = path_scratch + path_weight_floats(D, H) * sizeof(float);
-    const int staged = path_full <= 200 * 1024 ? 1 : 0;
+    const bool staged = path_full <= 200 * 1024;
     const size_t path_smem = staged ? path_full : path_scratch;
-    launch(k_path_forward, dim3(B), kPathThreads, path_smem, stream, true, 1, a, staged);
+    if (staged) launch(k_path_forward<true>, dim3(B), kPathThreads, path_full, stream, true, 1, a);
+    else launch(k_path_forward<false>, dim3(B), kPathThreads, path_scratch + kPathBuffer * sizeof(float), stream, true, 1, a);
     {
         float* dhx = back ? ws + o.dhx : nullptr;
         const auto run = [&](auto tile) {

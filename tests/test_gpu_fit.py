@@ -183,3 +183,9 @@ def test_step_at_the_edges_of_tiles_and_of_shared_memory(N, D, H, lag, B):
         denom = max(float(np.max(np.abs(want_g[name]))), 1e-6)
         err = float(np.max(np.abs(got[name].astype(np.float64) - want_g[name]))) / denom
         assert err <= 2e-4, f"{name}: {err:.2e}"
+
+
+# Matrices that pass through shared memory in pieces (wide networks), one step and several, rows that are not a multiple of 16 bytes.
+@pytest.mark.parametrize("N,D,H,lag,B", [(16, 64, 256, 1, 40), (9, 32, 1023, 0, 7), (9, 5, 1021, 2, 3)])
+def test_matrices_in_pieces_match_the_oracle(N, D, H, lag, B):
+    test_step_at_the_edges_of_tiles_and_of_shared_memory(N, D, H, lag, B)
