@@ -8,7 +8,8 @@
 // What bounds a step is the number of dependent launches and the length of its chains, not its arithmetic (64 windows of
 // the n1024 model: 1.0 G multiply-adds, 28 us at the FMA rate), so the step is laid out by what depends on what.  Only the
 // recurrences depend on the previous step of a window, and only within the window: one CTA walks through all of a
-// window's steps, a cluster through those of a few windows' RNN, in one launch.  Everything else is one product over all
+// window's steps, a cluster through those of a few windows' RNN, in one launch (the forward RNNs of wide networks and large
+// batches: a product per step).  Everything else is one product over all
 // B*W (window, step) rows: the input projections, the emission head with its density in the epilogue, the input gradient
 // of that head, and the weight gradients as a list of products in one launch.
 //
@@ -307,6 +308,40 @@ __global__ void __launch_bounds__(256) k_rnn_forward(RnnArgs a) {
         }
         cluster_sync();
         float* swap = cur; cur = next; next = swap;
+    }
+}
+
+// One step of both recurrences as a product over all windows, for batches so large that the clusters would take turns: a tile of
+// windows x units per CTA, a launch per step.  The same chain per result as above.
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(T::kThreads) k_rnn_step(RnnArgs a, int s) {
+    __shared__ __align__(16) Slabs<T, true, true> sm;
+    dependency_wait();
+    const int H = a.H, W = a.W, dir = blockIdx.y, t = dir ? W - 1 - s : s, unit_tiles = (H + T::TN - 1) / T::TN;
+    const int m0 = static_cast<int>(blockIdx.x) / unit_tiles * T::TM, n0 = static_cast<int>(blockIdx.x) % unit_tiles * T::TN;
+    const long long pitch = static_cast<long long>(W + 1) * H;             // from one window's states to the next's
+    float* const state = a.state[dir];
+    float* const before = state + static_cast<long long>(dir ? t + 1 : t) * H;
+    float* const after = state + static_cast<long long>(dir ? t : t + 1) * H;
+    // the initial state is the same for every window
+    const Operand x{s == 0 ? a.init[dir] : before, s == 0 ? 0 : pitch, 0, a.B};
+    const auto copy_b = [&](uint32_t dst, int k0, int) { copy_slab<T, T::TN, true, VEC>(dst, a.Wh[dir], H, H, n0, k0, H); };
+    float acc[T::RM][T::RN] = {};
+    float unused = 0.f;
+    tile_product<T, true, true, VEC, false, false>(sm, x, m0, H, 1, copy_b, acc, unused);
+    const int tx = threadIdx.x % T::TX, ty = threadIdx.x / T::TX;
+#pragma unroll
+    for (int i = 0; i < T::RM; ++i) {
+        const int b = m0 + result_at<T::RM, T::TY, true>(ty, i);
+        if (b >= a.B) continue;
+#pragma unroll
+        for (int j = 0; j < T::RN; ++j) {
+            const int h = n0 + result_at<T::RN, T::TX, true>(tx, j);
+            if (h >= H) continue;
+            const float p = a.proj[(static_cast<long long>(b) * W + t) * 2 * H + dir * H + h] + a.bias[dir][h];
+            after[b * pitch + h] = fmaxf(acc[i][j] + p, 0.f);
+            if (s == 0) state[b * pitch + static_cast<long long>(dir ? W : 0) * H + h] = a.init[dir][h];
+        }
     }
 }
 

@@ -133,6 +133,12 @@ inline RnnPlan rnn_plan(int B, int H) {
     return p;
 }
 
+// Whether the forward recurrence runs as products over all windows, a launch per step (k_rnn_step), instead: where the clusters
+// would take several turns on the GPU.  Forward passes of five steps, N=64, D=4, clusters and products: H=192 1024 windows 226 and
+// 225 us, 4096 744 and 537; H=256 256 windows 176 and 204, 512 250 and 225; H=512 64 windows 302 and 306, 256 698 and 328; H=1024 16
+// windows 483 and 493, 64 776 and 532, 1024 6038 and 2387; H=128 4096 windows 369 and 382.
+inline bool rnn_by_steps(int B, int H) { return H >= 192 && static_cast<long long>(B) * H * H > 40 << 20; }
+
 // Enqueue forward (+ backward if grads) on `stream`.  All pointers are device pointers.
 inline void elbo_grad(int N, int D, int H, int W, int B, const float* p, const float* xhat, const float* eps, float* elbo,
                       float* grads, float* ws, cudaStream_t stream) {
@@ -159,7 +165,13 @@ inline void elbo_grad(int N, int D, int H, int W, int B, const float* p, const f
     r.d_pre[0] = ws + o.dpf; r.d_pre[1] = ws + o.dpb; r.carry_out[0] = ws + o.ca; r.carry_out[1] = ws + o.cb;
     const RnnPlan rp = rnn_plan(B, H);
     r.B = B; r.W = W; r.H = H; r.cluster = rp.cluster; r.units = rp.units; r.chunk = rp.chunk;
-    launch(rp.rw == 2 ? k_rnn_forward<2> : k_rnn_forward<4>, rp.grid, rp.threads, rp.smem, stream, true, rp.cluster, r);
+    if (rnn_by_steps(B, H)) {
+        const dim3 grid(static_cast<unsigned>(tiles_of(B, LargeTile::TM) * tiles_of(H, LargeTile::TN)), 2);
+        for (int s = 0; s < W; ++s)
+            launch(vec ? k_rnn_step<LargeTile, true> : k_rnn_step<LargeTile, false>, grid, LargeTile::kThreads, 0, stream, true, 1, r, s);
+    } else {
+        launch(rp.rw == 2 ? k_rnn_forward<2> : k_rnn_forward<4>, rp.grid, rp.threads, rp.smem, stream, true, rp.cluster, r);
+    }
     PathArgs a{};
     a.Wz = w(iWz); a.bz = w(ibz); a.Wmu = w(iWmu); a.bmu = w(ibmu); a.Wsig = w(iWsig); a.bsig = w(ibsig); a.z0 = w(iz0);
     a.W1 = w(iW1); a.b1 = w(ib1); a.W2 = w(iW2); a.b2 = w(ib2); a.W3 = w(iW3); a.b3 = w(ib3);

@@ -189,3 +189,23 @@ def test_step_at_the_edges_of_tiles_and_of_shared_memory(N, D, H, lag, B):
 @pytest.mark.parametrize("N,D,H,lag,B", [(16, 64, 256, 1, 40), (9, 32, 1023, 0, 7), (9, 5, 1021, 2, 3)])
 def test_matrices_in_pieces_match_the_oracle(N, D, H, lag, B):
     test_step_at_the_edges_of_tiles_and_of_shared_memory(N, D, H, lag, B)
+
+
+# The recurrence as products over all windows (wide networks, large batches): edges of the 64 x 64 tiles, rows that are not a multiple of
+# 16 bytes, one step and several.  A window's ELBO does not depend on the batch it is in, to the last bit: a small batch goes
+# through the clusters.
+@pytest.mark.parametrize("N,D,H,lag,B", [(16, 4, 192, 0, 1150), (20, 5, 201, 2, 1050), (16, 64, 256, 1, 650), (9, 4, 1024, 2, 41), (9, 32, 1023, 1, 64)])
+def test_windows_do_not_depend_on_the_batch(N, D, H, lag, B):
+    import torch
+    w, x, eps = _case(N, D, H, lag, B, seed=H)
+    whole = binding.Fitter(N, D, H, lag, B, w)
+    elbo, _ = whole.elbo_grad(torch.from_numpy(x).cuda(), torch.from_numpy(eps).cuda(), want_grad=False)
+    for first in (0, B // 2, B - 5):
+        part = binding.Fitter(N, D, H, lag, 5, w)
+        some, _ = part.elbo_grad(torch.from_numpy(x[first:first + 5]).cuda(), torch.from_numpy(eps[first:first + 5]).cuda(), want_grad=False)
+        assert torch.equal(some, elbo[first:first + 5])
+
+
+@pytest.mark.parametrize("N,D,H,lag,B", [(9, 4, 1024, 2, 41), (20, 5, 201, 1, 1050)])
+def test_the_recurrence_as_products_matches_the_oracle(N, D, H, lag, B):
+    test_step_at_the_edges_of_tiles_and_of_shared_memory(N, D, H, lag, B)
