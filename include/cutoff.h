@@ -269,7 +269,7 @@ int cutoff_set_option(cutoff_ctx* ctx, const char* name, int64_t value);
  * units, for local samples k0 .. k0+count-1 (x_out, host, count*N floats).  Does not advance the
  * decision counter.  Returns WARMUP before lag+1 pushes.
  *
- * cutoff_debug_sort: the library's sorting network applied to caller rows.  rows (host,
+ * cutoff_debug_sort: the register sorting network applied to caller rows, with positions.  rows (host,
  * n_rows*n floats) -> keys_out (host, sorted ascending) and perm_out (host, int32, the original
  * position of each sorted key; equal keys keep their original order). */
 int cutoff_debug_normals(int device, uint64_t seed, uint32_t step, uint32_t stream, int64_t k0,
@@ -280,9 +280,9 @@ int cutoff_debug_samples(cutoff_ctx* ctx, int64_t k0, int64_t count, float* x_ou
 int cutoff_debug_window(cutoff_ctx* ctx, float* window_out);
 int cutoff_debug_sort(cutoff_ctx* ctx, const float* rows, int64_t n_rows, int32_t n,
                       float* keys_out, int32_t* perm_out);
-/* cutoff_debug_sort_values: the same networks in the instantiation the decision itself runs (plain
- * fp32 keys, rows padded with +infinity), the sorted rows returned instead of summed (Section 3.1.1,
- * last paragraph: "sort").  rows (host, n_rows*n floats, any finite values, +-0 and +infinity
+/* cutoff_debug_sort_values: the sort a decision of n_rows samples over n workers runs (the network up to 128
+ * keys, and up to 256 for less than 8192 rows; by distribution beyond), the sorted rows returned instead of
+ * summed (Section 3.1.1, last paragraph: "sort").  rows (host, n_rows*n floats, any finite values, +-0 and +infinity
  * included) -> keys_out (host, n_rows*n floats, each row ascending).  n <= 4096. */
 int cutoff_debug_sort_values(cutoff_ctx* ctx, const float* rows, int64_t n_rows, int32_t n, float* keys_out);
 

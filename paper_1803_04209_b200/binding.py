@@ -349,7 +349,7 @@ class Cutoff:
         return keys, perm
 
     def debug_sort_values(self, rows: np.ndarray) -> np.ndarray:
-        """Rows sorted ascending by the fp32 network of the decision path."""
+        """Rows sorted ascending by the sort a decision of as many samples runs."""
         r = np.ascontiguousarray(rows, dtype=np.float32)
         keys = np.empty_like(r)
         self._check(self._lib.cutoff_debug_sort_values(self._h, r.ctypes.data, r.shape[0], r.shape[1], keys.ctypes.data),

@@ -563,4 +563,52 @@ k_bucket_sum_cta(const float* __restrict__ x, int ldx, int n, int count, float* 
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Test hook: the sorts above, the sorted rows written out instead of summed.  Rows come in by plain copies; a warp (a CTA) sorts
+// several rows one after the other, so that a row meets the map of the one before it.
+// ---------------------------------------------------------------------------------------------
+constexpr int kDebugBucketWarps = 4;
+
+template <int E>
+__global__ void __launch_bounds__(kDebugBucketWarps * 32) k_debug_bucket_warp(const float* __restrict__ rows, int n, int n_rows,
+                                                                              float* __restrict__ keys) {
+    constexpr size_t kWarpFloats = bucket_warp_floats<E>();
+    __shared__ __align__(128) float data[kDebugBucketWarps * kWarpFloats];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* const mine = data + warp * kWarpFloats;
+    const uint32_t row_s = async::smem_u32(mine), hist = row_s + 32 * E * 4;
+    for (int i = lane; i < 32 * BucketShape<E>::kLaneWords; i += 32) mine[32 * E + i] = 0.0f;
+    BucketMap map{};
+    const int row0 = blockIdx.x * kDebugBucketWarps + warp;
+    for (int row = row0; row < n_rows; row += gridDim.x * kDebugBucketWarps) {
+        for (int e = lane; e < n; e += 32) mine[e] = rows[static_cast<size_t>(row) * n + e];
+        __syncwarp();
+        float v[E];
+        warp_bucket_sort<E>(v, row_s, hist, n, lane, row == row0, map, [] { __syncwarp(); });
+#pragma unroll
+        for (int r = 0; r < E; ++r)
+            if (lane * E + r < n) keys[static_cast<size_t>(row) * n + lane * E + r] = v[r];
+    }
+}
+
+template <int E>
+__global__ void __launch_bounds__(128) k_debug_bucket_cta(const float* __restrict__ rows, int n, int n_rows, float* __restrict__ keys) {
+    constexpr int kCounters = 128 * BucketShape<E>::kLaneWords;
+    __shared__ __align__(128) float data[4096 + kCounters];
+    __shared__ uint32_t red[16];
+    const int t = threadIdx.x;
+    for (int i = t; i < kCounters; i += 128) data[4096 + i] = 0.0f;
+    BucketMap map{};
+    for (int row = blockIdx.x; row < n_rows; row += gridDim.x) {
+        for (int e = t; e < n; e += 128) data[e] = rows[static_cast<size_t>(row) * n + e];
+        __syncthreads();
+        float v[E];
+        cta_bucket_sort<E>(v, async::smem_u32(data), data, async::smem_u32(data + 4096), red, n, true, row == static_cast<int>(blockIdx.x), map,
+                           [] { __syncthreads(); });
+#pragma unroll
+        for (int r = 0; r < E; ++r)
+            if (t * E + r < n) keys[static_cast<size_t>(row) * n + t * E + r] = v[r];
+    }
+}
+
 }  // namespace cutoff

@@ -1,6 +1,7 @@
 // C ABI and host orchestration of the cutoff library (see include/cutoff.h).
 #include "../../include/cutoff.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1887,19 +1888,37 @@ int cutoff_debug_sort_values(cutoff_ctx* c, const float* rows, int64_t n_rows, i
     if (cudaMalloc(&d_rows, elems * 4) != cudaSuccess || cudaMalloc(&d_keys, elems * 4) != cudaSuccess) rc = CUTOFF_ERR_NOMEM;
     if (!rc && cudaMemcpyAsync(d_rows, rows, elems * 4, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) rc = CUTOFF_ERR_CUDA;
     if (!rc) {
-        const int P = next_pow2(n) < 32 ? 32 : next_pow2(n);
         const int rows_i = static_cast<int>(n_rows);
-        const int grid_w = ceil_div(rows_i, kSortWarps) < 4 * c->sm_count ? ceil_div(rows_i, kSortWarps) : 4 * c->sm_count;
-        const int grid_c = rows_i < 4 * c->sm_count ? rows_i : 4 * c->sm_count;
-        switch (P) {
-            case 32: k_debug_sort_values_warp<1><<<grid_w, kSortWarps * 32, 0, c->stream>>>(d_rows, n, rows_i, d_keys); break;
-            case 64: k_debug_sort_values_warp<2><<<grid_w, kSortWarps * 32, 0, c->stream>>>(d_rows, n, rows_i, d_keys); break;
-            case 128: k_debug_sort_values_warp<4><<<grid_w, kSortWarps * 32, 0, c->stream>>>(d_rows, n, rows_i, d_keys); break;
-            case 256: k_debug_sort_values_warp<8><<<grid_w, kSortWarps * 32, 0, c->stream>>>(d_rows, n, rows_i, d_keys); break;
-            case 512: k_debug_sort_values_warp<16><<<grid_w, kSortWarps * 32, 0, c->stream>>>(d_rows, n, rows_i, d_keys); break;
-            case 1024: k_debug_sort_values_warp<32><<<grid_w, kSortWarps * 32, 0, c->stream>>>(d_rows, n, rows_i, d_keys); break;
-            case 2048: k_debug_sort_values_cta<2><<<grid_c, 64, 0, c->stream>>>(d_rows, n, rows_i, d_keys); break;
-            default: k_debug_sort_values_cta<4><<<grid_c, 128, 0, c->stream>>>(d_rows, n, rows_i, d_keys);
+        const auto grid = [&](int rows_per_cta) { return std::min(ceil_div(rows_i, rows_per_cta), 4 * c->sm_count); };
+        const auto network = [&](auto* kernel) { kernel<<<grid(kSortWarps), kSortWarps * 32, 0, c->stream>>>(d_rows, n, rows_i, d_keys); };
+        const auto warps = [&](auto* kernel) { kernel<<<grid(8 * kDebugBucketWarps), kDebugBucketWarps * 32, 0, c->stream>>>(d_rows, n, rows_i, d_keys); };
+        const auto ctas = [&](auto* kernel) { kernel<<<grid(8), 128, 0, c->stream>>>(d_rows, n, rows_i, d_keys); };
+        if (n > 1024) {
+            switch (keys_per_thread(n, 128)) {
+                case 12: ctas(k_debug_bucket_cta<12>); break;
+                case 16: ctas(k_debug_bucket_cta<16>); break;
+                case 20: ctas(k_debug_bucket_cta<20>); break;
+                case 24: ctas(k_debug_bucket_cta<24>); break;
+                case 28: ctas(k_debug_bucket_cta<28>); break;
+                default: ctas(k_debug_bucket_cta<32>); break;
+            }
+        } else if (by_buckets(n, n_rows)) {
+            switch (keys_per_thread(n, 32)) {
+                case 8: warps(k_debug_bucket_warp<8>); break;
+                case 12: warps(k_debug_bucket_warp<12>); break;
+                case 16: warps(k_debug_bucket_warp<16>); break;
+                case 20: warps(k_debug_bucket_warp<20>); break;
+                case 24: warps(k_debug_bucket_warp<24>); break;
+                case 28: warps(k_debug_bucket_warp<28>); break;
+                default: warps(k_debug_bucket_warp<32>); break;
+            }
+        } else {
+            switch (n <= 32 ? 32 : next_pow2(n)) {
+                case 32: network(k_debug_sort_values_warp<1>); break;
+                case 64: network(k_debug_sort_values_warp<2>); break;
+                case 128: network(k_debug_sort_values_warp<4>); break;
+                default: network(k_debug_sort_values_warp<8>); break;
+            }
         }
         c->launches += 1;
         if (cudaMemcpyAsync(keys_out, d_keys, elems * 4, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||

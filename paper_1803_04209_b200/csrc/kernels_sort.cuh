@@ -608,9 +608,8 @@ __global__ void __launch_bounds__(WPR * 32) k_debug_sort_cta(const float* __rest
 }
 
 // ---------------------------------------------------------------------------------------------
-// Test hook: the float instantiation of the networks -- the one the decision path runs -- applied to
-// caller rows, the sorted rows written out instead of summed.  Rows are loaded, padded and sorted
-// exactly as k_sort_sum_* do it.
+// Test hook: the float instantiation of the network, as decisions run it on short rows, applied to caller rows, the sorted rows
+// written out instead of summed.  Rows are loaded, padded and sorted exactly as k_sort_sum_* do it.
 // ---------------------------------------------------------------------------------------------
 template <int E>
 __global__ void __launch_bounds__(kSortWarps * 32) k_debug_sort_values_warp(const float* __restrict__ rows, int n, int n_rows,
@@ -627,27 +626,6 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_debug_sort_values_warp(cons
 #pragma unroll
         for (int r = 0; r < E; ++r) {
             const int idx = lane * E + r;
-            if (idx < n) keys[static_cast<size_t>(row) * n + idx] = v[r];
-        }
-    }
-}
-
-template <int WPR>
-__global__ void __launch_bounds__(WPR * 32) k_debug_sort_values_cta(const float* __restrict__ rows, int n, int n_rows,
-                                                                     float* __restrict__ keys) {
-    __shared__ float xch[WPR * 1024];
-    constexpr int E = 32, T_ = WPR * 32;
-    for (int row = blockIdx.x; row < n_rows; row += gridDim.x) {
-        float v[E];
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int e = r * T_ + threadIdx.x;
-            v[r] = e < n ? rows[static_cast<size_t>(row) * n + e] : INFINITY;
-        }
-        cta_bitonic_sort<float, WPR>(v, xch);
-#pragma unroll
-        for (int r = 0; r < E; ++r) {
-            const int idx = threadIdx.x * E + r;
             if (idx < n) keys[static_cast<size_t>(row) * n + idx] = v[r];
         }
     }

@@ -111,7 +111,7 @@ def test_sort_permutation_bit_exact(n):
 
 @pytest.mark.parametrize("n", [1, 2, 33, 158, 512, 1024, 1025, 2175, 4096])
 def test_float_sort_rows_bit_exact(n):
-    # the fp32 instantiation of the network -- the one every decision runs -- row by row against numpy's sort:
+    # the sort that decisions run (network or buckets, by the row's length) row by row against numpy's sort:
     # continuous keys, many equal keys, both zeros, infinities among the keys, already sorted and reversed rows
     rng = np.random.default_rng(1000 + n)
     rows = [rng.standard_normal(n), rng.lognormal(0.0, 0.5, size=n), rng.integers(-3, 4, size=n) * 0.5,

@@ -200,3 +200,26 @@ def test_rows_that_change_between_spread_and_not(n, rows):
     sums = torch.empty(n, dtype=torch.float64, device="cuda")
     binding.sorted_row_sums_static(torch.from_numpy(x).cuda(), sums)
     _check(sums.cpu().numpy(), x)
+
+
+# Row by row and bit for bit, at the edges of the keys per thread: a warp (CTA) sorts rows of all kinds in turn, so that rows meet the
+# bucket map of another kind and scale.  129 to 256 keys take the buckets from 8192 rows on.
+@pytest.mark.parametrize("n,rows", [(128, 90), (129, 8192), (200, 8191), (256, 8200)] +
+                         [(n, 90) for e in range(8, 32, 4) for n in (32 * e, 32 * e + 1)] + [(1023, 90), (1024, 90)] +
+                         [(n, 90) for e in range(8, 32, 4) for n in (128 * e + 1, 128 * e + 128 * 4)] + [(2175, 90), (4095, 90)])
+def test_sorted_rows_bit_for_bit(n, rows):
+    rng = np.random.default_rng(n)
+    kinds = [_rows(k, rows, n, rng) for k in ("plain", "ties", "equal rows", "far clusters", "heavy tails", "changing scale", "infinities")]
+    kinds.append(np.where(rng.random((rows, n)) < 0.5, 0.0, -0.0).astype(np.float32))
+    kinds.append(np.sort(kinds[0], axis=1)[:, ::-1])
+    x = np.stack(kinds)[rng.integers(0, len(kinds), rows), np.arange(rows)]
+    ctx = binding.Cutoff(16, 4, 32, 1, 64)
+    got, want = ctx.debug_sort_values(x), np.sort(x, axis=1)
+    nonzero = want != 0
+    assert np.array_equal(got, want)
+    assert np.array_equal(got.view(np.uint32)[nonzero], want.view(np.uint32)[nonzero])
+    zeros = ~nonzero
+    assert np.array_equal(np.signbit(got).sum(axis=1), np.signbit(x).sum(axis=1))           # -0 before +0, none lost
+    for r in np.flatnonzero(zeros.any(axis=1)):
+        sign = np.signbit(got[r][zeros[r]])
+        assert np.all(sign[:-1] >= sign[1:])
