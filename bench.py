@@ -33,10 +33,6 @@ UNIT = "worker-times/s"
 SM_COUNT = 148
 FP32_LANES_PER_SM = 128          # fused multiply-add lanes per SM per clock
 MINMAX_LANES_PER_SM = 64         # fp32 min / max lanes per SM per clock (ALU pipe: 16 per sub-partition)
-# DRAM bytes per launch of the dominant kernel, from the ncu capture summarised under profiles/ (valid for the
-# kernel as committed with that summary; set to None when the kernel changes): the sample matrix read once
-# (grows with S) plus the partial rows written (one per CTA: does not grow with S).
-NCU_TRAFFIC = {}
 PRECISION_NAMES = {0: "f32", 1: "tf32", 2: "tf32(bf16 weights)"}
 
 
@@ -559,10 +555,8 @@ def main():
         peak_src = (f"{rates['source']}: {rates['fma']:.3f} fp32 FMA warp-instructions per clock per SM x 32 lanes "
                     f"x {SM_COUNT} SMs x {clock_mhz:.0f} MHz")
     achieved = amount / dur / 1e12
-    traffic = None if literal else NCU_TRAFFIC.get((wl.name, dominant))
     roofline = {"bound": bound, "kernel": dominant, "achieved": achieved, "peak": peak, "unit": unit,
-                "frac": achieved / peak, "traffic": traffic["bytes_per_sample"] * wl.S + traffic["bytes_fixed"] if traffic else None,
-                "traffic_source": traffic["source"] if traffic else None,
+                "frac": achieved / peak, "traffic": None, "traffic_source": None,        # DRAM bytes: profiles/
                 "algorithmic_per_launch": amount, "peak_source": peak_src,
                 "stage_ms": {k: round(v, 4) for k, v in stage_avg.items()}}
     # The path's model time: the slowest of the three resources the whole decision needs -- tensor cores (every

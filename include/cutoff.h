@@ -90,8 +90,9 @@ typedef struct {
     int32_t device;             /* CUDA device ordinal                                             */
     int32_t flags;              /* CUTOFF_FLAG_*                                                   */
     int64_t sample_offset;      /* index of this context's first sample in the global draw         */
-    int64_t total_samples;      /* samples of the whole decision (0 means n_samples); used only to
-                                   normalise when several contexts share one decision              */
+    int64_t total_samples;      /* samples of the whole decision (0 means n_samples); normalises when
+                                   several contexts share one decision, and chooses the kernel that
+                                   computes the samples, so that all of them draw alike              */
     void*   stream;             /* cudaStream_t the kernels run on; NULL = the default stream (with
                                    CUTOFF_FLAG_GRAPH: a stream the context creates, because the
                                    default stream cannot be captured)                              */

@@ -80,8 +80,8 @@ struct cutoff_ctx {
     bool have_std = false;
     double* d_sums = nullptr;       // [N]
 
-    CUtensorMap map_v{};            // TMA view of d_v   [alloc_rows][H]
-    CUtensorMap map_w4{};           // TMA view of W4    [2N][H]
+    CUtensorMap map_v{};            // TMA view of d_v16 [alloc_rows][H]
+    CUtensorMap map_w4{};           // TMA view of d_w16 [2N][H]
 
     bool literal = false;           // the networks as Section 3.1.3 prints them (CUTOFF_FLAG_LITERAL)
     LiteralDev lit{};
@@ -93,7 +93,7 @@ struct cutoff_ctx {
     float* d_W4T = nullptr;         // [H][2][ldx]        fp32 compact path: W4 with the columns of both heads contiguous
     float* d_M = nullptr;           // [H][H]             M, before it becomes rows of d_w16
     float* d_Mb = nullptr;          // [H]                b' = Wj1 bi2 + bj1 (tensor-core path: Wj1 I + bj1 = M u + b' with M = Wj1 Wi2)
-    CUtensorMap map_r{};            // TMA view of d_r [alloc_rows][H]
+    CUtensorMap map_r{};            // TMA view of d_r16 [alloc_rows][H]
     CUtensorMap map_wi2{}, map_M{}, map_wj2{};
     bool use_tc = false;            // emission output layer on tensor cores
     int pair_clusters = 0;          // clusters of two CTAs of the two-SM emission kernel that fit the GPU at once
@@ -1932,8 +1932,8 @@ int cutoff_debug_sort_values(cutoff_ctx* c, const float* rows, int64_t n_rows, i
 
 // Device memory for the duration of one call that has no context: taken from and returned to a memory pool of the
 // library's own, in the order of the call's stream, so calls on other threads and streams do not meet in it.  The pool keeps at
-// most kPoolKeeps bytes between calls (what exceeds that goes back to the driver at the next synchronisation; the
-// rest when another allocation of the process needs it): cudaMalloc and cudaFree took 1 to 10 ms per call, the kernels 60 us.
+// most kPoolKeeps bytes between calls, until the process ends (what exceeds that goes back to the driver at the next
+// synchronisation): cudaMalloc and cudaFree took 1 to 10 ms per call, the kernels 60 us.
 namespace {
 constexpr uint64_t kPoolKeeps = 64ull << 20;
 constexpr int kPoolDevices = 64;

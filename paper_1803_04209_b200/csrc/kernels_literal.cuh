@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(ChainShape<D>::kThreads) k_chain_literal(Model
 // CTA, 4 x 4 per thread.  K, lda and ldb are multiples of 4; entries of A and B beyond the logical K
 // must be zero (padded rows).
 //   kEpiAffine      out = acc + bias
-//   kEpiRelu        out = relu(acc + bias)                      (rounded to tf32 if round_out)
+//   kEpiRelu        out = relu(acc + bias)
 //   kEpiScaleNoise  out = add + softplus(acc + bias) * eps      (add: [M][ld_out]; eps: emission stream)
 // ---------------------------------------------------------------------------------------------
 enum { kEpiAffine = 0, kEpiRelu = 1, kEpiScaleNoise = 2 };
@@ -177,7 +177,6 @@ struct GemmFmaArgs {
     const float* add;
     float* out; int ld_out;
     int M, Nout, K;
-    int round_out;
     const DevState* st;
     NoiseKey key;
     uint32_t sample_base;
@@ -239,10 +238,7 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_fma(GemmFmaArgs a) {
             if (j >= a.Nout) continue;
             const size_t o = static_cast<size_t>(k) * a.ld_out + j;
             float v = acc[s][c] + a.bias[j];
-            if (EPI == kEpiRelu) {
-                v = fmaxf(v, 0.0f);
-                if (a.round_out) v = round_tf32(v);
-            }
+            if (EPI == kEpiRelu) v = fmaxf(v, 0.0f);
             if (EPI == kEpiScaleNoise) v = fmaf(softplusf(v), eps[c], a.add[o]);
             a.out[o] = v;
         }
