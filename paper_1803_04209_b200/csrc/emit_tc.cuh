@@ -16,10 +16,10 @@
 // epilogue (warp w reads TMEM lanes 32*(w%4).., the 32 workers of column group (w-2)/4).
 //
 // What bounds it, at N = 1024, S = 65536, H = 256 and at N = 4096, S = 32768, H = 512: as four-byte operands, the stream from
-// L2 to shared memory (0.148 and 0.432 ms).  As halves the stream and the tensor time are a half (0.122 and 0.297 ms); with the
-// weights resident (H = 256) a third of that stream remains (0.113 ms; H = 512: 0.290 ms).  Now no single
-// resource: issue slots 57 %, shared-memory and store wavefronts 64 %, tensor pipe 28 % (N = 1024); the drawing alone, without
-// operands and products, takes 0.104 and 0.200 ms, without the stores 0.111 and 0.295, without the products 0.112 and 0.241.
+// L2 to shared memory (0.148 and 0.432 ms); as halves, and with the weights resident (H = 256), it takes 0.122 and 0.309 ms.  Now no
+// single resource: issue slots 57 %, shared-memory and store wavefronts 65 %, tensor pipe 28 % (N = 1024).  Shares, from an
+// earlier capture in which it took 0.113 and 0.290: streamed weights 0.122 and 0.297, the drawing alone, without operands and
+// products, 0.104 and 0.200, without the stores 0.111 and 0.295, without the products 0.112 and 0.241.
 // 28 epilogue warps of 64 registers, with the generator's words in tables of the whole CTA, were slower (0.142 and 0.330 ms):
 // more instructions for the indexing than the occupancy gives.
 //
