@@ -257,7 +257,8 @@ int64_t cutoff_launch_count(cutoff_ctx* ctx);
  * captured (STATE).  "pair_emission": 1 = run the emission output layer (Section 3.1.3, x ~ N(I(z), J(z))) with
  * tensor-core instructions that span two SMs, so that each SM loads only half of every weight tile (compact variant
  * on a tensor-core precision only: UNSUPPORTED otherwise; same results as 0, the default, which is the faster one
- * as measured); not once a graph has been captured (STATE).  Errors: BAD_ARG, STATE, UNSUPPORTED. */
+ * as measured); not once a graph has been captured (STATE).  "order_stat_std" allocates device memory for more than
+ * 1024 workers.  Errors: BAD_ARG, STATE, UNSUPPORTED, NOMEM, CUDA. */
 int cutoff_set_option(cutoff_ctx* ctx, const char* name, int64_t value);
 
 /* ---- test hooks ----------------------------------------------------------------------------
