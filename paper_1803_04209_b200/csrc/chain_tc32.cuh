@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
                 if (!ok) break;
                 ++nz;
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint64_t a_desc = make_smem_desc(t_z);
                     const uint64_t b_lo = make_smem_desc(t_ra), b_hi = make_smem_desc(t_ra + 256u * 128u);
 #pragma unroll
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
                         if (!ok) break;
                     }
                     tc_fence_after();
-                    if (lane == 0) {
+                    if (elect_one()) {
                         const uint64_t a_desc = make_smem_desc(t_hb + b * 16384u);
                         const uint64_t b_first = make_smem_desc(t_rb + c * 4096u);          // Wmu, or the mean rows of W2
 #pragma unroll
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
                     if (!ok) break;
                     ++nz;
                     tc_fence_after();
-                    if (lane == 0) {
+                    if (elect_one()) {
                         const uint64_t a_desc = make_smem_desc(t_z), b_desc = make_smem_desc(t_ws);
 #pragma unroll
                         for (int k = 0; k < 4; ++k) umma_tf32(tmem_base, a_desc + 2 * k, b_desc + 2 * k, idesc_32, k != 0 ? 1u : 0u);
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
             }
         }
         if (!ok) {
-            if (lane == 0) umma_commit(bar_drain);
+            if (elect_one()) umma_commit(bar_drain);
             __syncwarp();
             mbar_wait_quiet(bar_drain, 0u);
         }

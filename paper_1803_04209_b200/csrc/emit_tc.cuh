@@ -16,7 +16,8 @@
 // epilogue (warp w reads TMEM lanes 32*(w%4).., the 32 workers of column group (w-2)/4).
 //
 // What bounds it, at N = 1024, S = 65536, H = 256 and at N = 4096, S = 32768, H = 512: as four-byte operands, the stream from
-// L2 to shared memory (0.148 and 0.432 ms); as halves, and with the weights resident (H = 256), it takes 0.122 and 0.309 ms.  Now no
+// L2 to shared memory (0.148 and 0.432 ms); as halves, with the weights resident (H = 256) and the
+// MMAs issued at their rate, it takes 0.119 and 0.282 ms.  Now no
 // single resource: issue slots 57 %, shared-memory and store wavefronts 65 %, tensor pipe 28 % (N = 1024).  Shares, from an
 // earlier capture in which it took 0.113 and 0.290: streamed weights 0.122 and 0.297, the drawing alone, without operands and
 // products, 0.104 and 0.200, without the stores 0.111 and 0.295, without the products 0.112 and 0.241.
@@ -75,6 +76,15 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr) {
     return d;
 }
 
+// True in one lane of the warp, always the same.  MMAs are issued from a branch on it: their operands are uniform registers, and only of
+// such a branch does the compiler know that one thread runs it; from a branch on a lane number each MMA takes 140 cycles to issue instead of 40,
+// more than the 128 that one of N = 256 occupies the tensor cores (emission at N = 4096, S = 32768, H = 512: 301 us so, 282 now; of the literal
+// networks at N = 1024, S = 65536: 165 and 152; N = 1024, H = 256: 121 and 119; the chain of D = 32, H = 512, S = 32768: 174 and 162).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t yes;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(yes));
+    return yes != 0;
+}
 __device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                           uint32_t accumulate) {
     asm volatile(
@@ -374,7 +384,7 @@ __device__ __forceinline__ void multiply_operands(const Pipeline& p, int lane) {
                  mbar_wait(p.full(stage), phase, p.abort_flag, p.st);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t a_addr = p.ring(stage), b_addr = p.resident ? p.tiles + kb * kBBytes : a_addr + A * kABytes;
                 const uint64_t a_desc = make_smem_desc(a_addr), b_desc = make_smem_desc(b_addr);
 #pragma unroll
@@ -401,7 +411,7 @@ __device__ __forceinline__ void multiply_operands(const Pipeline& p, int lane) {
     }
     if (!ok) {
         // make sure no MMA is still running before TMEM is released (bounded)
-        if (lane == 0) umma_commit(p.drain());
+        if (elect_one()) umma_commit(p.drain());
         __syncwarp();
         mbar_wait_quiet(p.drain(), 0u);
     }

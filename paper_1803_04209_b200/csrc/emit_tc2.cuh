@@ -177,7 +177,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
                 ok = mbar_wait(bar_full + 8 * stage, phase, abort_flag, a.st);
                 if (!ok) break;
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
 #pragma unroll
                     for (int j = 0; j < kStageK2; ++j) {
                         const uint32_t a_addr = tiles + stage * kStage2Bytes + j * (kABytes + kBBytes / 2);
@@ -196,7 +196,7 @@ k_emit_tc2(const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CU
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (!ok) {
-            if (lane == 0) umma_commit_pair(bar_drain, 1);
+            if (elect_one()) umma_commit_pair(bar_drain, 1);
             __syncwarp();
             const unsigned long long t0 = global_ns();
             while (!mbar_try_wait(bar_drain, 0u) && global_ns() - t0 < kWaitLimitNs) {}
