@@ -1,34 +1,48 @@
 // Per-sample chain (guide steps, transition, first emission layer) on the tcgen05 tensor cores,
-// for latent size 16 and hidden width 64..256, operands in tf32.  One kernel template serves both model
+// for latent size 16 and hidden width 64..256.  One kernel template serves both model
 // variants: the compact one (transition = one hidden layer with a [mean | logvar] head, then the emission's
 // hidden layer v) and the networks as Section 3.1.3 prints them (LITERAL: gated transition
 //      g = sigmoid(Wg2 relu(Wg1 z + bg1) + bg2)        h = Wh2 relu(Wh1 z + bh1) + bh2
 //      G = (1 - g) * (Wl z + bl) + g * h               H = softplus(Ws relu(G) + bs)        z' = G + H * eps
 // then the affine first layer of the emission mean, u = Wi1 z' + bi1).
 //
-// A CTA walks over tiles of 128 samples; sample r of the tile is TMEM lane r.  Every layer pair
-//      hidden = act(A z + a)          (M=128, N=H, K=16)
-//      out    = B hidden (+ b)        (M=128, N=16 or 32, K=H)
-// is two UMMA groups.  The first writes the hidden pre-activations to TMEM columns [0, H); the
-// epilogue warps read them 64 hidden units ("chunk") at a time, apply bias and activation, round
-// to tf32 and store the chunk as two K-major, 128-byte-swizzled A operand tiles in the buffer of
-// the tile's slot; the MMA warp multiplies that chunk with the matching K blocks of B while the
-// epilogue produces the same chunk of the other tile in flight.  The second result (mu; mean | logvar; gate;
-// proposal) is read back by all epilogue warps, which draw the noise, form the next latent and store it as the
-// next A operand.  In the literal variant the proposal's result is combined with the gate and the linear map
-// (computed by the epilogue threads from the latent tile) into G, relu(G) then takes the place of the latent
-// tile and one more small product with Ws gives the scale.
-// The last layer's hidden vector (v, or u) goes to global memory as halves for the emission output GEMMs (half_operand.cuh),
-// its scale from the largest |latent| of the sample.
+// A CTA walks over tiles of samples; a sample is a TMEM lane.  Every layer pair
+//      hidden = act(A z + a)          (M=128, N=H, K=16, tf32)
+//      out    = B hidden (+ b)        (M=128, N=16 or 32, K=H, halves)
+// is two UMMA groups.  The first writes the hidden pre-activations to TMEM columns [0, H) of the tile's slot.  Each
+// epilogue warp reads its lanes' quarter of the columns, applies bias and activation and writes the result as packed
+// halves over the columns that it has just read: the hidden layer is the A operand of the second product straight from tensor
+// memory and never passes through shared memory.  The second result (mu; mean | logvar; gate; proposal) is read back by all
+// epilogue warps, which draw the noise, form the next latent and store it as the next A operand of a first layer (shared
+// memory, tf32).  In the literal variant the proposal's result is combined with the gate and the linear map (computed by the
+// epilogue threads from the latent tile) into G, relu(G) then takes the place of the latent tile and one more small product
+// with Ws gives the scale.
+//
+// The halves carry the 11 bits of a tf32 value (half_operand.cuh): hidden values of the guide lie in [-1, 1] and are scaled by
+// 2^14, those of the other layers by a power of two from the sample's largest |latent|, rows of weights by one each.  Of the
+// guide's h_out = (tanh + h_left + h_right) / 3 only the tanh differs between samples, so only it is an operand:
+//      mu = (Wmu tanh) / 3 + [Wmu (h_left + h_right) / 3 + bmu],
+// the bracket, one vector of 16 per step, is formed in fp32 from the unrounded weights when the kernel starts.  The scale's linear
+// map Wsig mu + bsig comes out of the same product: its rows are those of Wsig Wmu, formed in double and split into two halves
+// each (together 22 bits), and a bracket of its own.  The first step starts from one latent for all samples, so its tanh is one vector
+// too and joins the bracket: that step is only noise.
+//
+// What bounds it: with two tiles in flight the special-function pipe, 256 tanh per sample and step and about 60 logarithms, sines and the
+// like for its noise (S=65536, D=16, H=256, lag 4: 68 us, of which 21 at that pipe's rate of 16 a clock; the rest is each step's round
+// trip, two products and the noise in between, which the other tile covers in part).  With the hidden layer through shared memory as
+// tf32, 64 units at a time, four steps of handshakes each, it took 108.  With one tile per SM, the steps' latency: 3700 cycles, of
+// which 1400 are the tanh (S=8192: 41 -> 27 us; 35 with tiles of 128).
 //
 // All weight operands live in shared memory for the whole kernel: the host prepares their
 // swizzled image once, the CTA copies it in at start.  Latent rows are 128 bytes wide (32 tf32)
 // although K = 16: two first-layer matrices share one tile (columns 0..15 and 16..31: [Wz | W1], or
 // [Wz | Wg1] and [Wh1 | Wi1]), so the MMA for the second of them simply starts 64 bytes into the rows.
+// The last layer's hidden vector (v, or u) goes to global memory as halves for the emission output GEMMs.
 //
-// Warp 0 issues the MMAs and owns TMEM; warps 1..16 are the epilogue: warp w serves TMEM lanes
-// 32*(w%4).. and column group cg = (w-1)/4: 16 of each chunk's 64 columns and the latent
-// dimensions 4cg..4cg+3 (one Philox call per stream and sample, as everywhere else).
+// A tile is the work of one warp that issues its MMAs and of 8 or 16 epilogue warps: warp w serves TMEM lanes 32*(w%4).. and one of
+// two or four column groups, that is its share of the hidden units and 8 or 4 of the latent dimensions (whole Philox calls).  Two tiles
+// of 8 warps each run side by side without knowing of each other, so that one's tanh meets the other's noise, products and waits;
+// a CTA with only one tile gives it all 16 warps.
 // Every mbarrier wait is bounded (see async.cuh).
 #pragma once
 #include "emit_tc.cuh"
@@ -37,34 +51,47 @@ namespace cutoff {
 namespace tc {
 
 constexpr int kChainEpiWarps = 16;
-constexpr int kChainTcThreads = (1 + kChainEpiWarps) * 32;
+constexpr int kChainTcThreads = (2 + kChainEpiWarps) * 32;
 constexpr int kChainD = 16;
+constexpr float kTanhScale = 16384.0f;       // a tanh as an operand: normal halves down to 2^-28
 
 struct ChainTcArgs {
-    // swizzled operand tiles.  compact: [Wz|W1] (H x 32), W3 (H x 32), Wmu (H/32 x 16 x 32), W2 (H/32 x 32 x 32);
-    // literal: [Wz|Wg1] (H x 32), [Wh1|Wi1] (H x 32), Wmu, Wg2, Wh2 (H/32 x 16 x 32 each), Ws (16 x 32)
-    const float* image;
+    // swizzled operand tiles.  compact: [Wz|W1] (H x 32 floats), W3 (H x 32), then halves: Wmu and the two parts of Wsig Wmu (H/64 x 48 x 64),
+    // W2 (H/64 x 32 x 64);  literal: [Wz|Wg1], [Wh1|Wi1] (H x 32 floats each), halves as before (H/64 x 48 x 64), Wg2, Wh2
+    // (H/64 x 16 x 64 each), Ws (16 x 32 floats).  Behind them, floats: the inverse scales of the rows of halves, in that order,
+    // then Wsig bmu + bsig (16) and Wsig Wmu (16 x H).
+    const uint8_t* image;
     // compact: b1, b3 = biases of the transition's and the emission's hidden layer, b2 = [mean | logvar] bias (32);
     // literal: b1 = bg1, b3 = bh1, b2 unused
-    const float *bz, *b1, *b3, *bmu, *bsig, *Wsig, *b2, *z0;
+    const float *bz, *b1, *b3, *bmu, *b2, *z0;
     const float *bi1, *bg2, *bh2, *Wl, *bl, *bs;       // literal variant only
+    const float *WzT, *Wmu;     // [16][H] each, fp32
     const float* hlr;           // [2][W][H] h_left, h_right
+    const float* bounds;        // [2][2] of the transition's hidden layer (literal: of the gate's and the proposal's), as HalfRows::bound
     DevState* st;
     NoiseKey key;
     uint32_t sample_base;
     int count, H, W;
-    HalfRows v_out;             // v (literal: u), rounded to tf32 and scaled
+    HalfRows v_out;             // v (literal: u), scaled
 };
 
-inline size_t chain_tc_image_floats(int H, bool literal = false) {
-    return literal ? static_cast<size_t>(H) * (32 + 32 + 16 + 16 + 16) + 16 * 32 : static_cast<size_t>(H) * (32 + 32 + 16 + 32);
-}
+// Bytes of the operand tiles, and floats behind them.
+inline size_t chain_tc_image_bytes(int H, bool literal) { return static_cast<size_t>(H) * 416 + (literal ? 16 * 128 : 0); }
+constexpr int kChainTcScales = 80;
+inline size_t chain_tc_image_floats(int H) { return kChainTcScales + 16 + 16 * static_cast<size_t>(H); }
 
 inline size_t chain_tc_smem_bytes(int H, int W, bool literal = false) {
-    const size_t tiles = chain_tc_image_floats(H, literal) * 4 + 2 * 128 * 128 /*Z x2*/ + 4 * 128 * 128 /*hidden chunks: 2 per slot*/;
-    const size_t floats = literal ? 4 * static_cast<size_t>(H) + static_cast<size_t>(W) * H + 2 * 16 * 16 + 7 * 16
-                                  : 3 * static_cast<size_t>(H) + static_cast<size_t>(W) * H + 16 * 16 + 16 + 16 + 32 + 16;
-    return 1024 + tiles + floats * 4 + 256;
+    const size_t floats = (literal ? 4 : 3) * static_cast<size_t>(H) + 4 * 128 + static_cast<size_t>(W) * (H + 32) + (literal ? 256 : 0) + kChainTcScales +
+                          (literal ? 64 : 32) + 32;
+    return 1024 + chain_tc_image_bytes(H, literal) + 2 * 16384 + floats * 4;
+}
+
+// Which windows: those whose states the kernel could hold beside its operands when it kept both in shared memory.  Longer ones
+// (H=256: from 14 steps on) have always gone through the fp32 kernels, and what is computed in fp32 stays so.
+inline bool chain_tc_window(int H, int W, bool literal) {
+    const size_t tiles = static_cast<size_t>(H) * 448 + (literal ? 2048 : 0) + 6 * 16384;
+    const size_t floats = literal ? 4 * static_cast<size_t>(H) + static_cast<size_t>(W) * H + 624 : 3 * static_cast<size_t>(H) + static_cast<size_t>(W) * H + 336;
+    return 1024 + tiles + floats * 4 + 256 <= 227 * 1024;
 }
 
 // byte offset of the 16-byte chunk `chunk` of row `row` in a K-major tile with 128-byte swizzled rows
@@ -113,8 +140,7 @@ __device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
     return v;
 }
 
-// The largest |latent| of a thread's dimensions, into the hidden-chunk buffer: all its chunks have been multiplied by now,
-// and the next one is written when every warp has begun the next tile, that is, finished the last layer, which reads it.
+// The largest |latent| of a thread's dimensions.
 template <int N>
 __device__ __forceinline__ void put_largest(uint32_t addr, const float (&z)[N]) {
     float m = 0.0f;
@@ -123,27 +149,86 @@ __device__ __forceinline__ void put_largest(uint32_t addr, const float (&z)[N]) 
     asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(m) : "memory");
 }
 
-// 16 consecutive halves: the two 16-byte halves of one sector.
+// 16 consecutive halves: one sector.
 __device__ __forceinline__ void store8(__half* p, const uint32_t (&w)[8]) {
-    *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-    *reinterpret_cast<uint4*>(p + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
 }
 
-// One of the two tiles a CTA has in flight: its shared-memory operands, TMEM columns and barriers,
-// and how many times each barrier has completed (both roles count the same sequence).
-struct ChainSlot {
-    uint32_t t_z;            // latent A operand [128 x 128 B]
-    uint32_t t_hb;           // two hidden-chunk A operands [128 x 128 B] each
-    uint32_t tmem;           // first of the slot's 256 TMEM columns
-    uint32_t bar_z, bar_p, bar_h, bar_hfree, bar_acc2;     // bar_h, bar_hfree: two barriers each
-    uint32_t nz, np, na, nu;
-    int tile;                // current tile, -1 if the slot is idle
-};
+// Sixteen consecutive accumulator columns of a warp's 32 lanes as they are spread by .32x32b (a lane's 16 columns in its thread), or
+// of its first 16 lanes by .16x256b: the thread's rows are lane / 4 and lane / 4 + 8, its columns 2 (lane % 4) and the one behind it, of each 8.
+// What is written back as packed halves takes the .32x32b and .16x128b spreads, under which a thread owns the pairs that it has read.
+__device__ __forceinline__ void tmem_ld16_half(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+}
+__device__ __forceinline__ void tmem_st8_half(uint32_t taddr, const uint32_t (&r)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x2.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-template <bool LITERAL>
+__device__ __forceinline__ void tmem_ld_dims(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld_dims(uint32_t taddr, uint32_t (&r)[8]) { tmem_ld8(taddr, r); }
+
+// D += A B with A in tensor memory (lanes = rows, two halves per column).
+__device__ __forceinline__ void umma_f16_tmem(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+
+__device__ __forceinline__ float tanh_hw(float x) {
+    float t;
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(x));
+    return t;
+}
+// tanh of two biased accumulators as a word of two scaled halves.
+__device__ __forceinline__ uint32_t tanh_pair(uint32_t acc0, uint32_t acc1, unsigned long long bias) {
+    float x0, x1;
+    unpack2(add2(pack2(__uint_as_float(acc0), __uint_as_float(acc1)), bias), x0, x1);
+    unpack2(mul2(pack2(tanh_hw(x0), tanh_hw(x1)), pack2(kTanhScale, kTanhScale)), x0, x1);
+    return pack_half2(x0, x1);
+}
+// The same of a ReLU layer (or an affine one), scaled by the sample's power of two.
+template <bool RELU>
+__device__ __forceinline__ uint32_t scaled_pair(uint32_t acc0, uint32_t acc1, unsigned long long bias, unsigned long long scale) {
+    float x0, x1;
+    unpack2(mul2(add2(pack2(__uint_as_float(acc0), __uint_as_float(acc1)), bias), scale), x0, x1);
+    return RELU ? pack_half2(fmaxf(x0, 0.0f), fmaxf(x1, 0.0f)) : pack_half2(x0, x1);
+}
+// Biases of 16 columns, from shared memory.
+__device__ __forceinline__ void load_bias(const float* bias, ulonglong2 (&b)[4]) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) b[g] = *reinterpret_cast<const ulonglong2*>(bias + 4 * g);
+}
+// Eight words from 16 columns of one lane.  act(acc0, acc1, bias pair).
+template <typename Act>
+__device__ __forceinline__ void pack_columns(const uint32_t (&acc)[16], const ulonglong2 (&b)[4], uint32_t (&w)[8], Act act) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        w[2 * g] = act(acc[4 * g], acc[4 * g + 1], b[g].x);
+        w[2 * g + 1] = act(acc[4 * g + 2], acc[4 * g + 3], b[g].y);
+    }
+}
+
+// WARPS: epilogue warps of a tile.  HALF: tiles of 64 samples, 16 lanes of each quarter of the tensor memory, for decisions that leave SMs
+// without a tile of 128.  A warp then spreads the 16 lanes' guide columns over its 32 threads; all else runs as in a full tile, the
+// other lanes on values that nobody reads.  The results of a sample are the same to the last bit in every shape.
+template <bool LITERAL, int WARPS, bool HALF>
 __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) {
     extern __shared__ uint8_t smem_raw[];
-    const int H = a.H, W = a.W;
+    constexpr int kRows = HALF ? 64 : 128;                        // samples per tile
+    constexpr int kSlots = kChainEpiWarps / WARPS, kGroups = WARPS / 4, kDims = kChainD / kGroups;
+    const int H = a.H, W = a.W, Hg = H / kGroups;                 // hidden units per column group
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* gen = smem_raw + (base - raw);
@@ -151,55 +236,53 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
     const uint32_t t_in0 = base;                                  // [Wz | W1]   or [Wz | Wg1]
     const uint32_t t_in1 = t_in0 + H * 128;                       // W3          or [Wh1 | Wi1]
     const uint32_t t_wmu = t_in1 + H * 128;
-    const uint32_t t_out1 = t_wmu + H * 64;                       // W2 (32 rows per K block) or Wg2 (16 rows)
-    const uint32_t t_out2 = t_out1 + H * 64;                      // literal: Wh2
-    const uint32_t t_ws = t_out2 + H * 64;                        // literal: Ws, 16 rows x 128 bytes
-    const uint32_t image_bytes = static_cast<uint32_t>(H) * 448u + (LITERAL ? 2048u : 0u);
-    const uint32_t t_act = base + image_bytes;                    // Z0, Z1, then 4 hidden-chunk buffers: 6 x 16 KB
+    const uint32_t t_out1 = t_wmu + H * 96;                       // W2 (32 rows per K block) or Wg2 (16 rows)
+    const uint32_t t_out2 = t_out1 + H * 32;                      // literal: Wh2
+    const uint32_t t_ws = t_out2 + H * 32;                        // literal: Ws, 16 rows x 128 bytes
+    const uint32_t image_bytes = static_cast<uint32_t>(H) * 416u + (LITERAL ? 2048u : 0u);
+    const uint32_t t_act = base + image_bytes;                    // latent tiles, one per slot
     // fp32 side tables
-    float* sbzs = reinterpret_cast<float*>(gen + image_bytes + 6 * 16384);    // bz
+    float* sbzs = reinterpret_cast<float*>(gen + image_bytes + 2 * 16384);    // bz
     float* sb1 = sbzs + H;
     float* sb3 = sb1 + H;
     float* sbi1 = sb3 + H;                   // literal only
-    float* slr = sb3 + (LITERAL ? 2 : 1) * H;        // [W][H]  (h_left + h_right) / 3
-    float* sWsig = slr + W * H;              // [16][16]
-    float* sWl = sWsig + 256;                // [16][16], literal only
-    float* sbmu = sWsig + (LITERAL ? 512 : 256);
-    float* sbsig = sbmu + 16;
-    float* sb2 = sbsig + 16;                 // compact: [32]
-    float* sbg2 = sbsig + 16;                // literal: bg2, bh2, bl, bs, 16 each
+    float* szmax = sb3 + (LITERAL ? 2 : 1) * H;      // [slot][column group][row] largest |latent| of a thread's dimensions
+    float* slr = szmax + 4 * 128;        // [W][H]  h_left + h_right (first step: + tanh)
+    float* sct = slr + W * H;                // [W][16]  Wmu (h_left + h_right) / 3 + bmu
+    float* spt = sct + W * 16;               // [W][16]  the same of the scale: Wsig times that, + bsig
+    float* sWl = spt + W * 16;               // [16][16], literal only
+    // what the products of halves are multiplied with: mu 16, the two parts of the scale's map 16 each, then W2 32 or Wg2, Wh2 16 each
+    float* sscale = sWl + (LITERAL ? 256 : 0);
+    float* sb2 = sscale + kChainTcScales;                // compact: [32]
+    float* sbg2 = sscale + kChainTcScales;               // literal: bg2, bh2, bl, bs, 16 each
     float* sbh2 = sbg2 + 16;
     float* sbl = sbh2 + 16;
     float* sbs = sbl + 16;
-    float* sz0 = LITERAL ? sbs + 16 : sb2 + 32;      // [16]
-    const uint32_t bars = smem_u32(sz0 + 16);                     // 2 slots x 7 barriers, then the drain barrier
-    const uint32_t bar_drain = bars + 2 * 56;
-    const uint32_t bar_img = bar_drain + 8;                       // the operand image has landed
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sz0 + 16 + 32);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(sz0 + 16 + 34);
+    float* sbar = LITERAL ? sbs + 16 : sb2 + 32;
+    const uint32_t bars = smem_u32(sbar);                         // 2 slots x 4 barriers, then the drain barriers
+    const uint32_t bar_img = bars + 2 * 40;                       // the operand image has landed
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sbar + 24);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(sbar + 25);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // ---- one-time set-up: barriers, operand image (bulk copies, while the side tables are filled), TMEM ----------
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < 2; ++s) {
-            const uint32_t b0 = bars + 56 * s;
-            mbar_init(b0, kChainEpiWarps);           // latent tile (or relu(G)) ready
+            const uint32_t b0 = bars + 40 * s;
+            mbar_init(b0, WARPS);                    // latent tile (or relu(G)) ready
             mbar_init(b0 + 8, 1);                    // hidden pre-activations ready
-            mbar_init(b0 + 16, kChainEpiWarps);      // hidden chunk buffer 0 written
-            mbar_init(b0 + 24, kChainEpiWarps);      // hidden chunk buffer 1 written
-            mbar_init(b0 + 32, 1);                   // hidden chunk buffer 0 multiplied
-            mbar_init(b0 + 40, 1);                   // hidden chunk buffer 1 multiplied
-            mbar_init(b0 + 48, 1);                   // second result ready
+            mbar_init(b0 + 16, WARPS);               // hidden layer written
+            mbar_init(b0 + 24, 1);                   // second result ready
+            mbar_init(b0 + 32, 1);                   // drained
         }
-        mbar_init(bar_drain, 1);
         mbar_init(bar_img, 1);
         *abort_flag = 0;
         fence_barrier_init();
         mbar_arrive_expect_tx(bar_img, image_bytes);
         for (uint32_t off = 0; off < image_bytes; off += 32768u) {
             const uint32_t n = image_bytes - off < 32768u ? image_bytes - off : 32768u;
-            bulk_load_1d(base + off, reinterpret_cast<const uint8_t*>(a.image) + off, n, bar_img);
+            bulk_load_1d(base + off, a.image + off, n, bar_img);
         }
     }
     if (warp == 0) {
@@ -207,34 +290,74 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                      ::"r"(smem_u32(const_cast<uint32_t*>(tmem_slot))), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    const float* const tail = reinterpret_cast<const float*>(a.image + image_bytes);
+    for (int i = threadIdx.x; i < H; i += kChainTcThreads) {
+        sbzs[i] = a.bz[i];
+        sb1[i] = a.b1[i];
+        sb3[i] = a.b3[i];
+        if (LITERAL) sbi1[i] = a.bi1[i];
+    }
+    if (LITERAL)
+        for (int i = threadIdx.x; i < 256; i += kChainTcThreads) sWl[i] = a.Wl[i];
+    if (threadIdx.x < kChainTcScales) {
+        const float inv = tail[threadIdx.x];
+        sscale[threadIdx.x] = threadIdx.x < 48 ? inv * (1.0f / (3.0f * kTanhScale)) : inv;
+    }
+    if (LITERAL && threadIdx.x < 16) {
+        sbg2[threadIdx.x] = a.bg2[threadIdx.x];
+        sbh2[threadIdx.x] = a.bh2[threadIdx.x];
+        sbl[threadIdx.x] = a.bl[threadIdx.x];
+        sbs[threadIdx.x] = a.bs[threadIdx.x];
+    }
+    if (!LITERAL && threadIdx.x < 32) sb2[threadIdx.x] = a.b2[threadIdx.x];
+    // hidden unit i of the first step, the same for every sample
+    float first_tanh = 0.0f;
+    if (threadIdx.x < H) {
+        float s = a.bz[threadIdx.x];
+#pragma unroll
+        for (int d = 0; d < 16; ++d) s = fmaf(a.WzT[d * H + threadIdx.x], a.z0[d], s);
+        first_tanh = tanhf(s);
+    }
+    // epilogue warp 2 + d: rows d of Wmu and of Wsig Wmu, for the parts of mu and of the scale that no sample changes
+    float wmu[8], wsm[8], bmu = 0.0f, bsm = 0.0f;
+    if (warp > 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int at = (warp - 2) * H + 32 * i + lane;
+            wmu[i] = 32 * i < H ? a.Wmu[at] : 0.0f;
+            wsm[i] = 32 * i < H ? tail[kChainTcScales + 16 + at] : 0.0f;
+        }
+        bmu = a.bmu[warp - 2];
+        bsm = tail[kChainTcScales + warp - 2];
+    }
     // up to here nothing an earlier kernel of the stream writes has been touched (the image and the biases are
     // weights): the encoder's states and the device state come after this point
     dependency_wait();
     launch_dependents();
-    {
-        for (int i = threadIdx.x; i < H; i += kChainTcThreads) {
-            sbzs[i] = a.bz[i];
-            sb1[i] = a.b1[i];
-            sb3[i] = a.b3[i];
-            if (LITERAL) sbi1[i] = a.bi1[i];
-        }
-        for (int i = threadIdx.x; i < W * H; i += kChainTcThreads) slr[i] = (a.hlr[i] + a.hlr[W * H + i]) * (1.0f / 3.0f);
-        for (int i = threadIdx.x; i < 256; i += kChainTcThreads) {
-            sWsig[i] = a.Wsig[i];
-            if (LITERAL) sWl[i] = a.Wl[i];
-        }
-        if (threadIdx.x < 16) {
-            sbmu[threadIdx.x] = a.bmu[threadIdx.x];
-            sbsig[threadIdx.x] = a.bsig[threadIdx.x];
-            sz0[threadIdx.x] = a.z0[threadIdx.x];
-            if (LITERAL) {
-                sbg2[threadIdx.x] = a.bg2[threadIdx.x];
-                sbh2[threadIdx.x] = a.bh2[threadIdx.x];
-                sbl[threadIdx.x] = a.bl[threadIdx.x];
-                sbs[threadIdx.x] = a.bs[threadIdx.x];
+    for (int i = threadIdx.x; i < W * H; i += kChainTcThreads) slr[i] = a.hlr[i] + a.hlr[W * H + i] + (i < H ? first_tanh : 0.0f);
+    __syncthreads();
+    if (warp > 1) {
+        // not unrolled: a launch finds the instruction caches cold, and this code runs once
+#pragma unroll 1
+        for (int t = 0; t < W; ++t) {
+            float s = 0.0f, p = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (32 * i < H) {
+                    const float v = slr[t * H + 32 * i + lane];
+                    s = fmaf(wmu[i], v, s);
+                    p = fmaf(wsm[i], v, p);
+                }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, off);
+                p += __shfl_xor_sync(0xffffffffu, p, off);
+            }
+            if (lane == 0) {
+                sct[t * 16 + warp - 2] = fmaf(s, 1.0f / 3.0f, bmu);
+                spt[t * 16 + warp - 2] = fmaf(p, 1.0f / 3.0f, bsm);
             }
         }
-        if (!LITERAL && threadIdx.x < 32) sb2[threadIdx.x] = a.b2[threadIdx.x];
     }
     tc_fence_before();
     __syncthreads();
@@ -243,339 +366,300 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
     // nothing starts before the weights are in place; if they never arrive every role skips its loop
     const bool image_ok = mbar_wait(bar_img, 0u, abort_flag, a.st);
 
-    ChainSlot slot[2];
-#pragma unroll
-    for (uint32_t s = 0; s < 2; ++s) {
-        const uint32_t b0 = bars + 56 * s;
-        slot[s].t_z = t_act + s * 16384u;
-        slot[s].t_hb = t_act + 2 * 16384u + s * 32768u;
-        slot[s].tmem = tmem_base + s * 256u;
-        slot[s].bar_z = b0; slot[s].bar_p = b0 + 8; slot[s].bar_h = b0 + 16; slot[s].bar_hfree = b0 + 32;
-        slot[s].bar_acc2 = b0 + 48;
-        slot[s].nz = slot[s].np = slot[s].na = slot[s].nu = 0;
-        slot[s].tile = -1;
-    }
-    const int n_tiles = image_ok ? ceil_div(a.count, 128) : 0;
+    const int n_tiles = image_ok ? ceil_div(a.count, kRows) : 0;
     // phases: W guide steps, then transition and emission hidden layer -- or gate, proposal (+ scale), first emission layer
     const int n_phases = LITERAL ? W + 3 : W + 2;
     const int ph_last = n_phases - 1;                             // its hidden layer goes to global memory, no second GEMM
-    // The second result of a tile (16 columns; mean | logvar: 32) reuses the first columns of the tile's
-    // pre-activation block: those are multiplied only after every warp has read chunk 0.
+    // A column group's hidden units stand, packed, in the first half of the columns of its pre-activations, group 1's in the second half.
+    // The second result (at most 48 columns) takes columns that hold neither: the other halves of groups 0 and 1 where H = 256 fills the slot.
+    const uint32_t acc2_col = H == 256 ? Hg / 2 : H;
 
-    // A hidden layer goes to the second GEMM in chunks of 64 units (two K blocks).  Each slot has one chunk buffer
-    // (its two 16 KB tiles); the chunks of the two tiles in flight are produced alternately -- (chunk 0, slot 0),
-    // (chunk 0, slot 1), (chunk 1, slot 0), ... -- so a slot's buffer is being multiplied while the other slot's is
-    // written, and both roles walk the same order.  sl.nu counts a slot's chunks: chunk n completes phase n of
-    // bar_h (written) and of bar_hfree (multiplied).
-    const int n_chunks64 = H / 64;
-
-    if (warp == 0) {
-        // ---------------- MMA issuer -------------------------------------------------------------------
-        const uint32_t idesc_h = instr_desc_tf32(H), idesc_16 = instr_desc_tf32(16), idesc_head = instr_desc_tf32(32);
-        bool ok = true;
-        for (int t0 = blockIdx.x; ok && t0 < n_tiles; t0 += 2 * gridDim.x) {
-            slot[0].tile = t0;
-            slot[1].tile = t0 + static_cast<int>(gridDim.x) < n_tiles ? t0 + static_cast<int>(gridDim.x) : -1;
-            for (int ph = 0; ok && ph < n_phases; ++ph) {
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {                       // first GEMM of both tiles
-                    ChainSlot& sl = slot[s];
-                    if (!ok || sl.tile < 0) continue;
-                    ok = mbar_wait(sl.bar_z, sl.nz & 1u, abort_flag, a.st);
-                    if (!ok) continue;
-                    ++sl.nz;
-                    tc_fence_after();
-                    if (lane == 0) {
-                        const uint32_t b_tile = ph < W ? t_in0 : (ph == W ? t_in0 + 64u : (ph == W + 1 ? t_in1 : t_in1 + 64u));
-                        const uint64_t a_desc = make_smem_desc(sl.t_z), b_desc = make_smem_desc(b_tile);
-                        umma_tf32(sl.tmem, a_desc, b_desc, idesc_h, 0u);
-                        umma_tf32(sl.tmem, a_desc + 2, b_desc + 2, idesc_h, 1u);
-                        umma_commit(sl.bar_p);
-                    }
-                    __syncwarp();
+    const int slot = warp < 2 ? warp : (warp - 2) / WARPS;
+    const uint32_t t_z = t_act + slot * 16384u;                   // latent A operand [128 x 128 B]
+    const uint32_t tmem = tmem_base + slot * 256u;                // first of the slot's 256 TMEM columns
+    const uint32_t bar_z = bars + 40 * slot, bar_p = bar_z + 8, bar_h = bar_z + 16, bar_acc2 = bar_z + 24, bar_drain = bar_z + 32;
+    const int tile0 = static_cast<int>(blockIdx.x) + slot * static_cast<int>(gridDim.x), tile_step = kSlots * static_cast<int>(gridDim.x);
+    bool ok = true;
+    if (warp < kSlots) {
+        // ---------------- MMA issuer of the slot ---------------------------------------------------------
+        const uint32_t idesc_h = instr_desc_tf32(H);
+        uint32_t nz = 0, nh = 0;
+        for (int tile = tile0; ok && tile < n_tiles; tile += tile_step) {
+            for (int ph = 1; ph < n_phases; ++ph) {
+                ok = mbar_wait(bar_z, nz & 1u, abort_flag, a.st);
+                if (!ok) break;
+                ++nz;
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint32_t b_tile = ph < W ? t_in0 : (ph == W ? t_in0 + 64u : (ph == W + 1 ? t_in1 : t_in1 + 64u));
+                    const uint64_t a_desc = make_smem_desc(t_z), b_desc = make_smem_desc(b_tile);
+                    umma_tf32(tmem, a_desc, b_desc, idesc_h, 0u);
+                    umma_tf32(tmem, a_desc + 2, b_desc + 2, idesc_h, 1u);
+                    umma_commit(bar_p);
                 }
+                __syncwarp();
                 if (ph == ph_last) continue;                       // the last hidden layer has no second GEMM here
-                const uint32_t b_base = ph < W ? t_wmu : (ph == W ? t_out1 : t_out2);
-                const uint32_t slab = LITERAL || ph < W ? 16u * 128u : 32u * 128u;
-                const uint32_t idesc2 = LITERAL || ph < W ? idesc_16 : idesc_head;
-                for (int c = 0; ok && c < n_chunks64; ++c) {        // second GEMM, chunk by chunk as the epilogue delivers
-#pragma unroll
-                    for (int s = 0; s < 2; ++s) {
-                        ChainSlot& sl = slot[s];
-                        if (!ok || sl.tile < 0) continue;
-                        ok = mbar_wait(sl.bar_h, sl.nu & 1u, abort_flag, a.st);
-                        if (!ok) continue;
-                        ++sl.nu;
-                        tc_fence_after();
-                        if (lane == 0) {
-#pragma unroll
-                            for (int kb = 0; kb < 2; ++kb) {
-                                const uint64_t a_desc = make_smem_desc(sl.t_hb + kb * 16384u);
-                                const uint64_t b_desc = make_smem_desc(b_base + (2 * c + kb) * slab);
-#pragma unroll
-                                for (int k = 0; k < 4; ++k)
-                                    umma_tf32(sl.tmem, a_desc + 2 * k, b_desc + 2 * k, idesc2, (c | kb | k) != 0 ? 1u : 0u);
-                            }
-                            umma_commit(sl.bar_hfree);
-                            if (c == n_chunks64 - 1) umma_commit(sl.bar_acc2);
+                ok = mbar_wait(bar_h, nh & 1u, abort_flag, a.st);
+                if (!ok) break;
+                ++nh;
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint32_t b_base = ph < W ? t_wmu : (ph == W ? t_out1 : t_out2);
+                    const uint32_t out_rows = ph < W ? 48u : (LITERAL ? 16u : 32u), idesc2 = instr_desc_f16(out_rows, 128);
+                    uint64_t b_desc = make_smem_desc(b_base);
+                    uint32_t more = 0, k = 0;
+                    for (int g = 0; g < kGroups; ++g) {
+                        const uint32_t packed = tmem + g * Hg + (g == 1 ? Hg / 2 : 0);
+                        for (int c = 0; c < Hg / 2; c += 8) {                // 16 hidden units: 8 columns, 32 bytes of a row of B
+                            umma_f16_tmem(tmem + acc2_col, packed + c, b_desc, idesc2, more);
+                            more = 1;
+                            k += 16;
+                            b_desc += k & 63 ? 2 : out_rows * 8 - 6;         // the next 32 bytes, or the next K block
                         }
-                        __syncwarp();
                     }
+                    umma_commit(bar_acc2);
                 }
+                __syncwarp();
                 if (!LITERAL || ph != W + 1) continue;
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {                       // scale: Ws relu(G), relu(G) sits in the latent tile
-                    ChainSlot& sl = slot[s];
-                    if (!ok || sl.tile < 0) continue;
-                    ok = mbar_wait(sl.bar_z, sl.nz & 1u, abort_flag, a.st);
-                    if (!ok) continue;
-                    ++sl.nz;
-                    tc_fence_after();
-                    if (lane == 0) {
-                        const uint64_t a_desc = make_smem_desc(sl.t_z), b_desc = make_smem_desc(t_ws);
-                        umma_tf32(sl.tmem, a_desc, b_desc, idesc_16, 0u);
-                        umma_tf32(sl.tmem, a_desc + 2, b_desc + 2, idesc_16, 1u);
-                        umma_commit(sl.bar_acc2);
-                    }
-                    __syncwarp();
+                // scale: Ws relu(G), relu(G) sits in the latent tile
+                ok = mbar_wait(bar_z, nz & 1u, abort_flag, a.st);
+                if (!ok) break;
+                ++nz;
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint64_t a_desc = make_smem_desc(t_z), b_desc = make_smem_desc(t_ws);
+                    umma_tf32(tmem + acc2_col, a_desc, b_desc, instr_desc_tf32(16), 0u);
+                    umma_tf32(tmem + acc2_col, a_desc + 2, b_desc + 2, instr_desc_tf32(16), 1u);
+                    umma_commit(bar_acc2);
                 }
+                __syncwarp();
             }
         }
         if (!ok) {
-            if (lane == 0) umma_commit(bar_drain);
+            if (elect_one()) umma_commit(bar_drain);
             __syncwarp();
             mbar_wait_quiet(bar_drain, 0u);
         }
         __syncwarp();
-    } else {
+    } else if (warp >= 2) {
         // ---------------- epilogue ---------------------------------------------------------------------
-        const int q = warp & 3, cg = (warp - 1) >> 2;
-        const int row = q * 32 + lane;                                            // TMEM lane = sample of the tile
+        const int q = warp & 3, cg = ((warp - 2) % WARPS) >> 2;
+        const int row = q * 32 + lane;                                            // TMEM lane, row of the latent tile
+        const int sample_row = HALF ? q * 16 + lane : row;                        // sample of the tile (HALF: lanes 0 .. 15)
+        const bool mine = !HALF || lane < 16;
         const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
         const uint32_t step = a.st->step;
-        const uint32_t hb_off = static_cast<uint32_t>(cg >> 1) * 16384u;          // K block of the chunk this warp writes
-        const int hb_chunk = 4 * (cg & 1);                                        // its first 16-byte chunk in a row
-        float gate_own[2][4], lin_own[2][4], G_own[2][4];     // literal: per tile in flight, latent dimensions 4cg..4cg+3
-        bool ok = true;
-        float v_scale[2] = {1.0f, 1.0f};                                          // per tile in flight: of its last layer's row
-        for (int t0 = blockIdx.x; ok && t0 < n_tiles; t0 += 2 * gridDim.x) {
-            slot[0].tile = t0;
-            slot[1].tile = t0 + static_cast<int>(gridDim.x) < n_tiles ? t0 + static_cast<int>(gridDim.x) : -1;
+        // 16 columns at a time, packed over columns that have been read: group 1 from its last ones on, towards the end of its columns
+        const int batches = Hg / 16, first = cg == 1 ? batches - 1 : 0, dir = cg == 1 ? -1 : 1;
+        const uint32_t cols = tmem + lane_off + static_cast<uint32_t>(cg * Hg), packed = cols + static_cast<uint32_t>(cg == 1 ? Hg / 2 : 0);
+        const uint32_t res = tmem + lane_off + acc2_col + kDims * cg;             // this thread's columns of a second result
+        const int d0 = kDims * cg;                                                // its latent dimensions
+        float* const largest = szmax + slot * kGroups * 128 + row;                // [column group][128]
+        float gate_own[kDims], lin_own[kDims], G_own[kDims];                      // literal
+        uint32_t np = 0, na = 0;
+        const auto arrive = [&](uint32_t bar) {                     // our reads and writes precede the MMAs that this unblocks
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar);
+        };
+        const auto store_latent = [&](const float (&z)[kDims]) {
 #pragma unroll
-            for (int s = 0; s < 2; ++s) {                           // initial latent z_{T-l-1} of both tiles
-                if (slot[s].tile < 0) continue;
-                st_shared_v4(slot[s].t_z + sw128(row, cg), tf32_rna(sz0[4 * cg + 0]), tf32_rna(sz0[4 * cg + 1]),
-                             tf32_rna(sz0[4 * cg + 2]), tf32_rna(sz0[4 * cg + 3]));
-                fence_proxy_async();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(slot[s].bar_z);
-            }
-            for (int ph = 0; ok && ph < n_phases; ++ph) {
-                const float* bias = ph < W ? sbzs : (ph == W ? sb1 : (ph == W + 1 ? sb3 : sbi1));
-                const float* lr = slr + (ph < W ? ph : 0) * H;
-                // ---- hidden layer of both tiles: bias, activation, next A operand (or v) -----------------
-                for (int c = 0; ok && c < n_chunks64; ++c) {
+            for (int c = 0; c < kDims; c += 4)
+                st_shared_v4(t_z + sw128(row, (d0 + c) / 4), tf32_rna(z[c]), tf32_rna(z[c + 1]), tf32_rna(z[c + 2]), tf32_rna(z[c + 3]));
+            fence_proxy_async();
+            arrive(bar_z);
+        };
+        for (int tile = tile0; ok && tile < n_tiles; tile += tile_step) {
+            const int k = tile * kRows + sample_row;
+            const uint32_t sample = a.sample_base + static_cast<uint32_t>(k);
+            float z_own[kDims], eps[kDims];
+            Philox4 words[kDims / 4];
+            const auto draw_words = [&](uint32_t stream) {
 #pragma unroll
-                    for (int s = 0; s < 2; ++s) {
-                        ChainSlot& sl = slot[s];
-                        if (!ok || sl.tile < 0) continue;
-                        if (c == 0) {
-                            ok = mbar_wait(sl.bar_p, sl.np & 1u, abort_flag, a.st);
-                            if (!ok) continue;
-                            ++sl.np;
-                            tc_fence_after();
-                            if (ph == ph_last) {                   // the four column groups' largest |latent| of this sample
-                                float zm = 0.0f, inv;
+                for (int c = 0; c < kDims / 4; ++c) words[c] = philox4x32_10(static_cast<uint32_t>(d0 / 4 + c), sample, stream, step, a.key.seed_lo, a.key.seed_hi);
+            };
+            const auto draw_normals = [&] {
 #pragma unroll
-                                for (int gg = 0; gg < 4; ++gg) zm = fmaxf(zm, ld_shared_f32(sl.t_hb + (gg * 128 + row) * 4));
-                                half_scale(a.v_out, zm, v_scale[s], inv);
-                                const int k = sl.tile * 128 + row;
-                                if (cg == 0 && k < a.count) a.v_out.inv_scale[k] = inv;
+                for (int c = 0; c < kDims; c += 4) {
+                    box_muller_fast(words[c / 4].x, words[c / 4].y, eps[c], eps[c + 1]);
+                    box_muller_fast(words[c / 4].z, words[c / 4].w, eps[c + 2], eps[c + 3]);
+                }
+            };
+            draw_words(0u);                                                       // the first guide step
+            draw_normals();
+#pragma unroll
+            for (int c = 0; c < kDims; ++c) z_own[c] = fmaf(softplus_fast(spt[d0 + c]), eps[c], sct[d0 + c]);
+            if (W == 1) put_largest(smem_u32(largest + cg * 128), z_own);
+            store_latent(z_own);
+            float h_inv = 1.0f;                                                   // inverse scale of the hidden layer
+            for (int ph = 1; ph < n_phases; ++ph) {
+                const float* bias = (ph < W ? sbzs : (ph == W ? sb1 : (ph == W + 1 ? sb3 : sbi1))) + cg * Hg;
+                // the generator's words while the pre-activations are formed: they depend on nothing (literal: the gate draws nothing)
+                if (ph != ph_last && (!LITERAL || ph != W)) draw_words(ph < W ? static_cast<uint32_t>(ph) : kStreamTransition);
+                // ---- hidden layer: bias, activation, next A operand (or v) -----------------
+                ok = mbar_wait(bar_p, np & 1u, abort_flag, a.st);
+                if (!ok) break;
+                ++np;
+                tc_fence_after();
+                if (HALF && ph < W) {
+                    const float* thread_bias = bias + 2 * (lane & 3);
+                    uint32_t acc[2][8];
+                    tmem_ld16_half(cols + 16 * first, acc[0]);
+#pragma unroll 1
+                    for (int b = 0; b < batches; b += 2) {
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            if (b + u >= batches) break;
+                            const int at = first + dir * (b + u);
+                            tmem_ld_wait();
+                            if (b + u + 1 < batches) tmem_ld16_half(cols + 16 * (at + dir), acc[u ^ 1]);
+                            uint32_t w[4];
+#pragma unroll
+                            for (int g = 0; g < 2; ++g) {
+                                const unsigned long long bv = *reinterpret_cast<const unsigned long long*>(thread_bias + 16 * at + 8 * g);
+                                w[2 * g] = tanh_pair(acc[u][4 * g], acc[u][4 * g + 1], bv);
+                                w[2 * g + 1] = tanh_pair(acc[u][4 * g + 2], acc[u][4 * g + 3], bv);
                             }
-                        }
-                        const int col0 = c * 64 + cg * 16;
-                        uint32_t acc[16];
-                        tmem_ld16(sl.tmem + lane_off + col0, acc);
-                        tmem_ld_wait();
-                        float h[16];
-#pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            const float4 bq = *reinterpret_cast<const float4*>(bias + col0 + 4 * g);
-                            const float bv[4] = {bq.x, bq.y, bq.z, bq.w};
-                            if (ph < W) {
-                                const float4 lq = *reinterpret_cast<const float4*>(lr + col0 + 4 * g);
-                                const float lv[4] = {lq.x, lq.y, lq.z, lq.w};
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {      // tanh, then (tanh + h_left + h_right) / 3
-                                    float t;
-                                    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(__uint_as_float(acc[4 * g + i]) + bv[i]));
-                                    h[4 * g + i] = fmaf(t, 1.0f / 3.0f, lv[i]);
-                                }
-                            } else if (LITERAL && ph == ph_last) {  // u = Wi1 z' + bi1: no activation
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) h[4 * g + i] = __uint_as_float(acc[4 * g + i]) + bv[i];
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) h[4 * g + i] = fmaxf(__uint_as_float(acc[4 * g + i]) + bv[i], 0.0f);
-                            }
-                        }
-                        if (ph != ph_last) {
-                            if (sl.nu >= 1) {                      // the buffer's previous contents must have been multiplied
-                                ok = mbar_wait(sl.bar_hfree, (sl.nu - 1u) & 1u, abort_flag, a.st);
-                                if (!ok) continue;
-                            }
-                            const uint32_t dst = sl.t_hb + hb_off;
-#pragma unroll
-                            for (int g = 0; g < 4; ++g)
-                                st_shared_v4(dst + sw128(row, hb_chunk + g), tf32_rna(h[4 * g]), tf32_rna(h[4 * g + 1]),
-                                             tf32_rna(h[4 * g + 2]), tf32_rna(h[4 * g + 3]));
-                            fence_proxy_async();
-                            tc_fence_before();                     // our TMEM reads of this chunk precede the MMAs it unblocks
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(sl.bar_h);
-                            ++sl.nu;
-                        } else {
-                            const int k = sl.tile * 128 + row;
-                            if (k < a.count) {
-                                uint32_t w[8];
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) w[i] = pack_half2(tf32_rna(h[2 * i]) * v_scale[s], tf32_rna(h[2 * i + 1]) * v_scale[s]);
-                                store8(a.v_out.p + static_cast<size_t>(k) * a.v_out.ld + col0, w);      // one whole 32-byte sector
-                            }
+                            tmem_st8_half(packed + 8 * at, w);
                         }
                     }
-                }
-                if (!ok || ph == ph_last) continue;
-                // ---- second result of both tiles: the next latent (literal: gate, then G and relu(G)) ------------
+                } else {
+                    unsigned long long scale2 = 0;
+                    if (ph >= W) {                                  // the column groups' largest |latent| of this sample
+                        float zm = 0.0f, scale;
 #pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    ChainSlot& sl = slot[s];
-                    if (!ok || sl.tile < 0) continue;
-                    const uint32_t sample = a.sample_base + static_cast<uint32_t>(sl.tile * 128 + row);
-                    float eps[4];                                   // drawn before the wait: the noise does not depend on the result
-                    if (!LITERAL || ph < W)
-                        normal4_fast(static_cast<uint32_t>(cg), sample, ph < W ? static_cast<uint32_t>(ph) : kStreamTransition, step,
-                                     a.key.seed_lo, a.key.seed_hi, eps);
-                    ok = mbar_wait(sl.bar_acc2, sl.na & 1u, abort_flag, a.st);
-                    if (!ok) continue;
-                    ++sl.na;
-                    tc_fence_after();
-                    float z_own[4];
-                    bool store_z = true;
-                    if (ph < W) {
-                        // guide: z = mu + softplus(Wsig mu + bsig) * eps
-                        uint32_t mu_bits[16];
-                        tmem_ld16(sl.tmem + lane_off, mu_bits);
-                        tmem_ld_wait();
-                        float mu[16];
-#pragma unroll
-                        for (int d = 0; d < 16; ++d) mu[d] = __uint_as_float(mu_bits[d]) + sbmu[d];
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const float* wrow = sWsig + (4 * cg + c) * 16;
-                            float pre = sbsig[4 * cg + c];
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) pre = fmaf(wrow[e], mu[e], pre);
-                            float own = 0.0f;
-#pragma unroll
-                            for (int gg = 0; gg < 4; ++gg)
-                                if (gg == cg) own = mu[4 * gg + c];
-                            z_own[c] = fmaf(softplus_fast(pre), eps[c], own);
+                        for (int gg = 0; gg < kGroups; ++gg) zm = fmaxf(zm, largest[gg * 128]);
+                        const float* bound = ph == ph_last ? a.v_out.bound : a.bounds + 2 * (ph - W);
+                        half_scale(1.01f * fmaf(__ldg(bound), zm, __ldg(bound + 1)), scale, h_inv);
+                        scale2 = pack2(scale, scale);
+                        if (ph == ph_last && cg == 0 && mine && k < a.count) a.v_out.inv_scale[k] = h_inv;
+                    }
+                    const auto act16 = [&](const uint32_t (&acc)[16], const ulonglong2 (&bv)[4], int at) {
+                        uint32_t w[8];
+                        if (ph < W) {
+                            pack_columns(acc, bv, w, [](uint32_t x0, uint32_t x1, unsigned long long b) { return tanh_pair(x0, x1, b); });
+                        } else if (LITERAL && ph == ph_last) {  // u = Wi1 z' + bi1: no activation
+                            pack_columns(acc, bv, w, [&](uint32_t x0, uint32_t x1, unsigned long long b) { return scaled_pair<false>(x0, x1, b, scale2); });
+                        } else {
+                            pack_columns(acc, bv, w, [&](uint32_t x0, uint32_t x1, unsigned long long b) { return scaled_pair<true>(x0, x1, b, scale2); });
                         }
-                    } else if constexpr (!LITERAL) {
-                        uint32_t mean_bits[16], lv_bits[16];
-                        tmem_ld16(sl.tmem + lane_off, mean_bits);
-                        tmem_ld16(sl.tmem + lane_off + 16, lv_bits);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            float mean = 0.0f, lv = 0.0f;
-#pragma unroll
-                            for (int gg = 0; gg < 4; ++gg)
-                                if (gg == cg) { mean = __uint_as_float(mean_bits[4 * gg + c]); lv = __uint_as_float(lv_bits[4 * gg + c]); }
-                            z_own[c] = fmaf(exp_half_fast(lv + sb2[16 + 4 * cg + c]), eps[c], mean + sb2[4 * cg + c]);
+                        if (ph != ph_last) tmem_st8(packed + 8 * at, w);
+                        else if (mine && k < a.count) store8(a.v_out.p + static_cast<size_t>(k) * a.v_out.ld + cg * Hg + 16 * at, w);   // one sector
+                    };
+                    uint32_t acc[2][16];
+                    ulonglong2 bv[2][4];
+                    if constexpr (WARPS == 8) {
+                        // 32 columns at a time (Hg is a multiple of 32): two warps per scheduler keep the special-function pipe busy only with that
+                        // many independent values each
+#pragma unroll 1
+                        for (int b = 0; b < batches; b += 2) {
+                            const int at = first + dir * b;
+                            tmem_ld16(cols + 16 * at, acc[0]);
+                            tmem_ld16(cols + 16 * (at + dir), acc[1]);
+                            load_bias(bias + 16 * at, bv[0]);
+                            load_bias(bias + 16 * (at + dir), bv[1]);
+                            tmem_ld_wait();
+                            act16(acc[0], bv[0], at);
+                            act16(acc[1], bv[1], at + dir);
                         }
                     } else {
-                        uint32_t res_bits[16];
-                        tmem_ld16(sl.tmem + lane_off, res_bits);
-                        tmem_ld_wait();
-                        float own[4];                               // this thread's four of the 16 results
+                        tmem_ld16(cols + 16 * first, acc[0]);
+                        load_bias(bias + 16 * first, bv[0]);
+#pragma unroll 1
+                        for (int b = 0; b < batches; b += 2) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            own[c] = 0.0f;
-#pragma unroll
-                            for (int gg = 0; gg < 4; ++gg)
-                                if (gg == cg) own[c] = __uint_as_float(res_bits[4 * gg + c]);
-                        }
-                        if (ph == W) {
-                            // gate g, and the linear map Wl z + bl from the latent tile (it stays as it is for the proposal)
-                            float z[16];
-#pragma unroll
-                            for (int e4 = 0; e4 < 4; ++e4) {
-                                const float4 zq = ld_shared_v4(sl.t_z + sw128(row, e4));
-                                z[4 * e4 + 0] = zq.x; z[4 * e4 + 1] = zq.y; z[4 * e4 + 2] = zq.z; z[4 * e4 + 3] = zq.w;
-                            }
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                gate_own[s][c] = sigmoid_fast(own[c] + sbg2[4 * cg + c]);
-                                const float* wrow = sWl + (4 * cg + c) * 16;
-                                float lin = sbl[4 * cg + c];
-#pragma unroll
-                                for (int e = 0; e < 16; ++e) lin = fmaf(wrow[e], z[e], lin);
-                                lin_own[s][c] = lin;
-                            }
-                            store_z = false;
-                        } else {
-                            // proposal h -> G = (1 - g) * lin + g * h; relu(G) replaces the latent tile for the scale product
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                const float prop = own[c] + sbh2[4 * cg + c];
-                                G_own[s][c] = fmaf(gate_own[s][c], prop - lin_own[s][c], lin_own[s][c]);
-                                z_own[c] = fmaxf(G_own[s][c], 0.0f);
+                            for (int u = 0; u < 2; ++u) {
+                                if (b + u >= batches) break;
+                                const int at = first + dir * (b + u);
+                                tmem_ld_wait();
+                                if (b + u + 1 < batches) {
+                                    tmem_ld16(cols + 16 * (at + dir), acc[u ^ 1]);
+                                    load_bias(bias + 16 * (at + dir), bv[u ^ 1]);
+                                }
+                                act16(acc[u], bv[u], at);
                             }
                         }
                     }
-                    if (!LITERAL && ph == W) put_largest(sl.t_hb + (cg * 128 + row) * 4, z_own);
-                    if (store_z) {
-                        st_shared_v4(sl.t_z + sw128(row, cg), tf32_rna(z_own[0]), tf32_rna(z_own[1]), tf32_rna(z_own[2]), tf32_rna(z_own[3]));
-                        fence_proxy_async();
-                    }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(sl.bar_z);
                 }
-                if (!LITERAL || !ok || ph != W + 1) continue;
-                // ---- literal: scale of both tiles, z' = G + softplus(Ws relu(G) + bs) * eps ------------------
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    ChainSlot& sl = slot[s];
-                    if (!ok || sl.tile < 0) continue;
-                    const uint32_t sample = a.sample_base + static_cast<uint32_t>(sl.tile * 128 + row);
-                    float eps[4], z_own[4];
-                    normal4_fast(static_cast<uint32_t>(cg), sample, kStreamTransition, step, a.key.seed_lo, a.key.seed_hi, eps);
-                    ok = mbar_wait(sl.bar_acc2, sl.na & 1u, abort_flag, a.st);
-                    if (!ok) continue;
-                    ++sl.na;
-                    tc_fence_after();
-                    uint32_t res_bits[16];
-                    tmem_ld16(sl.tmem + lane_off, res_bits);
+                if (ph == ph_last) continue;
+                tmem_st_wait();
+                arrive(bar_h);
+                // ---- second result: the next latent (literal: gate, then G and relu(G), then the scale) ------------
+                if (!LITERAL || ph != W) draw_normals();
+                ok = mbar_wait(bar_acc2, na & 1u, abort_flag, a.st);
+                if (!ok) break;
+                ++na;
+                tc_fence_after();
+                uint32_t r0[kDims];
+                tmem_ld_dims(res, r0);
+                if (ph < W) {
+                    // guide: z = mu + softplus(Wsig mu + bsig) * eps
+                    uint32_t hi[kDims], lo[kDims];
+                    tmem_ld_dims(res + 16, hi);
+                    tmem_ld_dims(res + 32, lo);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        float pre = 0.0f;
-#pragma unroll
-                        for (int gg = 0; gg < 4; ++gg)
-                            if (gg == cg) pre = __uint_as_float(res_bits[4 * gg + c]);
-                        z_own[c] = fmaf(softplus_fast(pre + sbs[4 * cg + c]), eps[c], G_own[s][c]);
+                    for (int c = 0; c < kDims; ++c) {
+                        const int d = d0 + c;
+                        const float pre = fmaf(__uint_as_float(hi[c]), sscale[16 + d], fmaf(__uint_as_float(lo[c]), sscale[32 + d], spt[ph * 16 + d]));
+                        z_own[c] = fmaf(softplus_fast(pre), eps[c], fmaf(__uint_as_float(r0[c]), sscale[d], sct[ph * 16 + d]));
                     }
-                    put_largest(sl.t_hb + (cg * 128 + row) * 4, z_own);
-                    st_shared_v4(sl.t_z + sw128(row, cg), tf32_rna(z_own[0]), tf32_rna(z_own[1]), tf32_rna(z_own[2]), tf32_rna(z_own[3]));
-                    fence_proxy_async();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(sl.bar_z);
+                    if (ph == W - 1) put_largest(smem_u32(largest + cg * 128), z_own);      // the next layer scales its halves by it
+                } else if constexpr (!LITERAL) {
+                    uint32_t lv[kDims];
+                    tmem_ld_dims(res + 16, lv);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int c = 0; c < kDims; ++c) {
+                        const int d = d0 + c;
+                        z_own[c] = fmaf(exp_half_fast(fmaf(__uint_as_float(lv[c]) * h_inv, sscale[64 + d], sb2[16 + d])), eps[c],
+                                        fmaf(__uint_as_float(r0[c]) * h_inv, sscale[48 + d], sb2[d]));
+                    }
+                    put_largest(smem_u32(largest + cg * 128), z_own);
+                } else {
+                    tmem_ld_wait();
+                    if (ph == W) {
+                        // gate g, and the linear map Wl z + bl from the latent tile (it stays as it is for the proposal)
+                        float z[16];
+#pragma unroll
+                        for (int e4 = 0; e4 < 4; ++e4) {
+                            const float4 zq = ld_shared_v4(t_z + sw128(row, e4));
+                            z[4 * e4 + 0] = zq.x; z[4 * e4 + 1] = zq.y; z[4 * e4 + 2] = zq.z; z[4 * e4 + 3] = zq.w;
+                        }
+#pragma unroll
+                        for (int c = 0; c < kDims; ++c) {
+                            gate_own[c] = sigmoid_fast(fmaf(__uint_as_float(r0[c]) * h_inv, sscale[48 + d0 + c], sbg2[d0 + c]));
+                            float lin = sbl[d0 + c];
+#pragma unroll
+                            for (int e4 = 0; e4 < 4; ++e4) {
+                                const float4 w = *reinterpret_cast<const float4*>(sWl + (d0 + c) * 16 + 4 * e4);
+                                lin = fmaf(w.w, z[4 * e4 + 3], fmaf(w.z, z[4 * e4 + 2], fmaf(w.y, z[4 * e4 + 1], fmaf(w.x, z[4 * e4], lin))));
+                            }
+                            lin_own[c] = lin;
+                        }
+                        arrive(bar_z);
+                        continue;
+                    }
+                    // proposal h -> G = (1 - g) * lin + g * h; relu(G) replaces the latent tile for the scale product
+#pragma unroll
+                    for (int c = 0; c < kDims; ++c) {
+                        const float prop = fmaf(__uint_as_float(r0[c]) * h_inv, sscale[64 + d0 + c], sbh2[d0 + c]);
+                        G_own[c] = fmaf(gate_own[c], prop - lin_own[c], lin_own[c]);
+                        z_own[c] = fmaxf(G_own[c], 0.0f);
+                    }
+                    store_latent(z_own);
+                    // z' = G + softplus(Ws relu(G) + bs) * eps
+                    ok = mbar_wait(bar_acc2, na & 1u, abort_flag, a.st);
+                    if (!ok) break;
+                    ++na;
+                    tc_fence_after();
+                    tmem_ld_dims(res, r0);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int c = 0; c < kDims; ++c) z_own[c] = fmaf(softplus_fast(__uint_as_float(r0[c]) + sbs[d0 + c]), eps[c], G_own[c]);
+                    put_largest(smem_u32(largest + cg * 128), z_own);
                 }
+                store_latent(z_own);
             }
         }
     }

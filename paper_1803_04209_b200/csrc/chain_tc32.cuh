@@ -29,6 +29,7 @@ namespace cutoff {
 namespace tc {
 
 constexpr int kChain32D = 32;
+constexpr int kChainTc32Threads = (1 + kChainEpiWarps) * 32;
 
 struct ChainTc32Args {
     const float* image;         // swizzled tiles: Wz, W1, W3 (H x 32 each), Wmu, W2 mean rows, W2 logvar rows (H/32 x 32 x 32 each)
@@ -62,7 +63,7 @@ __device__ __forceinline__ void stage_region(uint8_t* dst, const float* __restri
 }
 
 template <bool LITERAL>
-__global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args a) {
+__global__ void __launch_bounds__(kChainTc32Threads, 1) k_chain_tc32(ChainTc32Args a) {
     extern __shared__ uint8_t smem_raw[];
     const int H = a.H, W = a.W;
     const int n_chunks = H / 32;
@@ -109,12 +110,12 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int epi_thread = threadIdx.x - 32;               // 0..511 for the epilogue warps
 
-    for (int i = threadIdx.x; i < H; i += kChainTcThreads) {
+    for (int i = threadIdx.x; i < H; i += kChainTc32Threads) {
         sbzs[i] = a.bz[i];
         sb1[i] = a.b1[i];
         sb3[i] = a.b3[i];
     }
-    for (int i = threadIdx.x; i < 1024; i += kChainTcThreads) sWsig[i] = a.Wsig[i];
+    for (int i = threadIdx.x; i < 1024; i += kChainTc32Threads) sWsig[i] = a.Wsig[i];
     if (threadIdx.x < 32) {
         sbmu[threadIdx.x] = a.bmu[threadIdx.x];
         sbsig[threadIdx.x] = a.bsig[threadIdx.x];
@@ -123,8 +124,8 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
     if (!LITERAL) {
         if (threadIdx.x < 64) sb2[threadIdx.x] = a.b2[threadIdx.x];
     } else {
-        for (int i = threadIdx.x; i < H; i += kChainTcThreads) sbi1[i] = a.bi1[i];
-        for (int i = threadIdx.x; i < 1024; i += kChainTcThreads) {
+        for (int i = threadIdx.x; i < H; i += kChainTc32Threads) sbi1[i] = a.bi1[i];
+        for (int i = threadIdx.x; i < 1024; i += kChainTc32Threads) {
             sWl[i] = a.Wl[i];
             reinterpret_cast<float*>(gen + 2 * region_bytes + 3 * 16384)[i] = img_ws[i];    // the Ws tile stays resident
         }
@@ -154,7 +155,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc32(ChainTc32Args
     }
     dependency_wait();            // up to here: weights.  The encoder's states and the device state are earlier kernels'
     launch_dependents();
-    for (int i = threadIdx.x; i < W * H; i += kChainTcThreads) slr[i] = (a.hlr[i] + a.hlr[W * H + i]) * (1.0f / 3.0f);
+    for (int i = threadIdx.x; i < W * H; i += kChainTc32Threads) slr[i] = (a.hlr[i] + a.hlr[W * H + i]) * (1.0f / 3.0f);
     if (LITERAL) fence_proxy_async();                             // the Ws tile was written with ordinary stores
     tc_fence_before();
     __syncthreads();

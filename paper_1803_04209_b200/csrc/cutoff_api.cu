@@ -71,7 +71,9 @@ struct cutoff_ctx {
     float* d_v_inv = nullptr;       // [alloc_rows]
     __half* d_w16 = nullptr;        // weights: W4 [2N][ldh]; literal: Wi2 [N], Wj2 [N], M [H] rows
     float* d_w_inv = nullptr;       // their inverse scales
-    float* d_bound = nullptr;       // [4] bound of v's (u's) entries, slope * largest |latent| + offset; literal: of r's, from the largest |u|
+    // [8] bounds of hidden layers' entries, slope * largest |input| + offset each: v (u), from the largest |latent|; literal: r, from the
+    // largest |u|; the transition's (literal: the gate's and the proposal's), from the largest |latent|
+    float* d_bound = nullptr;
     float* d_x = nullptr;           // [chunk_rows][ldx]
     float* d_partial = nullptr;     // [n_chunks * sort_grid][N]; a second block of kPartialRows rows holds sums of squares
     float* d_std = nullptr;         // [N] spread of each order statistic (when asked for)
@@ -103,7 +105,7 @@ struct cutoff_ctx {
     bool chain_tc32 = false;        // the same for D = 32, H <= 512 (weights staged phase by phase)
     bool chain_tcl = false;         // the literal variant's chain on tensor cores (D = 16, H in {64, 128, 192, 256})
     bool chain_tcl32 = false;       // the same for D = 32, H <= 512 (weights staged phase by phase)
-    float* d_chain_image = nullptr; // swizzled tf32 operand tiles of the chain
+    uint8_t* d_chain_image = nullptr;   // swizzled operand tiles of the chain
 
     // pinned host memory that kernels read and write directly (one address on both sides); one block that begins with h_state
     uint8_t* h_mask = nullptr;      // [N] censoring mask of the push in progress
@@ -221,6 +223,31 @@ void put_second_layer(float* tiles, const float* w, size_t out_rows, size_t H, s
     for (size_t kb = 0; kb < H / 32; ++kb)
         for (size_t o = 0; o < out_rows; ++o)
             for (size_t jj = 0; jj < 32; ++jj) tiles[kb * block_rows * 32 + swz(o, jj)] = host_tf32(w[o * H + kb * 32 + jj]);
+}
+
+// The same as H / 64 K blocks of `block_rows` rows x 64 halves, each row multiplied by a power of two as k_half_rows does it; the
+// inverses go to `inv`.  `rest`: what the halves leave of the rows.
+void put_second_layer_half(uint8_t* tiles, float* inv, const double* w, size_t out_rows, size_t H, size_t row0, size_t block_rows, double* rest = nullptr) {
+    for (size_t o = 0; o < out_rows; ++o) {
+        float big = 0.0f;
+        for (size_t k = 0; k < H; ++k) big = std::fmax(big, static_cast<float>(std::fabs(w[o * H + k])));
+        uint32_t bits;
+        std::memcpy(&bits, &big, 4);
+        const int e = bits ? half_exponent(bits) : 0;
+        const size_t row = row0 + o;
+        for (size_t k = 0; k < H; ++k) {
+            const __half h = __float2half_rn(static_cast<float>(std::ldexp(w[o * H + k], e)));
+            const size_t at = k / 64 * block_rows * 128 + (row >> 3) * 1024 + (row & 7) * 128 + (((k % 64 >> 3) ^ (row & 7)) << 4) + (k & 7) * 2;
+            std::memcpy(tiles + at, &h, 2);
+            if (rest) rest[o * H + k] = w[o * H + k] - std::ldexp(static_cast<double>(__half2float(h)), -e);
+        }
+        inv[row] = std::ldexp(1.0f, -e);
+    }
+}
+void put_second_layer_half(uint8_t* tiles, float* inv, const float* w, size_t out_rows, size_t H, size_t block_rows) {
+    std::vector<double> rounded(out_rows * H);
+    for (size_t i = 0; i < rounded.size(); ++i) rounded[i] = host_tf32(w[i]);
+    put_second_layer_half(tiles, inv, rounded.data(), out_rows, H, 0, block_rows);
 }
 
 // `rows` rows of weights w [rows][H] on the device, already rounded to at most 11 significant bits, into the half-precision
@@ -427,26 +454,32 @@ void launch_chain_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
     tc::ChainTcArgs a{};
     const ModelDev& m = c->m;
     a.image = c->d_chain_image;
-    a.bz = m.bz; a.b1 = m.b1; a.b3 = m.b3; a.bmu = m.bmu; a.bsig = m.bsig; a.Wsig = m.Wsig; a.b2 = m.b2; a.z0 = m.z0;
+    a.bz = m.bz; a.b1 = m.b1; a.b3 = m.b3; a.bmu = m.bmu; a.b2 = m.b2; a.z0 = m.z0;
     if (c->chain_tcl) {
         const LiteralDev& l = c->lit;
         a.b1 = l.bg1; a.b3 = l.bh1; a.b2 = nullptr;
         a.bi1 = l.bi1; a.bg2 = l.bg2; a.bh2 = l.bh2; a.Wl = l.Wl; a.bl = l.bl; a.bs = l.bs;
     }
-    a.hlr = c->d_hlr; a.st = c->d_state;
+    a.hlr = c->d_hlr; a.WzT = m.WzT; a.Wmu = m.Wmu; a.bounds = c->d_bound + 4; a.st = c->d_state;
     a.key = NoiseKey{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.v_out = half_v(c);
-    const int tiles = ceil_div(count, 128);
-    const int grid = tiles < c->sm_count ? tiles : c->sm_count;
-    if (c->chain_tcl) launch_dependent(tc::k_chain_tc<true>, dim3(grid), dim3(tc::kChainTcThreads), tc::chain_tc_smem_bytes(c->H, c->W, true), c->stream, a);
-    else launch_dependent(tc::k_chain_tc<false>, dim3(grid), dim3(tc::kChainTcThreads), tc::chain_tc_smem_bytes(c->H, c->W), c->stream, a);
+    const auto run = [&](auto* kernel, int rows) {
+        const int tiles = ceil_div(count, rows);
+        launch_dependent(kernel, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kChainTcThreads),
+                         tc::chain_tc_smem_bytes(c->H, c->W, c->chain_tcl), c->stream, a);
+    };
+    // Half tiles as long as every one of them has an SM of its own (H=256, S=8192: 27 us, whole tiles on half the SMs 35), then whole tiles,
+    // each worked on by all warps of its SM, then two side by side (S=65536: 68 us; one after the other by all warps 76 to 90).
+    if (ceil_div(count, 64) <= c->sm_count) c->chain_tcl ? run(tc::k_chain_tc<true, 16, true>, 64) : run(tc::k_chain_tc<false, 16, true>, 64);
+    else if (ceil_div(count, 128) <= c->sm_count) c->chain_tcl ? run(tc::k_chain_tc<true, 16, false>, 128) : run(tc::k_chain_tc<false, 16, false>, 128);
+    else c->chain_tcl ? run(tc::k_chain_tc<true, 8, false>, 128) : run(tc::k_chain_tc<false, 8, false>, 128);
     c->launches += 1;
 }
 
 void launch_chain_tc32(cutoff_ctx* c, uint32_t sample_base, int count) {
     tc::ChainTc32Args a;
     const ModelDev& m = c->m;
-    a.image = c->d_chain_image;
+    a.image = reinterpret_cast<const float*>(c->d_chain_image);
     a.bz = m.bz; a.b1 = m.b1; a.b3 = m.b3; a.bmu = m.bmu; a.bsig = m.bsig; a.Wsig = m.Wsig; a.b2 = m.b2; a.z0 = m.z0;
     if (c->chain_tcl32) {
         const LiteralDev& l = c->lit;
@@ -458,8 +491,8 @@ void launch_chain_tc32(cutoff_ctx* c, uint32_t sample_base, int count) {
     a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.v_out = half_v(c);
     const int tiles = ceil_div(count, 128);
     const int grid = tiles < c->sm_count ? tiles : c->sm_count;
-    if (c->chain_tcl32) launch_dependent(tc::k_chain_tc32<true>, dim3(grid), dim3(tc::kChainTcThreads), tc::chain_tc32_smem_bytes(c->H, c->W, true), c->stream, a);
-    else launch_dependent(tc::k_chain_tc32<false>, dim3(grid), dim3(tc::kChainTcThreads), tc::chain_tc32_smem_bytes(c->H, c->W), c->stream, a);
+    if (c->chain_tcl32) launch_dependent(tc::k_chain_tc32<true>, dim3(grid), dim3(tc::kChainTc32Threads), tc::chain_tc32_smem_bytes(c->H, c->W, true), c->stream, a);
+    else launch_dependent(tc::k_chain_tc32<false>, dim3(grid), dim3(tc::kChainTc32Threads), tc::chain_tc32_smem_bytes(c->H, c->W), c->stream, a);
     c->launches += 1;
 }
 
@@ -763,8 +796,15 @@ cudaError_t allow_smem_chain(const cutoff_ctx* c) {
 cudaError_t set_kernel_attributes(const cutoff_ctx* c) {
     cudaError_t e = allow_smem_sort(c->N);
     if (e != cudaSuccess) return e;
-    if (c->chain_tc) e = allow_smem(tc::k_chain_tc<false>, 227 * 1024);
-    else if (c->chain_tcl) e = allow_smem(tc::k_chain_tc<true>, 227 * 1024);
+    if (c->chain_tc) {
+        e = allow_smem(tc::k_chain_tc<false, 16, true>, 227 * 1024);
+        if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<false, 16, false>, 227 * 1024);
+        if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<false, 8, false>, 227 * 1024);
+    } else if (c->chain_tcl) {
+        e = allow_smem(tc::k_chain_tc<true, 16, true>, 227 * 1024);
+        if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<true, 16, false>, 227 * 1024);
+        if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<true, 8, false>, 227 * 1024);
+    }
     else if (c->chain_tc32) e = allow_smem(tc::k_chain_tc32<false>, 227 * 1024);
     else if (c->chain_tcl32) e = allow_smem(tc::k_chain_tc32<true>, 227 * 1024);
     else switch (c->D) {
@@ -870,9 +910,9 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     plan_chunks(c, c->alloc_rows);
     c->use_tc = cfg->precision != CUTOFF_PRECISION_FP32;
     c->chain_tc = !c->literal && c->use_tc && c->D == tc::kChainD && c->H % 64 == 0 && c->H <= 256 &&
-                  tc::chain_tc_smem_bytes(c->H, c->W) <= 227 * 1024;
+                  tc::chain_tc_window(c->H, c->W, false);
     c->chain_tcl = c->literal && c->use_tc && c->D == tc::kChainD && c->H % 64 == 0 && c->H <= 256 &&
-                   tc::chain_tc_smem_bytes(c->H, c->W, true) <= 227 * 1024;
+                   tc::chain_tc_window(c->H, c->W, true);
     c->chain_tc32 = !c->literal && c->use_tc && c->D == tc::kChain32D && c->H % 32 == 0 && c->H <= 512 &&
                     (c->H <= 256 || (c->H - 256) % 16 == 0) && tc::chain_tc32_smem_bytes(c->H, c->W) <= 227 * 1024;
     c->chain_tcl32 = c->literal && c->use_tc && c->D == tc::kChain32D && c->H % 32 == 0 && c->H <= 512 &&
@@ -911,9 +951,9 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
         }
     }
     CREATE_CHECK(cudaMalloc(&c->d_WhR, sizeof(float) * 2 * c->H * c->H));
-    if (c->chain_tc) CREATE_CHECK(cudaMalloc(&c->d_chain_image, sizeof(float) * tc::chain_tc_image_floats(c->H)));
+    if (c->chain_tc || c->chain_tcl)
+        CREATE_CHECK(cudaMalloc(&c->d_chain_image, tc::chain_tc_image_bytes(c->H, c->chain_tcl) + tc::chain_tc_image_floats(c->H) * sizeof(float)));
     if (c->chain_tc32) CREATE_CHECK(cudaMalloc(&c->d_chain_image, sizeof(float) * tc::chain_tc32_image_floats(c->H)));
-    if (c->chain_tcl) CREATE_CHECK(cudaMalloc(&c->d_chain_image, sizeof(float) * tc::chain_tc_image_floats(c->H, true)));
     if (c->chain_tcl32) CREATE_CHECK(cudaMalloc(&c->d_chain_image, sizeof(float) * tc::chain_tc32_image_floats(c->H, true)));
     CREATE_CHECK(cudaMalloc(&c->d_ring, sizeof(float) * c->W * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_stage, sizeof(float) * c->N));
@@ -926,7 +966,7 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
         CREATE_CHECK(cudaMalloc(&c->d_v_inv, sizeof(float) * c->alloc_rows));
         CREATE_CHECK(cudaMalloc(&c->d_w16, sizeof(__half) * w_rows * c->ldh));
         CREATE_CHECK(cudaMalloc(&c->d_w_inv, sizeof(float) * w_rows));
-        CREATE_CHECK(cudaMalloc(&c->d_bound, 4 * sizeof(float)));
+        CREATE_CHECK(cudaMalloc(&c->d_bound, 8 * sizeof(float)));
     } else {
         CREATE_CHECK(cudaMalloc(&c->d_v, sizeof(float) * static_cast<size_t>(c->alloc_rows) * c->H));
         if (!c->literal) CREATE_CHECK(cudaMalloc(&c->d_W4T, sizeof(float) * 2 * static_cast<size_t>(c->H) * c->ldx));
@@ -1049,6 +1089,10 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         float bound[2];
         layer_bound(host.data() + off[first], host.data() + off[first + 1], H, D, !c->literal, bound);
         CU_CHECK(c, upload(c, c->d_bound, bound, sizeof(bound)));
+        for (size_t t = 0; t < (c->literal ? 2u : 1u); ++t) {                                            // W1, or Wg1 and Wh1
+            layer_bound(host.data() + off[15 + 4 * t], host.data() + off[16 + 4 * t], H, D, true, bound);
+            CU_CHECK(c, upload(c, c->d_bound + 4 + 2 * t, bound, sizeof(bound)));
+        }
     }
     if (!c->use_tc && !c->literal) {
         k_transpose_heads<<<dim3(ceil_div(c->ldx, 32), ceil_div(c->H, 32), 2), dim3(32, 8), 0, c->stream>>>(c->d_blob + off[21], c->N, c->H, c->ldx, c->d_W4T);
@@ -1094,48 +1138,68 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         const float* wh2 = lit ? host.data() + off[21] : nullptr;
         const float* ws = lit ? host.data() + off[25] : nullptr; // [D][D]
         const size_t tile = H * 32;
-        std::vector<float> img;
+        std::vector<uint8_t> img;
         if (c->chain_tc || c->chain_tcl) {
-            // D = 16: two first-layer matrices share a tile (columns 0..15 and 16..31); second-layer K blocks of 16 rows
-            // (W2: 32).  compact: [Wz|W1], W3, Wmu, W2;  literal: [Wz|Wg1], [Wh1|Wi1], Wmu, Wg2, Wh2, Ws (16 rows)
-            img.assign(tc::chain_tc_image_floats(c->H, lit), 0.0f);
-            float* t_in0 = img.data();
+            // D = 16: two first-layer matrices share a tile (columns 0..15 and 16..31); second layers as halves, K blocks of 16 rows
+            // (W2: 32).  compact: [Wz|W1], W3, Wmu, W2;  literal: [Wz|Wg1], [Wh1|Wi1], Wmu, Wg2, Wh2, Ws (16 rows of floats)
+            const size_t bytes = tc::chain_tc_image_bytes(c->H, lit);
+            img.assign(bytes + tc::chain_tc_image_floats(c->H) * sizeof(float), 0);
+            float* t_in0 = reinterpret_cast<float*>(img.data());
             float* t_in1 = t_in0 + tile;
-            float* t_wmu = t_in1 + tile;
-            float* t_out1 = t_wmu + H * 16;
+            uint8_t* t_wmu = img.data() + 2 * tile * sizeof(float);
+            uint8_t* t_out1 = t_wmu + H * 96;
+            float* inv = reinterpret_cast<float*>(img.data() + bytes);
             put_first_layer(t_in0, wz, H, D, 0);
             put_first_layer(t_in0, wa, H, D, 16);
             put_first_layer(t_in1, wb, H, D, 0);
-            put_second_layer(t_wmu, wmu, D, H, 16);
+            put_second_layer_half(t_wmu, inv, wmu, D, H, 48);
+            {
+                // Wsig Wmu as the sum of two halves; with Wsig bmu + bsig also in fp32
+                const float *wsig = host.data() + off[12], *bmu = host.data() + off[11], *bsig = host.data() + off[13];
+                std::vector<double> map(D * H, 0.0), rest(D * H);
+                for (size_t d = 0; d < D; ++d)
+                    for (size_t e = 0; e < D; ++e)
+                        for (size_t k = 0; k < H; ++k) map[d * H + k] += static_cast<double>(wsig[d * D + e]) * wmu[e * H + k];
+                put_second_layer_half(t_wmu, inv, map.data(), D, H, 16, 48, rest.data());
+                put_second_layer_half(t_wmu, inv, rest.data(), D, H, 32, 48);
+                float* const plain = inv + tc::kChainTcScales;
+                for (size_t d = 0; d < D; ++d) {
+                    double b = bsig[d];
+                    for (size_t e = 0; e < D; ++e) b += static_cast<double>(wsig[d * D + e]) * bmu[e];
+                    plain[d] = static_cast<float>(b);
+                    for (size_t k = 0; k < H; ++k) plain[16 + d * H + k] = static_cast<float>(map[d * H + k]);
+                }
+            }
             if (lit) {
-                float* t_out2 = t_out1 + H * 16;
+                uint8_t* t_out2 = t_out1 + H * 32;
                 put_first_layer(t_in1, wi1, H, D, 16);
-                put_second_layer(t_out1, wc, D, H, 16);
-                put_second_layer(t_out2, wh2, D, H, 16);
-                put_first_layer(t_out2 + H * 16, ws, D, D, 0);
+                put_second_layer_half(t_out1, inv + 48, wc, D, H, 16);
+                put_second_layer_half(t_out2, inv + 64, wh2, D, H, 16);
+                put_first_layer(reinterpret_cast<float*>(t_out2 + H * 32), ws, D, D, 0);
             } else {
-                put_second_layer(t_out1, wc, 2 * D, H, 32);
+                put_second_layer_half(t_out1, inv + 48, wc, 2 * D, H, 32);
             }
         } else {
             // D = 32: every matrix has a tile of H x 32 of its own, staged by the kernel phase by phase.
             // compact: Wz, W1, W3, Wmu, W2 mean rows, W2 log-variance rows;  literal: Wz, Wg1, Wh1, Wi1, Wmu, Wg2, Wh2, Ws
-            img.assign(tc::chain_tc32_image_floats(c->H, lit), 0.0f);
-            put_first_layer(img.data() + 0 * tile, wz, H, 32, 0);
-            put_first_layer(img.data() + 1 * tile, wa, H, 32, 0);
-            put_first_layer(img.data() + 2 * tile, wb, H, 32, 0);
+            img.assign(tc::chain_tc32_image_floats(c->H, lit) * sizeof(float), 0);
+            float* const t = reinterpret_cast<float*>(img.data());
+            put_first_layer(t + 0 * tile, wz, H, 32, 0);
+            put_first_layer(t + 1 * tile, wa, H, 32, 0);
+            put_first_layer(t + 2 * tile, wb, H, 32, 0);
             if (lit) {
-                put_first_layer(img.data() + 3 * tile, wi1, H, 32, 0);
-                put_second_layer(img.data() + 4 * tile, wmu, 32, H, 32);
-                put_second_layer(img.data() + 5 * tile, wc, 32, H, 32);
-                put_second_layer(img.data() + 6 * tile, wh2, 32, H, 32);
-                put_first_layer(img.data() + 7 * tile, ws, 32, 32, 0);
+                put_first_layer(t + 3 * tile, wi1, H, 32, 0);
+                put_second_layer(t + 4 * tile, wmu, 32, H, 32);
+                put_second_layer(t + 5 * tile, wc, 32, H, 32);
+                put_second_layer(t + 6 * tile, wh2, 32, H, 32);
+                put_first_layer(t + 7 * tile, ws, 32, 32, 0);
             } else {
-                put_second_layer(img.data() + 3 * tile, wmu, 32, H, 32);
-                put_second_layer(img.data() + 4 * tile, wc, 32, H, 32);
-                put_second_layer(img.data() + 5 * tile, wc + 32 * H, 32, H, 32);
+                put_second_layer(t + 3 * tile, wmu, 32, H, 32);
+                put_second_layer(t + 4 * tile, wc, 32, H, 32);
+                put_second_layer(t + 5 * tile, wc + 32 * H, 32, H, 32);
             }
         }
-        CU_CHECK(c, upload(c, c->d_chain_image, img.data(), img.size() * sizeof(float)));
+        CU_CHECK(c, upload(c, c->d_chain_image, img.data(), img.size()));
     }
 
     ModelDev& m = c->m;

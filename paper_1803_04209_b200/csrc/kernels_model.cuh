@@ -949,16 +949,6 @@ k_chain_wide(ModelDev m, const float* __restrict__ hlr, const DevState* __restri
 constexpr int kEmitThreads = 64, kEmitTN = 64, kEmitTK = 8, kEmitSlabs = 5;
 constexpr int kEmitPitchA = kEmitTK + 4, kEmitPitchB = 2 * kEmitTN + 4;
 
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-// Two fused multiply-adds in one instruction.
-__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-
 // W4 [2N][H] as [H][2][ldn], so that the columns of a slab are contiguous (when weights are loaded).
 __global__ void k_transpose_heads(const float* __restrict__ W4, int N, int H, int ldn, float* __restrict__ out) {
     __shared__ float tile[32][33];

@@ -1,0 +1,61 @@
+"""The chain on tensor cores (latent size 16): every hidden width, windows of one step and longer, sample counts at the edges of its
+tiles (64 samples, 128 samples with 16 or 8 warps) and of the rules that choose between them, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import cutoff_oracle as O
+from paper_1803_04209_b200 import binding, build, inputs
+
+pytestmark = pytest.mark.gpu
+
+SMS = 148
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    assert torch.cuda.is_available(), "these tests need a GPU"
+    build.build()
+    return binding.load_library()
+
+
+# the compact model takes this chain from 2369 samples on, the literal one always
+@pytest.mark.parametrize("H,lag,S,literal", [(64, 0, 2369, False), (128, 1, 2400, False), (192, 2, 64 * SMS, False), (256, 4, 64 * SMS + 1, False),
+                                             (64, 3, 128 * SMS, False), (192, 0, 128 * SMS + 1, False), (128, 12, 256 * SMS + 129, False),
+                                             (256, 12, 40000, False), (64, 0, 1, True), (256, 4, 63, True), (128, 1, 65, True), (192, 5, 300, True),
+                                             (256, 0, 64 * SMS + 1, True), (192, 2, 128 * SMS + 65, True), (64, 6, 256 * SMS + 1, True)])
+def test_tensor_core_chain_meets_the_oracle(H, lag, S, literal):
+    N, D = 20, 16
+    make = inputs.make_weights_literal if literal else inputs.make_weights
+    w = make(N, D, H, seed=H + lag, fan_in_ref=32)
+    gpu = binding.Cutoff(N, D, H, lag, S, precision=1, seed=3, flags=binding.FLAG_LITERAL if literal else 0)
+    gpu.load_weights(w)
+    orc = O.CutoffOracle(w, lag, S, seed=3)
+    for x in inputs.make_trace(N, lag + 3, seed=S, sigma=0.25):
+        gpu.push(x)
+        orc.push(x)
+    x = gpu.debug_samples(0, S)
+    rows = np.unique(np.concatenate([np.linspace(0, S - 1, 150).astype(int), np.arange(max(0, S - 70), S)]))
+    ref = orc.samples(rows)
+    assert np.max(np.abs(x[rows] - ref) / np.maximum(np.abs(ref), np.abs(ref).mean())) <= 2e-3
+    # a sample does not depend on the tile that it is part of
+    for first, n in ((0, 1), (S // 3, 65), (S // 2, 64 * SMS + 3)):
+        n = min(n, S - first)
+        assert np.array_equal(gpu.debug_samples(first, n), x[first:first + n])
+
+
+def test_hidden_layers_keep_their_bits_at_any_scale():
+    # the transition's hidden layer times 2^a against output weights times 2^-a: powers of two, so the same samples to the last bit
+    N, D, H, lag, S = 20, 16, 128, 2, 2500
+    trace = inputs.make_trace(N, lag + 2, seed=4, sigma=0.25)
+    out = []
+    for a in (0, -40, 40):
+        w = inputs.make_weights(N, D, H, seed=9, fan_in_ref=32)
+        for k, p in (("W1", a), ("b1", a), ("W2", -a)):
+            w[k] = (w[k] * np.float32(2.0 ** p)).astype(np.float32)
+        gpu = binding.Cutoff(N, D, H, lag, S, precision=1, seed=3)
+        gpu.load_weights(w)
+        for x in trace:
+            gpu.push(x)
+        out.append(gpu.debug_samples(0, S))
+    assert np.array_equal(out[1], out[0]) and np.array_equal(out[2], out[0])
