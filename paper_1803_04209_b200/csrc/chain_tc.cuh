@@ -1,5 +1,5 @@
 // Per-sample chain (guide steps, transition, first emission layer) on the tcgen05 tensor cores,
-// for latent size 16 and hidden width 64..256.  One kernel template serves both model
+// for latent size 16 and hidden width 64..256, or latent size 32 and hidden width up to 512.  One kernel template serves both model
 // variants: the compact one (transition = one hidden layer with a [mean | logvar] head, then the emission's
 // hidden layer v) and the networks as Section 3.1.3 prints them (LITERAL: gated transition
 //      g = sigmoid(Wg2 relu(Wg1 z + bg1) + bg2)        h = Wh2 relu(Wh1 z + bh1) + bh2
@@ -7,8 +7,8 @@
 // then the affine first layer of the emission mean, u = Wi1 z' + bi1).
 //
 // A CTA walks over tiles of samples; a sample is a TMEM lane.  Every layer pair
-//      hidden = act(A z + a)          (M=128, N=H, K=16, tf32)
-//      out    = B hidden (+ b)        (M=128, N=16 or 32, K=H, halves)
+//      hidden = act(A z + a)          (M=128, N=H, K=D, tf32)
+//      out    = B hidden (+ b)        (M=128, N=D to 3D, K=H, halves)
 // is two UMMA groups.  The first writes the hidden pre-activations to TMEM columns [0, H) of the tile's slot.  Each
 // epilogue warp reads its lanes' quarter of the columns, applies bias and activation and writes the result as packed
 // halves over the columns that it has just read: the hidden layer is the A operand of the second product straight from tensor
@@ -31,12 +31,14 @@
 // like for its noise (S=65536, D=16, H=256, lag 4: 68 us, of which 21 at that pipe's rate of 16 a clock; the rest is each step's round
 // trip, two products and the noise in between, which the other tile covers in part).  With the hidden layer through shared memory as
 // tf32, 64 units at a time, four steps of handshakes each, it took 108.  With one tile per SM, the steps' latency: 3700 cycles, of
-// which 1400 are the tanh (S=8192: 41 -> 27 us; 35 with tiles of 128).
+// which 1400 are the tanh (S=8192: 41 -> 27 us; 35 with tiles of 128).  D=32, with one tile per SM: S=32768, H=512, lag 4 162 -> 92 us (of
+// which 35 at the special-function pipe's rate), S=8192, H=256 60 -> 35 us; its weights were copied by the epilogue's threads before.
 //
-// All weight operands live in shared memory for the whole kernel: the host prepares their
-// swizzled image once, the CTA copies it in at start.  Latent rows are 128 bytes wide (32 tf32)
-// although K = 16: two first-layer matrices share one tile (columns 0..15 and 16..31: [Wz | W1], or
-// [Wz | Wg1] and [Wh1 | Wi1]), so the MMA for the second of them simply starts 64 bytes into the rows.
+// The host prepares a swizzled image of the weight operands once.  Latent rows are 128 bytes wide (32 tf32).  D = 16: all operands live in
+// shared memory for the whole kernel, and two first-layer matrices share one tile (columns 0..15 and 16..31: [Wz | W1], or
+// [Wz | Wg1] and [Wh1 | Wi1]), so the MMA for the second of them simply starts 64 bytes into the rows.  D = 32: they are too large
+// (352 KB at H = 512), so one first-layer and one second-layer matrix are there at a time and the issuing warp has each replaced by
+// the next phase's as soon as its last product is done, while the epilogue is still at work on the result.
 // The last layer's hidden vector (v, or u) goes to global memory as halves for the emission output GEMMs.
 //
 // A tile is the work of one warp that issues its MMAs and of 8 or 16 epilogue warps: warp w serves TMEM lanes 32*(w%4).. and one of
@@ -52,20 +54,20 @@ namespace tc {
 
 constexpr int kChainEpiWarps = 16;
 constexpr int kChainTcThreads = (2 + kChainEpiWarps) * 32;
-constexpr int kChainD = 16;
+constexpr int kChainD = 16, kChain32D = 32;
 constexpr float kTanhScale = 16384.0f;       // a tanh as an operand: normal halves down to 2^-28
 
 struct ChainTcArgs {
-    // swizzled operand tiles.  compact: [Wz|W1] (H x 32 floats), W3 (H x 32), then halves: Wmu and the two parts of Wsig Wmu (H/64 x 48 x 64),
-    // W2 (H/64 x 32 x 64);  literal: [Wz|Wg1], [Wh1|Wi1] (H x 32 floats each), halves as before (H/64 x 48 x 64), Wg2, Wh2
-    // (H/64 x 16 x 64 each), Ws (16 x 32 floats).  Behind them, floats: the inverse scales of the rows of halves, in that order,
-    // then Wsig bmu + bsig (16) and Wsig Wmu (16 x H).
+    // swizzled operand tiles: first-layer matrices in floats (D = 16: [Wz|W1], [W3] or [Wz|Wg1], [Wh1|Wi1]; D = 32: Wz, W1, W3 or Wz, Wg1,
+    // Wh1, Wi1; H x 32 each), then second-layer ones in halves, K blocks of 64: Wmu and the two parts of Wsig Wmu (3D rows), W2 (2D rows) or
+    // Wg2 and Wh2 (D rows each); literal: Ws (D x 32 floats).  Behind them, floats: the inverse scales of the rows of halves, in that order
+    // (5D), then Wsig bmu + bsig (D) and Wsig Wmu (D x H).
     const uint8_t* image;
-    // compact: b1, b3 = biases of the transition's and the emission's hidden layer, b2 = [mean | logvar] bias (32);
+    // compact: b1, b3 = biases of the transition's and the emission's hidden layer, b2 = [mean | logvar] bias (2D);
     // literal: b1 = bg1, b3 = bh1, b2 unused
     const float *bz, *b1, *b3, *bmu, *b2, *z0;
     const float *bi1, *bg2, *bh2, *Wl, *bl, *bs;       // literal variant only
-    const float *WzT, *Wmu;     // [16][H] each, fp32
+    const float *WzT, *Wmu;     // [D][H] each, fp32
     const float* hlr;           // [2][W][H] h_left, h_right
     const float* bounds;        // [2][2] of the transition's hidden layer (literal: of the gate's and the proposal's), as HalfRows::bound
     DevState* st;
@@ -75,22 +77,31 @@ struct ChainTcArgs {
     HalfRows v_out;             // v (literal: u), scaled
 };
 
-// Bytes of the operand tiles, and floats behind them.
-inline size_t chain_tc_image_bytes(int H, bool literal) { return static_cast<size_t>(H) * 416 + (literal ? 16 * 128 : 0); }
-constexpr int kChainTcScales = 80;
-inline size_t chain_tc_image_floats(int H) { return kChainTcScales + 16 + 16 * static_cast<size_t>(H); }
+// Bytes of D rows of halves (whole K blocks), of the first-layer tiles, of all operand tiles, and floats behind them.
+__host__ __device__ constexpr uint32_t chain_tc_row_bytes(int D, int H) { return static_cast<uint32_t>((H + 63) / 64) * 128u * static_cast<uint32_t>(D); }
+__host__ __device__ constexpr uint32_t chain_tc_first_bytes(int D, int H, bool literal) { return static_cast<uint32_t>(H) * 128u * (D == 16 ? 2u : (literal ? 4u : 3u)); }
+__host__ __device__ constexpr uint32_t chain_tc_image_bytes(int D, int H, bool literal) {
+    return chain_tc_first_bytes(D, H, literal) + 5u * chain_tc_row_bytes(D, H) + (literal ? static_cast<uint32_t>(D) * 128u : 0u);
+}
+inline size_t chain_tc_image_floats(int D, int H) { return 6 * static_cast<size_t>(D) + static_cast<size_t>(D) * H; }
+// What of them is in shared memory at a time: D = 16 all, D = 32 one first-layer tile, the guide's second layer or a smaller one, and Ws.
+__host__ __device__ constexpr uint32_t chain_tc_operand_bytes(int D, int H, bool literal) {
+    return D == 16 ? chain_tc_image_bytes(D, H, literal) : static_cast<uint32_t>(H) * 128u + 3u * chain_tc_row_bytes(D, H) + (literal ? 4096u : 0u);
+}
+constexpr int kChainLatentBytes = 2 * 16384;      // latent tiles of two slots
 
-inline size_t chain_tc_smem_bytes(int H, int W, bool literal = false) {
-    const size_t floats = (literal ? 4 : 3) * static_cast<size_t>(H) + 4 * 128 + static_cast<size_t>(W) * (H + 32) + (literal ? 256 : 0) + kChainTcScales +
-                          (literal ? 64 : 32) + 32;
-    return 1024 + chain_tc_image_bytes(H, literal) + 2 * 16384 + floats * 4;
+inline size_t chain_tc_smem_bytes(int D, int H, int W, bool literal) {
+    const size_t floats = (literal ? 4 : 3) * static_cast<size_t>(H) + 4 * 128 + 2 * static_cast<size_t>(W) * D + (literal ? D * D : 0) + 5 * D +
+                          (literal ? 4 : 2) * D + 32;
+    return 1024 + chain_tc_operand_bytes(D, H, literal) + kChainLatentBytes + floats * 4;
 }
 
-// Which windows: those whose states the kernel could hold beside its operands when it kept both in shared memory.  Longer ones
-// (H=256: from 14 steps on) have always gone through the fp32 kernels, and what is computed in fp32 stays so.
-inline bool chain_tc_window(int H, int W, bool literal) {
-    const size_t tiles = static_cast<size_t>(H) * 448 + (literal ? 2048 : 0) + 6 * 16384;
-    const size_t floats = literal ? 4 * static_cast<size_t>(H) + static_cast<size_t>(W) * H + 624 : 3 * static_cast<size_t>(H) + static_cast<size_t>(W) * H + 336;
+// Which windows: those whose states the kernels could hold beside their operands when they kept both in shared memory.  Longer ones
+// (D=16, H=256: from 14 steps on) have always gone through the fp32 kernels, and what is computed in fp32 stays so.
+inline bool chain_tc_window(int D, int H, int W, bool literal) {
+    const size_t states = static_cast<size_t>(W) * H;
+    const size_t tiles = D == 16 ? static_cast<size_t>(H) * 448 + (literal ? 2048 : 0) + 6 * 16384 : static_cast<size_t>(H) * 256 + 3 * 16384 + 4096;
+    const size_t floats = states + (D == 32 ? 4 * static_cast<size_t>(H) + 2336 : literal ? 4 * static_cast<size_t>(H) + 624 : 3 * static_cast<size_t>(H) + 336);
     return 1024 + tiles + floats * 4 + 256 <= 227 * 1024;
 }
 
@@ -223,48 +234,62 @@ __device__ __forceinline__ void pack_columns(const uint32_t (&acc)[16], const ul
 // WARPS: epilogue warps of a tile.  HALF: tiles of 64 samples, 16 lanes of each quarter of the tensor memory, for decisions that leave SMs
 // without a tile of 128.  A warp then spreads the 16 lanes' guide columns over its 32 threads; all else runs as in a full tile, the
 // other lanes on values that nobody reads.  The results of a sample are the same to the last bit in every shape.
-template <bool LITERAL, int WARPS, bool HALF>
+template <int D, bool LITERAL, int WARPS, bool HALF>
 __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) {
     extern __shared__ uint8_t smem_raw[];
     constexpr int kRows = HALF ? 64 : 128;                        // samples per tile
-    constexpr int kSlots = kChainEpiWarps / WARPS, kGroups = WARPS / 4, kDims = kChainD / kGroups;
-    const int H = a.H, W = a.W, Hg = H / kGroups;                 // hidden units per column group
+    constexpr int kSlots = kChainEpiWarps / WARPS, kGroups = WARPS / 4, kDims = D / kGroups;
+    constexpr bool kStaged = D == 32;
+    static_assert(!kStaged || kSlots == 1, "operands that come and go serve one tile");
+    const int H = a.H, W = a.W;
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t* gen = smem_raw + (base - raw);
     // weight operand tiles
-    const uint32_t t_in0 = base;                                  // [Wz | W1]   or [Wz | Wg1]
-    const uint32_t t_in1 = t_in0 + H * 128;                       // W3          or [Wh1 | Wi1]
-    const uint32_t t_wmu = t_in1 + H * 128;
-    const uint32_t t_out1 = t_wmu + H * 96;                       // W2 (32 rows per K block) or Wg2 (16 rows)
-    const uint32_t t_out2 = t_out1 + H * 32;                      // literal: Wh2
-    const uint32_t t_ws = t_out2 + H * 32;                        // literal: Ws, 16 rows x 128 bytes
-    const uint32_t image_bytes = static_cast<uint32_t>(H) * 416u + (LITERAL ? 2048u : 0u);
-    const uint32_t t_act = base + image_bytes;                    // latent tiles, one per slot
+    const uint32_t first_bytes = chain_tc_first_bytes(D, H, LITERAL);
+    const uint32_t image_bytes = chain_tc_image_bytes(D, H, LITERAL), operand_bytes = chain_tc_operand_bytes(D, H, LITERAL);
+    const uint32_t t_first = base;
+    const uint32_t t_guide = t_first + (kStaged ? H * 128u : first_bytes);    // Wmu and the parts of Wsig Wmu; staged: any second layer
+    const uint32_t row_bytes = chain_tc_row_bytes(D, H);
+    const uint32_t t_out1 = t_guide + 3 * row_bytes;              // W2 (2D rows per K block) or Wg2 (D rows)
+    const uint32_t t_out2 = t_out1 + row_bytes;                   // literal: Wh2
+    const uint32_t t_ws = base + operand_bytes - D * 128u;        // literal: Ws, D rows x 128 bytes
+    const uint32_t t_act = base + operand_bytes;                  // latent tiles, one per slot
     // fp32 side tables
-    float* sbzs = reinterpret_cast<float*>(gen + image_bytes + 2 * 16384);    // bz
+    float* sbzs = reinterpret_cast<float*>(gen + operand_bytes + kChainLatentBytes);     // bz
     float* sb1 = sbzs + H;
     float* sb3 = sb1 + H;
     float* sbi1 = sb3 + H;                   // literal only
     float* szmax = sb3 + (LITERAL ? 2 : 1) * H;      // [slot][column group][row] largest |latent| of a thread's dimensions
-    float* slr = szmax + 4 * 128;        // [W][H]  h_left + h_right (first step: + tanh)
-    float* sct = slr + W * H;                // [W][16]  Wmu (h_left + h_right) / 3 + bmu
-    float* spt = sct + W * 16;               // [W][16]  the same of the scale: Wsig times that, + bsig
-    float* sWl = spt + W * 16;               // [16][16], literal only
-    // what the products of halves are multiplied with: mu 16, the two parts of the scale's map 16 each, then W2 32 or Wg2, Wh2 16 each
-    float* sscale = sWl + (LITERAL ? 256 : 0);
-    float* sb2 = sscale + kChainTcScales;                // compact: [32]
-    float* sbg2 = sscale + kChainTcScales;               // literal: bg2, bh2, bl, bs, 16 each
-    float* sbh2 = sbg2 + 16;
-    float* sbl = sbh2 + 16;
-    float* sbs = sbl + 16;
-    float* sbar = LITERAL ? sbs + 16 : sb2 + 32;
-    const uint32_t bars = smem_u32(sbar);                         // 2 slots x 4 barriers, then the drain barriers
-    const uint32_t bar_img = bars + 2 * 40;                       // the operand image has landed
+    float* sct = szmax + 4 * 128;            // [W][D]  Wmu (h_left + h_right) / 3 + bmu
+    float* spt = sct + W * D;                // [W][D]  the same of the scale: Wsig times that, + bsig
+    float* sWl = spt + W * D;                // [D][D], literal only
+    // what the products of halves are multiplied with: mu D, the two parts of the scale's map D each, then W2 2D or Wg2, Wh2 D each
+    float* sscale = sWl + (LITERAL ? D * D : 0);
+    float* sb2 = sscale + 5 * D;             // compact: [2D]
+    float* sbg2 = sb2;                       // literal: bg2, bh2, bl, bs, D each
+    float* sbh2 = sbg2 + D;
+    float* sbl = sbh2 + D;
+    float* sbs = sbl + D;
+    float* sbar = sb2 + (LITERAL ? 4 : 2) * D;
+    const uint32_t bars = smem_u32(sbar);                         // 2 slots x 5 barriers
+    const uint32_t bar_img = bars + 2 * 40, bar_second = bar_img + 8;      // the operand image has landed; staged: a first layer, a second layer
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sbar + 24);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sbar + 25);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    // Staged operands.  First layers in the order of the image, one per kind of phase: guide, transition (gate), last layer (proposal), - (last
+    // layer).  Second layers: guide, W2 (Wg2), - (Wh2).
+    const auto phase_kind = [&](int ph) { return ph < W ? 0 : ph - W + 1; };
+    const auto load_operand = [&](uint32_t dst, uint32_t offset, uint32_t bytes, uint32_t bar) {
+        mbar_arrive_expect_tx(bar, bytes);
+        for (uint32_t off = 0; off < bytes; off += 32768u) bulk_load_1d(dst + off, a.image + offset + off, min(bytes - off, 32768u), bar);
+    };
+    const auto load_first = [&](int kind) { load_operand(t_first, static_cast<uint32_t>(kind) * H * 128u, H * 128u, bar_img); };
+    const auto load_second = [&](int kind) {
+        load_operand(t_guide, first_bytes + (kind == 0 ? 0u : kind == 1 ? 3u : 4u) * row_bytes, (kind == 0 ? 3u : (LITERAL ? 1u : 2u)) * row_bytes, bar_second);
+    };
 
     // ---- one-time set-up: barriers, operand image (bulk copies, while the side tables are filled), TMEM ----------
     if (threadIdx.x == 0) {
@@ -277,12 +302,14 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
             mbar_init(b0 + 32, 1);                   // drained
         }
         mbar_init(bar_img, 1);
+        mbar_init(bar_second, 1);
         *abort_flag = 0;
         fence_barrier_init();
-        mbar_arrive_expect_tx(bar_img, image_bytes);
-        for (uint32_t off = 0; off < image_bytes; off += 32768u) {
-            const uint32_t n = image_bytes - off < 32768u ? image_bytes - off : 32768u;
-            bulk_load_1d(base + off, a.image + off, n, bar_img);
+        if (kStaged) {
+            load_first(phase_kind(1));
+            load_second(phase_kind(1));
+        } else {
+            load_operand(base, 0u, image_bytes, bar_img);
         }
     }
     if (warp == 0) {
@@ -297,82 +324,105 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
         sb3[i] = a.b3[i];
         if (LITERAL) sbi1[i] = a.bi1[i];
     }
-    if (LITERAL)
-        for (int i = threadIdx.x; i < 256; i += kChainTcThreads) sWl[i] = a.Wl[i];
-    if (threadIdx.x < kChainTcScales) {
+    if (LITERAL) {
+        for (int i = threadIdx.x; i < D * D; i += kChainTcThreads) sWl[i] = a.Wl[i];
+        if (kStaged)                                              // Ws stays
+            for (int i = threadIdx.x; i < D * 32; i += kChainTcThreads)
+                reinterpret_cast<float*>(gen + operand_bytes - D * 128)[i] = reinterpret_cast<const float*>(a.image + image_bytes - D * 128)[i];
+        if (threadIdx.x < D) {
+            sbg2[threadIdx.x] = a.bg2[threadIdx.x];
+            sbh2[threadIdx.x] = a.bh2[threadIdx.x];
+            sbl[threadIdx.x] = a.bl[threadIdx.x];
+            sbs[threadIdx.x] = a.bs[threadIdx.x];
+        }
+    } else if (threadIdx.x < 2 * D) {
+        sb2[threadIdx.x] = a.b2[threadIdx.x];
+    }
+    if (threadIdx.x < 5 * D) {
         const float inv = tail[threadIdx.x];
-        sscale[threadIdx.x] = threadIdx.x < 48 ? inv * (1.0f / (3.0f * kTanhScale)) : inv;
+        sscale[threadIdx.x] = threadIdx.x < 3 * D ? inv * (1.0f / (3.0f * kTanhScale)) : inv;
     }
-    if (LITERAL && threadIdx.x < 16) {
-        sbg2[threadIdx.x] = a.bg2[threadIdx.x];
-        sbh2[threadIdx.x] = a.bh2[threadIdx.x];
-        sbl[threadIdx.x] = a.bl[threadIdx.x];
-        sbs[threadIdx.x] = a.bs[threadIdx.x];
-    }
-    if (!LITERAL && threadIdx.x < 32) sb2[threadIdx.x] = a.b2[threadIdx.x];
     // hidden unit i of the first step, the same for every sample
     float first_tanh = 0.0f;
     if (threadIdx.x < H) {
         float s = a.bz[threadIdx.x];
-#pragma unroll
-        for (int d = 0; d < 16; ++d) s = fmaf(a.WzT[d * H + threadIdx.x], a.z0[d], s);
+#pragma unroll 16
+        for (int d = 0; d < D; ++d) s = fmaf(a.WzT[d * H + threadIdx.x], a.z0[d], s);
         first_tanh = tanhf(s);
     }
-    // epilogue warp 2 + d: rows d of Wmu and of Wsig Wmu, for the parts of mu and of the scale that no sample changes
-    float wmu[8], wsm[8], bmu = 0.0f, bsm = 0.0f;
-    if (warp > 1) {
+    // epilogue warp 2 + w: rows w, w + 16 of Wmu and of Wsig Wmu, for the parts of mu and of the scale that no sample changes
+    constexpr int kPer = D == 16 ? 8 : 16;                        // hidden units per lane at most
+    float wmu[kPer], wsm[kPer];
+    const auto load_row = [&](int d) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int at = (warp - 2) * H + 32 * i + lane;
+        for (int i = 0; i < kPer; ++i) {
+            const int at = d * H + 32 * i + lane;
             wmu[i] = 32 * i < H ? a.Wmu[at] : 0.0f;
-            wsm[i] = 32 * i < H ? tail[kChainTcScales + 16 + at] : 0.0f;
+            wsm[i] = 32 * i < H ? tail[6 * D + at] : 0.0f;
         }
-        bmu = a.bmu[warp - 2];
-        bsm = tail[kChainTcScales + warp - 2];
-    }
+    };
+    if (warp > 1) load_row(warp - 2);
     // up to here nothing an earlier kernel of the stream writes has been touched (the image and the biases are
     // weights): the encoder's states and the device state come after this point
     dependency_wait();
     launch_dependents();
-    for (int i = threadIdx.x; i < W * H; i += kChainTcThreads) slr[i] = a.hlr[i] + a.hlr[W * H + i] + (i < H ? first_tanh : 0.0f);
-    __syncthreads();
-    if (warp > 1) {
-        // not unrolled: a launch finds the instruction caches cold, and this code runs once
+    // h_left + h_right (first step: + tanh) of as many steps as the place of the latent tiles holds, then the steps' vectors from them.
+    // Nothing is unrolled over steps or rows: a launch finds the instruction caches cold, and this code runs once.
+    float* const slr = reinterpret_cast<float*>(gen + operand_bytes);
+    const int per_round = kChainLatentBytes / 4 / H;
 #pragma unroll 1
-        for (int t = 0; t < W; ++t) {
-            float s = 0.0f, p = 0.0f;
+    for (int t0 = 0; t0 < W; t0 += per_round) {
+        const int steps = min(per_round, W - t0);
+        if (t0 > 0) __syncthreads();
+        for (int i = threadIdx.x; i < steps * H; i += kChainTcThreads)
+            slr[i] = a.hlr[t0 * H + i] + a.hlr[(W + t0) * H + i] + (t0 == 0 && i < H ? first_tanh : 0.0f);
+        __syncthreads();
+        if (warp > 1) {
+#pragma unroll 1
+            for (int d = warp - 2; d < D; d += 16) {
+                if (d != warp - 2 || (D == 32 && t0 > 0)) load_row(d);
+                const float bmu = a.bmu[d], bsm = tail[5 * D + d];
+#pragma unroll 1
+                for (int t = 0; t < steps; ++t) {
+                    float s = 0.0f, p = 0.0f;
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (32 * i < H) {
-                    const float v = slr[t * H + 32 * i + lane];
-                    s = fmaf(wmu[i], v, s);
-                    p = fmaf(wsm[i], v, p);
+                    for (int i = 0; i < kPer; ++i)
+                        if (32 * i < H) {
+                            const float v = slr[t * H + 32 * i + lane];
+                            s = fmaf(wmu[i], v, s);
+                            p = fmaf(wsm[i], v, p);
+                        }
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) {
+                        s += __shfl_xor_sync(0xffffffffu, s, off);
+                        p += __shfl_xor_sync(0xffffffffu, p, off);
+                    }
+                    if (lane == 0) {
+                        sct[(t0 + t) * D + d] = fmaf(s, 1.0f / 3.0f, bmu);
+                        spt[(t0 + t) * D + d] = fmaf(p, 1.0f / 3.0f, bsm);
+                    }
                 }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                s += __shfl_xor_sync(0xffffffffu, s, off);
-                p += __shfl_xor_sync(0xffffffffu, p, off);
-            }
-            if (lane == 0) {
-                sct[t * 16 + warp - 2] = fmaf(s, 1.0f / 3.0f, bmu);
-                spt[t * 16 + warp - 2] = fmaf(p, 1.0f / 3.0f, bsm);
             }
         }
     }
+    if (LITERAL && kStaged) fence_proxy_async();                  // Ws was written with ordinary stores
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    // nothing starts before the weights are in place; if they never arrive every role skips its loop
-    const bool image_ok = mbar_wait(bar_img, 0u, abort_flag, a.st);
-
+    // nothing starts before the weights are in place; if they never arrive every role skips its loop (staged: the issuing warp waits for each)
+    const bool image_ok = kStaged || mbar_wait(bar_img, 0u, abort_flag, a.st);
     const int n_tiles = image_ok ? ceil_div(a.count, kRows) : 0;
     // phases: W guide steps, then transition and emission hidden layer -- or gate, proposal (+ scale), first emission layer
     const int n_phases = LITERAL ? W + 3 : W + 2;
     const int ph_last = n_phases - 1;                             // its hidden layer goes to global memory, no second GEMM
-    // A column group's hidden units stand, packed, in the first half of the columns of its pre-activations, group 1's in the second half.
-    // The second result (at most 48 columns) takes columns that hold neither: the other halves of groups 0 and 1 where H = 256 fills the slot.
-    const uint32_t acc2_col = H == 256 ? Hg / 2 : H;
+    // The hidden units go to the column groups in blocks of 16.  A group's stand, packed, in the first half of the columns of its
+    // pre-activations, group 1's in the second half.  The second result (at most 3D columns) takes columns that hold neither: those behind the
+    // hidden layer, or the other halves of groups 0 and 1.
+    const int blocks = H / 16;
+    const auto group_block = [&](int g) { return g * blocks / kGroups; };
+    const auto packed_col = [&](int g) { return 16 * group_block(g) + (g == 1 ? 8 * (group_block(2) - group_block(1)) : 0); };
+    const uint32_t acc2_col = H + 3 * D <= 512 / kSlots ? H : 8 * group_block(1);
 
     const int slot = warp < 2 ? warp : (warp - 2) / WARPS;
     const uint32_t t_z = t_act + slot * 16384u;                   // latent A operand [128 x 128 B]
@@ -382,37 +432,69 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
     bool ok = true;
     if (warp < kSlots) {
         // ---------------- MMA issuer of the slot ---------------------------------------------------------
-        const uint32_t idesc_h = instr_desc_tf32(H);
-        uint32_t nz = 0, nh = 0;
+        const int n_lo = H < 256 ? H : 256, n_hi = H - n_lo;
+        const uint32_t idesc_lo = instr_desc_tf32(n_lo), idesc_hi = instr_desc_tf32(n_hi);
+        uint32_t nz = 0, nh = 0, np = 0, na = 0, n_first = 0, n_second = 0;
+        int first_kind = -1, second_kind = -1;                     // staged: the operands that have been waited for
         for (int tile = tile0; ok && tile < n_tiles; tile += tile_step) {
+            const bool last_tile = tile + tile_step >= n_tiles;
             for (int ph = 1; ph < n_phases; ++ph) {
+                const int kind = phase_kind(ph);
                 ok = mbar_wait(bar_z, nz & 1u, abort_flag, a.st);
                 if (!ok) break;
                 ++nz;
+                if (kStaged && first_kind != kind) {
+                    ok = mbar_wait(bar_img, n_first & 1u, abort_flag, a.st);
+                    if (!ok) break;
+                    ++n_first;
+                    first_kind = kind;
+                }
                 tc_fence_after();
                 if (elect_one()) {
-                    const uint32_t b_tile = ph < W ? t_in0 : (ph == W ? t_in0 + 64u : (ph == W + 1 ? t_in1 : t_in1 + 64u));
-                    const uint64_t a_desc = make_smem_desc(t_z), b_desc = make_smem_desc(b_tile);
-                    umma_tf32(tmem, a_desc, b_desc, idesc_h, 0u);
-                    umma_tf32(tmem, a_desc + 2, b_desc + 2, idesc_h, 1u);
+                    const uint32_t b_tile = kStaged || kind == 0 ? t_first : t_first + (kind >> 1) * H * 128u + (kind & 1) * 64u;
+                    const uint64_t a_desc = make_smem_desc(t_z), b_lo = make_smem_desc(b_tile);
+#pragma unroll
+                    for (int k = 0; k < D / 8; ++k) umma_tf32(tmem, a_desc + 2 * k, b_lo + 2 * k, idesc_lo, k != 0 ? 1u : 0u);
+                    if (D == 32 && n_hi > 0) {
+                        const uint64_t b_hi = make_smem_desc(b_tile + 256u * 128u);
+#pragma unroll
+                        for (int k = 0; k < D / 8; ++k) umma_tf32(tmem + 256u, a_desc + 2 * k, b_hi + 2 * k, idesc_hi, k != 0 ? 1u : 0u);
+                    }
                     umma_commit(bar_p);
                 }
                 __syncwarp();
+                if (kStaged) {
+                    const int next = ph < ph_last ? phase_kind(ph + 1) : (last_tile ? kind : phase_kind(1));
+                    if (next != kind) {
+                        ok = mbar_wait(bar_p, np & 1u, abort_flag, a.st);
+                        if (!ok) break;
+                        if (elect_one()) load_first(next);
+                        __syncwarp();
+                    }
+                    ++np;
+                }
                 if (ph == ph_last) continue;                       // the last hidden layer has no second GEMM here
                 ok = mbar_wait(bar_h, nh & 1u, abort_flag, a.st);
                 if (!ok) break;
                 ++nh;
+                if (kStaged && second_kind != kind) {
+                    ok = mbar_wait(bar_second, n_second & 1u, abort_flag, a.st);
+                    if (!ok) break;
+                    ++n_second;
+                    second_kind = kind;
+                }
                 tc_fence_after();
                 if (elect_one()) {
-                    const uint32_t b_base = ph < W ? t_wmu : (ph == W ? t_out1 : t_out2);
-                    const uint32_t out_rows = ph < W ? 48u : (LITERAL ? 16u : 32u), idesc2 = instr_desc_f16(out_rows, 128);
+                    const uint32_t b_base = kStaged || kind == 0 ? t_guide : (kind == 1 ? t_out1 : t_out2);
+                    const uint32_t out_rows = kind == 0 ? 3u * D : (LITERAL ? D : 2u * D), idesc2 = instr_desc_f16(out_rows, 128);
                     uint64_t b_desc = make_smem_desc(b_base);
                     uint32_t more = 0, k = 0;
                     for (int g = 0; g < kGroups; ++g) {
-                        const uint32_t packed = tmem + g * Hg + (g == 1 ? Hg / 2 : 0);
-                        for (int c = 0; c < Hg / 2; c += 8) {                // 16 hidden units: 8 columns, 32 bytes of a row of B
-                            umma_f16_tmem(tmem + acc2_col, packed + c, b_desc, idesc2, more);
+                        uint32_t packed = tmem + packed_col(g);
+                        for (int c = group_block(g); c < group_block(g + 1); ++c) {       // 16 hidden units: 8 columns, 32 bytes of a row of B
+                            umma_f16_tmem(tmem + acc2_col, packed, b_desc, idesc2, more);
                             more = 1;
+                            packed += 8;
                             k += 16;
                             b_desc += k & 63 ? 2 : out_rows * 8 - 6;         // the next 32 bytes, or the next K block
                         }
@@ -420,6 +502,16 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                     umma_commit(bar_acc2);
                 }
                 __syncwarp();
+                if (kStaged) {
+                    const int next = ph + 1 < ph_last ? phase_kind(ph + 1) : (last_tile ? kind : phase_kind(1));
+                    if (next != kind) {
+                        ok = mbar_wait(bar_acc2, na & 1u, abort_flag, a.st);
+                        if (!ok) break;
+                        if (elect_one()) load_second(next);
+                        __syncwarp();
+                    }
+                    ++na;
+                }
                 if (!LITERAL || ph != W + 1) continue;
                 // scale: Ws relu(G), relu(G) sits in the latent tile
                 ok = mbar_wait(bar_z, nz & 1u, abort_flag, a.st);
@@ -428,12 +520,18 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                 tc_fence_after();
                 if (elect_one()) {
                     const uint64_t a_desc = make_smem_desc(t_z), b_desc = make_smem_desc(t_ws);
-                    umma_tf32(tmem + acc2_col, a_desc, b_desc, instr_desc_tf32(16), 0u);
-                    umma_tf32(tmem + acc2_col, a_desc + 2, b_desc + 2, instr_desc_tf32(16), 1u);
+#pragma unroll
+                    for (int k = 0; k < D / 8; ++k) umma_tf32(tmem + acc2_col, a_desc + 2 * k, b_desc + 2 * k, instr_desc_tf32(D), k != 0 ? 1u : 0u);
                     umma_commit(bar_acc2);
                 }
                 __syncwarp();
+                ++na;
             }
+        }
+        if (kStaged && !ok) {
+            // wind down: let a copy that was asked for land before the CTA leaves (bounded)
+            mbar_wait_quiet(bar_img, n_first & 1u);
+            mbar_wait_quiet(bar_second, n_second & 1u);
         }
         if (!ok) {
             if (elect_one()) umma_commit(bar_drain);
@@ -450,8 +548,8 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
         const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
         const uint32_t step = a.st->step;
         // 16 columns at a time, packed over columns that have been read: group 1 from its last ones on, towards the end of its columns
-        const int batches = Hg / 16, first = cg == 1 ? batches - 1 : 0, dir = cg == 1 ? -1 : 1;
-        const uint32_t cols = tmem + lane_off + static_cast<uint32_t>(cg * Hg), packed = cols + static_cast<uint32_t>(cg == 1 ? Hg / 2 : 0);
+        const int hidden0 = 16 * group_block(cg), batches = group_block(cg + 1) - group_block(cg), first = cg == 1 ? batches - 1 : 0, dir = cg == 1 ? -1 : 1;
+        const uint32_t cols = tmem + lane_off + hidden0, packed = tmem + lane_off + packed_col(cg);
         const uint32_t res = tmem + lane_off + acc2_col + kDims * cg;             // this thread's columns of a second result
         const int d0 = kDims * cg;                                                // its latent dimensions
         float* const largest = szmax + slot * kGroups * 128 + row;                // [column group][128]
@@ -493,7 +591,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
             store_latent(z_own);
             float h_inv = 1.0f;                                                   // inverse scale of the hidden layer
             for (int ph = 1; ph < n_phases; ++ph) {
-                const float* bias = (ph < W ? sbzs : (ph == W ? sb1 : (ph == W + 1 ? sb3 : sbi1))) + cg * Hg;
+                const float* bias = (ph < W ? sbzs : (ph == W ? sb1 : (ph == W + 1 ? sb3 : sbi1))) + hidden0;
                 // the generator's words while the pre-activations are formed: they depend on nothing (literal: the gate draws nothing)
                 if (ph != ph_last && (!LITERAL || ph != W)) draw_words(ph < W ? static_cast<uint32_t>(ph) : kStreamTransition);
                 // ---- hidden layer: bias, activation, next A operand (or v) -----------------
@@ -504,7 +602,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                 if (HALF && ph < W) {
                     const float* thread_bias = bias + 2 * (lane & 3);
                     uint32_t acc[2][8];
-                    tmem_ld16_half(cols + 16 * first, acc[0]);
+                    if (batches > 0) tmem_ld16_half(cols + 16 * first, acc[0]);
 #pragma unroll 1
                     for (int b = 0; b < batches; b += 2) {
 #pragma unroll
@@ -544,12 +642,12 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                             pack_columns(acc, bv, w, [&](uint32_t x0, uint32_t x1, unsigned long long b) { return scaled_pair<true>(x0, x1, b, scale2); });
                         }
                         if (ph != ph_last) tmem_st8(packed + 8 * at, w);
-                        else if (mine && k < a.count) store8(a.v_out.p + static_cast<size_t>(k) * a.v_out.ld + cg * Hg + 16 * at, w);   // one sector
+                        else if (mine && k < a.count) store8(a.v_out.p + static_cast<size_t>(k) * a.v_out.ld + hidden0 + 16 * at, w);   // one sector
                     };
                     uint32_t acc[2][16];
                     ulonglong2 bv[2][4];
                     if constexpr (WARPS == 8) {
-                        // 32 columns at a time (Hg is a multiple of 32): two warps per scheduler keep the special-function pipe busy only with that
+                        // 32 columns at a time (D = 16: a group has a multiple of 32): two warps per scheduler keep the special-function pipe busy only with that
                         // many independent values each
 #pragma unroll 1
                         for (int b = 0; b < batches; b += 2) {
@@ -563,7 +661,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                             act16(acc[1], bv[1], at + dir);
                         }
                     } else {
-                        tmem_ld16(cols + 16 * first, acc[0]);
+                        if (batches > 0) tmem_ld16(cols + 16 * first, acc[0]);
                         load_bias(bias + 16 * first, bv[0]);
 #pragma unroll 1
                         for (int b = 0; b < batches; b += 2) {
@@ -595,47 +693,47 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                 if (ph < W) {
                     // guide: z = mu + softplus(Wsig mu + bsig) * eps
                     uint32_t hi[kDims], lo[kDims];
-                    tmem_ld_dims(res + 16, hi);
-                    tmem_ld_dims(res + 32, lo);
+                    tmem_ld_dims(res + D, hi);
+                    tmem_ld_dims(res + 2 * D, lo);
                     tmem_ld_wait();
 #pragma unroll
                     for (int c = 0; c < kDims; ++c) {
                         const int d = d0 + c;
-                        const float pre = fmaf(__uint_as_float(hi[c]), sscale[16 + d], fmaf(__uint_as_float(lo[c]), sscale[32 + d], spt[ph * 16 + d]));
-                        z_own[c] = fmaf(softplus_fast(pre), eps[c], fmaf(__uint_as_float(r0[c]), sscale[d], sct[ph * 16 + d]));
+                        const float pre = fmaf(__uint_as_float(hi[c]), sscale[D + d], fmaf(__uint_as_float(lo[c]), sscale[2 * D + d], spt[ph * D + d]));
+                        z_own[c] = fmaf(softplus_fast(pre), eps[c], fmaf(__uint_as_float(r0[c]), sscale[d], sct[ph * D + d]));
                     }
                     if (ph == W - 1) put_largest(smem_u32(largest + cg * 128), z_own);      // the next layer scales its halves by it
                 } else if constexpr (!LITERAL) {
                     uint32_t lv[kDims];
-                    tmem_ld_dims(res + 16, lv);
+                    tmem_ld_dims(res + D, lv);
                     tmem_ld_wait();
 #pragma unroll
                     for (int c = 0; c < kDims; ++c) {
                         const int d = d0 + c;
-                        z_own[c] = fmaf(exp_half_fast(fmaf(__uint_as_float(lv[c]) * h_inv, sscale[64 + d], sb2[16 + d])), eps[c],
-                                        fmaf(__uint_as_float(r0[c]) * h_inv, sscale[48 + d], sb2[d]));
+                        z_own[c] = fmaf(exp_half_fast(fmaf(__uint_as_float(lv[c]) * h_inv, sscale[4 * D + d], sb2[D + d])), eps[c],
+                                        fmaf(__uint_as_float(r0[c]) * h_inv, sscale[3 * D + d], sb2[d]));
                     }
                     put_largest(smem_u32(largest + cg * 128), z_own);
                 } else {
                     tmem_ld_wait();
                     if (ph == W) {
                         // gate g, and the linear map Wl z + bl from the latent tile (it stays as it is for the proposal)
-                        float z[16];
+                        float lin[kDims];
 #pragma unroll
-                        for (int e4 = 0; e4 < 4; ++e4) {
-                            const float4 zq = ld_shared_v4(t_z + sw128(row, e4));
-                            z[4 * e4 + 0] = zq.x; z[4 * e4 + 1] = zq.y; z[4 * e4 + 2] = zq.z; z[4 * e4 + 3] = zq.w;
+                        for (int c = 0; c < kDims; ++c) lin[c] = sbl[d0 + c];
+#pragma unroll
+                        for (int e4 = 0; e4 < D / 4; ++e4) {
+                            const float4 z = ld_shared_v4(t_z + sw128(row, e4));
+#pragma unroll
+                            for (int c = 0; c < kDims; ++c) {
+                                const float4 w = *reinterpret_cast<const float4*>(sWl + (d0 + c) * D + 4 * e4);
+                                lin[c] = fmaf(w.w, z.w, fmaf(w.z, z.z, fmaf(w.y, z.y, fmaf(w.x, z.x, lin[c]))));
+                            }
                         }
 #pragma unroll
                         for (int c = 0; c < kDims; ++c) {
-                            gate_own[c] = sigmoid_fast(fmaf(__uint_as_float(r0[c]) * h_inv, sscale[48 + d0 + c], sbg2[d0 + c]));
-                            float lin = sbl[d0 + c];
-#pragma unroll
-                            for (int e4 = 0; e4 < 4; ++e4) {
-                                const float4 w = *reinterpret_cast<const float4*>(sWl + (d0 + c) * 16 + 4 * e4);
-                                lin = fmaf(w.w, z[4 * e4 + 3], fmaf(w.z, z[4 * e4 + 2], fmaf(w.y, z[4 * e4 + 1], fmaf(w.x, z[4 * e4], lin))));
-                            }
-                            lin_own[c] = lin;
+                            gate_own[c] = sigmoid_fast(fmaf(__uint_as_float(r0[c]) * h_inv, sscale[3 * D + d0 + c], sbg2[d0 + c]));
+                            lin_own[c] = lin[c];
                         }
                         arrive(bar_z);
                         continue;
@@ -643,7 +741,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                     // proposal h -> G = (1 - g) * lin + g * h; relu(G) replaces the latent tile for the scale product
 #pragma unroll
                     for (int c = 0; c < kDims; ++c) {
-                        const float prop = fmaf(__uint_as_float(r0[c]) * h_inv, sscale[64 + d0 + c], sbh2[d0 + c]);
+                        const float prop = fmaf(__uint_as_float(r0[c]) * h_inv, sscale[4 * D + d0 + c], sbh2[d0 + c]);
                         G_own[c] = fmaf(gate_own[c], prop - lin_own[c], lin_own[c]);
                         z_own[c] = fmaxf(G_own[c], 0.0f);
                     }

@@ -17,7 +17,6 @@
 #include "emit_tc.cuh"
 #include "emit_tc2.cuh"
 #include "chain_tc.cuh"
-#include "chain_tc32.cuh"
 #include "kernels_literal.cuh"
 #include "gemm_tc.cuh"
 #include "pipe_rates.cuh"
@@ -101,10 +100,7 @@ struct cutoff_ctx {
     int pair_clusters = 0;          // clusters of two CTAs of the two-SM emission kernel that fit the GPU at once
     bool pair_emission = false;     // option "pair_emission": run the output layer on pairs of SMs (slower as measured; off)
     int chain_wide = 0;             // compact chain with D lanes per sample (few samples): samples per lane, 0 = another chain
-    bool chain_tc = false;          // per-sample chain on tensor cores as well (D = 16, H in {64, 128, 192, 256})
-    bool chain_tc32 = false;        // the same for D = 32, H <= 512 (weights staged phase by phase)
-    bool chain_tcl = false;         // the literal variant's chain on tensor cores (D = 16, H in {64, 128, 192, 256})
-    bool chain_tcl32 = false;       // the same for D = 32, H <= 512 (weights staged phase by phase)
+    bool chain_tc = false;          // per-sample chain on tensor cores as well (D = 16, H in {64, 128, 192, 256}; D = 32, H <= 512)
     uint8_t* d_chain_image = nullptr;   // swizzled operand tiles of the chain
 
     // pinned host memory that kernels read and write directly (one address on both sides); one block that begins with h_state
@@ -217,16 +213,8 @@ void put_first_layer(float* tile, const float* w, size_t rows, size_t cols, size
         for (size_t k = 0; k < cols; ++k) tile[swz(n, col0 + k)] = host_tf32(w[n * cols + k]);
 }
 
-// A second-layer matrix w [out_rows][H] as H / 32 K blocks of `block_rows` rows x 32 (out_rows <= block_rows; the
-// other rows stay as they are), swizzled and rounded to tf32: the B operand of out = W hidden, K = H.
-void put_second_layer(float* tiles, const float* w, size_t out_rows, size_t H, size_t block_rows) {
-    for (size_t kb = 0; kb < H / 32; ++kb)
-        for (size_t o = 0; o < out_rows; ++o)
-            for (size_t jj = 0; jj < 32; ++jj) tiles[kb * block_rows * 32 + swz(o, jj)] = host_tf32(w[o * H + kb * 32 + jj]);
-}
-
-// The same as H / 64 K blocks of `block_rows` rows x 64 halves, each row multiplied by a power of two as k_half_rows does it; the
-// inverses go to `inv`.  `rest`: what the halves leave of the rows.
+// A second-layer matrix w [out_rows][H] as K blocks of `block_rows` rows x 64 halves (the other rows stay as they are), swizzled, each
+// row multiplied by a power of two as k_half_rows does it; the inverses go to `inv`.  The B operand of out = W hidden, K = H.  `rest`: what the halves leave of the rows.
 void put_second_layer_half(uint8_t* tiles, float* inv, const double* w, size_t out_rows, size_t H, size_t row0, size_t block_rows, double* rest = nullptr) {
     for (size_t o = 0; o < out_rows; ++o) {
         float big = 0.0f;
@@ -455,7 +443,7 @@ void launch_chain_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
     const ModelDev& m = c->m;
     a.image = c->d_chain_image;
     a.bz = m.bz; a.b1 = m.b1; a.b3 = m.b3; a.bmu = m.bmu; a.b2 = m.b2; a.z0 = m.z0;
-    if (c->chain_tcl) {
+    if (c->literal) {
         const LiteralDev& l = c->lit;
         a.b1 = l.bg1; a.b3 = l.bh1; a.b2 = nullptr;
         a.bi1 = l.bi1; a.bg2 = l.bg2; a.bh2 = l.bh2; a.Wl = l.Wl; a.bl = l.bl; a.bs = l.bs;
@@ -466,33 +454,20 @@ void launch_chain_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
     const auto run = [&](auto* kernel, int rows) {
         const int tiles = ceil_div(count, rows);
         launch_dependent(kernel, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kChainTcThreads),
-                         tc::chain_tc_smem_bytes(c->H, c->W, c->chain_tcl), c->stream, a);
+                         tc::chain_tc_smem_bytes(c->D, c->H, c->W, c->literal), c->stream, a);
     };
-    // Half tiles as long as every one of them has an SM of its own (H=256, S=8192: 27 us, whole tiles on half the SMs 35), then whole tiles,
-    // each worked on by all warps of its SM, then two side by side (S=65536: 68 us; one after the other by all warps 76 to 90).
-    if (ceil_div(count, 64) <= c->sm_count) c->chain_tcl ? run(tc::k_chain_tc<true, 16, true>, 64) : run(tc::k_chain_tc<false, 16, true>, 64);
-    else if (ceil_div(count, 128) <= c->sm_count) c->chain_tcl ? run(tc::k_chain_tc<true, 16, false>, 128) : run(tc::k_chain_tc<false, 16, false>, 128);
-    else c->chain_tcl ? run(tc::k_chain_tc<true, 8, false>, 128) : run(tc::k_chain_tc<false, 8, false>, 128);
-    c->launches += 1;
-}
-
-void launch_chain_tc32(cutoff_ctx* c, uint32_t sample_base, int count) {
-    tc::ChainTc32Args a;
-    const ModelDev& m = c->m;
-    a.image = reinterpret_cast<const float*>(c->d_chain_image);
-    a.bz = m.bz; a.b1 = m.b1; a.b3 = m.b3; a.bmu = m.bmu; a.bsig = m.bsig; a.Wsig = m.Wsig; a.b2 = m.b2; a.z0 = m.z0;
-    if (c->chain_tcl32) {
-        const LiteralDev& l = c->lit;
-        a.b1 = l.bg1; a.b3 = l.bh1; a.b2 = nullptr;
-        a.bi1 = l.bi1; a.bg2 = l.bg2; a.bh2 = l.bh2; a.Wl = l.Wl; a.bl = l.bl; a.bs = l.bs;
+    // Half tiles as long as every one of them has an SM of its own (D=16, H=256, S=8192: 27 us, whole tiles on half the SMs 35), then whole
+    // tiles, each worked on by all warps of its SM, then, where all operands fit, two side by side (S=65536: 68 us; one after the other by
+    // all warps 76 to 90).
+    const bool half = ceil_div(count, 64) <= c->sm_count, one = ceil_div(count, 128) <= c->sm_count;
+    if (c->D == tc::kChain32D) {
+        if (c->literal) half ? run(tc::k_chain_tc<32, true, 16, true>, 64) : run(tc::k_chain_tc<32, true, 16, false>, 128);
+        else half ? run(tc::k_chain_tc<32, false, 16, true>, 64) : run(tc::k_chain_tc<32, false, 16, false>, 128);
+    } else if (c->literal) {
+        half ? run(tc::k_chain_tc<16, true, 16, true>, 64) : one ? run(tc::k_chain_tc<16, true, 16, false>, 128) : run(tc::k_chain_tc<16, true, 8, false>, 128);
+    } else {
+        half ? run(tc::k_chain_tc<16, false, 16, true>, 64) : one ? run(tc::k_chain_tc<16, false, 16, false>, 128) : run(tc::k_chain_tc<16, false, 8, false>, 128);
     }
-    a.hlr = c->d_hlr; a.st = c->d_state;
-    a.key = NoiseKey{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
-    a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.v_out = half_v(c);
-    const int tiles = ceil_div(count, 128);
-    const int grid = tiles < c->sm_count ? tiles : c->sm_count;
-    if (c->chain_tcl32) launch_dependent(tc::k_chain_tc32<true>, dim3(grid), dim3(tc::kChainTc32Threads), tc::chain_tc32_smem_bytes(c->H, c->W, true), c->stream, a);
-    else launch_dependent(tc::k_chain_tc32<false>, dim3(grid), dim3(tc::kChainTc32Threads), tc::chain_tc32_smem_bytes(c->H, c->W), c->stream, a);
     c->launches += 1;
 }
 
@@ -505,8 +480,7 @@ void launch_chain_literal_t(cutoff_ctx* c, uint32_t sample_base, int count) {
 }
 
 void launch_chain(cutoff_ctx* c, uint32_t sample_base, int count) {
-    if (c->chain_tcl) { launch_chain_tc(c, sample_base, count); return; }
-    if (c->chain_tcl32) { launch_chain_tc32(c, sample_base, count); return; }
+    if (c->chain_tc) { launch_chain_tc(c, sample_base, count); return; }
     if (c->literal) {
         switch (c->D) {
             case 4: launch_chain_literal_t<4>(c, sample_base, count); break;
@@ -517,8 +491,6 @@ void launch_chain(cutoff_ctx* c, uint32_t sample_base, int count) {
         c->launches += 1;
         return;
     }
-    if (c->chain_tc) { launch_chain_tc(c, sample_base, count); return; }
-    if (c->chain_tc32) { launch_chain_tc32(c, sample_base, count); return; }
     const size_t smem = chain_smem_floats(c->D, c->H, c->W) * sizeof(float);
     switch (c->D) {
         case 4: launch_chain_t<4>(c, sample_base, count, smem); break;
@@ -797,16 +769,16 @@ cudaError_t set_kernel_attributes(const cutoff_ctx* c) {
     cudaError_t e = allow_smem_sort(c->N);
     if (e != cudaSuccess) return e;
     if (c->chain_tc) {
-        e = allow_smem(tc::k_chain_tc<false, 16, true>, 227 * 1024);
-        if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<false, 16, false>, 227 * 1024);
-        if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<false, 8, false>, 227 * 1024);
-    } else if (c->chain_tcl) {
-        e = allow_smem(tc::k_chain_tc<true, 16, true>, 227 * 1024);
-        if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<true, 16, false>, 227 * 1024);
-        if (e == cudaSuccess) e = allow_smem(tc::k_chain_tc<true, 8, false>, 227 * 1024);
+        const auto allow = [&](auto* kernel) { if (e == cudaSuccess) e = allow_smem(kernel, 227 * 1024); };
+        if (c->D == tc::kChain32D) {
+            allow(c->literal ? tc::k_chain_tc<32, true, 16, true> : tc::k_chain_tc<32, false, 16, true>);
+            allow(c->literal ? tc::k_chain_tc<32, true, 16, false> : tc::k_chain_tc<32, false, 16, false>);
+        } else {
+            allow(c->literal ? tc::k_chain_tc<16, true, 16, true> : tc::k_chain_tc<16, false, 16, true>);
+            allow(c->literal ? tc::k_chain_tc<16, true, 16, false> : tc::k_chain_tc<16, false, 16, false>);
+            allow(c->literal ? tc::k_chain_tc<16, true, 8, false> : tc::k_chain_tc<16, false, 8, false>);
+        }
     }
-    else if (c->chain_tc32) e = allow_smem(tc::k_chain_tc32<false>, 227 * 1024);
-    else if (c->chain_tcl32) e = allow_smem(tc::k_chain_tc32<true>, 227 * 1024);
     else switch (c->D) {
         case 4: e = allow_smem_chain<4>(c); break;
         case 8: e = allow_smem_chain<8>(c); break;
@@ -909,14 +881,9 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     if (ceil_div(c->S, kMaxChunks) > c->alloc_rows) return fail(CUTOFF_ERR_UNSUPPORTED);   // S too large for the pass buffers
     plan_chunks(c, c->alloc_rows);
     c->use_tc = cfg->precision != CUTOFF_PRECISION_FP32;
-    c->chain_tc = !c->literal && c->use_tc && c->D == tc::kChainD && c->H % 64 == 0 && c->H <= 256 &&
-                  tc::chain_tc_window(c->H, c->W, false);
-    c->chain_tcl = c->literal && c->use_tc && c->D == tc::kChainD && c->H % 64 == 0 && c->H <= 256 &&
-                   tc::chain_tc_window(c->H, c->W, true);
-    c->chain_tc32 = !c->literal && c->use_tc && c->D == tc::kChain32D && c->H % 32 == 0 && c->H <= 512 &&
-                    (c->H <= 256 || (c->H - 256) % 16 == 0) && tc::chain_tc32_smem_bytes(c->H, c->W) <= 227 * 1024;
-    c->chain_tcl32 = c->literal && c->use_tc && c->D == tc::kChain32D && c->H % 32 == 0 && c->H <= 512 &&
-                     (c->H <= 256 || (c->H - 256) % 16 == 0) && tc::chain_tc32_smem_bytes(c->H, c->W, true) <= 227 * 1024;
+    c->chain_tc = c->use_tc && tc::chain_tc_window(c->D, c->H, c->W, c->literal) &&
+                  ((c->D == tc::kChainD && c->H % 64 == 0 && c->H <= 256) ||
+                   (c->D == tc::kChain32D && c->H % 32 == 0 && c->H <= 512));
     // D lanes per sample pay for few samples.  Where the alternative is the resident FMA kernel: one sample per lane up to 12 warps per
     // SM (H=64, lag 20: 4096 samples 28 us against 76; H=128, lag 2: 7000 samples 16.8 against 27), two up to 40 of those warps
     // (9000 samples 16.7 against 19.8 with one and 27; 16384: 24 against 29; 20000: 32 against 39, lag 20: 95 against 110; 36000: 42
@@ -928,8 +895,8 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     const int64_t few = 16 * static_cast<int64_t>(c->sm_count);
     const int64_t warps = total * c->D / 32;
     if (!c->literal && chain_resident_smem_floats(c->D, c->H, c->W) * sizeof(float) <= 200 * 1024)
-        c->chain_wide = c->chain_tc || c->chain_tc32 ? total <= few : warps <= 3 * few / 4 ? 1 : warps <= 5 * few / 2 && c->D <= 16 ? 2 : warps <= few ? 1 : 0;
-    if (c->chain_wide) c->chain_tc = c->chain_tc32 = false;
+        c->chain_wide = c->chain_tc ? total <= few : warps <= 3 * few / 4 ? 1 : warps <= 5 * few / 2 && c->D <= 16 ? 2 : warps <= few ? 1 : 0;
+    if (c->chain_wide) c->chain_tc = false;
 
     size_t blob_floats = 0;
     for (const auto& t : c->literal ? tensor_specs_literal(c->N, c->D, c->H) : tensor_specs(c->N, c->D, c->H))
@@ -951,10 +918,8 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
         }
     }
     CREATE_CHECK(cudaMalloc(&c->d_WhR, sizeof(float) * 2 * c->H * c->H));
-    if (c->chain_tc || c->chain_tcl)
-        CREATE_CHECK(cudaMalloc(&c->d_chain_image, tc::chain_tc_image_bytes(c->H, c->chain_tcl) + tc::chain_tc_image_floats(c->H) * sizeof(float)));
-    if (c->chain_tc32) CREATE_CHECK(cudaMalloc(&c->d_chain_image, sizeof(float) * tc::chain_tc32_image_floats(c->H)));
-    if (c->chain_tcl32) CREATE_CHECK(cudaMalloc(&c->d_chain_image, sizeof(float) * tc::chain_tc32_image_floats(c->H, true)));
+    if (c->chain_tc)
+        CREATE_CHECK(cudaMalloc(&c->d_chain_image, tc::chain_tc_image_bytes(c->D, c->H, c->literal) + tc::chain_tc_image_floats(c->D, c->H) * sizeof(float)));
     CREATE_CHECK(cudaMalloc(&c->d_ring, sizeof(float) * c->W * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_stage, sizeof(float) * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_state, sizeof(DevState)));
@@ -1127,8 +1092,8 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
     }
     // Operand tiles of the tensor-core chain kernels as they will sit in shared memory: tf32 (nearest, ties away),
     // K-major rows of 32 values, 16-byte chunks XOR-swizzled with the row index modulo 8.
-    if (c->chain_tc || c->chain_tcl || c->chain_tc32 || c->chain_tcl32) {
-        const bool lit = c->chain_tcl || c->chain_tcl32;
+    if (c->chain_tc) {
+        const bool lit = c->literal;
         const float* wz = host.data() + off[8];                  // first layers, [H][D]: Wz; W1 or Wg1; W3 or Wh1; Wi1
         const float* wa = host.data() + off[15];
         const float* wb = host.data() + off[19];
@@ -1137,67 +1102,48 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         const float* wc = host.data() + off[17];
         const float* wh2 = lit ? host.data() + off[21] : nullptr;
         const float* ws = lit ? host.data() + off[25] : nullptr; // [D][D]
-        const size_t tile = H * 32;
-        std::vector<uint8_t> img;
-        if (c->chain_tc || c->chain_tcl) {
-            // D = 16: two first-layer matrices share a tile (columns 0..15 and 16..31); second layers as halves, K blocks of 16 rows
-            // (W2: 32).  compact: [Wz|W1], W3, Wmu, W2;  literal: [Wz|Wg1], [Wh1|Wi1], Wmu, Wg2, Wh2, Ws (16 rows of floats)
-            const size_t bytes = tc::chain_tc_image_bytes(c->H, lit);
-            img.assign(bytes + tc::chain_tc_image_floats(c->H) * sizeof(float), 0);
-            float* t_in0 = reinterpret_cast<float*>(img.data());
-            float* t_in1 = t_in0 + tile;
-            uint8_t* t_wmu = img.data() + 2 * tile * sizeof(float);
-            uint8_t* t_out1 = t_wmu + H * 96;
-            float* inv = reinterpret_cast<float*>(img.data() + bytes);
-            put_first_layer(t_in0, wz, H, D, 0);
-            put_first_layer(t_in0, wa, H, D, 16);
-            put_first_layer(t_in1, wb, H, D, 0);
-            put_second_layer_half(t_wmu, inv, wmu, D, H, 48);
-            {
-                // Wsig Wmu as the sum of two halves; with Wsig bmu + bsig also in fp32
-                const float *wsig = host.data() + off[12], *bmu = host.data() + off[11], *bsig = host.data() + off[13];
-                std::vector<double> map(D * H, 0.0), rest(D * H);
-                for (size_t d = 0; d < D; ++d)
-                    for (size_t e = 0; e < D; ++e)
-                        for (size_t k = 0; k < H; ++k) map[d * H + k] += static_cast<double>(wsig[d * D + e]) * wmu[e * H + k];
-                put_second_layer_half(t_wmu, inv, map.data(), D, H, 16, 48, rest.data());
-                put_second_layer_half(t_wmu, inv, rest.data(), D, H, 32, 48);
-                float* const plain = inv + tc::kChainTcScales;
-                for (size_t d = 0; d < D; ++d) {
-                    double b = bsig[d];
-                    for (size_t e = 0; e < D; ++e) b += static_cast<double>(wsig[d * D + e]) * bmu[e];
-                    plain[d] = static_cast<float>(b);
-                    for (size_t k = 0; k < H; ++k) plain[16 + d * H + k] = static_cast<float>(map[d * H + k]);
-                }
-            }
-            if (lit) {
-                uint8_t* t_out2 = t_out1 + H * 32;
-                put_first_layer(t_in1, wi1, H, D, 16);
-                put_second_layer_half(t_out1, inv + 48, wc, D, H, 16);
-                put_second_layer_half(t_out2, inv + 64, wh2, D, H, 16);
-                put_first_layer(reinterpret_cast<float*>(t_out2 + H * 32), ws, D, D, 0);
-            } else {
-                put_second_layer_half(t_out1, inv + 48, wc, 2 * D, H, 32);
-            }
+        const size_t tile = H * 32, bytes = tc::chain_tc_image_bytes(c->D, c->H, lit);
+        std::vector<uint8_t> img(bytes + tc::chain_tc_image_floats(c->D, c->H) * sizeof(float), 0);
+        float* const first = reinterpret_cast<float*>(img.data());
+        if (D == 16) {                                           // two matrices share a tile (columns 0..15 and 16..31)
+            put_first_layer(first, wz, H, D, 0);
+            put_first_layer(first, wa, H, D, 16);
+            put_first_layer(first + tile, wb, H, D, 0);
+            if (lit) put_first_layer(first + tile, wi1, H, D, 16);
         } else {
-            // D = 32: every matrix has a tile of H x 32 of its own, staged by the kernel phase by phase.
-            // compact: Wz, W1, W3, Wmu, W2 mean rows, W2 log-variance rows;  literal: Wz, Wg1, Wh1, Wi1, Wmu, Wg2, Wh2, Ws
-            img.assign(tc::chain_tc32_image_floats(c->H, lit) * sizeof(float), 0);
-            float* const t = reinterpret_cast<float*>(img.data());
-            put_first_layer(t + 0 * tile, wz, H, 32, 0);
-            put_first_layer(t + 1 * tile, wa, H, 32, 0);
-            put_first_layer(t + 2 * tile, wb, H, 32, 0);
-            if (lit) {
-                put_first_layer(t + 3 * tile, wi1, H, 32, 0);
-                put_second_layer(t + 4 * tile, wmu, 32, H, 32);
-                put_second_layer(t + 5 * tile, wc, 32, H, 32);
-                put_second_layer(t + 6 * tile, wh2, 32, H, 32);
-                put_first_layer(t + 7 * tile, ws, 32, 32, 0);
-            } else {
-                put_second_layer(t + 3 * tile, wmu, 32, H, 32);
-                put_second_layer(t + 4 * tile, wc, 32, H, 32);
-                put_second_layer(t + 5 * tile, wc + 32 * H, 32, H, 32);
+            put_first_layer(first, wz, H, D, 0);
+            put_first_layer(first + tile, wa, H, D, 0);
+            put_first_layer(first + 2 * tile, wb, H, D, 0);
+            if (lit) put_first_layer(first + 3 * tile, wi1, H, D, 0);
+        }
+        const size_t rows = tc::chain_tc_row_bytes(c->D, c->H);
+        uint8_t* const guide = img.data() + tc::chain_tc_first_bytes(c->D, c->H, lit);
+        uint8_t* const out = guide + 3 * rows;
+        float* const inv = reinterpret_cast<float*>(img.data() + bytes);
+        put_second_layer_half(guide, inv, wmu, D, H, 3 * D);
+        {
+            // Wsig Wmu as the sum of two halves; with Wsig bmu + bsig also in fp32
+            const float *wsig = host.data() + off[12], *bmu = host.data() + off[11], *bsig = host.data() + off[13];
+            std::vector<double> map(D * H, 0.0), rest(D * H);
+            for (size_t d = 0; d < D; ++d)
+                for (size_t e = 0; e < D; ++e)
+                    for (size_t k = 0; k < H; ++k) map[d * H + k] += static_cast<double>(wsig[d * D + e]) * wmu[e * H + k];
+            put_second_layer_half(guide, inv, map.data(), D, H, D, 3 * D, rest.data());
+            put_second_layer_half(guide, inv, rest.data(), D, H, 2 * D, 3 * D);
+            float* const plain = inv + 5 * D;
+            for (size_t d = 0; d < D; ++d) {
+                double b = bsig[d];
+                for (size_t e = 0; e < D; ++e) b += static_cast<double>(wsig[d * D + e]) * bmu[e];
+                plain[d] = static_cast<float>(b);
+                for (size_t k = 0; k < H; ++k) plain[D + d * H + k] = static_cast<float>(map[d * H + k]);
             }
+        }
+        if (lit) {
+            put_second_layer_half(out, inv + 3 * D, wc, D, H, D);
+            put_second_layer_half(out + rows, inv + 4 * D, wh2, D, H, D);
+            put_first_layer(reinterpret_cast<float*>(out + 2 * rows), ws, D, D, 0);
+        } else {
+            put_second_layer_half(out, inv + 3 * D, wc, 2 * D, H, 2 * D);
         }
         CU_CHECK(c, upload(c, c->d_chain_image, img.data(), img.size()));
     }

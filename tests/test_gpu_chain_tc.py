@@ -1,4 +1,4 @@
-"""The chain on tensor cores (latent size 16): every hidden width, windows of one step and longer, sample counts at the edges of its
+"""The chain on tensor cores: latent size 16 with every hidden width, latent size 32 with widths that fill and split blocks, windows of one step and longer, sample counts at the edges of its
 tiles (64 samples, 128 samples with 16 or 8 warps) and of the rules that choose between them, against the oracle."""
 import numpy as np
 import pytest
@@ -20,12 +20,15 @@ def _lib():
 
 
 # the compact model takes this chain from 2369 samples on, the literal one always
+@pytest.mark.parametrize("D", [16, 32])
 @pytest.mark.parametrize("H,lag,S,literal", [(64, 0, 2369, False), (128, 1, 2400, False), (192, 2, 64 * SMS, False), (256, 4, 64 * SMS + 1, False),
                                              (64, 3, 128 * SMS, False), (192, 0, 128 * SMS + 1, False), (128, 12, 256 * SMS + 129, False),
                                              (256, 12, 40000, False), (64, 0, 1, True), (256, 4, 63, True), (128, 1, 65, True), (192, 5, 300, True),
                                              (256, 0, 64 * SMS + 1, True), (192, 2, 128 * SMS + 65, True), (64, 6, 256 * SMS + 1, True)])
-def test_tensor_core_chain_meets_the_oracle(H, lag, S, literal):
-    N, D = 20, 16
+def test_tensor_core_chain_meets_the_oracle(D, H, lag, S, literal):
+    if D == 32:                                          # and widths of other multiples of 32, more than one half of 256
+        H = {64: 32, 128: 160, 192: 512, 256: 288 if S % 2 else 448}[H]
+    N = 20
     make = inputs.make_weights_literal if literal else inputs.make_weights
     w = make(N, D, H, seed=H + lag, fan_in_ref=32)
     gpu = binding.Cutoff(N, D, H, lag, S, precision=1, seed=3, flags=binding.FLAG_LITERAL if literal else 0)
