@@ -631,15 +631,16 @@ void refresh_projections(cutoff_ctx* c) {
 
 void launch_encoder(cutoff_ctx* c) {
     refresh_projections(c);
-    // H <= 128: one CTA per direction with the recurrence matrix in registers.  From H = 256 on a thread's share no
-    // longer fits its registers, and a cluster of 8 CTAs per direction does the step in less time than one CTA that
-    // keeps part of the matrix in shared memory (H = 256: 17 against 21 us).
+    // H = 32, 64, 128: one CTA per direction with the recurrence matrix in registers.  Other widths in whole warps: a cluster of 8 CTAs per
+    // direction (H = 256: a thread's share no longer fits its registers, and one CTA that keeps part of the matrix in shared memory takes 21
+    // us against 17; H = 192 with one CTA that reads the matrix from L2 in every step, lag 6:
+    // 62 us, so 17; H = 96, lag 3: 17 and 12).
     const size_t cluster_smem = enc_rnn_cluster_smem_floats(c->H, c->W) * sizeof(float);
     const size_t resident_smem = enc_rnn_resident_smem_floats(c->H, c->W) * sizeof(float);
     if (c->H == 32 && resident_smem <= 200 * 1024) launch_rnn_resident<8>(c);
     else if (c->H == 64 && resident_smem <= 200 * 1024) launch_rnn_resident<16>(c);
     else if (c->H == 128 && resident_smem <= 200 * 1024) launch_rnn_resident<32>(c);
-    else if (c->H >= 256 && c->H % 32 == 0 && c->H <= 1024 && cluster_smem <= 200 * 1024)
+    else if (c->H % 32 == 0 && cluster_smem <= 200 * 1024)
         launch_dependent(k_enc_rnn_cluster, dim3(2 * kRnnClusterSize), dim3(c->H), cluster_smem, c->stream, c->m, c->d_proj, c->d_state, c->d_hlr);
     else
         launch_dependent(k_enc_rnn, dim3(2), dim3(kRnnThreads), 2 * c->H * sizeof(float), c->stream, c->m, c->d_proj, c->d_state, c->d_hlr);
@@ -790,8 +791,8 @@ cudaError_t set_kernel_attributes(const cutoff_ctx* c) {
         case 32: e = allow_smem(k_enc_rnn_resident<8>, 200 * 1024); break;
         case 64: e = allow_smem(k_enc_rnn_resident<16>, 200 * 1024); break;
         case 128: e = allow_smem(k_enc_rnn_resident<32>, 200 * 1024); break;
-        default: if (c->H >= 256) e = allow_smem(k_enc_rnn_cluster, 200 * 1024);
     }
+    if (e == cudaSuccess && c->H % 32 == 0) e = allow_smem(k_enc_rnn_cluster, 200 * 1024);
     if (e != cudaSuccess || !c->use_tc) return e;
     if (!c->literal) {
         e = allow_smem(tc::k_emit_tc, tc::kSmemBytes);
