@@ -129,7 +129,7 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, float a, float b, fl
 __device__ __forceinline__ float softplus_fast(float x) {          // ln(1 + e^x)
     float e;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * 1.4426950408889634f));
-    return x > 15.0f ? x : 0.6931471805599453f * __log2f(1.0f + e);
+    return x > 15.0f ? x : 0.6931471805599453f * log2_fast(1.0f + e);
 }
 
 __device__ __forceinline__ float sigmoid_fast(float x) {
@@ -579,8 +579,10 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
             const auto draw_normals = [&] {
 #pragma unroll
                 for (int c = 0; c < kDims; c += 4) {
-                    box_muller_fast(words[c / 4].x, words[c / 4].y, eps[c], eps[c + 1]);
-                    box_muller_fast(words[c / 4].z, words[c / 4].w, eps[c + 2], eps[c + 3]);
+                    float four[4];
+                    box_muller_fast(words[c / 4], four);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) eps[c + i] = four[i];
                 }
             };
             draw_words(0u);                                                       // the first guide step

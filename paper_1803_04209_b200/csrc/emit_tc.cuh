@@ -17,7 +17,7 @@
 //
 // What bounds it, at N = 1024, S = 65536, H = 256 and at N = 4096, S = 32768, H = 512: as four-byte operands, the stream from
 // L2 to shared memory (0.148 and 0.432 ms); as halves, with the weights resident (H = 256) and the
-// MMAs issued at their rate, it takes 0.119 and 0.282 ms.  Now no
+// MMAs issued at their rate, it takes 0.118 and 0.276 ms.  Now no
 // single resource: issue slots 57 %, shared-memory and store wavefronts 65 %, tensor pipe 28 % (N = 1024).  Shares, from an
 // earlier capture in which it took 0.113 and 0.290: streamed weights 0.122 and 0.297, the drawing alone, without operands and
 // products, 0.104 and 0.200, without the stores 0.111 and 0.295, without the products 0.112 and 0.241.
@@ -157,9 +157,9 @@ __device__ __forceinline__ void noise_epilogue_tile(float* __restrict__ x, int l
         tmem_ld8(taddr + c8, lo);
         tmem_ld8(taddr + kBW + c8, hi);
         const int jw = jw0 + c8;
-        float eps[8], out[8];
-        normal4_row_column_fast(noise, columns[c8 / 4], key.seed_lo, key.seed_hi, eps);
-        normal4_row_column_fast(noise, columns[c8 / 4 + 1], key.seed_lo, key.seed_hi, eps + 4);
+        float eps[2][4], out[8];
+        normal4_row_column_fast(noise, columns[c8 / 4], key.seed_lo, key.seed_hi, eps[0]);
+        normal4_row_column_fast(noise, columns[c8 / 4 + 1], key.seed_lo, key.seed_hi, eps[1]);
         tmem_ld_wait();
         if (c8 == 24) {
             tc_fence_before();
@@ -186,9 +186,15 @@ __device__ __forceinline__ void put_noise_columns(float* table, int j0, int lane
         reinterpret_cast<uint4*>(table + 128)[lane] = philox_column(static_cast<uint32_t>((j0 >> 2) + lane), kStreamEmission, step, key.seed_lo, key.seed_hi);
 }
 
-__device__ __forceinline__ void load8(float (&r)[8], const float* p) {
-    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-    r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w; r[4] = b.x; r[5] = b.y; r[6] = b.z; r[7] = b.w;
+// Eight floats of a table as pairs.
+__device__ __forceinline__ void load8(unsigned long long (&r)[4], const float* p) {
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(p), b = *reinterpret_cast<const ulonglong2*>(p + 4);
+    r[0] = a.x; r[1] = a.y; r[2] = b.x; r[3] = b.y;
+}
+// acc * row * column + bias of two accumulators, in this order.
+__device__ __forceinline__ unsigned long long unscale2(uint32_t acc0, uint32_t acc1, unsigned long long row, unsigned long long column, unsigned long long bias) {
+    fma2(bias, mul2(pack2(__uint_as_float(acc0), __uint_as_float(acc1)), row), column);
+    return bias;
 }
 
 // A warp's table for the 32 workers from j0 on: mean and log-variance biases, then the inverse scales of the same rows of W4
@@ -206,16 +212,17 @@ __device__ __forceinline__ void stage_emission_tables(const EmitArgs& a, float* 
 __device__ __forceinline__ void emit_epilogue_tile(const EmitArgs& a, uint32_t taddr, int row, int j0, int lane, uint32_t bar_acc_empty,
                                                    const float* table, float v_inv) {
     noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, table, taddr, j0, lane, bar_acc_empty,
-                        [&](const uint32_t (&mean)[8], const uint32_t (&logvar)[8], const float (&eps)[8], int c8, float (&out)[8]) {
-        float bm[8], bl[8], sm[8], sl[8];
+                        [&](const uint32_t (&mean)[8], const uint32_t (&logvar)[8], const float (&eps)[2][4], int c8, float (&out)[8]) {
+        unsigned long long bm[4], bl[4], sm[4], sl[4];
         load8(bm, table + c8);
         load8(bl, table + 32 + c8);
         load8(sm, table + 64 + c8);
         load8(sl, table + 96 + c8);
+        const unsigned long long row_inv = pack2(v_inv, v_inv);
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-            out[c] = fmaf(exp_half_fast(fmaf(__uint_as_float(logvar[c]) * v_inv, sl[c], bl[c])), eps[c],
-                          fmaf(__uint_as_float(mean[c]) * v_inv, sm[c], bm[c]));
+        for (int c = 0; c < 8; c += 2)
+            unpack2(scale_noise2(unscale2(logvar[c], logvar[c + 1], row_inv, sl[c / 2], bl[c / 2]), eps[c / 4][c % 4], eps[c / 4][c % 4 + 1],
+                                 unscale2(mean[c], mean[c + 1], row_inv, sm[c / 2], bm[c / 2])), out[c], out[c + 1]);
     });
 }
 

@@ -129,16 +129,21 @@ struct EmitDualArgs {
 __device__ __forceinline__ void dual_epilogue_tile(const EmitDualArgs& a, uint32_t taddr, int row, int j0, int lane, uint32_t bar_acc_empty,
                                                    const float* table, float u_inv, float r_inv) {
     noise_epilogue_tile(a.x, a.ldx, a.N, row < a.count, row, a.sample_base + static_cast<uint32_t>(row), a.key, table, taddr, j0, lane, bar_acc_empty,
-                        [&](const uint32_t (&mean)[8], const uint32_t (&scale)[8], const float (&eps)[8], int c8, float (&out)[8]) {
-        float bm[8], bs[8], im[8], is[8];
+                        [&](const uint32_t (&mean)[8], const uint32_t (&scale)[8], const float (&eps)[2][4], int c8, float (&out)[8]) {
+        unsigned long long bm[4], bs[4], im[4], is[4];
         load8(bm, table + c8);
         load8(bs, table + 32 + c8);
         load8(im, table + 64 + c8);
         load8(is, table + 96 + c8);
+        const unsigned long long u2 = pack2(u_inv, u_inv), r2 = pack2(r_inv, r_inv);
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-            out[c] = fmaf(softplus_fast(fmaf(__uint_as_float(scale[c]) * r_inv, is[c], bs[c])), eps[c],
-                          fmaf(__uint_as_float(mean[c]) * u_inv, im[c], bm[c]));
+        for (int c = 0; c < 8; c += 2) {
+            float s0, s1;
+            unpack2(unscale2(scale[c], scale[c + 1], r2, is[c / 2], bs[c / 2]), s0, s1);
+            unsigned long long x = unscale2(mean[c], mean[c + 1], u2, im[c / 2], bm[c / 2]);
+            fma2(x, pack2(softplus_fast(s0), softplus_fast(s1)), pack2(eps[c / 4][c % 4], eps[c / 4][c % 4 + 1]));
+            unpack2(x, out[c], out[c + 1]);
+        }
     });
 }
 
