@@ -961,6 +961,166 @@ __global__ void k_transpose_heads(const float* __restrict__ W4, int N, int H, in
             out[(static_cast<size_t>(k0 + r) * 2 + head) * ldn + j0 + threadIdx.x] = tile[threadIdx.x][r];
 }
 
+// ---------------------------------------------------------------------------------------------
+// The same layer with the weights of a CTA's workers resident in shared memory: one persistent CTA per SM, 4 TX workers per CTA,
+// (32 / TX) RM samples at a time per warp, and no warp waits for another.  A thread has RM samples x 4 workers, both heads.
+// What bounds it is the issue of instructions: per k 4 RM paired multiply-adds (two columns each), RM / 2 loads of two hidden values and
+// two of weights.  A hidden value is stored twice in a row, so that a load brings the pair that an instruction multiplies two
+// columns with; made in registers, the pairs took as many moves as there are multiply-adds to four columns.  The warps of a
+// CTA lie evenly on the four schedulers, and CTAs of this size cannot crowd on the SMs that the chain leaves free: the CTAs of 64 threads of
+// the kernel below did both (N=16, S=1024: 128 of them on 19 SMs).  Emission stage before and after: N=16 S=60000 33.6 and 15.1 us,
+// N=30 S=30000 23.6 and 15.4, N=50 S=8000 23.6 and 15.1, N=16 S=1024 9.1 and 7.2.  With several worker tiles of 32 the reads of the
+// pairs cost more than it gains (four cycles of the shared-memory pipe for 16 bytes a lane): N=100 S=60000 79 and 87, N=250 S=1500 17 and 23.
+// ---------------------------------------------------------------------------------------------
+constexpr int kEmitRowsWarps = 16, kEmitRowsTK = 16, kEmitRowsPitch = 2 * kEmitRowsTK + 4;
+
+// Shared memory: the weights [H][2][4 TX], and per warp its samples' hidden values of 16 k.  Never less than half an SM's: one CTA per SM.
+template <int TX, int RM> __host__ __device__ constexpr int emit_rows_warp_floats() {
+    const int hidden = 32 / TX * RM * kEmitRowsPitch, results = (RM < 4 ? RM : 4) * 8 * 32;
+    return hidden > results ? hidden : results;
+}
+template <int TX, int RM> constexpr size_t emit_rows_smem_bytes(int H) {
+    const size_t bytes = sizeof(float) * (static_cast<size_t>(H) * 8 * TX + kEmitRowsWarps * emit_rows_warp_floats<TX, RM>());
+    return bytes < 116 * 1024 ? 116 * 1024 : bytes;
+}
+
+template <int TX, int RM>
+__global__ void __launch_bounds__(kEmitRowsWarps * 32, 1) k_emit_rows(ModelDev m, const float* __restrict__ v, const float* __restrict__ W4T, int ldn,
+                                                            const DevState* __restrict__ st, NoiseKey key,
+                                                            uint32_t sample_base, int count,
+                                                            float* __restrict__ x, int ldx) {
+    constexpr int TN = 4 * TX, TY = 32 / TX, TM = TY * RM, TK = kEmitRowsTK, kPitch = kEmitRowsPitch;
+    constexpr int kQuads = TM * TK / 4, kLoads = (kQuads + 31) / 32;     // 16-byte pieces of a slab, and how many a lane moves
+    constexpr int kStage = RM < 4 ? RM : 4;                              // samples whose results wait in shared memory for their draws
+    static_assert(kStage * 8 * 32 <= emit_rows_warp_floats<TX, RM>(), "results fit where the hidden values were");
+    extern __shared__ __align__(16) float sm_rows[];
+    const int H = m.H, N = m.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tx = lane % TX, ty = lane / TX;
+    const int worker_tiles = ceil_div(N, TN), wt = static_cast<int>(blockIdx.x) % worker_tiles, part = static_cast<int>(blockIdx.x) / worker_tiles;
+    const int parts = (static_cast<int>(gridDim.x) - wt + worker_tiles - 1) / worker_tiles;      // CTAs that share these workers
+    const int j0 = wt * TN, jbase = j0 + 4 * tx;
+    float* const weights = sm_rows;
+    float* const hidden = sm_rows + static_cast<size_t>(H) * 2 * TN + warp * emit_rows_warp_floats<TX, RM>();
+    const uint32_t weights_s = fma32::smem_addr(weights);
+    for (int i = threadIdx.x; i < H * 2 * TX; i += kEmitRowsWarps * 32) {
+        const int k2 = i / TX, j = j0 + i % TX * 4;                       // k2: k and head
+        fma32::copy4<true>(weights_s + 16 * i, j < ldn ? W4T + static_cast<size_t>(k2) * ldn + j : W4T, ldn - j);
+    }
+    dependency_wait();            // up to here: weights.  No launch_dependents: the row sort after this kernel has a few CTAs per SM, and placed
+                                  // early they crowd on the SMs that happen to have room
+    fma32::copies_landed();
+    __syncthreads();
+    const int tiles = ceil_div(count, TM);
+    const uint4 column = philox_column(static_cast<uint32_t>(jbase >> 2), kStreamEmission, st->step, key.seed_lo, key.seed_hi);
+    const float* const wp = weights + 4 * tx;
+    const float* const hp = hidden + ty * kPitch;
+    float2* const own = reinterpret_cast<float2*>(hidden) + lane;
+    // consecutive tiles go to different CTAs, so that a small decision still spreads over all SMs
+#pragma unroll 1
+    for (int tile = part + parts * warp; tile < tiles; tile += parts * kEmitRowsWarps) {
+        const int row0 = tile * TM;
+        float4 next[kLoads];
+        const auto request = [&](int k0) {
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u) {
+                const int q = u * 32 + lane, r = q / (TK / 4), k = k0 + q % (TK / 4) * 4;
+                next[u] = q < kQuads && row0 + r < count && k < H ? *reinterpret_cast<const float4*>(v + static_cast<size_t>(row0 + r) * H + k)
+                                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        };
+        unsigned long long sums[RM][4] = {};                     // means of workers 0, 1 and 2, 3, then their log-variances
+        request(0);
+#pragma unroll 1
+        for (int k0 = 0; k0 < H; k0 += TK) {
+            __syncwarp();                                        // everyone has finished with the values before these
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u) {
+                const int q = u * 32 + lane, r = q / (TK / 4), c = q % (TK / 4) * 4;
+                if (q < kQuads) {
+                    float4* const dst = reinterpret_cast<float4*>(hidden + r * kPitch + 2 * c);
+                    dst[0] = make_float4(next[u].x, next[u].x, next[u].y, next[u].y);
+                    dst[1] = make_float4(next[u].z, next[u].z, next[u].w, next[u].w);
+                }
+            }
+            __syncwarp();
+            if (k0 + TK < H) request(k0 + TK);
+            const float* w = wp + static_cast<size_t>(k0) * 2 * TN;
+#pragma unroll
+            for (int k = 0; k < TK; k += 4) {
+                if (k0 + k >= H) break;                          // H is a multiple of 4
+#pragma unroll
+                for (int p = 0; p < 4; p += 2) {
+                    ulonglong2 a[RM];
+#pragma unroll
+                    for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(hp + i * TY * kPitch + 2 * (k + p));
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const ulonglong2 mean = *reinterpret_cast<const ulonglong2*>(w + (k + p + q) * 2 * TN);
+                        const ulonglong2 logvar = *reinterpret_cast<const ulonglong2*>(w + (k + p + q) * 2 * TN + TN);
+#pragma unroll
+                        for (int i = 0; i < RM; ++i) {
+                            const unsigned long long s2 = q == 0 ? a[i].x : a[i].y;
+                            fma2(sums[i][0], s2, mean.x);
+                            fma2(sums[i][1], s2, mean.y);
+                            fma2(sums[i][2], s2, logvar.x);
+                            fma2(sums[i][3], s2, logvar.y);
+                        }
+                    }
+                }
+            }
+        }
+        // The draws one sample at a time, results through shared memory (each lane its own), four samples of the lane at once:
+        // unrolled, the generator and its logarithms and sines would be 30 KB of instructions, which a call that finds the caches cold
+        // fetches from memory.
+        float b_mean[4], b_logvar[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            b_mean[c] = jbase + c < N ? m.b4[jbase + c] : 0.f;
+            b_logvar[c] = jbase + c < N ? m.b4[N + jbase + c] : 0.f;
+        }
+#pragma unroll 1
+        for (int i0 = 0; i0 < RM; i0 += kStage) {
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < kStage; ++i)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    float2 pair;
+                    unpack2(sums[i][c], pair.x, pair.y);
+                    own[(4 * i + c) * 32] = pair;
+                }
+#pragma unroll 1
+            for (int i = 0; i < kStage; ++i) {
+                const int k = row0 + ty + TY * (i0 + i);
+                if (k >= count || jbase >= N) break;
+                float eps[4], mean[4], logvar[4], out[4];
+                normal4_row_column(philox_row(sample_base + static_cast<uint32_t>(k), kStreamEmission, key.seed_lo), column, key.seed_lo, key.seed_hi, eps);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const float2 mp = own[(4 * i + c) * 32], lp = own[(4 * i + 2 + c) * 32];
+                    mean[2 * c] = mp.x; mean[2 * c + 1] = mp.y;
+                    logvar[2 * c] = lp.x; logvar[2 * c + 1] = lp.y;
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) out[c] = fmaf(expf(0.5f * (logvar[c] + b_logvar[c])), eps[c], mean[c] + b_mean[c]);
+                float* dst = x + static_cast<size_t>(k) * ldx + jbase;           // the row pitch is a multiple of 8 floats
+                if (jbase + 3 < N) {
+                    *reinterpret_cast<float4*>(dst) = make_float4(out[0], out[1], out[2], out[3]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (jbase + c < N) dst[c] = out[c];
+                }
+            }
+            if constexpr (RM > kStage) {
+#pragma unroll
+                for (int i = 0; i < kStage; ++i)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) sums[i][c] = sums[i + kStage][c];
+            }
+        }
+    }
+}
+
 template <int RM>
 __global__ void __launch_bounds__(kEmitThreads, RM == 8 ? 7 : 8) k_emit_fma(ModelDev m, const float* __restrict__ v, const float* __restrict__ W4T, int ldn,
                                                             const DevState* __restrict__ st, NoiseKey key,

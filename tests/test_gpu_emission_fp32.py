@@ -18,10 +18,13 @@ def _lib():
     return binding.load_library()
 
 
-# worker counts around a tile of 64 and around the row pitch, hidden widths that are not whole slabs of 8, sample counts around
-# the tiles of 8 and 32, and calls large enough (296 tiles of 32 x 64) for the large tile
+# worker counts around the tiles of 16, 32 and 64 and around the row pitch, hidden widths that are not whole slabs of 16, sample counts around
+# the tiles of 4 to 64, calls at the borders between the tiles (1776 of them: 12 for each of 148 SMs),
+# and hidden widths up to the largest whose weights stay in shared memory (N <= 16: 664, else 620) and beyond
 @pytest.mark.parametrize("N,D,H,S", [(1, 4, 4, 7), (3, 4, 12, 9), (63, 4, 20, 33), (64, 4, 8, 9472), (65, 4, 36, 4737), (130, 8, 8, 3200),
-                                     (257, 8, 24, 2049), (4096, 4, 16, 161)])
+                                     (257, 8, 24, 2049), (4096, 4, 16, 161),
+                                     (16, 4, 32, 14201), (17, 4, 32, 7101), (33, 4, 28, 28417), (16, 4, 32, 113700), (15, 4, 664, 65), (9, 4, 668, 65),
+                                     (32, 4, 620, 130), (40, 4, 624, 130), (128, 8, 128, 16384), (4096, 16, 592, 37)])
 def test_every_tile_gives_the_same_draws(N, D, H, S):
     w = inputs.make_weights(N, D, H, seed=N, fan_in_ref=32)
     gpu = binding.Cutoff(N, D, H, 1, S, seed=5)
