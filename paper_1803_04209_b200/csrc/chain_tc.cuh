@@ -91,7 +91,7 @@ __host__ __device__ constexpr uint32_t chain_tc_operand_bytes(int D, int H, bool
 constexpr int kChainLatentBytes = 2 * 16384;      // latent tiles of two slots
 
 inline size_t chain_tc_smem_bytes(int D, int H, int W, bool literal) {
-    const size_t floats = (literal ? 4 : 3) * static_cast<size_t>(H) + 4 * 128 + 2 * static_cast<size_t>(W) * D + (literal ? D * D : 0) + 5 * D +
+    const size_t floats = (literal ? 4 : 3) * static_cast<size_t>(H) + 2 * 4 * 128 + 2 * static_cast<size_t>(W) * D + (literal ? D * D : 0) + 5 * D +
                           (literal ? 4 : 2) * D + 32;
     return 1024 + chain_tc_operand_bytes(D, H, literal) + kChainLatentBytes + floats * 4;
 }
@@ -260,8 +260,12 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
     float* sb1 = sbzs + H;
     float* sb3 = sb1 + H;
     float* sbi1 = sb3 + H;                   // literal only
-    float* szmax = sb3 + (LITERAL ? 2 : 1) * H;      // [slot][column group][row] largest |latent| of a thread's dimensions
-    float* sct = szmax + 4 * 128;            // [W][D]  Wmu (h_left + h_right) / 3 + bmu
+    // [guide, transition][slot][column group][row] largest |latent| of a thread's dimensions.  Two arrays, because nobody waits between the
+    // last layer's reads of the transition's and, in a window of one step, the next tile's writes of the guide's: a warp that is ahead would
+    // change what another has yet to read.  So both arrays' writes are a barrier that all warps arrive at away from their readers: the guide's are
+    // read before the arrivals on bar_z that the last layer's product waits for, the transition's before those on bar_h of the next tile.
+    float* szmax = sb3 + (LITERAL ? 2 : 1) * H;
+    float* sct = szmax + 2 * 4 * 128;        // [W][D]  Wmu (h_left + h_right) / 3 + bmu
     float* spt = sct + W * D;                // [W][D]  the same of the scale: Wsig times that, + bsig
     float* sWl = spt + W * D;                // [D][D], literal only
     // what the products of halves are multiplied with: mu D, the two parts of the scale's map D each, then W2 2D or Wg2, Wh2 D each
@@ -552,7 +556,8 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
         const uint32_t cols = tmem + lane_off + hidden0, packed = tmem + lane_off + packed_col(cg);
         const uint32_t res = tmem + lane_off + acc2_col + kDims * cg;             // this thread's columns of a second result
         const int d0 = kDims * cg;                                                // its latent dimensions
-        float* const largest = szmax + slot * kGroups * 128 + row;                // [column group][128]
+        float* const z_largest = szmax + slot * kGroups * 128 + row;              // [column group][128]: the guide's latent
+        float* const t_largest = z_largest + 4 * 128;                             // the transition's
         float gate_own[kDims], lin_own[kDims], G_own[kDims];                      // literal
         uint32_t np = 0, na = 0;
         const auto arrive = [&](uint32_t bar) {                     // our reads and writes precede the MMAs that this unblocks
@@ -589,7 +594,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
             draw_normals();
 #pragma unroll
             for (int c = 0; c < kDims; ++c) z_own[c] = fmaf(softplus_fast(spt[d0 + c]), eps[c], sct[d0 + c]);
-            if (W == 1) put_largest(smem_u32(largest + cg * 128), z_own);
+            if (W == 1) put_largest(smem_u32(z_largest + cg * 128), z_own);
             store_latent(z_own);
             float h_inv = 1.0f;                                                   // inverse scale of the hidden layer
             for (int ph = 1; ph < n_phases; ++ph) {
@@ -626,6 +631,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                 } else {
                     unsigned long long scale2 = 0;
                     if (ph >= W) {                                  // the column groups' largest |latent| of this sample
+                        const float* const largest = ph == ph_last ? t_largest : z_largest;
                         float zm = 0.0f, scale;
 #pragma unroll
                         for (int gg = 0; gg < kGroups; ++gg) zm = fmaxf(zm, largest[gg * 128]);
@@ -704,7 +710,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                         const float pre = fmaf(__uint_as_float(hi[c]), sscale[D + d], fmaf(__uint_as_float(lo[c]), sscale[2 * D + d], spt[ph * D + d]));
                         z_own[c] = fmaf(softplus_fast(pre), eps[c], fmaf(__uint_as_float(r0[c]), sscale[d], sct[ph * D + d]));
                     }
-                    if (ph == W - 1) put_largest(smem_u32(largest + cg * 128), z_own);      // the next layer scales its halves by it
+                    if (ph == W - 1) put_largest(smem_u32(z_largest + cg * 128), z_own);      // the next layer scales its halves by it
                 } else if constexpr (!LITERAL) {
                     uint32_t lv[kDims];
                     tmem_ld_dims(res + D, lv);
@@ -715,7 +721,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                         z_own[c] = fmaf(exp_half_fast(fmaf(__uint_as_float(lv[c]) * h_inv, sscale[4 * D + d], sb2[D + d])), eps[c],
                                         fmaf(__uint_as_float(r0[c]) * h_inv, sscale[3 * D + d], sb2[d]));
                     }
-                    put_largest(smem_u32(largest + cg * 128), z_own);
+                    put_largest(smem_u32(t_largest + cg * 128), z_own);
                 } else {
                     tmem_ld_wait();
                     if (ph == W) {
@@ -757,7 +763,7 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
                     tmem_ld_wait();
 #pragma unroll
                     for (int c = 0; c < kDims; ++c) z_own[c] = fmaf(softplus_fast(__uint_as_float(r0[c]) + sbs[d0 + c]), eps[c], G_own[c]);
-                    put_largest(smem_u32(largest + cg * 128), z_own);
+                    put_largest(smem_u32(t_largest + cg * 128), z_own);
                 }
                 store_latent(z_own);
             }

@@ -47,6 +47,24 @@ def test_tensor_core_chain_meets_the_oracle(D, H, lag, S, literal):
         assert np.array_equal(gpu.debug_samples(first, n), x[first:first + n])
 
 
+# A window of one step is the one in which the tiles of a slot follow each other without a guide step in between: three tiles and more
+# for each slot (D = 16: two slots per SM, D = 32: one), all samples against calls that give an SM one tile at most.
+@pytest.mark.parametrize("literal", [False, True])
+@pytest.mark.parametrize("D,H", [(16, 64), (16, 256), (32, 32), (32, 512)])
+def test_tiles_of_a_slot_in_windows_of_one_step(D, H, literal):
+    N, S = 20, (256 if D == 16 else 128) * SMS * 3 + 65
+    make = inputs.make_weights_literal if literal else inputs.make_weights
+    gpu = binding.Cutoff(N, D, H, 0, S, precision=1, seed=7, flags=binding.FLAG_LITERAL if literal else 0)
+    gpu.load_weights(make(N, D, H, seed=H, fan_in_ref=32))
+    for x in inputs.make_trace(N, 2, seed=D, sigma=0.25):
+        gpu.push(x)
+    x = gpu.debug_samples(0, S)
+    assert np.isfinite(x).all()
+    for first in range(0, S, 128 * SMS):
+        n = min(128 * SMS, S - first)
+        assert np.array_equal(gpu.debug_samples(first, n), x[first:first + n])
+
+
 def test_hidden_layers_keep_their_bits_at_any_scale():
     # the transition's hidden layer times 2^a against output weights times 2^-a: powers of two, so the same samples to the last bit
     N, D, H, lag, S = 20, 16, 128, 2, 2500
