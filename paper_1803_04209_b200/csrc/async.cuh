@@ -43,15 +43,17 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// Bounded wait.  Returns false if it gave up or if another role already aborted.
+// Bounded wait of a whole warp.  Returns false, in all lanes, if it gave up or if another role already aborted: what follows a wait (an election,
+// tensor-memory reads, warp barriers) takes all lanes of the warp, so they may not part ways on its result.  The lanes read the
+// barrier, the flag and the clock each for itself, therefore the votes.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, DevState* st) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     const unsigned long long t0 = global_ns();
     for (uint32_t it = 1;; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
         if ((it & 63u) == 0u) {
-            if (*abort_flag) return false;
-            if (global_ns() - t0 > kWaitLimitNs) {
+            if (__any_sync(0xffffffffu, *abort_flag)) return false;
+            if (__any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) {
                 *abort_flag = 1;
                 atomicOr(&st->error_flags, kErrTimeout);
                 return false;
