@@ -595,9 +595,9 @@ void launch_emission_literal(cutoff_ctx* c, uint32_t sample_base, int count) {
 }
 
 // The fp32 emission keeps its weights in shared memory for up to 64 workers (N=70, S=3000: 19 us either way; N=50, S=8000: 15 against 24;
-// N=100, S=60000: 87 against 79), where they fit beside the hidden values (32 workers: H <= 620, 16: H <= 664).
+// N=100, S=60000: 87 against 79), where they fit beside the hidden values (32 workers: H <= 652, 16: every H).
 bool emission_rows(const cutoff_ctx* c) {
-    return !c->literal && !c->use_tc && c->N <= 64 && (c->N <= 16 ? emit_rows_smem_bytes<4, 8>(c->H) : emit_rows_smem_bytes<8, 8>(c->H)) <= 227 * 1024;
+    return !c->literal && !c->use_tc && c->N <= 64 && (c->N <= 16 ? emit_rows_smem_bytes<4, 4>(c->H) : emit_rows_smem_bytes<8, 4>(c->H)) <= 227 * 1024;
 }
 
 void launch_emission(cutoff_ctx* c, uint32_t sample_base, int count) {
@@ -605,7 +605,9 @@ void launch_emission(cutoff_ctx* c, uint32_t sample_base, int count) {
     if (c->use_tc) { launch_emission_tc(c, sample_base, count); return; }
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     if (emission_rows(c)) {
-        // As many samples per lane as still give most warps of the GPU a tile: fewer read the weights and hidden values more often.
+        // As many samples per lane as still give most warps of the GPU a tile: fewer read the weights and hidden values more often.  Not more
+        // than four: with eight, tiles twice as large spill and leave twice as much of the GPU idle in their last round (N=64, H=320,
+        // S=38500: 134 us against 111 with four and 113 without resident weights; S=65536: 168 and 162).
         const int worker_tiles = ceil_div(c->N, c->N <= 16 ? 16 : 32), sample_lanes = c->N <= 16 ? 8 : 4, enough = 12 * c->sm_count;
         const auto full = [&](int per_lane) { return worker_tiles * ceil_div(count, sample_lanes * per_lane) >= enough; };
         const auto run = [&](auto* kernel, size_t smem) {
@@ -613,13 +615,11 @@ void launch_emission(cutoff_ctx* c, uint32_t sample_base, int count) {
                              c->ldx, c->d_state, key, sample_base, count, c->d_x, c->ldx);
         };
         if (c->N <= 16) {
-            if (full(8)) run(k_emit_rows<4, 8>, emit_rows_smem_bytes<4, 8>(c->H));
-            else if (full(4)) run(k_emit_rows<4, 4>, emit_rows_smem_bytes<4, 4>(c->H));
+            if (full(4)) run(k_emit_rows<4, 4>, emit_rows_smem_bytes<4, 4>(c->H));
             else if (full(2)) run(k_emit_rows<4, 2>, emit_rows_smem_bytes<4, 2>(c->H));
             else run(k_emit_rows<4, 1>, emit_rows_smem_bytes<4, 1>(c->H));
         } else {
-            if (full(8)) run(k_emit_rows<8, 8>, emit_rows_smem_bytes<8, 8>(c->H));
-            else if (full(4)) run(k_emit_rows<8, 4>, emit_rows_smem_bytes<8, 4>(c->H));
+            if (full(4)) run(k_emit_rows<8, 4>, emit_rows_smem_bytes<8, 4>(c->H));
             else if (full(2)) run(k_emit_rows<8, 2>, emit_rows_smem_bytes<8, 2>(c->H));
             else run(k_emit_rows<8, 1>, emit_rows_smem_bytes<8, 1>(c->H));
         }
@@ -823,7 +823,6 @@ cudaError_t set_kernel_attributes(const cutoff_ctx* c) {
     if (e == cudaSuccess && c->H % 32 == 0) e = allow_smem(k_enc_rnn_cluster, 200 * 1024);
     if (emission_rows(c)) {
         const auto allow = [&](auto* kernel) { if (e == cudaSuccess) e = allow_smem(kernel, 227 * 1024); };
-        allow(c->N <= 16 ? k_emit_rows<4, 8> : k_emit_rows<8, 8>);
         allow(c->N <= 16 ? k_emit_rows<4, 4> : k_emit_rows<8, 4>);
         allow(c->N <= 16 ? k_emit_rows<4, 2> : k_emit_rows<8, 2>);
         allow(c->N <= 16 ? k_emit_rows<4, 1> : k_emit_rows<8, 1>);

@@ -976,7 +976,7 @@ constexpr int kEmitRowsWarps = 16, kEmitRowsTK = 16, kEmitRowsPitch = 2 * kEmitR
 
 // Shared memory: the weights [H][2][4 TX], and per warp its samples' hidden values of 16 k.  Never less than half an SM's: one CTA per SM.
 template <int TX, int RM> __host__ __device__ constexpr int emit_rows_warp_floats() {
-    const int hidden = 32 / TX * RM * kEmitRowsPitch, results = (RM < 4 ? RM : 4) * 8 * 32;
+    const int hidden = 32 / TX * RM * kEmitRowsPitch, results = RM * 8 * 32;
     return hidden > results ? hidden : results;
 }
 template <int TX, int RM> constexpr size_t emit_rows_smem_bytes(int H) {
@@ -991,8 +991,6 @@ __global__ void __launch_bounds__(kEmitRowsWarps * 32, 1) k_emit_rows(ModelDev m
                                                             float* __restrict__ x, int ldx) {
     constexpr int TN = 4 * TX, TY = 32 / TX, TM = TY * RM, TK = kEmitRowsTK, kPitch = kEmitRowsPitch;
     constexpr int kQuads = TM * TK / 4, kLoads = (kQuads + 31) / 32;     // 16-byte pieces of a slab, and how many a lane moves
-    constexpr int kStage = RM < 4 ? RM : 4;                              // samples whose results wait in shared memory for their draws
-    static_assert(kStage * 8 * 32 <= emit_rows_warp_floats<TX, RM>(), "results fit where the hidden values were");
     extern __shared__ __align__(16) float sm_rows[];
     const int H = m.H, N = m.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tx = lane % TX, ty = lane / TX;
     const int worker_tiles = ceil_div(N, TN), wt = static_cast<int>(blockIdx.x) % worker_tiles, part = static_cast<int>(blockIdx.x) / worker_tiles;
@@ -1068,54 +1066,44 @@ __global__ void __launch_bounds__(kEmitRowsWarps * 32, 1) k_emit_rows(ModelDev m
                 }
             }
         }
-        // The draws one sample at a time, results through shared memory (each lane its own), four samples of the lane at once:
-        // unrolled, the generator and its logarithms and sines would be 30 KB of instructions, which a call that finds the caches cold
-        // fetches from memory.
+        // The draws one sample at a time, results through shared memory (each lane its own): unrolled, the generator, its logarithms and
+        // sines would be RM copies of their code, which a call that finds the caches cold fetches from memory.
         float b_mean[4], b_logvar[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             b_mean[c] = jbase + c < N ? m.b4[jbase + c] : 0.f;
             b_logvar[c] = jbase + c < N ? m.b4[N + jbase + c] : 0.f;
         }
-#pragma unroll 1
-        for (int i0 = 0; i0 < RM; i0 += kStage) {
-            __syncwarp();
+        __syncwarp();
 #pragma unroll
-            for (int i = 0; i < kStage; ++i)
+        for (int i = 0; i < RM; ++i)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float2 pair;
-                    unpack2(sums[i][c], pair.x, pair.y);
-                    own[(4 * i + c) * 32] = pair;
-                }
-#pragma unroll 1
-            for (int i = 0; i < kStage; ++i) {
-                const int k = row0 + ty + TY * (i0 + i);
-                if (k >= count || jbase >= N) break;
-                float eps[4], mean[4], logvar[4], out[4];
-                normal4_row_column(philox_row(sample_base + static_cast<uint32_t>(k), kStreamEmission, key.seed_lo), column, key.seed_lo, key.seed_hi, eps);
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const float2 mp = own[(4 * i + c) * 32], lp = own[(4 * i + 2 + c) * 32];
-                    mean[2 * c] = mp.x; mean[2 * c + 1] = mp.y;
-                    logvar[2 * c] = lp.x; logvar[2 * c + 1] = lp.y;
-                }
-#pragma unroll
-                for (int c = 0; c < 4; ++c) out[c] = fmaf(expf(0.5f * (logvar[c] + b_logvar[c])), eps[c], mean[c] + b_mean[c]);
-                float* dst = x + static_cast<size_t>(k) * ldx + jbase;           // the row pitch is a multiple of 8 floats
-                if (jbase + 3 < N) {
-                    *reinterpret_cast<float4*>(dst) = make_float4(out[0], out[1], out[2], out[3]);
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (jbase + c < N) dst[c] = out[c];
-                }
+            for (int c = 0; c < 4; ++c) {
+                float2 pair;
+                unpack2(sums[i][c], pair.x, pair.y);
+                own[(4 * i + c) * 32] = pair;
             }
-            if constexpr (RM > kStage) {
+#pragma unroll 1
+        for (int i = 0; i < RM; ++i) {
+            const int k = row0 + ty + TY * i;
+            if (k >= count || jbase >= N) break;
+            float eps[4], mean[4], logvar[4], out[4];
+            normal4_row_column(philox_row(sample_base + static_cast<uint32_t>(k), kStreamEmission, key.seed_lo), column, key.seed_lo, key.seed_hi, eps);
 #pragma unroll
-                for (int i = 0; i < kStage; ++i)
+            for (int c = 0; c < 2; ++c) {
+                const float2 mp = own[(4 * i + c) * 32], lp = own[(4 * i + 2 + c) * 32];
+                mean[2 * c] = mp.x; mean[2 * c + 1] = mp.y;
+                logvar[2 * c] = lp.x; logvar[2 * c + 1] = lp.y;
+            }
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) sums[i][c] = sums[i + kStage][c];
+            for (int c = 0; c < 4; ++c) out[c] = fmaf(expf(0.5f * (logvar[c] + b_logvar[c])), eps[c], mean[c] + b_mean[c]);
+            float* dst = x + static_cast<size_t>(k) * ldx + jbase;           // the row pitch is a multiple of 8 floats
+            if (jbase + 3 < N) {
+                *reinterpret_cast<float4*>(dst) = make_float4(out[0], out[1], out[2], out[3]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (jbase + c < N) dst[c] = out[c];
             }
         }
     }

@@ -20,11 +20,12 @@ def _lib():
 
 # worker counts around the tiles of 16, 32 and 64 and around the row pitch, hidden widths that are not whole slabs of 16, sample counts around
 # the tiles of 4 to 64, calls at the borders between the tiles (1776 of them: 12 for each of 148 SMs),
-# and hidden widths up to the largest whose weights stay in shared memory (N <= 16: 664, else 620) and beyond
+# and hidden widths up to the largest whose weights stay in shared memory (N <= 16: any, else 652) and beyond
 @pytest.mark.parametrize("N,D,H,S", [(1, 4, 4, 7), (3, 4, 12, 9), (63, 4, 20, 33), (64, 4, 8, 9472), (65, 4, 36, 4737), (130, 8, 8, 3200),
                                      (257, 8, 24, 2049), (4096, 4, 16, 161),
                                      (16, 4, 32, 14201), (17, 4, 32, 7101), (33, 4, 28, 28417), (16, 4, 32, 113700), (15, 4, 664, 65), (9, 4, 668, 65),
-                                     (32, 4, 620, 130), (40, 4, 624, 130), (128, 8, 128, 16384), (4096, 16, 592, 37)])
+                                     (32, 4, 620, 130), (40, 4, 624, 130), (16, 4, 1024, 14300), (17, 4, 652, 7200), (64, 4, 652, 3700),
+                                     (33, 4, 656, 130), (64, 8, 128, 14201), (64, 4, 32, 18945), (128, 8, 128, 16384), (4096, 16, 592, 37)])
 def test_every_tile_gives_the_same_draws(N, D, H, S):
     w = inputs.make_weights(N, D, H, seed=N, fan_in_ref=32)
     gpu = binding.Cutoff(N, D, H, 1, S, seed=5)
