@@ -438,6 +438,22 @@ void launch_chain_t(cutoff_ctx* c, uint32_t sample_base, int count, size_t smem)
     }
 }
 
+// The tensor-core chain of a call of `count` samples, and how many of them are a tile.  Half tiles as long as every one of them has an SM of
+// its own (D=16, H=256, S=8192: 27 us, whole tiles on half the SMs 35), then whole tiles, each worked on by all warps of its SM, then, where
+// all operands fit, two side by side (S=65536: 68 us; one after the other by all warps 76 to 90).
+struct ChainTcChoice {
+    void (*kernel)(tc::ChainTcArgs);
+    int rows;
+};
+template <bool LITERAL>
+ChainTcChoice chain_tc_choice(const cutoff_ctx* c, int count) {
+    const bool wide = c->D == tc::kChain32D;
+    if (ceil_div(count, 64) <= c->sm_count) return {wide ? tc::k_chain_tc<32, LITERAL, 16, true> : tc::k_chain_tc<16, LITERAL, 16, true>, 64};
+    if (wide) return {tc::k_chain_tc<32, LITERAL, 16, false>, 128};
+    return {ceil_div(count, 128) <= c->sm_count ? tc::k_chain_tc<16, LITERAL, 16, false> : tc::k_chain_tc<16, LITERAL, 8, false>, 128};
+}
+ChainTcChoice chain_tc_choice(const cutoff_ctx* c, int count) { return c->literal ? chain_tc_choice<true>(c, count) : chain_tc_choice<false>(c, count); }
+
 void launch_chain_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
     tc::ChainTcArgs a{};
     const ModelDev& m = c->m;
@@ -451,23 +467,10 @@ void launch_chain_tc(cutoff_ctx* c, uint32_t sample_base, int count) {
     a.hlr = c->d_hlr; a.WzT = m.WzT; a.Wmu = m.Wmu; a.bounds = c->d_bound + 4; a.st = c->d_state;
     a.key = NoiseKey{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     a.sample_base = sample_base; a.count = count; a.H = c->H; a.W = c->W; a.v_out = half_v(c);
-    const auto run = [&](auto* kernel, int rows) {
-        const int tiles = ceil_div(count, rows);
-        launch_dependent(kernel, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kChainTcThreads),
-                         tc::chain_tc_smem_bytes(c->D, c->H, c->W, c->literal), c->stream, a);
-    };
-    // Half tiles as long as every one of them has an SM of its own (D=16, H=256, S=8192: 27 us, whole tiles on half the SMs 35), then whole
-    // tiles, each worked on by all warps of its SM, then, where all operands fit, two side by side (S=65536: 68 us; one after the other by
-    // all warps 76 to 90).
-    const bool half = ceil_div(count, 64) <= c->sm_count, one = ceil_div(count, 128) <= c->sm_count;
-    if (c->D == tc::kChain32D) {
-        if (c->literal) half ? run(tc::k_chain_tc<32, true, 16, true>, 64) : run(tc::k_chain_tc<32, true, 16, false>, 128);
-        else half ? run(tc::k_chain_tc<32, false, 16, true>, 64) : run(tc::k_chain_tc<32, false, 16, false>, 128);
-    } else if (c->literal) {
-        half ? run(tc::k_chain_tc<16, true, 16, true>, 64) : one ? run(tc::k_chain_tc<16, true, 16, false>, 128) : run(tc::k_chain_tc<16, true, 8, false>, 128);
-    } else {
-        half ? run(tc::k_chain_tc<16, false, 16, true>, 64) : one ? run(tc::k_chain_tc<16, false, 16, false>, 128) : run(tc::k_chain_tc<16, false, 8, false>, 128);
-    }
+    const ChainTcChoice choice = chain_tc_choice(c, count);
+    const int tiles = ceil_div(count, choice.rows);
+    launch_dependent(choice.kernel, dim3(tiles < c->sm_count ? tiles : c->sm_count), dim3(tc::kChainTcThreads),
+                     tc::chain_tc_smem_bytes(c->D, c->H, c->W, c->literal), c->stream, a);
     c->launches += 1;
 }
 
@@ -600,29 +603,31 @@ bool emission_rows(const cutoff_ctx* c) {
     return !c->literal && !c->use_tc && c->N <= 64 && (c->N <= 16 ? emit_rows_smem_bytes<4, 4>(c->H) : emit_rows_smem_bytes<8, 4>(c->H)) <= 227 * 1024;
 }
 
+// Its kernel for a call of `count` samples, and the shared memory that this takes.  As many samples per lane as still give most warps of the GPU
+// a tile: fewer read the weights and hidden values more often.  Not more than four: with eight, tiles twice as large spill and leave
+// twice as much of the GPU idle in their last round (N=64, H=320, S=38500: 134 us against 111 with four and 113 without resident
+// weights; S=65536: 168 and 162).
+struct EmitRowsChoice {
+    decltype(&k_emit_rows<4, 4>) kernel;
+    size_t smem;
+};
+template <int TX>
+EmitRowsChoice emit_rows_choice(const cutoff_ctx* c, int count) {
+    const auto full = [&](int per_lane) { return ceil_div(c->N, 4 * TX) * ceil_div(count, 32 / TX * per_lane) >= 12 * c->sm_count; };
+    if (full(4)) return {k_emit_rows<TX, 4>, emit_rows_smem_bytes<TX, 4>(c->H)};
+    if (full(2)) return {k_emit_rows<TX, 2>, emit_rows_smem_bytes<TX, 2>(c->H)};
+    return {k_emit_rows<TX, 1>, emit_rows_smem_bytes<TX, 1>(c->H)};
+}
+EmitRowsChoice emit_rows_choice(const cutoff_ctx* c, int count) { return c->N <= 16 ? emit_rows_choice<4>(c, count) : emit_rows_choice<8>(c, count); }
+
 void launch_emission(cutoff_ctx* c, uint32_t sample_base, int count) {
     if (c->literal) { launch_emission_literal(c, sample_base, count); return; }
     if (c->use_tc) { launch_emission_tc(c, sample_base, count); return; }
     const NoiseKey key{static_cast<uint32_t>(c->cfg.seed), static_cast<uint32_t>(c->cfg.seed >> 32)};
     if (emission_rows(c)) {
-        // As many samples per lane as still give most warps of the GPU a tile: fewer read the weights and hidden values more often.  Not more
-        // than four: with eight, tiles twice as large spill and leave twice as much of the GPU idle in their last round (N=64, H=320,
-        // S=38500: 134 us against 111 with four and 113 without resident weights; S=65536: 168 and 162).
-        const int worker_tiles = ceil_div(c->N, c->N <= 16 ? 16 : 32), sample_lanes = c->N <= 16 ? 8 : 4, enough = 12 * c->sm_count;
-        const auto full = [&](int per_lane) { return worker_tiles * ceil_div(count, sample_lanes * per_lane) >= enough; };
-        const auto run = [&](auto* kernel, size_t smem) {
-            launch_dependent(kernel, dim3(c->sm_count > worker_tiles ? c->sm_count : worker_tiles), dim3(kEmitRowsWarps * 32), smem, c->stream, c->m, c->d_v, c->d_W4T,
-                             c->ldx, c->d_state, key, sample_base, count, c->d_x, c->ldx);
-        };
-        if (c->N <= 16) {
-            if (full(4)) run(k_emit_rows<4, 4>, emit_rows_smem_bytes<4, 4>(c->H));
-            else if (full(2)) run(k_emit_rows<4, 2>, emit_rows_smem_bytes<4, 2>(c->H));
-            else run(k_emit_rows<4, 1>, emit_rows_smem_bytes<4, 1>(c->H));
-        } else {
-            if (full(4)) run(k_emit_rows<8, 4>, emit_rows_smem_bytes<8, 4>(c->H));
-            else if (full(2)) run(k_emit_rows<8, 2>, emit_rows_smem_bytes<8, 2>(c->H));
-            else run(k_emit_rows<8, 1>, emit_rows_smem_bytes<8, 1>(c->H));
-        }
+        const EmitRowsChoice choice = emit_rows_choice(c, count);
+        launch_dependent(choice.kernel, dim3(c->sm_count), dim3(kEmitRowsWarps * 32), choice.smem, c->stream, c->m, c->d_v, c->d_W4T, c->ldx,
+                         c->d_state, key, sample_base, count, c->d_x, c->ldx);
         c->launches += 1;
         return;
     }
@@ -657,19 +662,27 @@ void refresh_projections(cutoff_ctx* c) {
     c->proj_stale = false;
 }
 
+// H = 32, 64, 128: one CTA per direction with the recurrence matrix in registers.  Other widths in whole warps, as far as the matrix fits the
+// shared memories of a cluster of 8 CTAs (H <= 608, at windows of more than 41 steps less): one of these per direction (H = 256: a thread's share no longer fits its registers, and
+// one CTA that keeps part of the matrix in shared memory takes 21 us against 17; H = 192 with one CTA that reads the matrix from
+// L2 in every step, lag 6: 62 us, so 17; H = 96, lag 3: 17 and 12).
+bool encoder_resident(const cutoff_ctx* c) {
+    return (c->H == 32 || c->H == 64 || c->H == 128) && enc_rnn_resident_smem_floats(c->H, c->W) * sizeof(float) <= 200 * 1024;
+}
+bool encoder_cluster(const cutoff_ctx* c) {
+    return !encoder_resident(c) && c->H % 32 == 0 && enc_rnn_cluster_smem_floats(c->H, c->W) * sizeof(float) <= 200 * 1024;
+}
+
 void launch_encoder(cutoff_ctx* c) {
     refresh_projections(c);
-    // H = 32, 64, 128: one CTA per direction with the recurrence matrix in registers.  Other widths in whole warps: a cluster of 8 CTAs per
-    // direction (H = 256: a thread's share no longer fits its registers, and one CTA that keeps part of the matrix in shared memory takes 21
-    // us against 17; H = 192 with one CTA that reads the matrix from L2 in every step, lag 6:
-    // 62 us, so 17; H = 96, lag 3: 17 and 12).
-    const size_t cluster_smem = enc_rnn_cluster_smem_floats(c->H, c->W) * sizeof(float);
-    const size_t resident_smem = enc_rnn_resident_smem_floats(c->H, c->W) * sizeof(float);
-    if (c->H == 32 && resident_smem <= 200 * 1024) launch_rnn_resident<8>(c);
-    else if (c->H == 64 && resident_smem <= 200 * 1024) launch_rnn_resident<16>(c);
-    else if (c->H == 128 && resident_smem <= 200 * 1024) launch_rnn_resident<32>(c);
-    else if (c->H % 32 == 0 && cluster_smem <= 200 * 1024)
-        launch_dependent(k_enc_rnn_cluster, dim3(2 * kRnnClusterSize), dim3(c->H), cluster_smem, c->stream, c->m, c->d_proj, c->d_state, c->d_hlr);
+    if (encoder_resident(c)) {
+        if (c->H == 32) launch_rnn_resident<8>(c);
+        else if (c->H == 64) launch_rnn_resident<16>(c);
+        else launch_rnn_resident<32>(c);
+    }
+    else if (encoder_cluster(c))
+        launch_dependent(k_enc_rnn_cluster, dim3(2 * kRnnClusterSize), dim3(c->H), enc_rnn_cluster_smem_floats(c->H, c->W) * sizeof(float), c->stream,
+                         c->m, c->d_proj, c->d_state, c->d_hlr);
     else
         launch_dependent(k_enc_rnn, dim3(2), dim3(kRnnThreads), 2 * c->H * sizeof(float), c->stream, c->m, c->d_proj, c->d_state, c->d_hlr);
     c->launches += 1;
@@ -739,9 +752,8 @@ int collect_timing(cutoff_ctx* c) {
 
 bool valid_latent(int D) { return D == 4 || D == 8 || D == 16 || D == 32; }
 
-// Kernels that need more than 48 KB of dynamic shared memory must be told so once per device.  Done at
-// context creation, with the context's device current, for every kernel this context's shape can launch
-// (a function attribute belongs to the device's copy of the kernel, not to the process).
+// Kernels that need more than 48 KB of dynamic shared memory must be told so once per device, with the context's
+// device current (a function attribute belongs to the device's copy of the kernel, not to the process).
 template <typename Kernel>
 cudaError_t allow_smem(Kernel kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
@@ -793,40 +805,39 @@ cudaError_t allow_smem_chain(const cutoff_ctx* c) {
     return allow_smem(k_chain<D>, 220 * 1024);
 }
 
-// Only for the kernels this context runs: each one is loaded by the driver when it is first named.
+// The kernels that depend on how many samples a call draws: named for the passes of the context's decisions, anew when these change, and for
+// the draws that a caller asks for by number.
+cudaError_t set_call_attributes(const cutoff_ctx* c, int count) {
+    cudaError_t e = cudaSuccess;
+    if (c->chain_tc) e = allow_smem(chain_tc_choice(c, count).kernel, 227 * 1024);
+    if (e == cudaSuccess && emission_rows(c)) e = allow_smem(emit_rows_choice(c, count).kernel, 227 * 1024);
+    return e;
+}
+cudaError_t set_pass_attributes(const cutoff_ctx* c) {
+    const cudaError_t e = set_call_attributes(c, c->chunk_rows);
+    return e == cudaSuccess ? set_call_attributes(c, c->S - (c->n_chunks - 1) * c->chunk_rows) : e;      // the last pass may be smaller
+}
+
+// Only for the kernels that this context runs, or that an option makes it run: each one is loaded by the driver when it is first named.
 cudaError_t set_kernel_attributes(const cutoff_ctx* c) {
     cudaError_t e = allow_smem_sort(c->N);
-    if (e != cudaSuccess) return e;
-    if (c->chain_tc) {
-        const auto allow = [&](auto* kernel) { if (e == cudaSuccess) e = allow_smem(kernel, 227 * 1024); };
-        if (c->D == tc::kChain32D) {
-            allow(c->literal ? tc::k_chain_tc<32, true, 16, true> : tc::k_chain_tc<32, false, 16, true>);
-            allow(c->literal ? tc::k_chain_tc<32, true, 16, false> : tc::k_chain_tc<32, false, 16, false>);
-        } else {
-            allow(c->literal ? tc::k_chain_tc<16, true, 16, true> : tc::k_chain_tc<16, false, 16, true>);
-            allow(c->literal ? tc::k_chain_tc<16, true, 16, false> : tc::k_chain_tc<16, false, 16, false>);
-            allow(c->literal ? tc::k_chain_tc<16, true, 8, false> : tc::k_chain_tc<16, false, 8, false>);
+    if (e == cudaSuccess) e = set_pass_attributes(c);
+    if (e == cudaSuccess && !c->chain_tc) {
+        switch (c->D) {
+            case 4: e = allow_smem_chain<4>(c); break;
+            case 8: e = allow_smem_chain<8>(c); break;
+            case 16: e = allow_smem_chain<16>(c); break;
+            default: e = allow_smem_chain<32>(c); break;
         }
     }
-    else switch (c->D) {
-        case 4: e = allow_smem_chain<4>(c); break;
-        case 8: e = allow_smem_chain<8>(c); break;
-        case 16: e = allow_smem_chain<16>(c); break;
-        default: e = allow_smem_chain<32>(c); break;
+    if (e == cudaSuccess && encoder_resident(c)) {
+        switch (c->H) {
+            case 32: e = allow_smem(k_enc_rnn_resident<8>, 200 * 1024); break;
+            case 64: e = allow_smem(k_enc_rnn_resident<16>, 200 * 1024); break;
+            default: e = allow_smem(k_enc_rnn_resident<32>, 200 * 1024); break;
+        }
     }
-    if (e != cudaSuccess) return e;
-    switch (c->H) {
-        case 32: e = allow_smem(k_enc_rnn_resident<8>, 200 * 1024); break;
-        case 64: e = allow_smem(k_enc_rnn_resident<16>, 200 * 1024); break;
-        case 128: e = allow_smem(k_enc_rnn_resident<32>, 200 * 1024); break;
-    }
-    if (e == cudaSuccess && c->H % 32 == 0) e = allow_smem(k_enc_rnn_cluster, 200 * 1024);
-    if (emission_rows(c)) {
-        const auto allow = [&](auto* kernel) { if (e == cudaSuccess) e = allow_smem(kernel, 227 * 1024); };
-        allow(c->N <= 16 ? k_emit_rows<4, 4> : k_emit_rows<8, 4>);
-        allow(c->N <= 16 ? k_emit_rows<4, 2> : k_emit_rows<8, 2>);
-        allow(c->N <= 16 ? k_emit_rows<4, 1> : k_emit_rows<8, 1>);
-    }
+    if (e == cudaSuccess && encoder_cluster(c)) e = allow_smem(k_enc_rnn_cluster, 200 * 1024);
     if (e != cudaSuccess || !c->use_tc) return e;
     if (!c->literal) {
         e = allow_smem(tc::k_emit_tc, tc::kSmemBytes);
@@ -1784,8 +1795,11 @@ int cutoff_set_option(cutoff_ctx* c, const char* name, int64_t value) {
     if (std::strcmp(name, "pass_rows") == 0) {
         if (value < 1024 || value > 0x7fffffffll) return CUTOFF_ERR_BAD_ARG;
         if (c->graph_exec || c->graph_dev_exec) return CUTOFF_ERR_STATE;   // the captured graph replays the old split
+        DeviceGuard guard(c->cfg.device);
+        CU_CHECK(c, guard.err);
         plan_chunks(c, static_cast<int>(value));
         c->draws_valid = false;
+        CU_CHECK(c, set_pass_attributes(c));
         return CUTOFF_OK;
     }
     return CUTOFF_ERR_BAD_ARG;
@@ -1858,6 +1872,7 @@ int cutoff_debug_samples(cutoff_ctx* c, int64_t k0, int64_t count, float* x_out)
     for (int64_t done = 0; done < count; done += c->chunk_rows) {
         const int n = static_cast<int>(count - done < c->chunk_rows ? count - done : c->chunk_rows);
         const uint32_t base = static_cast<uint32_t>(c->cfg.sample_offset + k0 + done);
+        CU_CHECK(c, set_call_attributes(c, n));
         launch_chain(c, base, n);
         launch_emission(c, base, n);
         CU_CHECK(c, cudaMemcpy2DAsync(x_out + done * c->N, sizeof(float) * c->N, c->d_x, sizeof(float) * c->ldx,

@@ -336,7 +336,7 @@ inline size_t enc_rnn_resident_smem_floats(int H, int W) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Encoder, part 2, for multiples of 32 up to about 640 that k_enc_rnn_resident does not serve: the recurrence matrix of a direction is split over the shared
+// Encoder, part 2, for multiples of 32 up to 608 that k_enc_rnn_resident does not serve: the recurrence matrix of a direction is split over the shared
 // memories of a cluster of 8 CTAs (H/8 rows each), so it is read from global memory once.  Every CTA
 // keeps the whole state (double-buffered); after a step each row's new value is written into the next
 // state buffer of all 8 CTAs through distributed shared memory, and one cluster barrier (a hardware

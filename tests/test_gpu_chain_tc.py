@@ -65,6 +65,26 @@ def test_tiles_of_a_slot_in_windows_of_one_step(D, H, literal):
         assert np.array_equal(gpu.debug_samples(first, n), x[first:first + n])
 
 
+# Decisions in passes whose sizes take other kernels than the whole does, chosen after the context was made: whole tiles side by side, then
+# one tile per SM and half tiles; the fp32 model with 4, 2 and 1 samples per lane in the emission.
+@pytest.mark.parametrize("N,D,H,S,precision,literal", [(20, 16, 128, 40000, 1, False), (20, 16, 128, 40000, 1, True), (20, 32, 64, 40000, 1, False),
+                                                       (20, 32, 64, 40000, 1, True), (16, 8, 64, 60000, 0, False), (40, 8, 64, 16000, 0, False)])
+def test_decisions_in_passes_of_other_sizes(N, D, H, S, precision, literal):
+    make = inputs.make_weights_literal if literal else inputs.make_weights
+    gpu = binding.Cutoff(N, D, H, 1, S, precision=precision, seed=7, flags=binding.FLAG_LITERAL if literal else 0)
+    gpu.load_weights(make(N, D, H, seed=H, fan_in_ref=32))
+    for x in inputs.make_trace(N, 3, seed=D, sigma=0.25):
+        gpu.push(x)
+    state = gpu.save_state()
+    want = np.sort(gpu.debug_samples(0, S).astype(np.float64), axis=1).sum(axis=0)
+    for rows in (15000, 8000, 1024):
+        gpu.restore_state(state)                                      # the same decision again
+        gpu.set_option("pass_rows", rows)
+        assert gpu.predict()[0] == binding.OK
+        # a warp of the sort adds at most 26 rows (60000 over 296 CTAs of 8) in single precision, warps are added in double: 26 / 2^24
+        assert np.max(np.abs(gpu.get_partial_sums() - want)) <= 1.6e-6 * np.abs(want).max()
+
+
 def test_hidden_layers_keep_their_bits_at_any_scale():
     # the transition's hidden layer times 2^a against output weights times 2^-a: powers of two, so the same samples to the last bit
     N, D, H, lag, S = 20, 16, 128, 2, 2500
