@@ -222,12 +222,13 @@ void put_second_layer_half(uint8_t* tiles, float* inv, const double* w, size_t o
         uint32_t bits;
         std::memcpy(&bits, &big, 4);
         const int e = bits ? half_exponent(bits) : 0;
+        const double up = std::ldexp(1.0, e), down = std::ldexp(1.0, -e);       // exact factors, as the function itself would be too slow here
         const size_t row = row0 + o;
         for (size_t k = 0; k < H; ++k) {
-            const __half h = __float2half_rn(static_cast<float>(std::ldexp(w[o * H + k], e)));
+            const __half h = __float2half_rn(static_cast<float>(w[o * H + k] * up));
             const size_t at = k / 64 * block_rows * 128 + (row >> 3) * 1024 + (row & 7) * 128 + (((k % 64 >> 3) ^ (row & 7)) << 4) + (k & 7) * 2;
             std::memcpy(tiles + at, &h, 2);
-            if (rest) rest[o * H + k] = w[o * H + k] - std::ldexp(static_cast<double>(__half2float(h)), -e);
+            if (rest) rest[o * H + k] = w[o * H + k] - static_cast<double>(__half2float(h)) * down;
         }
         inv[row] = std::ldexp(1.0f, -e);
     }
