@@ -27,12 +27,12 @@
 // each (together 22 bits), and a bracket of its own.  The first step starts from one latent for all samples, so its tanh is one vector
 // too and joins the bracket: that step is only noise.
 //
-// What bounds it: with two tiles in flight the special-function pipe, 256 tanh per sample and step and about 60 logarithms, sines and the
-// like for its noise (S=65536, D=16, H=256, lag 4: 68 us, of which 21 at that pipe's rate of 16 a clock; the rest is each step's round
-// trip, two products and the noise in between, which the other tile covers in part).  With the hidden layer through shared memory as
-// tf32, 64 units at a time, four steps of handshakes each, it took 108.  With one tile per SM, the steps' latency: 3700 cycles, of
-// which 1400 are the tanh (S=8192: 41 -> 27 us; 35 with tiles of 128).  D=32, with one tile per SM: S=32768, H=512, lag 4 162 -> 92 us (of
-// which 35 at the special-function pipe's rate), S=8192, H=256 60 -> 35 us; its weights were copied by the epilogue's threads before.
+// What bounds it: each step's round trip, two products and the noise in between, which a second tile covers in part; no unit is busy.  Of
+// them the special-function pipe is the first (256 tanh per sample and step and about 60 logarithms, sines and the like for its
+// noise): S=65536, D=16, H=256, lag 4 67 us, special-function pipe 37 % busy, issue slots 44 %, shared-memory wavefronts 29 %, tensor pipe
+// 11 %.  With the hidden layer through shared memory as tf32, 64 units at a time, four steps of handshakes each, it took 108.  With
+// one tile per SM, S=8192 41 -> 27 us (35 with tiles of 128).  D=32, with one tile per SM: S=32768, H=512, lag 4 162 -> 92 us,
+// S=8192, H=256 60 -> 35 us; its weights were copied by the epilogue's threads before.
 //
 // The host prepares a swizzled image of the weight operands once.  Latent rows are 128 bytes wide (32 tf32).  D = 16: all operands live in
 // shared memory for the whole kernel, and two first-layer matrices share one tile (columns 0..15 and 16..31: [Wz | W1], or
@@ -83,7 +83,7 @@ __host__ __device__ constexpr uint32_t chain_tc_first_bytes(int D, int H, bool l
 __host__ __device__ constexpr uint32_t chain_tc_image_bytes(int D, int H, bool literal) {
     return chain_tc_first_bytes(D, H, literal) + 5u * chain_tc_row_bytes(D, H) + (literal ? static_cast<uint32_t>(D) * 128u : 0u);
 }
-inline size_t chain_tc_image_floats(int D, int H) { return 6 * static_cast<size_t>(D) + static_cast<size_t>(D) * H; }
+inline size_t chain_tc_tail_floats(int D, int H) { return 6 * static_cast<size_t>(D) + static_cast<size_t>(D) * H; }
 // What of them is in shared memory at a time: D = 16 all, D = 32 one first-layer tile, the guide's second layer or a smaller one, and Ws.
 __host__ __device__ constexpr uint32_t chain_tc_operand_bytes(int D, int H, bool literal) {
     return D == 16 ? chain_tc_image_bytes(D, H, literal) : static_cast<uint32_t>(H) * 128u + 3u * chain_tc_row_bytes(D, H) + (literal ? 4096u : 0u);
@@ -96,13 +96,15 @@ inline size_t chain_tc_smem_bytes(int D, int H, int W, bool literal) {
     return 1024 + chain_tc_operand_bytes(D, H, literal) + kChainLatentBytes + floats * 4;
 }
 
-// Which windows: those whose states the kernels could hold beside their operands when they kept both in shared memory.  Longer ones
-// (D=16, H=256: from 14 steps on) have always gone through the fp32 kernels, and what is computed in fp32 stays so.
+// The longest window, in steps: D = 16 13 at H = 256 (literal 9), 56 (51) at 192, 141 (134) at 128; D = 32 96 at H = 256, 14 at 512.  The line is
+// one of precision, not of room: longer windows have always been computed by the fp32 kernels (the RNN states of these, W H floats, used
+// to stand beside the operands), and what is computed in fp32 stays so.  This kernel itself would take longer ones (D = 16, H = 256, 13 steps:
+// 150 of 227 KB).
+inline int chain_tc_longest_window(int D, int H, bool literal) {
+    return D == 32 ? 42144 / H - 68 : literal ? 32080 / H - 116 : 32880 / H - 115;
+}
 inline bool chain_tc_window(int D, int H, int W, bool literal) {
-    const size_t states = static_cast<size_t>(W) * H;
-    const size_t tiles = D == 16 ? static_cast<size_t>(H) * 448 + (literal ? 2048 : 0) + 6 * 16384 : static_cast<size_t>(H) * 256 + 3 * 16384 + 4096;
-    const size_t floats = states + (D == 32 ? 4 * static_cast<size_t>(H) + 2336 : literal ? 4 * static_cast<size_t>(H) + 624 : 3 * static_cast<size_t>(H) + 336);
-    return 1024 + tiles + floats * 4 + 256 <= 227 * 1024;
+    return W <= chain_tc_longest_window(D, H, literal) && chain_tc_smem_bytes(D, H, W, literal) <= 227 * 1024;
 }
 
 // byte offset of the 16-byte chunk `chunk` of row `row` in a K-major tile with 128-byte swizzled rows
@@ -142,12 +144,6 @@ __device__ __forceinline__ float sigmoid_fast(float x) {
 __device__ __forceinline__ float4 ld_shared_v4(uint32_t addr) {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
     return v;
 }
 

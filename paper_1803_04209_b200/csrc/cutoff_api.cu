@@ -935,9 +935,11 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     // SM (H=64, lag 20: 4096 samples 28 us against 76; H=128, lag 2: 7000 samples 16.8 against 27), two up to 40 of those warps
     // (9000 samples 16.7 against 19.8 with one and 27; 16384: 24 against 29; 20000: 32 against 39, lag 20: 95 against 110; 36000: 42
     // against 41; D=16, H=128, lag 4: 4700 samples 23 against 27 with one and 39, 10000: 46 against 54; D=32 has no registers for
-    // two).  Where it is a tensor-core chain, whose time hardly depends on the samples, up to 16 samples per SM (D=16, H=128, lag 20:
-    // 2048 samples 43 us against 75; D=16, H=256, lag 4: 25 against 36, 4096 samples 41 against 35; D=32, H=128, lag 4: 29
-    // against 45, 4096 samples 50 against 45).
+    // two).  Where it is a tensor-core chain, whose time hardly depends on the samples, up to 16 samples per SM.  Both are equal at (D=16)
+    // H=128 2700 samples (lag 4: 23 us) or 3000 (lag 20: 60), H=192 2000 (lag 4: 25) or 2500 (lag 20: 66), H=256 1500 (lag 4: 27), (D=32)
+    // H=128 1700 (lag 4: 30) or 2000 (lag 20: 83): one line for all of them.  At its 2368 samples, this one against the tensor-core chain:
+    // D=16, lag 4 22 and 23 us at H=128, 27 and 25 at 192, 32 and 27 at 256, lag 20 51 and 60, 64 and 66; D=32, H=128 36 and 30, 91 and 83;
+    // in windows of one step 15 and 15, 17 and 15, 19 and 16, at D=32 21 and 17, H=256 30 and 19.
     const int64_t total = cfg->total_samples > 0 ? cfg->total_samples : c->S;       // the same for every shard of a decision, as its draws must be
     const int64_t few = 16 * static_cast<int64_t>(c->sm_count);
     const int64_t warps = total * c->D / 32;
@@ -966,7 +968,7 @@ int cutoff_create(cutoff_ctx** out, const cutoff_config* cfg) {
     }
     CREATE_CHECK(cudaMalloc(&c->d_WhR, sizeof(float) * 2 * c->H * c->H));
     if (c->chain_tc)
-        CREATE_CHECK(cudaMalloc(&c->d_chain_image, tc::chain_tc_image_bytes(c->D, c->H, c->literal) + tc::chain_tc_image_floats(c->D, c->H) * sizeof(float)));
+        CREATE_CHECK(cudaMalloc(&c->d_chain_image, tc::chain_tc_image_bytes(c->D, c->H, c->literal) + tc::chain_tc_tail_floats(c->D, c->H) * sizeof(float)));
     CREATE_CHECK(cudaMalloc(&c->d_ring, sizeof(float) * c->W * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_stage, sizeof(float) * c->N));
     CREATE_CHECK(cudaMalloc(&c->d_state, sizeof(DevState)));
@@ -1150,7 +1152,7 @@ int cutoff_load_weights(cutoff_ctx* c, const void* blob, size_t nbytes) {
         const float* wh2 = lit ? host.data() + off[21] : nullptr;
         const float* ws = lit ? host.data() + off[25] : nullptr; // [D][D]
         const size_t tile = H * 32, bytes = tc::chain_tc_image_bytes(c->D, c->H, lit);
-        std::vector<uint8_t> img(bytes + tc::chain_tc_image_floats(c->D, c->H) * sizeof(float), 0);
+        std::vector<uint8_t> img(bytes + tc::chain_tc_tail_floats(c->D, c->H) * sizeof(float), 0);
         float* const first = reinterpret_cast<float*>(img.data());
         if (D == 16) {                                           // two matrices share a tile (columns 0..15 and 16..31)
             put_first_layer(first, wz, H, D, 0);

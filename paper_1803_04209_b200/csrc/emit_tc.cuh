@@ -18,8 +18,8 @@
 // What bounds it, at N = 1024, S = 65536, H = 256 and at N = 4096, S = 32768, H = 512: as four-byte operands, the stream from
 // L2 to shared memory (0.148 and 0.432 ms); as halves, with the weights resident (H = 256) and the
 // MMAs issued at their rate, it takes 0.118 and 0.276 ms.  Now no
-// single resource: issue slots 57 %, shared-memory and store wavefronts 65 %, tensor pipe 28 % (N = 1024).  Shares, from an
-// earlier capture in which it took 0.113 and 0.290: streamed weights 0.122 and 0.297, the drawing alone, without operands and
+// single resource: shared-memory and store wavefronts 67 %, issue slots 47 %, special-function pipe 45 %, tensor pipe 29 % (N = 1024).  Shares,
+// of an earlier version that took 0.113 and 0.290: streamed weights 0.122 and 0.297, the drawing alone, without operands and
 // products, 0.104 and 0.200, without the stores 0.111 and 0.295, without the products 0.112 and 0.241.
 // 28 epilogue warps of 64 registers, with the generator's words in tables of the whole CTA, were slower (0.142 and 0.330 ms):
 // more instructions for the indexing than the occupancy gives.
@@ -76,10 +76,10 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr) {
     return d;
 }
 
-// True in one lane of the warp, always the same.  MMAs are issued from a branch on it: their operands are uniform registers, and only of
-// such a branch does the compiler know that one thread runs it; from a branch on a lane number each MMA takes 140 cycles to issue instead of 40,
-// more than the 128 that one of N = 256 occupies the tensor cores (emission at N = 4096, S = 32768, H = 512: 301 us so, 282 now; of the literal
-// networks at N = 1024, S = 65536: 165 and 152; N = 1024, H = 256: 121 and 119; the chain of D = 32, H = 512, S = 32768: 174 and 162).
+// True in one lane of the warp, always the same; takes all 32 lanes.  MMAs are issued from a branch on it: their operands are uniform
+// registers, and only of such a branch does the compiler know that one thread runs it; from a branch on a lane number every MMA takes longer to
+// issue (emission at N = 4096, S = 32768, H = 512: 301 us so, 282 with the election; of the literal networks at N = 1024, S = 65536: 165 and
+// 152; N = 1024, H = 256: 121 and 119; the chain of D = 32, H = 512, S = 32768: 174 and 162).
 __device__ __forceinline__ bool elect_one() {
     uint32_t yes;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(yes));

@@ -964,13 +964,14 @@ __global__ void k_transpose_heads(const float* __restrict__ W4, int N, int H, in
 // ---------------------------------------------------------------------------------------------
 // The same layer with the weights of a CTA's workers resident in shared memory: one persistent CTA per SM, 4 TX workers per CTA,
 // (32 / TX) RM samples at a time per warp, and no warp waits for another.  A thread has RM samples x 4 workers, both heads.
-// What bounds it is the issue of instructions: per k 4 RM paired multiply-adds (two columns each), RM / 2 loads of two hidden values and
-// two of weights.  A hidden value is stored twice in a row, so that a load brings the pair that an instruction multiplies two
+// Per k a thread issues 4 RM paired multiply-adds (two columns each), RM / 2 loads of two hidden values and two of weights.  What bounds it: the
+// reads of shared memory first (N=64, H=128, S=60000: wavefronts 69 % busy, issue slots 52 %, multiply-adds 49 %; N=16: 52, 44 and 40 %).  A
+// hidden value is stored twice in a row, so that a load brings the pair that an instruction multiplies two
 // columns with; made in registers, the pairs took as many moves as there are multiply-adds to four columns.  The warps of a
 // CTA lie evenly on the four schedulers, and CTAs of this size cannot crowd on the SMs that the chain leaves free: the CTAs of 64 threads of
 // the kernel below did both (N=16, S=1024: 128 of them on 19 SMs).  Emission stage before and after: N=16 S=60000 33.6 and 15.1 us,
-// N=30 S=30000 23.6 and 15.4, N=50 S=8000 23.6 and 15.1, N=16 S=1024 9.1 and 7.2.  With several worker tiles of 32 the reads of the
-// pairs cost more than it gains (four cycles of the shared-memory pipe for 16 bytes a lane): N=100 S=60000 79 and 87, N=250 S=1500 17 and 23.
+// N=30 S=30000 23.6 and 15.4, N=50 S=8000 23.6 and 15.1, N=16 S=1024 9.1 and 7.2;
+// N=64 S=60000, H=128 73.7 and 73.1.  With more worker tiles of 32 the reads of the pairs cost more than it gains (four cycles of the shared-memory pipe for 16 bytes a lane): N=100 S=60000 79 and 87, N=250 S=1500 17 and 23.
 // ---------------------------------------------------------------------------------------------
 constexpr int kEmitRowsWarps = 16, kEmitRowsTK = 16, kEmitRowsPitch = 2 * kEmitRowsTK + 4;
 
