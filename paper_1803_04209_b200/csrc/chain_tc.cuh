@@ -29,7 +29,7 @@
 //
 // What bounds it: each step's round trip, two products and the noise in between, which a second tile covers in part; no unit is busy.  Of
 // them the special-function pipe is the first (256 tanh per sample and step and about 60 logarithms, sines and the like for its
-// noise): S=65536, D=16, H=256, lag 4 67 us, special-function pipe 37 % busy, issue slots 44 %, shared-memory wavefronts 29 %, tensor pipe
+// noise): S=65536, D=16, H=256, lag 4 66 us, special-function pipe 37 % busy, issue slots 44 %, shared-memory wavefronts 29 %, tensor pipe
 // 11 %.  With the hidden layer through shared memory as tf32, 64 units at a time, four steps of handshakes each, it took 108.  With
 // one tile per SM, S=8192 41 -> 27 us (35 with tiles of 128).  D=32, with one tile per SM: S=32768, H=512, lag 4 162 -> 92 us,
 // S=8192, H=256 60 -> 35 us; its weights were copied by the epilogue's threads before.

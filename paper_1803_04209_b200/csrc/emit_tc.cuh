@@ -17,7 +17,7 @@
 //
 // What bounds it, at N = 1024, S = 65536, H = 256 and at N = 4096, S = 32768, H = 512: as four-byte operands, the stream from
 // L2 to shared memory (0.148 and 0.432 ms); as halves, with the weights resident (H = 256) and the
-// MMAs issued at their rate, it takes 0.118 and 0.276 ms.  Now no
+// MMAs issued at their rate, it takes 0.118 and 0.282 ms.  Now no
 // single resource: shared-memory and store wavefronts 67 %, issue slots 47 %, special-function pipe 45 %, tensor pipe 29 % (N = 1024).  Shares,
 // of an earlier version that took 0.113 and 0.290: streamed weights 0.122 and 0.297, the drawing alone, without operands and
 // products, 0.104 and 0.200, without the stores 0.111 and 0.295, without the products 0.112 and 0.241.
