@@ -533,11 +533,6 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
             mbar_wait_quiet(bar_img, n_first & 1u);
             mbar_wait_quiet(bar_second, n_second & 1u);
         }
-        if (!ok) {
-            if (elect_one()) umma_commit(bar_drain);
-            __syncwarp();
-            mbar_wait_quiet(bar_drain, 0u);
-        }
         __syncwarp();
     } else if (warp >= 2) {
         // ---------------- epilogue ---------------------------------------------------------------------
@@ -765,6 +760,14 @@ __global__ void __launch_bounds__(kChainTcThreads, 1) k_chain_tc(ChainTcArgs a) 
     }
     tc_fence_before();
     __syncthreads();
+    if (*abort_flag) {                                            // nobody has waited for the last products: let them end (bounded)
+        if (warp < kSlots) {
+            if (elect_one()) umma_commit(bar_drain);
+            __syncwarp();
+            mbar_wait_quiet(bar_drain, 0u);
+        }
+        __syncthreads();
+    }
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
